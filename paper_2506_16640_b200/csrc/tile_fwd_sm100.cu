@@ -959,8 +959,8 @@ cudaError_t launch_tile_impl(const Problem& p, const void* q, const void* k, con
   if (err != cudaSuccess) return err;
   err = make_tile_map(&map_v, v, p.D, p.N, p.H, p.B, p.sn, p.sh, p.sb);
   if (err != cudaSuccess) return err;
-  CUtensorMap map_ks = map_k;   // short sequences never take the sampled start
-  if (p.N >= kSampleMinTiles * TN) {
+  CUtensorMap map_ks = map_k;   // sequences whose longest Q tile sees too few K tiles never take the sampled start
+  if (args.tiles_per_head >= kSampleMinTiles) {
     err = make_sampled_tile_map(&map_ks, k, p.D, p.N, p.H, p.B, p.sn, p.sh, p.sb, kTileSampleStride);
     if (err != cudaSuccess) return err;
   }

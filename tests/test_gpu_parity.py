@@ -96,6 +96,18 @@ def test_dense_tiles_on_tensor_cores(N, d, causal, alpha):
     assert int(got["status"][binding.STATUS_DENSE_ROWS]) > N
 
 
+@pytest.mark.parametrize("N", [1920, 1921, 2047])
+def test_dense_tiles_sampled_start_at_a_partial_last_tile(N):
+    # the sampled start begins at the Q tile that sees 16 K tiles, the last of which may be a partial one: 1920 keys do
+    # not have it, 1921 do (the sampled view of K has to exist from there on, not from 16 whole tiles on)
+    inp = make_inputs(_small("dense_sampled_edge", N, 64, True, use_scale=True, sigma=0.03, seed=N))
+    got = parity.run_fwd(inp, 1.5)
+    assert int(got["status"][binding.STATUS_DENSE_ROWS]) > N // 2
+    rows = np.unique(np.concatenate([np.arange(0, N, 53), np.arange(max(0, N - 20), N)]))
+    for bh in range(inp.workload.H):
+        parity.check_fwd_rows(inp, 1.5, got, bh, rows)
+
+
 @pytest.mark.parametrize("sigma,expect", [(0.55, 200), (0.3, 1000), (0.18, 4000)])
 def test_dense_path_at_supports_of_hundreds_to_thousands(sigma, expect):
     # long rows whose supports run to about 200, 1000 and 4000 keys (fixed temperature, logits of std sigma^2): forward
