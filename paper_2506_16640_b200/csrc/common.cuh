@@ -49,7 +49,7 @@ struct Problem {
 };
 
 struct WsLayout {
-  size_t scale, row_cnt, half_cnt, half_thr, entries, fb_count, sweep_counter, tile_count, fb_list, tile_flag, tile_list, tile_mask, alibi_blob, alibi_kmax, scratch, acc_dk, acc_dv, dc_rows, total;
+  size_t scale, row_cnt, half_cnt, half_thr, entries, fb_count, sweep_counter, tile_count, grad_counter, tile_flag, tile_list, tile_mask, fb_list, alibi_blob, alibi_kmax, scratch, acc_dk, acc_dv, dc_rows, total;
   int scratch_ctas;     // CTAs of the dense-row kernels (each owns scratch_floats floats)
   size_t scratch_floats;
 };
@@ -186,8 +186,9 @@ __device__ __forceinline__ void atomic_add_slice(float* p, const float (&x)[PER]
 }
 
 // ---- launchers (each enqueues on `stream` and returns the cudaError_t of the launch) -------------
-cudaError_t launch_scale_table(const Problem& p, const float* beta, const float* gamma, const float* delta,
-                               float* scale, int32_t* status, cudaStream_t stream);
+// scale table c_i [H,N] (scale == nullptr: none) and n_clear words of zeros at `clear`, one launch
+cudaError_t launch_prologue(const Problem& p, const float* beta, const float* gamma, const float* delta, float* scale,
+                            int32_t* clear, size_t n_clear, int32_t* status, cudaStream_t stream);
 
 // dense-row path (CUDA cores): all rows (row_list == nullptr) or the rows in row_list[0 .. *row_count)
 cudaError_t launch_dense_fwd(const Problem& p, const void* q, const void* k, const void* v, const float* scale,
@@ -198,12 +199,14 @@ cudaError_t launch_dense_bwd(const Problem& p, const void* q, const void* k, con
                              const float* scale, const float* tau, void* dq, float* acc_dk, float* acc_dv,
                              float* dc_rows, const int32_t* row_list, const int32_t* row_count, float* scratch,
                              size_t scratch_floats, int ctas, cudaStream_t stream);
-// dbeta, dgamma, ddelta [H] from the per-row scale gradients dc_rows [B,H,N]
+// dbeta, dgamma, ddelta [H] from the per-row scale gradients dc_rows [B,H,N]; partial: 3 * H * ceil(N / 256) doubles of
+// scratch at most; *counter must be zero on entry
 cudaError_t launch_scale_grad(const Problem& p, const float* beta, const float* gamma, const float* dc_rows,
-                              float* dbeta, float* dgamma, float* ddelta, cudaStream_t stream);
+                              double* partial, int32_t* counter, float* dbeta, float* dgamma, float* ddelta,
+                              cudaStream_t stream);
 
 // tcgen05 score sweep (bf16): fills the per-row candidate lists.
-//   mode 0: threshold search (forward); mode 1: threshold given in tau_in (backward)
+//   mode 0: threshold search (forward); mode 1: threshold given in tau_in (backward); *work_counter must be zero on entry
 cudaError_t launch_sweep(const Problem& p, const void* q, const void* k, const float* scale, const float* tau_in,
                          int mode, int32_t* half_cnt, float* half_thr, Entry* entries, int32_t* work_counter,
                          float* dump, int dump_bh, float* alibi_blob, float* alibi_kmax, int32_t* status,

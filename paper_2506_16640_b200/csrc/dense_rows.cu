@@ -2,8 +2,8 @@
 //
 // Used for (1) float32 problems, where fp32 FMA dot products meet the tighter threshold tolerance that
 // bf16 tensor-core inputs cannot, and (2) the rows of a bf16 problem whose support does not fit the
-// sparse per-row list of the tensor-core sweep.  Also holds the ASEntmax scale-table kernel and the
-// gradient store kernel.
+// sparse per-row list of the tensor-core sweep.  Also holds the prologue kernel (ASEntmax scale
+// table, cleared counters), the scale gradient kernel and the gradient store kernel.
 //
 // Threshold solve: f(tau) = sum_j [y_j - tau]_+^e - 1 with y = (alpha-1) s and e = 1/(alpha-1) >= 1 is
 // convex and decreasing (Eq. 1 of the paper with the sum-to-one condition).  Newton steps started at
@@ -278,63 +278,97 @@ __global__ void __launch_bounds__(kThreads) dense_bwd_kernel(Problem p, const T*
 
 // dbeta_h, dgamma_h, ddelta_h from the per-row scale gradients: c_i = delta + beta L^gamma with L = ln n_i
 // (rows with n_i = 1 have c_i = delta), so d/ddelta = 1, d/dbeta = L^gamma, d/dgamma = beta L^gamma ln L.
-// One CTA per head, fp64 accumulation in a fixed order (reproducible).
-__global__ void __launch_bounds__(256) scale_grad_kernel(Problem p, const float* __restrict__ beta,
-                                                        const float* __restrict__ gamma,
-                                                        const float* __restrict__ dc_rows, float* __restrict__ dbeta,
-                                                        float* __restrict__ dgamma, float* __restrict__ ddelta) {
-  __shared__ double red[3][256];
-  const int h = blockIdx.x;
+// fp64 throughout.  What bounds it is the fp64 logarithms and exponentials (one L^gamma per head and position, after the
+// batch has been summed), so the positions of a head are spread over as many CTAs as it takes to reach every SM; each
+// leaves three partial sums, and the CTA that finishes last adds them in a fixed order (reproducible).  One CTA per head
+// and a pow per (batch, head, position) took 178 us at 16 heads x 32768 and 350 us at 8 x 65536; this takes 14 and 18 us.
+constexpr int kScaleGradThreads = 256;
+__device__ __forceinline__ double block_sum_fp64(double x, double* red) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = x;
+  __syncthreads();
+  double r = 0.0;
+#pragma unroll
+  for (int w = 0; w < kScaleGradThreads / 32; ++w) r += red[w];
+  return r;
+}
+__global__ void __launch_bounds__(kScaleGradThreads) scale_grad_kernel(Problem p, const float* __restrict__ beta,
+                                                                       const float* __restrict__ gamma,
+                                                                       const float* __restrict__ dc_rows,
+                                                                       double* __restrict__ partial, int32_t* counter,
+                                                                       float* __restrict__ dbeta,
+                                                                       float* __restrict__ dgamma,
+                                                                       float* __restrict__ ddelta) {
+  __shared__ double red[kScaleGradThreads / 32];
+  __shared__ int last;
+  const int h = blockIdx.y;
   const double b = beta[h], g = gamma[h];
   double sb = 0.0, sg = 0.0, sd = 0.0;
-  for (long t = threadIdx.x; t < (long)p.B * p.N; t += blockDim.x) {
-    const long bb = t / p.N;
-    const int i = (int)(t - bb * p.N);
-    const double dc = dc_rows[((size_t)bb * p.H + h) * p.N + i];
-    const long n = (p.n_mode || !p.causal) ? p.N : i + 1;
+  for (int i = blockIdx.x * kScaleGradThreads + threadIdx.x; i < p.N; i += gridDim.x * kScaleGradThreads) {
+    double dc = 0.0;
+    for (int bb = 0; bb < p.B; ++bb) dc += dc_rows[((size_t)bb * p.H + h) * p.N + i];
+    const int n = (p.n_mode || !p.causal) ? p.N : i + 1;
     sd += dc;
     if (n > 1) {
-      const double L = log((double)n);
-      const double Lg = pow(L, g);
-      sb += dc * Lg;
-      sg += dc * b * Lg * log(L);
+      const double lnL = log(log((double)n));
+      const double t = dc * exp(g * lnL);
+      sb += t;
+      sg += t * b * lnL;
     }
   }
-  red[0][threadIdx.x] = sb;
-  red[1][threadIdx.x] = sg;
-  red[2][threadIdx.x] = sd;
-  __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o) {
-      red[0][threadIdx.x] += red[0][threadIdx.x + o];
-      red[1][threadIdx.x] += red[1][threadIdx.x + o];
-      red[2][threadIdx.x] += red[2][threadIdx.x + o];
-    }
-    __syncthreads();
-  }
+  sb = block_sum_fp64(sb, red);
+  sg = block_sum_fp64(sg, red);
+  sd = block_sum_fp64(sd, red);
   if (threadIdx.x == 0) {
-    dbeta[h] = (float)red[0][0];
-    dgamma[h] = (float)red[1][0];
-    ddelta[h] = (float)red[2][0];
+    double* mine = partial + 3 * ((size_t)h * gridDim.x + blockIdx.x);
+    mine[0] = sb;
+    mine[1] = sg;
+    mine[2] = sd;
+    __threadfence();
+    last = atomicAdd(counter, 1) == (int)(gridDim.x * gridDim.y) - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  for (int t = threadIdx.x; t < 3 * p.H; t += kScaleGradThreads) {
+    const int hh = t / 3, which = t - 3 * hh;
+    double sum = 0.0;
+    for (unsigned c = 0; c < gridDim.x; ++c) sum += __ldcg(partial + 3 * ((size_t)hh * gridDim.x + c) + which);
+    (which == 0 ? dbeta : which == 1 ? dgamma : ddelta)[hh] = (float)sum;
   }
 }
 
-// c_i = delta_h + beta_h (ln n_i)^gamma_h in fp64, rounded once to fp32 (Eq. "asentmax").
-__global__ void scale_table_kernel(Problem p, const float* __restrict__ beta, const float* __restrict__ gamma,
-                                   const float* __restrict__ delta, float* __restrict__ scale,
-                                   int32_t* __restrict__ status) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= p.H * p.N) return;
-  float c = 1.0f;
-  if (p.has_scale) {
-    const int h = idx / p.N, i = idx - h * p.N;
-    const long n = (p.n_mode || !p.causal) ? p.N : i + 1;
-    double cd = (double)delta[h];
-    if (n > 1) cd += (double)beta[h] * pow(log((double)n), (double)gamma[h]);
-    c = (float)cd;
-    if (!isfinite(c) && status) atomicOr(status + ENTMAX_ATTN_STATUS_FLAGS, ENTMAX_ATTN_FLAG_BAD_SCALE);
+// c_i = delta_h + beta_h (ln n_i)^gamma_h in fp64, rounded once to fp32 (Eq. "asentmax").  A thread takes one position of
+// kScaleHeads heads: the two logarithms do not depend on the head, one exponential per head is left (a pow per entry took
+// 9.3 us at 16 heads x 32768, this 5.4 us).  The same launch clears the call's counters and flags (`clear`, n_clear words),
+// which used to be memsets of their own: about 2 us of stream time each.
+constexpr int kScaleHeads = 4;
+__global__ void __launch_bounds__(256) prologue_kernel(Problem p, const float* __restrict__ beta,
+                                                       const float* __restrict__ gamma, const float* __restrict__ delta,
+                                                       float* __restrict__ scale, int32_t* __restrict__ clear, int n_clear,
+                                                       int32_t* __restrict__ status) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (blockIdx.y == 0)
+    for (int t = i; t < n_clear; t += gridDim.x * blockDim.x) clear[t] = 0;
+  if (!scale || i >= p.N) return;
+  const int h0 = blockIdx.y * kScaleHeads;
+  const int n = (p.n_mode || !p.causal) ? p.N : i + 1;
+  const double lnL = p.has_scale && n > 1 ? log(log((double)n)) : 0.0;
+#pragma unroll
+  for (int t = 0; t < kScaleHeads; ++t) {
+    const int h = h0 + t;
+    if (h >= p.H) break;
+    float c = 1.0f;
+    if (p.has_scale) {
+      double cd = (double)delta[h];
+      if (n > 1) cd += (double)beta[h] * exp((double)gamma[h] * lnL);
+      c = (float)cd;
+      if (!isfinite(c) && status) atomicOr(status + ENTMAX_ATTN_STATUS_FLAGS, ENTMAX_ATTN_FLAG_BAD_SCALE);
+    }
+    scale[(size_t)h * p.N + i] = c;
   }
-  scale[idx] = c;
 }
 
 template <typename T>
@@ -356,10 +390,11 @@ __global__ void store_grad_kernel(Problem p, const float* __restrict__ acc, T* _
 
 }  // namespace
 
-cudaError_t launch_scale_table(const Problem& p, const float* beta, const float* gamma, const float* delta,
-                               float* scale, int32_t* status, cudaStream_t stream) {
-  const int total = p.H * p.N;
-  scale_table_kernel<<<(total + 255) / 256, 256, 0, stream>>>(p, beta, gamma, delta, scale, status);
+cudaError_t launch_prologue(const Problem& p, const float* beta, const float* gamma, const float* delta, float* scale,
+                            int32_t* clear, size_t n_clear, int32_t* status, cudaStream_t stream) {
+  const int most = scale ? p.N : (int)(n_clear < 256 * 148 ? n_clear : 256 * 148);
+  const dim3 grid((most + 255) / 256, scale ? (p.H + kScaleHeads - 1) / kScaleHeads : 1);
+  prologue_kernel<<<grid, 256, 0, stream>>>(p, beta, gamma, delta, scale, clear, (int)n_clear, status);
   return cudaGetLastError();
 }
 
@@ -399,8 +434,14 @@ cudaError_t launch_dense_bwd(const Problem& p, const void* q, const void* k, con
 }
 
 cudaError_t launch_scale_grad(const Problem& p, const float* beta, const float* gamma, const float* dc_rows,
-                              float* dbeta, float* dgamma, float* ddelta, cudaStream_t stream) {
-  scale_grad_kernel<<<p.H, 256, 0, stream>>>(p, beta, gamma, dc_rows, dbeta, dgamma, ddelta);
+                              double* partial, int32_t* counter, float* dbeta, float* dgamma, float* ddelta,
+                              cudaStream_t stream) {
+  // CTAs per head: enough for four per SM over all heads, none without a position of its own
+  int ctas = (148 * 4 + p.H - 1) / p.H;
+  const int most = (p.N + kScaleGradThreads - 1) / kScaleGradThreads;
+  if (ctas > most) ctas = most;
+  scale_grad_kernel<<<dim3(ctas, p.H), kScaleGradThreads, 0, stream>>>(p, beta, gamma, dc_rows, partial, counter, dbeta,
+                                                                       dgamma, ddelta);
   return cudaGetLastError();
 }
 

@@ -136,11 +136,13 @@ WsLayout make_layout(const Problem& p, bool is_bwd) {
   l.fb_count = take(256);
   l.sweep_counter = l.fb_count + 64;   // same 256-byte block: [0] dense-row count, [16] sweep work counter,
   l.tile_count = l.fb_count + 128;     // [32] number of listed dense tiles, [48] the dense-tile kernels' work counter
-  l.fb_list = take(rows * sizeof(int32_t));
+  l.grad_counter = l.fb_count + 32;    // [8] CTAs of the scale gradient that have finished
+  // tile flags, list and masks right behind the counters: what a call has to clear is one range
   const size_t q_tiles = (size_t)p.B * p.H * ((p.N + 127) / 128);
   l.tile_flag = take(q_tiles * sizeof(int32_t));
   l.tile_list = take(q_tiles * sizeof(int32_t));
   l.tile_mask = take(q_tiles * 4 * sizeof(uint32_t));   // 128 row bits per Q tile (dense-tile backward)
+  l.fb_list = take(rows * sizeof(int32_t));
   // ALiBi window of the score sweep: slopes [H] + first K tile of every 256-row work item; key norms per 256-key tile
   const size_t items = (size_t)p.B * p.H * ((p.N + 255) / 256);
   l.alibi_blob = take(((size_t)p.H + items) * sizeof(float));
@@ -232,14 +234,19 @@ int fwd_impl(const entmax_attn_params* params, const void* q, const void* k, con
     err = cudaMemsetAsync(device_status, 0, sizeof(int32_t) * ENTMAX_ATTN_STATUS_WORDS, stream);
     if (err != cudaSuccess) return fail_cuda(err);
   }
+  const bool bf16 = p.dtype == ENTMAX_ATTN_DTYPE_BF16;
+  const size_t q_tiles = (size_t)p.B * p.H * ((p.N + 127) / 128);
   if (c_rows) {
     scale = c_rows;
     p.scale_sb = (int64_t)p.H * p.N;
-  } else {
-    err = launch_scale_table(p, beta, gamma, delta, reinterpret_cast<float*>(ws + lay.scale), device_status, stream);
+  }
+  if (bf16 || !c_rows) {
+    // the scale table, and (bf16) the counters and tile flags of this call cleared
+    err = launch_prologue(p, beta, gamma, delta, c_rows ? nullptr : reinterpret_cast<float*>(ws + lay.scale), fb_count,
+                          bf16 ? (lay.tile_flag - lay.fb_count) / 4 + q_tiles : 0, device_status, stream);
     if (err != cudaSuccess) return fail_cuda(err);
   }
-  if (p.dtype == ENTMAX_ATTN_DTYPE_FP32) {
+  if (!bf16) {
     err = launch_dense_fwd(p, q, k, v, scale, o, tau, row_cnt, half_cnt, entries, nullptr, nullptr, scratch, lay.scratch_floats,
                            lay.scratch_ctas, stream);
     return err == cudaSuccess ? ENTMAX_ATTN_OK : fail_cuda(err);
@@ -247,10 +254,6 @@ int fwd_impl(const entmax_attn_params* params, const void* q, const void* k, con
   int32_t* tile_flag = reinterpret_cast<int32_t*>(ws + lay.tile_flag);
   int32_t* tile_list = reinterpret_cast<int32_t*>(ws + lay.tile_list);
   int32_t* tile_count = reinterpret_cast<int32_t*>(ws + lay.tile_count);
-  err = cudaMemsetAsync(fb_count, 0, 256, stream);   // the whole counter block
-  if (err != cudaSuccess) return fail_cuda(err);
-  err = cudaMemsetAsync(tile_flag, 0, (size_t)p.B * p.H * ((p.N + 127) / 128) * sizeof(int32_t), stream);
-  if (err != cudaSuccess) return fail_cuda(err);
   if (g_prof_start[0]) cudaEventRecord(g_prof_start[0], stream);
   err = launch_sweep(p, q, k, scale, nullptr, 0, half_cnt, half_thr, entries, sweep_counter, nullptr, -1,
                      reinterpret_cast<float*>(ws + lay.alibi_blob), reinterpret_cast<float*>(ws + lay.alibi_kmax),
@@ -366,14 +369,17 @@ int bwd_impl(const entmax_attn_params* params, const void* q, const void* k, con
     err = cudaMemsetAsync(acc_dv, 0, acc_bytes, stream);
     if (err != cudaSuccess) return fail_cuda(err);
   }
+  const bool bf16 = p.dtype == ENTMAX_ATTN_DTYPE_BF16;
+  const size_t q_tiles = (size_t)p.B * p.H * ((p.N + 127) / 128);
   if (c_rows) {
     scale = c_rows;
     p.scale_sb = (int64_t)p.H * p.N;
-  } else {
-    err = launch_scale_table(p, beta, gamma, delta, reinterpret_cast<float*>(ws + lay.scale), device_status, stream);
-    if (err != cudaSuccess) return fail_cuda(err);
   }
-  if (p.dtype == ENTMAX_ATTN_DTYPE_FP32) {
+  // the scale table, and the counters (bf16: with the tile flags, list and masks behind them) of this call cleared
+  err = launch_prologue(p, beta, gamma, delta, c_rows ? nullptr : reinterpret_cast<float*>(ws + lay.scale), fb_count,
+                        bf16 ? (lay.tile_mask - lay.fb_count) / 4 + 4 * q_tiles : 64, device_status, stream);
+  if (err != cudaSuccess) return fail_cuda(err);
+  if (!bf16) {
     err = launch_dense_bwd(p, q, k, v, d_o, scale, tau, dq, acc_dk, acc_dv, dc_rows, nullptr, nullptr, scratch,
                            lay.scratch_floats, lay.scratch_ctas, stream);
     if (err != cudaSuccess) return fail_cuda(err);
@@ -382,12 +388,6 @@ int bwd_impl(const entmax_attn_params* params, const void* q, const void* k, con
     int32_t* tile_list = reinterpret_cast<int32_t*>(ws + lay.tile_list);
     int32_t* tile_count = reinterpret_cast<int32_t*>(ws + lay.tile_count);
     uint32_t* tile_mask = reinterpret_cast<uint32_t*>(ws + lay.tile_mask);
-    const size_t q_tiles = (size_t)p.B * p.H * ((p.N + 127) / 128);
-    err = cudaMemsetAsync(fb_count, 0, 256, stream);   // the whole counter block
-    if (err != cudaSuccess) return fail_cuda(err);
-    // tile flags, tile list and tile masks are adjacent in the workspace: one memset clears all three
-    err = cudaMemsetAsync(tile_flag, 0, lay.tile_mask + q_tiles * 4 * sizeof(uint32_t) - lay.tile_flag, stream);
-    if (err != cudaSuccess) return fail_cuda(err);
     if (saved_supports) {
       // the compact copy of the forward call's supports: no score sweep; rows it does not hold count as dense
       const SavedLayout sl = saved_layout(p);
@@ -428,7 +428,9 @@ int bwd_impl(const entmax_attn_params* params, const void* q, const void* k, con
   err = launch_store_grad(p, acc_dv, dv, stream);
   if (err != cudaSuccess) return fail_cuda(err);
   if (n_param_grads) {
-    err = launch_scale_grad(p, beta, gamma, dc_rows, dbeta, dgamma, ddelta, stream);
+    // (the partial sums go where the list entries were: 2 KB per row, no longer needed)
+    err = launch_scale_grad(p, beta, gamma, dc_rows, reinterpret_cast<double*>(entries),
+                            reinterpret_cast<int32_t*>(ws + lay.grad_counter), dbeta, dgamma, ddelta, stream);
     if (err != cudaSuccess) return fail_cuda(err);
   }
   return ENTMAX_ATTN_OK;
@@ -502,7 +504,8 @@ int entmax_attn_scores_debug(const entmax_attn_params* params, const void* q, co
     err = cudaMemsetAsync(device_status, 0, sizeof(int32_t) * ENTMAX_ATTN_STATUS_WORDS, stream);
     if (err != cudaSuccess) return fail_cuda(err);
   }
-  err = launch_scale_table(p, nullptr, nullptr, nullptr, scale, device_status, stream);
+  err = launch_prologue(p, nullptr, nullptr, nullptr, scale, reinterpret_cast<int32_t*>(ws + lay.fb_count), 64, device_status,
+                        stream);
   if (err != cudaSuccess) return fail_cuda(err);
   err = launch_sweep(p, q, k, scale, nullptr, 0, reinterpret_cast<int32_t*>(ws + lay.half_cnt),
                      reinterpret_cast<float*>(ws + lay.half_thr), reinterpret_cast<Entry*>(ws + lay.entries),

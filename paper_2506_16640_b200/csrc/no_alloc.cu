@@ -89,7 +89,7 @@ extern "C" int entmax_attn_fwd_static(const entmax_attn_params* params, const vo
   // and every CTA fills its score row for the keys of a query before it reads them.
   float* scale = scratch;
   float* score_rows = scratch + scale_floats;
-  err = launch_scale_table(p, beta, gamma, delta, scale, device_status, stream);
+  err = launch_prologue(p, beta, gamma, delta, scale, nullptr, 0, device_status, stream);
   if (err != cudaSuccess) return fail_cuda(err);
   err = launch_dense_fwd(p, q, k, v, scale, o, tau, nullptr, nullptr, nullptr, nullptr, nullptr, score_rows, row_floats,
                          (int)ctas, stream);

@@ -80,7 +80,7 @@ struct SweepArgs {
                         // argument block, and with it the register allocation of the plain kernel, unchanged
   int dump_bh;
   int32_t* status;
-  int32_t* work_counter;  // zeroed before the launch
+  int32_t* work_counter;  // zero on entry
   int items_per_bh;     // ceil(N / kItemRows)
   int n_items;
 };
@@ -925,8 +925,6 @@ cudaError_t launch_impl(const Problem& p, const void* q, const void* k, SweepArg
   err = cudaGetDevice(&dev);
   if (err != cudaSuccess) return err;
   err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (err != cudaSuccess) return err;
-  err = cudaMemsetAsync(args.work_counter, 0, sizeof(int32_t), stream);
   if (err != cudaSuccess) return err;
   const int grid = args.n_items < sms ? args.n_items : sms;
   sweep_kernel<HD, kDump, kAlibi><<<grid, kThreads, Cfg<HD>::kSmemBytes, stream>>>(map_q, map_k, map_ks, args);
