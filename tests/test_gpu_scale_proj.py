@@ -52,6 +52,14 @@ def test_projection_forward_and_backward_match_the_oracle(B, H, N, dm, causal, n
     assert np.abs(dx.cpu().double().numpy() - rdx).max() <= dx_tol
 
 
+# widths that take the scalar loads (not a multiple of four) and the vector ones past one pass of the CTA's columns, head
+# counts on and off the rounds of four, token counts around the chunk of 32
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("B,H,N,dm", [(1, 7, 33, 37), (1, 4, 32, 514), (2, 9, 31, 516), (1, 64, 5, 130)])
+def test_projection_at_the_edges_of_its_tiles(B, H, N, dm, dtype):
+    test_projection_forward_and_backward_match_the_oracle(B, H, N, dm, True, 0, dtype)
+
+
 def test_projection_chained_with_the_per_query_attention_calls():
     # x -> c (projection) -> attention with a per-query scale table -> dL/dc -> dL/dw_beta, dL/dw_gamma, dL/ddelta, dL/dx;
     # the oracle walks the same chain in fp64
