@@ -50,8 +50,7 @@ struct Problem {
 
 struct WsLayout {
   size_t scale, row_cnt, half_cnt, half_thr, entries, fb_count, sweep_counter, tile_count, grad_counter, tile_flag, tile_list, tile_mask, fb_list, alibi_blob, alibi_kmax, scratch, acc_dk, acc_dv, dc_rows, total;
-  int scratch_ctas;     // CTAs of the dense-row kernels (each owns scratch_floats floats)
-  size_t scratch_floats;
+  int scratch_ctas;     // CTAs of the float32 kernels (each owns sixteen score rows of the scratch)
 };
 
 WsLayout make_layout(const Problem& p, bool is_bwd);
@@ -190,15 +189,19 @@ __device__ __forceinline__ void atomic_add_slice(float* p, const float (&x)[PER]
 cudaError_t launch_prologue(const Problem& p, const float* beta, const float* gamma, const float* delta, float* scale,
                             int32_t* clear, size_t n_clear, int32_t* status, cudaStream_t stream);
 
-// dense-row path (CUDA cores): all rows (row_list == nullptr) or the rows in row_list[0 .. *row_count)
-cudaError_t launch_dense_fwd(const Problem& p, const void* q, const void* k, const void* v, const float* scale,
-                             void* o, float* tau, int32_t* row_cnt, int32_t* dense_cnt, Entry* entries, const int32_t* row_list,
-                             const int32_t* row_count, float* scratch, size_t scratch_floats, int ctas,
-                             cudaStream_t stream);
-cudaError_t launch_dense_bwd(const Problem& p, const void* q, const void* k, const void* v, const void* d_o,
-                             const float* scale, const float* tau, void* dq, float* acc_dk, float* acc_dv,
-                             float* dc_rows, const int32_t* row_list, const int32_t* row_count, float* scratch,
-                             size_t scratch_floats, int ctas, cudaStream_t stream);
+// dense-row forward on CUDA cores, one score row of scratch per CTA
+cudaError_t launch_dense_fwd(const Problem& p, const void* q, const void* k, const void* v, const float* scale, void* o,
+                             float* tau, float* scratch, size_t scratch_floats, int ctas, cudaStream_t stream);
+// float32 problems; scratch: fp32_scratch_ctas() CTAs of sixteen score rows of fp32_scratch_pitch() floats each.
+// acc_dk, acc_dv: fp32 [B,H,N,D] contiguous, zero on entry
+int fp32_scratch_pitch(const Problem& p);
+int fp32_scratch_ctas(const Problem& p);
+cudaError_t launch_fp32_fwd(const Problem& p, const float* q, const float* k, const float* v, const float* scale, float* o,
+                            float* tau, int32_t* row_cnt, int32_t* dense_cnt, Entry* entries, float* scratch, int ctas,
+                            cudaStream_t stream);
+cudaError_t launch_fp32_bwd(const Problem& p, const float* q, const float* k, const float* v, const float* d_o,
+                            const float* scale, const float* tau, float* dq, float* acc_dk, float* acc_dv, float* dc_rows,
+                            float* scratch, int ctas, cudaStream_t stream);
 // dbeta, dgamma, ddelta [H] from the per-row scale gradients dc_rows [B,H,N]; partial: 3 * H * ceil(N / 256) doubles of
 // scratch at most; *counter must be zero on entry
 cudaError_t launch_scale_grad(const Problem& p, const float* beta, const float* gamma, const float* dc_rows,

@@ -1,8 +1,5 @@
-// Dense-row path on CUDA cores: one CTA per query row, every visible key visited.
-//
-// Used for (1) float32 problems, where fp32 FMA dot products meet the tighter threshold tolerance that
-// bf16 tensor-core inputs cannot, and (2) the rows of a bf16 problem whose support does not fit the
-// sparse per-row list of the tensor-core sweep.  Also holds the prologue kernel (ASEntmax scale
+// Dense-row forward on CUDA cores: one CTA per query row, every visible key visited, with a scratch of one score row per CTA.
+// It is what entmax_attn_fwd_static runs (its fixed scratch holds no more).  Also holds the prologue kernel (ASEntmax scale
 // table, cleared counters), the scale gradient kernel and the gradient store kernel.
 //
 // Threshold solve: f(tau) = sum_j [y_j - tau]_+^e - 1 with y = (alpha-1) s and e = 1/(alpha-1) >= 1 is
@@ -124,32 +121,24 @@ template <typename T, int D>
 __global__ void __launch_bounds__(kThreads) dense_fwd_kernel(Problem p, const T* __restrict__ q, const T* __restrict__ k,
                                                              const T* __restrict__ v, const float* __restrict__ scale,
                                                              T* __restrict__ o, float* __restrict__ tau_out,
-                                                             int32_t* __restrict__ row_cnt, int32_t* __restrict__ dense_cnt,
-                                                             Entry* __restrict__ entries,
-                                                             const int32_t* __restrict__ row_list,
-                                                             const int32_t* __restrict__ row_count,
-                                                             float* __restrict__ scratch, size_t scratch_floats) {
+                                                             float* scratch, size_t scratch_floats) {
   constexpr int PER = D / 32;
   __shared__ float red[2 * kWarps];
   __shared__ float opart[kWarps][D];
-  __shared__ int supp_count;
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  const int total = row_list ? *row_count : p.B * p.H * p.N;
+  const int total = p.B * p.H * p.N;
   float* ybuf = scratch + (size_t)blockIdx.x * scratch_floats;
   for (int ridx = blockIdx.x; ridx < total; ridx += gridDim.x) {
-    const RowCtx r = make_row(p, scale, row_list ? row_list[ridx] : ridx);
+    const RowCtx r = make_row(p, scale, ridx);
     float qs[PER];
     load_slice<PER>(q + r.base + (size_t)r.i * p.sn + l * PER, qs);
-    if (threadIdx.x == 0) supp_count = 0;
     const float ymax = score_pass<T, D>(p, r, k, qs, ybuf, red);
     const float tau = newton_tau(p, ybuf, r.nv, ymax, red);
     float acc[PER];
 #pragma unroll
     for (int t = 0; t < PER; ++t) acc[t] = 0.f;
-    Entry* list = entries ? entries + (size_t)r.grow * kListCap : nullptr;
     for (int j = w; j < r.nv; j += kWarps) {
-      const float yj = ybuf[j];
-      const float y = yj - tau;
+      const float y = ybuf[j] - tau;
       if (y > 0.f) {
         float pe, pe1;
         pow_pair(y, p.expo_class, p.expo, pe, pe1);
@@ -157,10 +146,6 @@ __global__ void __launch_bounds__(kThreads) dense_fwd_kernel(Problem p, const T*
         load_slice<PER>(v + r.base + (size_t)j * p.sn + l * PER, vs);
 #pragma unroll
         for (int t = 0; t < PER; ++t) acc[t] = fmaf(pe, vs[t], acc[t]);
-        if (l == 0) {
-          int slot = atomicAdd(&supp_count, 1);
-          if (list && slot < kListCap) { list[slot].y = yj; list[slot].j = j; }
-        }
       }
     }
 #pragma unroll
@@ -177,101 +162,7 @@ __global__ void __launch_bounds__(kThreads) dense_fwd_kernel(Problem p, const T*
       }
       store_slice<PER>(o + r.base + (size_t)r.i * p.sn + threadIdx.x * PER, out);
     }
-    if (threadIdx.x == 0) {
-      tau_out[r.grow] = tau;
-      if (row_cnt) row_cnt[r.grow] = supp_count <= kListCap ? supp_count : -2;
-      // a support too long for the list: its size alone is kept (same place and form as the dense-tile kernel's)
-      if (dense_cnt && supp_count > kListCap) { dense_cnt[2 * (size_t)r.grow] = supp_count; dense_cnt[2 * (size_t)r.grow + 1] = 0; }
-    }
-    __syncthreads();
-  }
-}
-
-template <typename T, int D>
-__global__ void __launch_bounds__(kThreads) dense_bwd_kernel(Problem p, const T* __restrict__ q, const T* __restrict__ k,
-                                                             const T* __restrict__ v, const T* __restrict__ d_o,
-                                                             const float* __restrict__ scale, const float* __restrict__ tau_in,
-                                                             T* __restrict__ dq, float* __restrict__ acc_dk,
-                                                             float* __restrict__ acc_dv, float* __restrict__ dc_rows,
-                                                             const int32_t* __restrict__ row_list,
-                                                             const int32_t* __restrict__ row_count,
-                                                             float* __restrict__ scratch, size_t scratch_floats) {
-  constexpr int PER = D / 32;
-  __shared__ float red[2 * kWarps];
-  __shared__ float qpart[kWarps][D];
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  const int total = row_list ? *row_count : p.B * p.H * p.N;
-  float* ybuf = scratch + (size_t)blockIdx.x * scratch_floats;
-  float* dpbuf = ybuf + scratch_floats / 2;
-  for (int ridx = blockIdx.x; ridx < total; ridx += gridDim.x) {
-    const RowCtx r = make_row(p, scale, row_list ? row_list[ridx] : ridx);
-    float qs[PER], gs[PER];
-    load_slice<PER>(q + r.base + (size_t)r.i * p.sn + l * PER, qs);
-    load_slice<PER>(d_o + r.base + (size_t)r.i * p.sn + l * PER, gs);
-    (void)score_pass<T, D>(p, r, k, qs, ybuf, red);
-    const float tau = tau_in[r.grow];
-    // sum_j u_ij and sum_j u_ij dP_ij over the support
-    float su = 0.f, sud = 0.f;
-    for (int j = w; j < r.nv; j += kWarps) {
-      const float y = ybuf[j] - tau;
-      if (y > 0.f) {
-        float vs[PER];
-        load_slice<PER>(v + r.base + (size_t)j * p.sn + l * PER, vs);
-        float dp = 0.f;
-#pragma unroll
-        for (int t = 0; t < PER; ++t) dp = fmaf(gs[t], vs[t], dp);
-        dp = warp_sum(dp);
-        float pe, u;
-        pow_pair(y, p.expo_class, p.expo, pe, u);
-        if (l == 0) { dpbuf[j] = dp; su += u; sud += u * dp; }
-      }
-    }
-    const float2 s = block_sum2(su, sud, red);
-    const float rho = s.x > 0.f ? s.y / s.x : 0.f;
-    float dcp = 0.f;                                  // sum_j dS_ij y_ij (lane 0 of every warp)
-    float acc[PER];
-#pragma unroll
-    for (int t = 0; t < PER; ++t) acc[t] = 0.f;
-    const size_t arow = (size_t)r.bh * p.N;
-    for (int j = w; j < r.nv; j += kWarps) {
-      const float y = ybuf[j] - tau;
-      if (y > 0.f) {
-        float pe, u;
-        pow_pair(y, p.expo_class, p.expo, pe, u);
-        const float gds = r.g * u * (dpbuf[j] - rho);
-        if (l == 0) dcp = fmaf(u * (dpbuf[j] - rho), ybuf[j], dcp);
-        float ks[PER], dkv[PER], dvv[PER];
-        load_slice<PER>(k + r.base + (size_t)j * p.sn + l * PER, ks);
-#pragma unroll
-        for (int t = 0; t < PER; ++t) {
-          acc[t] = fmaf(gds, ks[t], acc[t]);
-          dkv[t] = gds * qs[t];
-          dvv[t] = pe * gs[t];
-        }
-        atomic_add_slice<PER>(acc_dk + (arow + j) * D + l * PER, dkv);
-        atomic_add_slice<PER>(acc_dv + (arow + j) * D + l * PER, dvv);
-      }
-    }
-#pragma unroll
-    for (int t = 0; t < PER; ++t) qpart[w][l * PER + t] = acc[t];
-    __syncthreads();
-    if (threadIdx.x < D / PER) {
-      float out[PER];
-#pragma unroll
-      for (int t = 0; t < PER; ++t) {
-        float sacc = 0.f;
-#pragma unroll
-        for (int ww = 0; ww < kWarps; ++ww) sacc += qpart[ww][threadIdx.x * PER + t];
-        out[t] = sacc;
-      }
-      store_slice<PER>(dq + r.base + (size_t)r.i * p.sn + threadIdx.x * PER, out);
-    }
-    if (dc_rows) {
-      // dL/dc_i = sum_j dS_ij z_ij, z_ij = y_ij / ((alpha-1) c_i)  (y = (alpha-1) c z)
-      const float2 t = block_sum2(dcp, 0.f, red);
-      const float denom = (p.alpha - 1.0f) * r.c;
-      if (threadIdx.x == 0) dc_rows[r.grow] = denom != 0.f ? t.x / denom : 0.f;
-    }
+    if (threadIdx.x == 0) tau_out[r.grow] = tau;
     __syncthreads();
   }
 }
@@ -398,32 +289,11 @@ cudaError_t launch_prologue(const Problem& p, const float* beta, const float* ga
   return cudaGetLastError();
 }
 
-cudaError_t launch_dense_fwd(const Problem& p, const void* q, const void* k, const void* v, const float* scale,
-                             void* o, float* tau, int32_t* row_cnt, int32_t* dense_cnt, Entry* entries,
-                             const int32_t* row_list, const int32_t* row_count, float* scratch, size_t scratch_floats,
-                             int ctas, cudaStream_t stream) {
-#define ENTMAX_LAUNCH(T, D)                                                                                        \
-  dense_fwd_kernel<T, D><<<ctas, kThreads, 0, stream>>>(p, (const T*)q, (const T*)k, (const T*)v, scale, (T*)o, \
-                                                        tau, row_cnt, dense_cnt, entries, row_list, row_count, scratch, \
-                                                        scratch_floats)
-  if (p.dtype == ENTMAX_ATTN_DTYPE_FP32) {
-    if (p.D == 64) ENTMAX_LAUNCH(float, 64); else ENTMAX_LAUNCH(float, 128);
-  } else {
-    if (p.D == 64) ENTMAX_LAUNCH(__nv_bfloat16, 64); else ENTMAX_LAUNCH(__nv_bfloat16, 128);
-  }
-#undef ENTMAX_LAUNCH
-  return cudaGetLastError();
-}
-
-cudaError_t launch_dense_bwd(const Problem& p, const void* q, const void* k, const void* v, const void* d_o,
-                             const float* scale, const float* tau, void* dq, float* acc_dk, float* acc_dv,
-                             float* dc_rows, const int32_t* row_list, const int32_t* row_count, float* scratch,
-                             size_t scratch_floats, int ctas, cudaStream_t stream) {
+cudaError_t launch_dense_fwd(const Problem& p, const void* q, const void* k, const void* v, const float* scale, void* o,
+                             float* tau, float* scratch, size_t scratch_floats, int ctas, cudaStream_t stream) {
 #define ENTMAX_LAUNCH(T, D)                                                                                      \
-  dense_bwd_kernel<T, D><<<ctas, kThreads, 0, stream>>>(p, (const T*)q, (const T*)k, (const T*)v, (const T*)d_o, \
-                                                        scale, tau, (T*)dq, acc_dk, acc_dv, dc_rows, row_list,    \
-                                                        row_count,                                                 \
-                                                        scratch, scratch_floats)
+  dense_fwd_kernel<T, D><<<ctas, kThreads, 0, stream>>>(p, (const T*)q, (const T*)k, (const T*)v, scale, (T*)o, \
+                                                        tau, scratch, scratch_floats)
   if (p.dtype == ENTMAX_ATTN_DTYPE_FP32) {
     if (p.D == 64) ENTMAX_LAUNCH(float, 64); else ENTMAX_LAUNCH(float, 128);
   } else {

@@ -147,12 +147,13 @@ WsLayout make_layout(const Problem& p, bool is_bwd) {
   const size_t items = (size_t)p.B * p.H * ((p.N + 255) / 256);
   l.alibi_blob = take(((size_t)p.H + items) * sizeof(float));
   l.alibi_kmax = take(items * sizeof(float));
-  // dense-row CTAs: enough to fill the machine, few enough that their score rows stay modest
-  l.scratch_floats = align_up((size_t)p.N, 32) * (is_bwd ? 2 : 1);   // scores (+ dP in backward)
-  size_t ctas = 148 * 4;
-  if (ctas > rows) ctas = rows;
-  l.scratch_ctas = (int)ctas;
-  l.scratch = take(ctas * l.scratch_floats * sizeof(float));
+  // score rows of the float32 kernels
+  l.scratch_ctas = 0;
+  l.scratch = off;
+  if (p.dtype == ENTMAX_ATTN_DTYPE_FP32) {
+    l.scratch_ctas = fp32_scratch_ctas(p);
+    l.scratch = take((size_t)l.scratch_ctas * 16 * fp32_scratch_pitch(p) * sizeof(float));
+  }
   l.acc_dk = l.acc_dv = l.dc_rows = 0;
   if (is_bwd) {
     l.acc_dk = take(rows * p.D * sizeof(float));
@@ -247,8 +248,8 @@ int fwd_impl(const entmax_attn_params* params, const void* q, const void* k, con
     if (err != cudaSuccess) return fail_cuda(err);
   }
   if (!bf16) {
-    err = launch_dense_fwd(p, q, k, v, scale, o, tau, row_cnt, half_cnt, entries, nullptr, nullptr, scratch, lay.scratch_floats,
-                           lay.scratch_ctas, stream);
+    err = launch_fp32_fwd(p, static_cast<const float*>(q), static_cast<const float*>(k), static_cast<const float*>(v), scale,
+                          static_cast<float*>(o), tau, row_cnt, half_cnt, entries, scratch, lay.scratch_ctas, stream);
     return err == cudaSuccess ? ENTMAX_ATTN_OK : fail_cuda(err);
   }
   int32_t* tile_flag = reinterpret_cast<int32_t*>(ws + lay.tile_flag);
@@ -340,8 +341,11 @@ int bwd_impl(const entmax_attn_params* params, const void* q, const void* k, con
   int32_t* fb_count = reinterpret_cast<int32_t*>(ws + lay.fb_count);
   int32_t* fb_list = reinterpret_cast<int32_t*>(ws + lay.fb_list);
   float* scratch = reinterpret_cast<float*>(ws + lay.scratch);
-  float* acc_dk = reinterpret_cast<float*>(ws + lay.acc_dk);
-  float* acc_dv = reinterpret_cast<float*>(ws + lay.acc_dv);
+  // contiguous float32 outputs are their own accumulators
+  const bool in_place = p.dtype == ENTMAX_ATTN_DTYPE_FP32 && p.sn == p.D && p.sh == (int64_t)p.N * p.D &&
+                        p.sb == (int64_t)p.H * p.N * p.D;
+  float* acc_dk = in_place ? static_cast<float*>(dk) : reinterpret_cast<float*>(ws + lay.acc_dk);
+  float* acc_dv = in_place ? static_cast<float*>(dv) : reinterpret_cast<float*>(ws + lay.acc_dv);
   const size_t acc_bytes = (size_t)p.B * p.H * p.N * p.D * sizeof(float);
   // per-row scale gradients: into the caller's array, else (when only the parameter gradients are wanted)
   // into the workspace, else not computed
@@ -380,8 +384,9 @@ int bwd_impl(const entmax_attn_params* params, const void* q, const void* k, con
                         bf16 ? (lay.tile_mask - lay.fb_count) / 4 + 4 * q_tiles : 64, device_status, stream);
   if (err != cudaSuccess) return fail_cuda(err);
   if (!bf16) {
-    err = launch_dense_bwd(p, q, k, v, d_o, scale, tau, dq, acc_dk, acc_dv, dc_rows, nullptr, nullptr, scratch,
-                           lay.scratch_floats, lay.scratch_ctas, stream);
+    err = launch_fp32_bwd(p, static_cast<const float*>(q), static_cast<const float*>(k), static_cast<const float*>(v),
+                          static_cast<const float*>(d_o), scale, tau, static_cast<float*>(dq), acc_dk, acc_dv, dc_rows,
+                          scratch, lay.scratch_ctas, stream);
     if (err != cudaSuccess) return fail_cuda(err);
   } else {
     int32_t* tile_flag = reinterpret_cast<int32_t*>(ws + lay.tile_flag);
@@ -423,10 +428,12 @@ int bwd_impl(const entmax_attn_params* params, const void* q, const void* k, con
                           acc_dk, acc_dv, dc_rows, device_status, stream);
     if (err != cudaSuccess) return fail_cuda(err);
   }
-  err = launch_store_grad(p, acc_dk, dk, stream);
-  if (err != cudaSuccess) return fail_cuda(err);
-  err = launch_store_grad(p, acc_dv, dv, stream);
-  if (err != cudaSuccess) return fail_cuda(err);
+  if (!in_place) {
+    err = launch_store_grad(p, acc_dk, dk, stream);
+    if (err != cudaSuccess) return fail_cuda(err);
+    err = launch_store_grad(p, acc_dv, dv, stream);
+    if (err != cudaSuccess) return fail_cuda(err);
+  }
   if (n_param_grads) {
     // (the partial sums go where the list entries were: 2 KB per row, no longer needed)
     err = launch_scale_grad(p, beta, gamma, dc_rows, reinterpret_cast<double*>(entries),

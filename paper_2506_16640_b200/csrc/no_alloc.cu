@@ -91,7 +91,6 @@ extern "C" int entmax_attn_fwd_static(const entmax_attn_params* params, const vo
   float* score_rows = scratch + scale_floats;
   err = launch_prologue(p, beta, gamma, delta, scale, nullptr, 0, device_status, stream);
   if (err != cudaSuccess) return fail_cuda(err);
-  err = launch_dense_fwd(p, q, k, v, scale, o, tau, nullptr, nullptr, nullptr, nullptr, nullptr, score_rows, row_floats,
-                         (int)ctas, stream);
+  err = launch_dense_fwd(p, q, k, v, scale, o, tau, score_rows, row_floats, (int)ctas, stream);
   return err == cudaSuccess ? ENTMAX_ATTN_OK : fail_cuda(err);
 }

@@ -108,6 +108,21 @@ def test_dense_tiles_sampled_start_at_a_partial_last_tile(N):
         parity.check_fwd_rows(inp, 1.5, got, bh, rows)
 
 
+@pytest.mark.parametrize("N,d,H,causal,sigma", [(8, 64, 2, True, 1.0), (9, 128, 2, False, 1.0), (255, 64, 2, True, 1.0),
+                                                 (257, 128, 10, False, 1.0), (1201, 64, 2, True, 0.05),
+                                                 (1300, 128, 4, False, 0.05)])
+def test_fp32_row_tiles_at_their_edges(N, d, H, causal, sigma):
+    # float32 problems: row tiles of 8 and 16, K tiles of 256 and their remainders, lists in shared memory, and (sigma 0.05,
+    # where every key is in the support) rows longer than those lists, which the forward pass walks in the score row and the
+    # backward pass in stretches
+    inp = make_inputs(_small("fp32_edges", N, d, causal, dtype="fp32", H=H, sigma=sigma, backward=True, seed=N + d))
+    got = parity.run_fwd(inp, 1.5)
+    bwd = parity.run_bwd(inp, 1.5, got["tau"], got["dev"])
+    for bh in (0, H - 1):
+        parity.check_fwd_rows(inp, 1.5, got, bh, np.unique(np.concatenate([np.arange(0, N, 7), [N - 1]])))
+        parity.check_bwd_head(inp, 1.5, bwd, bh)
+
+
 @pytest.mark.parametrize("sigma,expect", [(0.55, 200), (0.3, 1000), (0.18, 4000)])
 def test_dense_path_at_supports_of_hundreds_to_thousands(sigma, expect):
     # long rows whose supports run to about 200, 1000 and 4000 keys (fixed temperature, logits of std sigma^2): forward
