@@ -22,13 +22,12 @@ from . import binding
 class _EntmaxAttention(torch.autograd.Function):
     @staticmethod
     def forward(ctx, q, k, v, beta, gamma, delta, c_rows, alibi_slopes, alpha, causal, sm_scale, keep_supports):
-        params = binding.make_params(q, alpha, causal, sm_scale, 0)
-        ws = binding.alloc_workspace(params, False, q.device) if keep_supports and q.dtype == torch.bfloat16 else None
-        keep_supports = ws is not None
-        det = lambda t: None if t is None else t.detach()
-        o, tau = binding.entmax_attn_fwd_ex(q.detach(), k.detach(), v.detach(), alpha, causal, det(beta), det(gamma),
-                                            det(delta), c_rows=det(c_rows), alibi_slopes=det(alibi_slopes),
-                                            sm_scale=sm_scale, workspace=ws)
+        keep_supports = keep_supports and q.dtype == torch.bfloat16
+        ws = binding.alloc_workspace(binding.make_params(q, alpha, causal, sm_scale, 0), False, q.device) if keep_supports \
+            else None
+        # (no detach: gradients are off inside forward and backward, and the binding only takes addresses)
+        o, tau = binding.entmax_attn_fwd_ex(q, k, v, alpha, causal, beta, gamma, delta, c_rows=c_rows,
+                                            alibi_slopes=alibi_slopes, sm_scale=sm_scale, workspace=ws)
         saved = binding.entmax_attn_save_supports(q, alpha, causal, ws, sm_scale=sm_scale) if keep_supports else None
         ctx.save_for_backward(q, k, v, beta, gamma, delta, c_rows, alibi_slopes, tau)
         ctx.alpha, ctx.causal, ctx.sm_scale, ctx.saved_supports = alpha, causal, sm_scale, saved
@@ -38,12 +37,11 @@ class _EntmaxAttention(torch.autograd.Function):
     @staticmethod
     def backward(ctx, d_o, _d_tau):
         q, k, v, beta, gamma, delta, c_rows, alibi_slopes, tau = ctx.saved_tensors
-        det = lambda t: None if t is None else t.detach()
         want_params = beta is not None and any(ctx.needs_input_grad[3:6])
         want_rows = c_rows is not None and ctx.needs_input_grad[6]
         dq, dk, dv, dc, grads = binding.entmax_attn_bwd_ex(
-            q.detach(), k.detach(), v.detach(), tau, d_o.contiguous(), ctx.alpha, ctx.causal, det(beta), det(gamma),
-            det(delta), c_rows=det(c_rows), alibi_slopes=det(alibi_slopes), saved_supports=ctx.saved_supports,
+            q, k, v, tau, d_o.contiguous(), ctx.alpha, ctx.causal, beta, gamma, delta, c_rows=c_rows,
+            alibi_slopes=alibi_slopes, saved_supports=ctx.saved_supports,
             want_scale_rows=want_rows, want_param_grads=want_params, sm_scale=ctx.sm_scale)
         ctx.saved_supports = None
         db, dg, dd = grads if grads is not None else (None, None, None)

@@ -133,7 +133,7 @@ def _check(rc: int, what: str):
 
 
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()      # the argtypes say c_void_p: a plain int converts fastest
 
 
 def make_params(q: torch.Tensor, alpha: float, causal: bool, sm_scale: float = 0.0, n_mode: int = 0) -> Params:
@@ -145,16 +145,17 @@ def make_params(q: torch.Tensor, alpha: float, causal: bool, sm_scale: float = 0
         dt = DTYPE_FP32
     else:
         raise EntmaxAttnError("dtype must be bfloat16 or float32")
-    if q.stride(3) != 1:
+    sb, sh, sn, sd = q.stride()
+    if sd != 1:
         raise EntmaxAttnError("head_dim must be the innermost, contiguous dimension")
     B, H, N, D = q.shape
-    return Params(B, H, N, D, dt, int(bool(causal)), int(n_mode), float(alpha), float(sm_scale),
-                  q.stride(0), q.stride(1), q.stride(2))
+    return Params(B, H, N, D, dt, int(bool(causal)), int(n_mode), float(alpha), float(sm_scale), sb, sh, sn)
 
 
 def _same_layout(ref: torch.Tensor, *others):
+    shape, stride, dtype, device = ref.shape, ref.stride(), ref.dtype, ref.device
     for t in others:
-        if t.shape != ref.shape or t.stride() != ref.stride() or t.dtype != ref.dtype or t.device != ref.device:
+        if t.shape != shape or t.stride() != stride or t.dtype != dtype or t.device != device:
             raise EntmaxAttnError("all [B,H,N,D] tensors of a call must share shape, strides, dtype and device")
 
 
@@ -176,8 +177,12 @@ def alloc_workspace(params: Params, is_bwd: bool, device) -> torch.Tensor:
 
 
 def _stream_ptr(stream):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if not torch.cuda.is_initialized():
+        torch.cuda.init()
+    # the current stream's handle without a Stream object around it (5 us of the 21 a small call took)
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def entmax_attn_fwd(q, k, v, alpha, causal, beta=None, gamma=None, delta=None, *, sm_scale=0.0, n_mode=0,
@@ -281,7 +286,7 @@ def entmax_attn_bwd_scale(q, k, v, tau, d_o, alpha, causal, beta, gamma, delta, 
         d_scale_rows = torch.empty((B, H, N), dtype=torch.float32, device=q.device)
     grads = None
     if want_param_grads:
-        grads = tuple(torch.empty((H,), dtype=torch.float32, device=q.device) for _ in range(3))
+        grads = torch.empty((3, H), dtype=torch.float32, device=q.device).unbind(0)
     if workspace is None:
         workspace = alloc_workspace(params, True, q.device)
     g = grads if grads is not None else (None, None, None)
@@ -332,10 +337,6 @@ def entmax_attn_bwd_rowscale(q, k, v, c_rows, tau, d_o, alpha, causal, *, sm_sca
     return dq, dk, dv, d_scale_rows
 
 
-def _dp(t):
-    return None if t is None else t.data_ptr()
-
-
 def entmax_attn_fwd_ex(q, k, v, alpha, causal, beta=None, gamma=None, delta=None, *, c_rows=None, alibi_slopes=None,
                        sm_scale=0.0, n_mode=0, o=None, tau=None, workspace=None, status=None, stream=None):
     """Extended forward pass: optional per-query scale table and ALiBi slopes.  Returns (o, tau)."""
@@ -347,7 +348,7 @@ def entmax_attn_fwd_ex(q, k, v, alpha, causal, beta=None, gamma=None, delta=None
         tau = torch.empty((B, H, N), dtype=torch.float32, device=q.device)
     if workspace is None:
         workspace = alloc_workspace(params, False, q.device)
-    ex = Extras(_dp(c_rows), _dp(alibi_slopes), None, None, None, None, None)
+    ex = Extras(_ptr(c_rows), _ptr(alibi_slopes), None, None, None, None, None)
     rc = load().entmax_attn_fwd_ex(ctypes.byref(params), _ptr(q), _ptr(k), _ptr(v), _ptr(beta), _ptr(gamma), _ptr(delta),
                                    ctypes.byref(ex), _ptr(o), _ptr(tau), _ptr(workspace), workspace.numel(),
                                    _ptr(status), _stream_ptr(stream))
@@ -383,12 +384,12 @@ def entmax_attn_bwd_ex(q, k, v, tau, d_o, alpha, causal, beta=None, gamma=None, 
     dk = torch.empty_like(q) if dk is None else dk
     dv = torch.empty_like(q) if dv is None else dv
     dc = torch.empty((B, H, N), dtype=torch.float32, device=q.device) if want_scale_rows else None
-    grads = tuple(torch.empty((H,), dtype=torch.float32, device=q.device) for _ in range(3)) if want_param_grads else None
+    grads = torch.empty((3, H), dtype=torch.float32, device=q.device).unbind(0) if want_param_grads else None
     g = grads if grads is not None else (None, None, None)
     if workspace is None:
         workspace = alloc_workspace(params, True, q.device)
-    ex = Extras(_dp(c_rows), _dp(alibi_slopes), _dp(dc), _dp(g[0]), _dp(g[1]), _dp(g[2]), _dp(fwd_workspace),
-                _dp(saved_supports))
+    ex = Extras(_ptr(c_rows), _ptr(alibi_slopes), _ptr(dc), _ptr(g[0]), _ptr(g[1]), _ptr(g[2]), _ptr(fwd_workspace),
+                _ptr(saved_supports))
     rc = load().entmax_attn_bwd_ex(ctypes.byref(params), _ptr(q), _ptr(k), _ptr(v), _ptr(beta), _ptr(gamma), _ptr(delta),
                                    ctypes.byref(ex), _ptr(tau), _ptr(d_o), _ptr(dq), _ptr(dk), _ptr(dv), _ptr(workspace),
                                    workspace.numel(), _ptr(status), _stream_ptr(stream))
