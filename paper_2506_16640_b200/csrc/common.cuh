@@ -10,16 +10,13 @@
 
 namespace entmax {
 
-// Sparse row lists.  The score sweep splits the keys of a row between two threads; each owns one half
-// of the row's kListCap list slots: capacity kHalfCap, the fill level at which the sweep tightens the
-// threshold and filters the half-list (checked after every 32 keys, so the capacity is never exceeded),
-// and the length a filtered half-list may keep -- a row that cannot be brought down to it is handed to
-// the dense path.  The row kernels merge the two halves and leave the support compacted from slot 0.
-constexpr int kHalfCap = 128;
-constexpr int kHalfTrigger = 88;
-constexpr int kHalfKeep = 72;
-static_assert(kHalfTrigger + 32 <= kHalfCap && kHalfKeep < kHalfTrigger, "half-list bounds");
-constexpr int kListCap = 2 * kHalfCap;
+// Sparse row lists: kListCap slots per row, the fill level at which the sweep tightens the threshold and filters the list
+// (checked after every K tile), and the length a filtered list may keep -- a row that cannot be brought down to it is
+// handed to the dense path.  The row kernels leave the support compacted from slot 0.
+constexpr int kListCap = 256;
+constexpr int kListTrigger = 112;
+constexpr int kListKeep = 96;
+static_assert(kListTrigger + 64 <= kListCap && kListKeep < kListTrigger, "list bounds");
 
 // One list slot: y = (alpha-1) * s_ij (or the raw accumulator while a sweep is running), j = key index.
 struct __align__(8) Entry {
@@ -49,7 +46,7 @@ struct Problem {
 };
 
 struct WsLayout {
-  size_t scale, row_cnt, half_cnt, half_thr, entries, fb_count, sweep_counter, tile_count, grad_counter, tile_flag, tile_list, tile_mask, fb_list, alibi_blob, alibi_kmax, scratch, acc_dk, acc_dv, dc_rows, total;
+  size_t scale, row_cnt, list_cnt, list_thr, entries, fb_count, sweep_counter, tile_count, grad_counter, tile_flag, tile_list, tile_mask, fb_list, alibi_blob, alibi_kmax, scratch, acc_dk, acc_dv, dc_rows, total;
   int scratch_ctas;     // CTAs of the float32 kernels (each owns sixteen score rows of the scratch)
 };
 
@@ -211,7 +208,7 @@ cudaError_t launch_scale_grad(const Problem& p, const float* beta, const float* 
 // tcgen05 score sweep (bf16): fills the per-row candidate lists.
 //   mode 0: threshold search (forward); mode 1: threshold given in tau_in (backward); *work_counter must be zero on entry
 cudaError_t launch_sweep(const Problem& p, const void* q, const void* k, const float* scale, const float* tau_in,
-                         int mode, int32_t* half_cnt, float* half_thr, Entry* entries, int32_t* work_counter,
+                         int mode, int32_t* list_cnt, float* list_thr, Entry* entries, int32_t* work_counter,
                          float* dump, int dump_bh, float* alibi_blob, float* alibi_kmax, int32_t* status,
                          cudaStream_t stream);
 
@@ -242,11 +239,11 @@ cudaError_t launch_tile_bwd(const Problem& p, const void* q, const void* k, cons
 // per-row solve + gather kernels working on the lists (bf16 path); the forward one also lists the
 // 128-row Q tiles that hold rows for the dense-tile path (tile_flag must be zero on entry)
 cudaError_t launch_row_fwd(const Problem& p, const void* v, const float* scale, int32_t* row_cnt,
-                           const int32_t* half_cnt, const float* half_thr, Entry* entries, void* o, float* tau, int32_t* fb_count,
+                           const int32_t* list_cnt, const float* list_thr, Entry* entries, void* o, float* tau, int32_t* fb_count,
                            int32_t* fb_list, int32_t* tile_flag, int32_t* tile_list, int32_t* tile_count, int32_t* status,
                            cudaStream_t stream);
 cudaError_t launch_row_bwd(const Problem& p, const void* q, const void* k, const void* v, const void* d_o,
-                           const float* scale, const float* tau, const int32_t* half_cnt, Entry* entries, void* dq,
+                           const float* scale, const float* tau, const int32_t* list_cnt, Entry* entries, void* dq,
                            float* acc_dk, float* acc_dv, float* dc_rows, int32_t* fb_count, int32_t* fb_list,
                            int32_t* status, int saved, int pitch, cudaStream_t stream);
 // compact copy of the forward call's supports (see entmax_attn_save_supports)

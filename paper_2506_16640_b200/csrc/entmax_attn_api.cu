@@ -130,8 +130,8 @@ WsLayout make_layout(const Problem& p, bool is_bwd) {
   auto take = [&off](size_t bytes) { size_t at = off; off = align_up(off + bytes, 256); return at; };
   l.scale = take((size_t)p.H * p.N * sizeof(float));
   l.row_cnt = take(rows * sizeof(int32_t));
-  l.half_cnt = take(rows * 2 * sizeof(int32_t));
-  l.half_thr = take(rows * 2 * sizeof(float));
+  l.list_cnt = take(rows * 2 * sizeof(int32_t));
+  l.list_thr = take(rows * sizeof(float));
   l.entries = take(rows * kListCap * sizeof(Entry));
   l.fb_count = take(256);
   l.sweep_counter = l.fb_count + 64;   // same 256-byte block: [0] dense-row count, [16] sweep work counter,
@@ -185,9 +185,9 @@ int entmax_attn_workspace_layout(const entmax_attn_params* params, entmax_attn_w
   out->row_count_offset = l.row_cnt;
   out->entries_offset = l.entries;
   out->scale_offset = l.scale;
-  out->dense_count_offset = l.half_cnt;
+  out->dense_count_offset = l.list_cnt;
   out->capacity = kListCap;
-  out->keep_limit = kHalfKeep;
+  out->keep_limit = kListKeep;
   return ENTMAX_ATTN_OK;
 }
 
@@ -223,8 +223,8 @@ int fwd_impl(const entmax_attn_params* params, const void* q, const void* k, con
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   const float* scale = reinterpret_cast<float*>(ws + lay.scale);
   int32_t* row_cnt = reinterpret_cast<int32_t*>(ws + lay.row_cnt);
-  int32_t* half_cnt = reinterpret_cast<int32_t*>(ws + lay.half_cnt);
-  float* half_thr = reinterpret_cast<float*>(ws + lay.half_thr);
+  int32_t* list_cnt = reinterpret_cast<int32_t*>(ws + lay.list_cnt);
+  float* list_thr = reinterpret_cast<float*>(ws + lay.list_thr);
   int32_t* sweep_counter = reinterpret_cast<int32_t*>(ws + lay.sweep_counter);
   Entry* entries = reinterpret_cast<Entry*>(ws + lay.entries);
   int32_t* fb_count = reinterpret_cast<int32_t*>(ws + lay.fb_count);
@@ -249,23 +249,23 @@ int fwd_impl(const entmax_attn_params* params, const void* q, const void* k, con
   }
   if (!bf16) {
     err = launch_fp32_fwd(p, static_cast<const float*>(q), static_cast<const float*>(k), static_cast<const float*>(v), scale,
-                          static_cast<float*>(o), tau, row_cnt, half_cnt, entries, scratch, lay.scratch_ctas, stream);
+                          static_cast<float*>(o), tau, row_cnt, list_cnt, entries, scratch, lay.scratch_ctas, stream);
     return err == cudaSuccess ? ENTMAX_ATTN_OK : fail_cuda(err);
   }
   int32_t* tile_flag = reinterpret_cast<int32_t*>(ws + lay.tile_flag);
   int32_t* tile_list = reinterpret_cast<int32_t*>(ws + lay.tile_list);
   int32_t* tile_count = reinterpret_cast<int32_t*>(ws + lay.tile_count);
   if (g_prof_start[0]) cudaEventRecord(g_prof_start[0], stream);
-  err = launch_sweep(p, q, k, scale, nullptr, 0, half_cnt, half_thr, entries, sweep_counter, nullptr, -1,
+  err = launch_sweep(p, q, k, scale, nullptr, 0, list_cnt, list_thr, entries, sweep_counter, nullptr, -1,
                      reinterpret_cast<float*>(ws + lay.alibi_blob), reinterpret_cast<float*>(ws + lay.alibi_kmax),
                      device_status, stream);
   if (err != cudaSuccess) return fail_cuda(err);
   if (g_prof_stop[0]) cudaEventRecord(g_prof_stop[0], stream);
-  err = launch_row_fwd(p, v, scale, row_cnt, half_cnt, half_thr, entries, o, tau, fb_count, fb_list, tile_flag, tile_list,
+  err = launch_row_fwd(p, v, scale, row_cnt, list_cnt, list_thr, entries, o, tau, fb_count, fb_list, tile_flag, tile_list,
                        tile_count, device_status, stream);
   if (err != cudaSuccess) return fail_cuda(err);
   // rows whose support does not fit the lists: dense tiles on the tensor cores
-  err = launch_tile_fwd(p, q, k, v, scale, tile_flag, tile_list, tile_count, tile_count + 16, row_cnt, half_cnt, o, tau,
+  err = launch_tile_fwd(p, q, k, v, scale, tile_flag, tile_list, tile_count, tile_count + 16, row_cnt, list_cnt, o, tau,
                         device_status, stream);
   return err == cudaSuccess ? ENTMAX_ATTN_OK : fail_cuda(err);
 }
@@ -334,8 +334,8 @@ int bwd_impl(const entmax_attn_params* params, const void* q, const void* k, con
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   const float* scale = reinterpret_cast<float*>(ws + lay.scale);
-  int32_t* half_cnt = reinterpret_cast<int32_t*>(ws + lay.half_cnt);
-  float* half_thr = reinterpret_cast<float*>(ws + lay.half_thr);
+  int32_t* list_cnt = reinterpret_cast<int32_t*>(ws + lay.list_cnt);
+  float* list_thr = reinterpret_cast<float*>(ws + lay.list_thr);
   int32_t* sweep_counter = reinterpret_cast<int32_t*>(ws + lay.sweep_counter);
   Entry* entries = reinterpret_cast<Entry*>(ws + lay.entries);
   int32_t* fb_count = reinterpret_cast<int32_t*>(ws + lay.fb_count);
@@ -411,20 +411,20 @@ int bwd_impl(const entmax_attn_params* params, const void* q, const void* k, con
       if (err != cudaSuccess) return fail_cuda(err);
     } else {
       if (g_prof_start[1]) cudaEventRecord(g_prof_start[1], stream);
-      err = launch_sweep(p, q, k, scale, tau, 1, half_cnt, half_thr, entries, sweep_counter, nullptr, -1,
+      err = launch_sweep(p, q, k, scale, tau, 1, list_cnt, list_thr, entries, sweep_counter, nullptr, -1,
                          reinterpret_cast<float*>(ws + lay.alibi_blob), reinterpret_cast<float*>(ws + lay.alibi_kmax),
                          device_status, stream);
       if (err != cudaSuccess) return fail_cuda(err);
       if (g_prof_stop[1]) cudaEventRecord(g_prof_stop[1], stream);
       err = cudaStreamWaitEvent(stream, side->join, 0);     // the accumulators are clear from here on
       if (err != cudaSuccess) return fail_cuda(err);
-      err = launch_row_bwd(p, q, k, v, d_o, scale, tau, half_cnt, entries, dq, acc_dk, acc_dv, dc_rows, fb_count,
+      err = launch_row_bwd(p, q, k, v, d_o, scale, tau, list_cnt, entries, dq, acc_dk, acc_dv, dc_rows, fb_count,
                            fb_list, device_status, 0, kListCap, stream);
       if (err != cudaSuccess) return fail_cuda(err);
     }
     // rows whose support does not fit the lists: dense tiles on the tensor cores
     err = launch_tile_bwd(p, q, k, v, d_o, scale, tau, fb_list, fb_count, tile_mask, tile_flag, tile_list, tile_count, tile_count + 16,
-                          reinterpret_cast<float*>(ws + lay.half_thr) /* idle after the sweep: rho of the dense rows */, dq,
+                          reinterpret_cast<float*>(ws + lay.list_thr) /* idle after the sweep: rho of the dense rows */, dq,
                           acc_dk, acc_dv, dc_rows, device_status, stream);
     if (err != cudaSuccess) return fail_cuda(err);
   }
@@ -514,8 +514,8 @@ int entmax_attn_scores_debug(const entmax_attn_params* params, const void* q, co
   err = launch_prologue(p, nullptr, nullptr, nullptr, scale, reinterpret_cast<int32_t*>(ws + lay.fb_count), 64, device_status,
                         stream);
   if (err != cudaSuccess) return fail_cuda(err);
-  err = launch_sweep(p, q, k, scale, nullptr, 0, reinterpret_cast<int32_t*>(ws + lay.half_cnt),
-                     reinterpret_cast<float*>(ws + lay.half_thr), reinterpret_cast<Entry*>(ws + lay.entries),
+  err = launch_sweep(p, q, k, scale, nullptr, 0, reinterpret_cast<int32_t*>(ws + lay.list_cnt),
+                     reinterpret_cast<float*>(ws + lay.list_thr), reinterpret_cast<Entry*>(ws + lay.entries),
                      reinterpret_cast<int32_t*>(ws + lay.sweep_counter), s_out, bh, nullptr, nullptr, device_status, stream);
   return err == cudaSuccess ? ENTMAX_ATTN_OK : fail_cuda(err);
 }

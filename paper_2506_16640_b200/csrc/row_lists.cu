@@ -1,5 +1,5 @@
 // Per-row kernels of the bf16 path that work on the sparse candidate lists left by the tensor-core
-// score sweep (two half-lists per row, see common.cuh).
+// score sweep (see common.cuh).
 //
 // Forward: exact threshold on the candidates (Eq. 1 with the sum-to-one condition), probabilities, and
 // O_i = sum_j p_ij v_j as a gather over the support only -- every zero of P is skipped, not just
@@ -184,18 +184,18 @@ __device__ __forceinline__ float newton_warp(const Problem& p, const float (&y)[
 // Stage A on S*32 candidate slots.  Leaves the kept entries (y in Eq. 1's units) compacted from slot 0
 // of the row's list and returns how many there are.
 template <int S>
-__device__ __forceinline__ int prefilter_row(const Problem& p, Entry* list, int c0, int c1, float a, int lane,
+__device__ __forceinline__ int prefilter_row(const Problem& p, Entry* list, int n_list, float a, int lane,
                                              float bound) {
   float y[S];
   int jj[S];
   float ymax = -INFINITY;
 #pragma unroll
   for (int s = 0; s < S; ++s) {
-    const int e = lane + 32 * s;                   // dense numbering: first half-list, then second
+    const int e = lane + 32 * s;
     y[s] = -INFINITY;
     jj[s] = 0x7fffffff;
-    if (e < c0 + c1) {
-      const Entry en = list[e < c0 ? e : kHalfCap + e - c0];
+    if (e < n_list) {
+      const Entry en = list[e];
       y[s] = a * en.y;
       jj[s] = en.j;
     }
@@ -285,12 +285,12 @@ __device__ __forceinline__ void finish_row(const Problem& p, const __nv_bfloat16
 }
 
 // Out-of-line forms for the rare rows with more than 32 candidates (kept out of the hot loop's code)
-__device__ __noinline__ int prefilter_long(const Problem& p, Entry* list, int c0, int c1, float a, int lane,
+__device__ __noinline__ int prefilter_long(const Problem& p, Entry* list, int n_list, float a, int lane,
                                            float bound) {
-  const int n = c0 + c1;
-  if (n <= 64) return prefilter_row<2>(p, list, c0, c1, a, lane, bound);
-  if (n <= 128) return prefilter_row<4>(p, list, c0, c1, a, lane, bound);
-  return prefilter_row<kSlots>(p, list, c0, c1, a, lane, bound);
+  const int n = n_list;
+  if (n <= 64) return prefilter_row<2>(p, list, n_list, a, lane, bound);
+  if (n <= 128) return prefilter_row<4>(p, list, n_list, a, lane, bound);
+  return prefilter_row<kSlots>(p, list, n_list, a, lane, bound);
 }
 template <int D>
 __device__ __noinline__ void finish_long(const Problem& p, const __nv_bfloat16* __restrict__ vbase, Entry* list, int kept,
@@ -303,14 +303,14 @@ __device__ __noinline__ void finish_long(const Problem& p, const __nv_bfloat16* 
 // One row with the whole warp.
 template <int D>
 __device__ __forceinline__ void solve_row_full(const Problem& p, const __nv_bfloat16* __restrict__ vbase, Entry* list,
-                                               int c0, int c1, float a, float bound, __nv_bfloat16* o_row,
+                                               int n_list, float a, float bound, __nv_bfloat16* o_row,
                                                float* tau_slot, int32_t* cnt_slot, int lane) {
-  const int n = c0 + c1;
+  const int n = n_list;
   int kept;
-  if (n <= 32) kept = prefilter_row<1>(p, list, c0, c1, a, lane, bound);
-  else if (n <= 64) kept = prefilter_row<2>(p, list, c0, c1, a, lane, bound);
-  else if (n <= 128) kept = prefilter_row<4>(p, list, c0, c1, a, lane, bound);
-  else kept = prefilter_row<kSlots>(p, list, c0, c1, a, lane, bound);
+  if (n <= 32) kept = prefilter_row<1>(p, list, n_list, a, lane, bound);
+  else if (n <= 64) kept = prefilter_row<2>(p, list, n_list, a, lane, bound);
+  else if (n <= 128) kept = prefilter_row<4>(p, list, n_list, a, lane, bound);
+  else kept = prefilter_row<kSlots>(p, list, n_list, a, lane, bound);
   if (kept <= 32) finish_row<D, 1>(p, vbase, list, kept, o_row, tau_slot, cnt_slot, lane);
   else if (kept <= 64) finish_row<D, 2>(p, vbase, list, kept, o_row, tau_slot, cnt_slot, lane);
   else if (kept <= 128) finish_row<D, 4>(p, vbase, list, kept, o_row, tau_slot, cnt_slot, lane);
@@ -339,19 +339,19 @@ template <int D, int W>
 __device__ __forceinline__ void solve_rows_sub(const Problem& p, const __nv_bfloat16* __restrict__ v,
                                                 const float* __restrict__ scale, Entry* __restrict__ entries,
                                                 __nv_bfloat16* __restrict__ o, float* __restrict__ tau_out,
-                                                int32_t* __restrict__ row_cnt, const float* __restrict__ half_thr,
-                                                int grow, bool active, int c0, int c1, int lane) {
+                                                int32_t* __restrict__ row_cnt, const float* __restrict__ list_thr,
+                                                int grow, bool active, int n_list, int lane) {
   constexpr int PL = D / W;                        // elements of a V / O row per lane
   const int sl = lane & (W - 1);
   const int base = lane & (32 - W);
-  const int n = active ? c0 + c1 : 0;
+  const int n = active ? n_list : 0;
   const int bh = grow / p.N, i = grow - bh * p.N, b = bh / p.H, h = bh - b * p.H;
   const float a = active ? (p.alpha - 1.0f) * (scale[(size_t)b * p.scale_sb + (size_t)h * p.N + i] * p.sm_scale) : 1.0f;
   Entry* list = entries + (size_t)grow * kListCap;
   float y = -INFINITY;
   int j = 0x7fffffff;
   if (sl < n) {
-    const Entry en = list[sl < c0 ? sl : kHalfCap + sl - c0];
+    const Entry en = list[sl];
     y = a * en.y;
     j = en.j;
   }
@@ -360,8 +360,7 @@ __device__ __forceinline__ void solve_rows_sub(const Problem& p, const __nv_bflo
   // stage A starts from the bound the sweep ended with (see prefilter_row)
   float bound = -INFINITY;
   if (active) {
-    const float2 ht = *reinterpret_cast<const float2*>(half_thr + 2 * (size_t)grow);
-    bound = fmaxf(ht.x, ht.y);
+    bound = list_thr[grow];
     bound -= kKeepMargin * fmaxf(1.0f, fabsf(bound));
   }
   const float tau_a = newton_sub<W>(p, y, sub_max<W>(y), !active, bound);
@@ -434,19 +433,19 @@ __device__ __forceinline__ void solve_rows_sub(const Problem& p, const __nv_bflo
 // with U1, U2 the prefix sums of u and u^2; the support size k* is the number of k with u_k < t_k (they form a
 // prefix) and tau = y_max - t_{k*} -- Eq. 1's threshold without iterating.  Only the top k* entries enter the
 // result, so candidates outside the support, which differ from run to run, do not change a bit of it.
-// `prescaled`: the list already holds y in Eq. 1's units from slot 0 (c1 = 0).
+// `prescaled`: the list already holds y in Eq. 1's units from slot 0.
 template <int D, int W, int EC>
 __device__ __forceinline__ void solve_rows_closed(const Problem& p, const __nv_bfloat16* __restrict__ v,
                                                   const float* __restrict__ scale, Entry* __restrict__ entries,
                                                   __nv_bfloat16* __restrict__ o, float* __restrict__ tau_out,
-                                                  int32_t* __restrict__ row_cnt, int grow, bool active, int c0, int c1,
+                                                  int32_t* __restrict__ row_cnt, int grow, bool active, int n_list,
                                                   bool prescaled, int lane) {
   static_assert(EC == kExpo2 || EC == kExpo1, "closed forms exist for e = 2 and e = 1");
   constexpr int PL = D / W;                        // elements of a V / O row per lane
   constexpr unsigned kWMask = W == 32 ? 0xffffffffu : ((1u << (W & 31)) - 1u);
   const int sl = lane & (W - 1);
   const int base = lane & (32 - W);
-  const int n = active ? c0 + c1 : 0;
+  const int n = active ? n_list : 0;
   const int bh = grow / p.N, i = grow - bh * p.N, b = bh / p.H, h = bh - b * p.H;
   const float a = (active && !prescaled)
                       ? (p.alpha - 1.0f) * (scale[(size_t)b * p.scale_sb + (size_t)h * p.N + i] * p.sm_scale) : 1.0f;
@@ -454,7 +453,7 @@ __device__ __forceinline__ void solve_rows_closed(const Problem& p, const __nv_b
   float y = -INFINITY;
   int j = 0x7fffffff;
   if (sl < n) {
-    const Entry en = list[sl < c0 ? sl : kHalfCap + sl - c0];
+    const Entry en = list[sl];
     y = a * en.y;
     j = en.j;
   }
@@ -578,28 +577,27 @@ __device__ __forceinline__ void push_dense_tiles(const Problem& p, unsigned mask
 template <int D, int EC>
 __device__ __forceinline__ void row_fwd_whole_warp(const Problem& p, const __nv_bfloat16* __restrict__ v,
                                                    const float* __restrict__ scale, int32_t* __restrict__ row_cnt,
-                                                   const float* __restrict__ half_thr, Entry* __restrict__ entries,
+                                                   const float* __restrict__ list_thr, Entry* __restrict__ entries,
                                                    __nv_bfloat16* __restrict__ o, float* __restrict__ tau_out, int grow,
-                                                   int c0, int c1, int lane) {
+                                                   int n_list, int lane) {
   constexpr int PER = D / 32;
   constexpr bool kClosed = EC == kExpo2 || EC == kExpo1;
   const int bh = grow / p.N, i = grow - bh * p.N, b = bh / p.H, h = bh - b * p.H;
   const float a = (p.alpha - 1.0f) * (scale[(size_t)b * p.scale_sb + (size_t)h * p.N + i] * p.sm_scale);
   Entry* list = entries + (size_t)grow * kListCap;
-  const float2 ht = *reinterpret_cast<const float2*>(half_thr + 2 * (size_t)grow);
-  float bound = fmaxf(ht.x, ht.y);
+  float bound = list_thr[grow];
   bound -= kKeepMargin * fmaxf(1.0f, fabsf(bound));
   if constexpr (kClosed) {
     // up to 32 entries: closed form with the whole warp; more: Newton prefilter first, and the closed form
     // if what it keeps fits the warp
-    const int n = c0 + c1;
+    const int n = n_list;
     if (n <= 32) {
-      solve_rows_closed<D, 32, EC>(p, v, scale, entries, o, tau_out, row_cnt, grow, true, c0, c1, false, lane);
+      solve_rows_closed<D, 32, EC>(p, v, scale, entries, o, tau_out, row_cnt, grow, true, n_list, false, lane);
       return;
     }
-    const int kept = prefilter_long(p, list, c0, c1, a, lane, bound);
+    const int kept = prefilter_long(p, list, n_list, a, lane, bound);
     if (kept <= 32) {
-      solve_rows_closed<D, 32, EC>(p, v, scale, entries, o, tau_out, row_cnt, grow, true, kept, 0, true, lane);
+      solve_rows_closed<D, 32, EC>(p, v, scale, entries, o, tau_out, row_cnt, grow, true, kept, true, lane);
       return;
     }
     const __nv_bfloat16* vbase = v + (size_t)b * p.sb + (size_t)h * p.sh + lane * PER;
@@ -608,7 +606,7 @@ __device__ __forceinline__ void row_fwd_whole_warp(const Problem& p, const __nv_
   } else {
     const __nv_bfloat16* vbase = v + (size_t)b * p.sb + (size_t)h * p.sh + lane * PER;
     __nv_bfloat16* o_row = o + (size_t)b * p.sb + (size_t)h * p.sh + (size_t)i * p.sn + lane * PER;
-    solve_row_full<D>(p, vbase, list, c0, c1, a, bound, o_row, tau_out + grow, row_cnt + grow, lane);
+    solve_row_full<D>(p, vbase, list, n_list, a, bound, o_row, tau_out + grow, row_cnt + grow, lane);
   }
 }
 
@@ -617,8 +615,8 @@ template <int D, int EC>
 __global__ void __launch_bounds__(kWarpsPerCta * 32) row_fwd_long_kernel(Problem p, const __nv_bfloat16* __restrict__ v,
                                                                          const float* __restrict__ scale,
                                                                          int32_t* __restrict__ row_cnt,
-                                                                         const int32_t* __restrict__ half_cnt,
-                                                                         const float* __restrict__ half_thr,
+                                                                         const int32_t* __restrict__ list_cnt,
+                                                                         const float* __restrict__ list_thr,
                                                                          Entry* __restrict__ entries,
                                                                          __nv_bfloat16* __restrict__ o,
                                                                          float* __restrict__ tau_out,
@@ -629,8 +627,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32) row_fwd_long_kernel(Problem
   const int n_long = fb_count[kLongCounter];
   for (int t = blockIdx.x * kWarpsPerCta + (threadIdx.x >> 5); t < n_long; t += gridDim.x * kWarpsPerCta) {
     const int grow = fb_list[total - 1 - t];
-    const int2 c = *reinterpret_cast<const int2*>(half_cnt + 2 * (size_t)grow);
-    row_fwd_whole_warp<D, EC>(p, v, scale, row_cnt, half_thr, entries, o, tau_out, grow, c.x, c.y, lane);
+    row_fwd_whole_warp<D, EC>(p, v, scale, row_cnt, list_thr, entries, o, tau_out, grow, list_cnt[2 * (size_t)grow], lane);
   }
 }
 
@@ -639,8 +636,8 @@ template <int D, int EC>
 __global__ void __launch_bounds__(kWarpsPerCta * 32) row_fwd_kernel(Problem p, const __nv_bfloat16* __restrict__ v,
                                                                     const float* __restrict__ scale,
                                                                     int32_t* __restrict__ row_cnt,
-                                                                    const int32_t* __restrict__ half_cnt,
-                                                                    const float* __restrict__ half_thr,
+                                                                    const int32_t* __restrict__ list_cnt,
+                                                                    const float* __restrict__ list_thr,
                                                                     Entry* __restrict__ entries,
                                                                     __nv_bfloat16* __restrict__ o,
                                                                     float* __restrict__ tau_out, int32_t* fb_count,
@@ -656,14 +653,11 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32) row_fwd_kernel(Problem p, c
     // each (9..16 entries), the rest one by one with the whole warp.
     constexpr bool kClosed = EC == kExpo2 || EC == kExpo1;
     const int my_row = 16 * blk + (lane & 15);
-    int mc0 = 0, mc1 = 0;
+    int mc = 0;
     int cls = 3;                                     // 0: <= 8 entries, 1: <= 16, 2: whole warp / dense, 3: no row
     if (my_row < total) {
-      const int2 c = *reinterpret_cast<const int2*>(half_cnt + 2 * (size_t)my_row);
-      mc0 = c.x;
-      mc1 = c.y;
-      const int n = mc0 + mc1;
-      cls = (mc0 < 0 || mc1 < 0 || n < 1 || n > 16) ? 2 : n <= 8 ? 0 : 1;
+      mc = list_cnt[2 * (size_t)my_row];
+      cls = (mc < 1 || mc > 16) ? 2 : mc <= 8 ? 0 : 1;
     }
     unsigned m8 = __ballot_sync(0xffffffffu, lane < 16 && cls == 0);
     unsigned m16 = __ballot_sync(0xffffffffu, lane < 16 && cls == 1);
@@ -671,11 +665,11 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32) row_fwd_kernel(Problem p, c
     {
       // rows without a usable list go to the dense-tile path, all of the warp's at once
       const unsigned mdense =
-          __ballot_sync(0xffffffffu, lane < 16 && my_row < total && (mc0 < 0 || mc1 < 0 || mc0 + mc1 == 0));
+          __ballot_sync(0xffffffffu, lane < 16 && my_row < total && mc < 1);
       push_dense_tiles(p, mdense, my_row, row_cnt, fb_count, fb_list, tile_flag, tile_list, tile_count, status, lane);
       mfull &= ~mdense;
       // ... and the ones with long lists to a launch of their own
-      const unsigned mlong = __ballot_sync(0xffffffffu, lane < 16 && ((mfull >> lane) & 1u) && mc0 + mc1 > (kClosed ? kLongRow : 32));
+      const unsigned mlong = __ballot_sync(0xffffffffu, lane < 16 && ((mfull >> lane) & 1u) && mc > (kClosed ? kLongRow : 32));
       push_long_rows(mlong, my_row, total, fb_count, fb_list, lane);
       mfull &= ~mlong;
     }
@@ -683,18 +677,17 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32) row_fwd_kernel(Problem p, c
       while (m8) {
         const unsigned src = __fns(m8, 0, (lane >> 3) + 1);        // the row of this group of eight lanes
         const bool active = src < 32u;
-        const int c0 = __shfl_sync(0xffffffffu, mc0, active ? src : 0), c1 = __shfl_sync(0xffffffffu, mc1, active ? src : 0);
-        solve_rows_closed<D, 8, EC>(p, v, scale, entries, o, tau_out, row_cnt, active ? 16 * blk + (int)src : 0, active, c0,
-                                    c1, false, lane);
+        const int n_list = __shfl_sync(0xffffffffu, mc, active ? src : 0);
+        solve_rows_closed<D, 8, EC>(p, v, scale, entries, o, tau_out, row_cnt, active ? 16 * blk + (int)src : 0, active, n_list, false, lane);
 #pragma unroll
         for (int t = 0; t < 4; ++t) m8 &= m8 - 1;
       }
       while (m16) {
         const unsigned src = __fns(m16, 0, (lane >> 4) + 1);
         const bool active = src < 32u;
-        const int c0 = __shfl_sync(0xffffffffu, mc0, active ? src : 0), c1 = __shfl_sync(0xffffffffu, mc1, active ? src : 0);
+        const int n_list = __shfl_sync(0xffffffffu, mc, active ? src : 0);
         solve_rows_closed<D, 16, EC>(p, v, scale, entries, o, tau_out, row_cnt, active ? 16 * blk + (int)src : 0, active,
-                                     c0, c1, false, lane);
+                                     n_list, false, lane);
         m16 &= m16 - 1;
         m16 &= m16 - 1;
       }
@@ -708,9 +701,8 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32) row_fwd_kernel(Problem p, c
         if ((m8 & gm) != 0u && ((m8 | none) & gm) == gm) {
           const int src = 4 * g + (lane >> 3);
           const bool active = (m8 >> src) & 1u;
-          const int c0 = __shfl_sync(0xffffffffu, mc0, src), c1 = __shfl_sync(0xffffffffu, mc1, src);
-          solve_rows_sub<D, 8>(p, v, scale, entries, o, tau_out, row_cnt, half_thr, active ? 16 * blk + src : 0, active, c0,
-                               c1, lane);
+          const int n_list = __shfl_sync(0xffffffffu, mc, src);
+          solve_rows_sub<D, 8>(p, v, scale, entries, o, tau_out, row_cnt, list_thr, active ? 16 * blk + src : 0, active, n_list, lane);
         } else {
           mfull |= (m8 | m16) & gm;
         }
@@ -720,8 +712,8 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32) row_fwd_kernel(Problem p, c
       const int src = __ffs(mfull) - 1;
       mfull &= mfull - 1;
       const int grow = 16 * blk + src;
-      const int c0 = __shfl_sync(0xffffffffu, mc0, src), c1 = __shfl_sync(0xffffffffu, mc1, src);
-      row_fwd_whole_warp<D, EC>(p, v, scale, row_cnt, half_thr, entries, o, tau_out, grow, c0, c1, lane);
+      const int n_list = __shfl_sync(0xffffffffu, mc, src);
+      row_fwd_whole_warp<D, EC>(p, v, scale, row_cnt, list_thr, entries, o, tau_out, grow, n_list, lane);
     }
   }
 }
@@ -733,8 +725,7 @@ __device__ __noinline__ void bwd_row_full(const Problem& p, const __nv_bfloat16*
                                              const __nv_bfloat16* __restrict__ d_o, const float* __restrict__ scale,
                                              const float* __restrict__ tau_in, const Entry* __restrict__ entries,
                                              __nv_bfloat16* __restrict__ dq, float* __restrict__ acc_dk,
-                                             float* __restrict__ acc_dv, float* __restrict__ dc_rows, int grow, int c0,
-                                             int c1, bool saved, int pitch, int lane) {
+                                             float* __restrict__ acc_dv, float* __restrict__ dc_rows, int grow, int n_list, bool saved, int pitch, int lane) {
   constexpr int PER = D / 32;
   const int bh = grow / p.N, i = grow - bh * p.N, b = bh / p.H, h = bh - b * p.H;
   const float g = scale[(size_t)b * p.scale_sb + (size_t)h * p.N + i] * p.sm_scale;
@@ -749,13 +740,13 @@ __device__ __noinline__ void bwd_row_full(const Problem& p, const __nv_bfloat16*
   int jj[kSlots];
 #pragma unroll
   for (int s = 0; s < kSlots; ++s) {
-    const int e = lane + 32 * s;                     // dense numbering: first half-list, then second
+    const int e = lane + 32 * s;  
     yv[s] = -1.0f;
     jj[s] = 0;
     dpv[s] = 0.f;
     zz[s] = 0.f;
-    if (e < c0 + c1) {
-      const Entry en = list[e < c0 ? e : kHalfCap + e - c0];
+    if (e < n_list) {
+      const Entry en = list[e];
       // a list saved by the forward pass holds y = (alpha-1) s in Eq. 1's units, a fresh one raw <q_i, k_j>
       yv[s] = saved ? en.y - tau : fmaf(a, en.y, -tau);
       jj[s] = en.j;
@@ -894,12 +885,12 @@ __device__ __forceinline__ void bwd_rows_sub(const Problem& p, const __nv_bfloat
                                              const float* __restrict__ tau_in, const Entry* __restrict__ entries,
                                              __nv_bfloat16* __restrict__ dq, float* __restrict__ acc_dk,
                                              float* __restrict__ acc_dv, float* __restrict__ dc_rows, int grow,
-                                             bool active, int c0, int c1, bool saved, int pitch, int lane) {
+                                             bool active, int n_list, bool saved, int pitch, int lane) {
   constexpr int PL = D / W;                        // elements of a row per lane
   constexpr unsigned kWMask = W == 32 ? 0xffffffffu : ((1u << (W & 31)) - 1u);
   const int sl = lane & (W - 1);
   const int base = lane & (32 - W);
-  const int n = active ? c0 + c1 : 0;
+  const int n = active ? n_list : 0;
   const int bh = grow / p.N, i = grow - bh * p.N, b = bh / p.H, h = bh - b * p.H;
   const float g = active ? scale[(size_t)b * p.scale_sb + (size_t)h * p.N + i] * p.sm_scale : 0.f;
   const float a = (p.alpha - 1.0f) * g;
@@ -912,7 +903,7 @@ __device__ __forceinline__ void bwd_rows_sub(const Problem& p, const __nv_bfloat
   float yv = -1.0f, zz = 0.f;
   int j = 0;
   if (sl < n) {
-    const Entry en = list[sl < c0 ? sl : kHalfCap + sl - c0];
+    const Entry en = list[sl];
     // a list saved by the forward pass holds y = (alpha-1) s in Eq. 1's units, a fresh one raw <q_i, k_j>
     yv = saved ? en.y - tau : fmaf(a, en.y, -tau);
     j = en.j;
@@ -979,10 +970,10 @@ template <int D>
 __global__ void __launch_bounds__(kWarpsPerCta * 32, 4) row_bwd_kernel(
     Problem p, const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k,
     const __nv_bfloat16* __restrict__ v, const __nv_bfloat16* __restrict__ d_o, const float* __restrict__ scale,
-    const float* __restrict__ tau_in, const int32_t* __restrict__ half_cnt, const Entry* __restrict__ entries,
+    const float* __restrict__ tau_in, const int32_t* __restrict__ list_cnt, const Entry* __restrict__ entries,
     __nv_bfloat16* __restrict__ dq, float* __restrict__ acc_dk, float* __restrict__ acc_dv,
     float* __restrict__ dc_rows, int32_t* fb_count, int32_t* fb_list, int32_t* status, int saved, int pitch) {
-  // saved != 0: `half_cnt` is the forward pass's final support size per row (one int per row, -2 = dense
+  // saved != 0: `list_cnt` is the forward pass's final support size per row (one int per row, -2 = dense
   // row) and `entries` its compacted support lists; `pitch` = list slots per row in `entries`
   const int lane = threadIdx.x & 31;
   const int total = p.B * p.H * p.N;
@@ -991,18 +982,11 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 4) row_bwd_kernel(
     // A warp takes 16 consecutive rows; lane l (and l + 16) looks at row 16*blk + l.  Rows are served by list
     // length: four at a time (<= 8 entries), two at a time (<= 16), one at a time (<= 32, or the long form).
     const int my_row = 16 * blk + (lane & 15);
-    int mc0 = 0, mc1 = 0;
+    int mc = 0;
     int cls = 4;                                     // 0: <= 8 entries, 1: <= 16, 2: <= 32, 3: more / dense, 4: no row
     if (my_row < total) {
-      if (saved) {
-        mc0 = half_cnt[my_row];
-      } else {
-        const int2 c = *reinterpret_cast<const int2*>(half_cnt + 2 * (size_t)my_row);
-        mc0 = c.x;
-        mc1 = c.y;
-      }
-      const int n = mc0 + mc1;
-      cls = (mc0 < 0 || mc1 < 0 || n > 32) ? 3 : n <= 8 ? 0 : n <= 16 ? 1 : 2;
+      mc = list_cnt[saved ? (size_t)my_row : 2 * (size_t)my_row];
+      cls = (mc < 0 || mc > 32) ? 3 : mc <= 8 ? 0 : mc <= 16 ? 1 : 2;
     }
     unsigned m8 = __ballot_sync(0xffffffffu, lane < 16 && cls == 0);
     unsigned m16 = __ballot_sync(0xffffffffu, lane < 16 && cls == 1);
@@ -1010,7 +994,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 4) row_bwd_kernel(
     unsigned mlong = __ballot_sync(0xffffffffu, lane < 16 && cls == 3);
     {
       // rows without a usable list go to the dense path, all of the warp's at once
-      const unsigned mdense = __ballot_sync(0xffffffffu, lane < 16 && my_row < total && (mc0 < 0 || mc1 < 0));
+      const unsigned mdense = __ballot_sync(0xffffffffu, lane < 16 && my_row < total && mc < 0);
       push_dense_rows(mdense, my_row, fb_count, fb_list, status, lane);
       mlong &= ~mdense;
       // ... and the ones with long lists to a launch of their own (see push_long_rows)
@@ -1019,18 +1003,18 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 4) row_bwd_kernel(
     while (m8) {
       const unsigned src = __fns(m8, 0, (lane >> 3) + 1);          // the row of this group of eight lanes
       const bool active = src < 32u;
-      const int c0 = __shfl_sync(0xffffffffu, mc0, active ? src : 0), c1 = __shfl_sync(0xffffffffu, mc1, active ? src : 0);
+      const int n_list = __shfl_sync(0xffffffffu, mc, active ? src : 0);
       bwd_rows_sub<D, 8>(p, q, k, v, d_o, scale, tau_in, entries, dq, acc_dk, acc_dv, dc_rows,
-                         active ? 16 * blk + (int)src : 0, active, c0, c1, saved != 0, pitch, lane);
+                         active ? 16 * blk + (int)src : 0, active, n_list, saved != 0, pitch, lane);
 #pragma unroll
       for (int t = 0; t < 4; ++t) m8 &= m8 - 1;
     }
     while (m16) {
       const unsigned src = __fns(m16, 0, (lane >> 4) + 1);
       const bool active = src < 32u;
-      const int c0 = __shfl_sync(0xffffffffu, mc0, active ? src : 0), c1 = __shfl_sync(0xffffffffu, mc1, active ? src : 0);
+      const int n_list = __shfl_sync(0xffffffffu, mc, active ? src : 0);
       bwd_rows_sub<D, 16>(p, q, k, v, d_o, scale, tau_in, entries, dq, acc_dk, acc_dv, dc_rows,
-                          active ? 16 * blk + (int)src : 0, active, c0, c1, saved != 0, pitch, lane);
+                          active ? 16 * blk + (int)src : 0, active, n_list, saved != 0, pitch, lane);
       m16 &= m16 - 1;
       m16 &= m16 - 1;
     }
@@ -1042,7 +1026,7 @@ template <int D>
 __global__ void __launch_bounds__(kWarpsPerCta * 32, 4) row_bwd_long_kernel(
     Problem p, const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k,
     const __nv_bfloat16* __restrict__ v, const __nv_bfloat16* __restrict__ d_o, const float* __restrict__ scale,
-    const float* __restrict__ tau_in, const int32_t* __restrict__ half_cnt, const Entry* __restrict__ entries,
+    const float* __restrict__ tau_in, const int32_t* __restrict__ list_cnt, const Entry* __restrict__ entries,
     __nv_bfloat16* __restrict__ dq, float* __restrict__ acc_dk, float* __restrict__ acc_dv,
     float* __restrict__ dc_rows, const int32_t* __restrict__ fb_count, const int32_t* __restrict__ fb_list, int saved,
     int pitch) {
@@ -1051,19 +1035,12 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 4) row_bwd_long_kernel(
   const int n_long = fb_count[kLongCounter];
   for (int t = blockIdx.x * kWarpsPerCta + (threadIdx.x >> 5); t < n_long; t += gridDim.x * kWarpsPerCta) {
     const int grow = fb_list[total - 1 - t];
-    int c0, c1 = 0;
-    if (saved) {
-      c0 = half_cnt[grow];
-    } else {
-      const int2 c = *reinterpret_cast<const int2*>(half_cnt + 2 * (size_t)grow);
-      c0 = c.x;
-      c1 = c.y;
-    }
-    if (c0 + c1 <= 32)
-      bwd_rows_sub<D, 32>(p, q, k, v, d_o, scale, tau_in, entries, dq, acc_dk, acc_dv, dc_rows, grow, true, c0, c1,
+    const int n_list = list_cnt[saved ? (size_t)grow : 2 * (size_t)grow];
+    if (n_list <= 32)
+      bwd_rows_sub<D, 32>(p, q, k, v, d_o, scale, tau_in, entries, dq, acc_dk, acc_dv, dc_rows, grow, true, n_list,
                           saved != 0, pitch, lane);
     else
-      bwd_row_full<D>(p, q, k, v, d_o, scale, tau_in, entries, dq, acc_dk, acc_dv, dc_rows, grow, c0, c1, saved != 0,
+      bwd_row_full<D>(p, q, k, v, d_o, scale, tau_in, entries, dq, acc_dk, acc_dv, dc_rows, grow, n_list, saved != 0,
                       pitch, lane);
   }
 }
@@ -1093,13 +1070,13 @@ inline int row_grid(const Problem& p) {
 }  // namespace
 
 cudaError_t launch_row_fwd(const Problem& p, const void* v, const float* scale, int32_t* row_cnt,
-                           const int32_t* half_cnt, const float* half_thr, Entry* entries, void* o, float* tau,
+                           const int32_t* list_cnt, const float* list_thr, Entry* entries, void* o, float* tau,
                            int32_t* fb_count, int32_t* fb_list, int32_t* tile_flag, int32_t* tile_list,
                            int32_t* tile_count, int32_t* status, cudaStream_t stream) {
   const int grid = row_grid(p);
 #define ENTMAX_ROW_FWD(D, EC)                                                                                         \
-  row_fwd_kernel<D, EC><<<grid, kWarpsPerCta * 32, 0, stream>>>(p, (const __nv_bfloat16*)v, scale, row_cnt, half_cnt, \
-                                                                half_thr, entries, (__nv_bfloat16*)o, tau, fb_count,  \
+  row_fwd_kernel<D, EC><<<grid, kWarpsPerCta * 32, 0, stream>>>(p, (const __nv_bfloat16*)v, scale, row_cnt, list_cnt, \
+                                                                list_thr, entries, (__nv_bfloat16*)o, tau, fb_count,  \
                                                                 fb_list,                                              \
                                                                 tile_flag, tile_list, tile_count, status)
   if (p.D == 64) {
@@ -1118,7 +1095,7 @@ cudaError_t launch_row_fwd(const Problem& p, const void* v, const float* scale, 
   const int lgrid = grid < 148 * 4 ? grid : 148 * 4;
 #define ENTMAX_ROW_FWD_LONG(D, EC)                                                                                     \
   row_fwd_long_kernel<D, EC><<<lgrid, kWarpsPerCta * 32, 0, stream>>>(p, (const __nv_bfloat16*)v, scale, row_cnt,       \
-                                                                      half_cnt, half_thr, entries, (__nv_bfloat16*)o,  \
+                                                                      list_cnt, list_thr, entries, (__nv_bfloat16*)o,  \
                                                                       tau, fb_count, fb_list)
   if (p.D == 64) {
     if (p.expo_class == kExpo2) ENTMAX_ROW_FWD_LONG(64, kExpo2);
@@ -1143,18 +1120,18 @@ cudaError_t launch_save_supports(const Problem& p, int slots, const int32_t* row
 }
 
 cudaError_t launch_row_bwd(const Problem& p, const void* q, const void* k, const void* v, const void* d_o,
-                           const float* scale, const float* tau, const int32_t* half_cnt, Entry* entries, void* dq,
+                           const float* scale, const float* tau, const int32_t* list_cnt, Entry* entries, void* dq,
                            float* acc_dk, float* acc_dv, float* dc_rows, int32_t* fb_count, int32_t* fb_list,
                            int32_t* status, int saved, int pitch, cudaStream_t stream) {
   const int grid = row_grid(p);
   if (p.D == 64)
     row_bwd_kernel<64><<<grid, kWarpsPerCta * 32, 0, stream>>>(
         p, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, (const __nv_bfloat16*)d_o, scale,
-        tau, half_cnt, entries, (__nv_bfloat16*)dq, acc_dk, acc_dv, dc_rows, fb_count, fb_list, status, saved, pitch);
+        tau, list_cnt, entries, (__nv_bfloat16*)dq, acc_dk, acc_dv, dc_rows, fb_count, fb_list, status, saved, pitch);
   else
     row_bwd_kernel<128><<<grid, kWarpsPerCta * 32, 0, stream>>>(
         p, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, (const __nv_bfloat16*)d_o, scale,
-        tau, half_cnt, entries, (__nv_bfloat16*)dq, acc_dk, acc_dv, dc_rows, fb_count, fb_list, status, saved, pitch);
+        tau, list_cnt, entries, (__nv_bfloat16*)dq, acc_dk, acc_dv, dc_rows, fb_count, fb_list, status, saved, pitch);
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) return err;
   // the rows it listed as long, one warp each (normally none or a few: the launch then ends at once)
@@ -1162,11 +1139,11 @@ cudaError_t launch_row_bwd(const Problem& p, const void* q, const void* k, const
   if (p.D == 64)
     row_bwd_long_kernel<64><<<lgrid, kWarpsPerCta * 32, 0, stream>>>(
         p, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, (const __nv_bfloat16*)d_o, scale,
-        tau, half_cnt, entries, (__nv_bfloat16*)dq, acc_dk, acc_dv, dc_rows, fb_count, fb_list, saved, pitch);
+        tau, list_cnt, entries, (__nv_bfloat16*)dq, acc_dk, acc_dv, dc_rows, fb_count, fb_list, saved, pitch);
   else
     row_bwd_long_kernel<128><<<lgrid, kWarpsPerCta * 32, 0, stream>>>(
         p, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, (const __nv_bfloat16*)d_o, scale,
-        tau, half_cnt, entries, (__nv_bfloat16*)dq, acc_dk, acc_dv, dc_rows, fb_count, fb_list, saved, pitch);
+        tau, list_cnt, entries, (__nv_bfloat16*)dq, acc_dk, acc_dv, dc_rows, fb_count, fb_list, saved, pitch);
   return cudaGetLastError();
 }
 

@@ -41,14 +41,19 @@ namespace {
 
 constexpr int BM = 128;          // query rows per Q tile = TMEM lanes
 constexpr int BN = 256;          // keys per K tile = N of one MMA = TMEM columns of one accumulator
-constexpr int kHalfCols = BN / 2;   // columns of a K tile one consumer thread scans
 constexpr int kQTiles = 2;       // Q tiles per item
 constexpr int kItemRows = BM * kQTiles;
-constexpr int kConsumerWarps = 8 * kQTiles;
+constexpr int kConsumerWarps = 4 * kQTiles;   // one thread per query row
 constexpr int kThreads = (2 + kConsumerWarps) * 32;
 constexpr int kTmemCols = kQTiles * BN;
 constexpr int kSchedSlots = 2;
-static_assert(kTmemCols == 512 && kHalfCols == 128, "TMEM budget / consumer split");
+static_assert(kTmemCols == 512, "TMEM budget");
+
+// Slots per consumer thread for what its scan of a tile found: eight consecutive accumulators of its row that hold at least
+// one candidate.  Slot s of a warp: two float4 arrays.
+constexpr int kSlots = 4;
+constexpr int kSlotHi = 32 * 16, kSlotStep = 2 * kSlotHi;
+constexpr int kSlotBytes = kSlots * kSlotStep;
 
 template <int HD>
 struct Cfg {
@@ -56,9 +61,10 @@ struct Cfg {
   static constexpr int kQBytes = BM * HD * 2;
   static constexpr int kKBytes = BN * HD * 2;
   static constexpr int kStages = HD == 128 ? 2 : 4;
-  static constexpr int kShareBytes = kQTiles * 2 * BM * 8;   // running maxima shared by the two halves of a row
   static constexpr int kBarBytes = 512;
-  static constexpr int kSmemBytes = kQTiles * kQBytes + kStages * kKBytes + kShareBytes + 1024 /*align*/ + kBarBytes;
+  static constexpr int kSmemBytes =
+      kQTiles * kQBytes + kStages * kKBytes + kConsumerWarps * kSlotBytes + 1024 /*align*/ + kBarBytes;
+  static_assert(kSmemBytes <= 232448, "shared memory of one CTA");
 };
 
 struct SweepArgs {
@@ -72,9 +78,9 @@ struct SweepArgs {
   const float* scale;   // [H, N] (scale_sb = 0) or [B, H, N] (scale_sb = H*N)
   long long scale_sb;
   const float* tau_in;  // [B*H*N] (mode 1)
-  int32_t* half_cnt;    // [B*H*N][2] list length of each half-row; -1 = hand the row to the dense path
-  float* half_thr;      // [B*H*N][2] lower bound on tau each half-row ended with (Eq. 1's units)
-  Entry* entries;       // [B*H*N][kListCap]; half h of a row owns slots [h*kHalfCap, (h+1)*kHalfCap)
+  int32_t* list_cnt;    // [B*H*N][2] list length of the row in the first word; -1 = hand the row to the dense path
+  float* list_thr;      // [B*H*N] lower bound on tau the row ended with (Eq. 1's units; forward)
+  Entry* entries;       // [B*H*N][kListCap]
   float* dump;          // kDump kernels: optional [N, N] raw accumulators of head dump_bh; kAlibi kernels: the
                         // [H] ALiBi slopes m_h (z_ij += m_h (j - i), j <= i).  One member for both keeps the
                         // argument block, and with it the register allocation of the plain kernel, unchanged
@@ -122,8 +128,9 @@ __device__ __forceinline__ int qtile_tiles(const SweepArgs& a, int item, int x) 
 // running maximum, about ln n of them per row; after a 1/16 sample about ln 16 are left; measured best among 8, 16, 32, 64).
 constexpr int kSampleStride = 8;
 constexpr int kSampleMinKeys = 4096;   // below this the stream is too short for the sample to pay
+template <bool kSearch>
 __device__ __forceinline__ int sample_tiles(const SweepArgs& a, int item) {
-  if (a.mode != 0) return 0;
+  if (!kSearch) return 0;
   int last_row = item * kItemRows + kItemRows - 1;
   if (last_row > a.N - 1) last_row = a.N - 1;
   const int n_vis = a.causal ? last_row + 1 : a.N;
@@ -152,19 +159,18 @@ __device__ __forceinline__ int first_tile(const SweepArgs& a, int k) {
 
 // ------------------------------------------------------------- consumer side: one half-row per thread
 struct RowState {
-  float thr;       // candidates are accumulators above this (accumulator units)
-  float m_run;     // running maximum accumulator (both halves of the row, as far as known)
+  float thr;       // candidates are accumulators above this (accumulator units); +inf: none any more
   int cnt;         // half-list length; -1 = handed to the dense path
 };
 
-// Warp-cooperative list shrink for the lanes whose half-list has grown past kHalfTrigger.  Accumulator
+// Warp-cooperative list shrink for the lanes whose list has grown past kListTrigger.  Accumulator
 // units are turned into Eq. 1's units with y = a * acc.  All 32 lanes must call this together.
 // Takes and returns the row state by value: a state whose address escaped would have to be kept in
 // local memory across every asm statement of the scan loop.
-__device__ __noinline__ RowState shrink_lists(RowState r, Entry* list, float a, float inv_a, unsigned need, int mode,
+__device__ __forceinline__ RowState shrink_lists(RowState r, Entry* list, float a, float inv_a, unsigned need, int mode,
                                               int expo_class, float expo) {
   const int lane = threadIdx.x & 31;
-  constexpr int kSlots = kHalfCap / 32;
+  constexpr int kPer = kListCap / 32;
   __syncwarp();   // the owner's list stores are ordered before the other lanes' loads
   while (need) {
     const int src = __ffs(need) - 1;
@@ -177,9 +183,9 @@ __device__ __noinline__ RowState shrink_lists(RowState r, Entry* list, float a, 
     float new_thr = INFINITY;
     int kept = -1;
     if (mode == 0) {
-      Entry e[kSlots];
+      Entry e[kPer];
 #pragma unroll
-      for (int s = 0; s < kSlots; ++s) {
+      for (int s = 0; s < kPer; ++s) {
         const int idx = lane + 32 * s;
         e[s].y = -INFINITY;
         e[s].j = 0;
@@ -187,22 +193,22 @@ __device__ __noinline__ RowState shrink_lists(RowState r, Entry* list, float a, 
       }
       // A sure case first.  With y_max the largest of the c listed keys, sum_j (y_max - tau)^e >= sum_j [y_j - tau]_+^e
       // = 1 at the list's own threshold tau*, so tau* <= y_max - c^(-1/e): every listed key above that is in the
-      // list's support.  If those alone are more than a half-list may keep, the row goes to the dense path without a
+      // list's support.  If those alone are more than a list may keep, the row goes to the dense path without a
       // solve (rows of flat logits, which would otherwise each pay a full Newton solve just to be handed over).
       bool sure_dense = false;
       {
         float ym = -INFINITY;
 #pragma unroll
-        for (int s = 0; s < kSlots; ++s) ym = fmaxf(ym, e[s].y);
+        for (int s = 0; s < kPer; ++s) ym = fmaxf(ym, e[s].y);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) ym = fmaxf(ym, __shfl_xor_sync(0xffffffffu, ym, o));
         const float width = expo_class == kExpo2 ? rsqrtf((float)c) : expo_class == kExpo1 ? 1.0f / (float)c
-                                                                                           : powf((float)c, -1.0f / expo);
+                                                                                           : __powf((float)c, -1.0f / expo);
         const float cut = ym - width * inv_aa;
         int sure = 0;
 #pragma unroll
-        for (int s = 0; s < kSlots; ++s) sure += __popc(__ballot_sync(0xffffffffu, e[s].y > cut));
-        sure_dense = sure > kHalfKeep;
+        for (int s = 0; s < kPer; ++s) sure += __popc(__ballot_sync(0xffffffffu, e[s].y > cut));
+        sure_dense = sure > kListKeep;
       }
       float tau = th * aa;
       if (sure_dense) {
@@ -211,19 +217,24 @@ __device__ __noinline__ RowState shrink_lists(RowState r, Entry* list, float a, 
         for (int it = 0; it < 8; ++it) {
           float s0 = 0.f, s1 = 0.f;
 #pragma unroll
-          for (int s = 0; s < kSlots; ++s) {
+          for (int s = 0; s < kPer; ++s) {
             const float y = fmaf(aa, e[s].y, -tau);
             if (y > 0.f) {
-              float ye, ye1;
-              pow_pair(y, expo_class, expo, ye, ye1);
-              s0 += ye;
+              float ye1 = y;
+              if (expo_class == kExpo1) ye1 = 1.0f;
+              else if (expo_class == kExpo4) ye1 = y * y * y;
+              else if (expo_class == kExpoGeneral) ye1 = __powf(y, expo - 1.0f);
+              s0 = fmaf(ye1, y, s0);
               s1 += ye1;
             }
           }
           s0 = warp_sum(s0);
           s1 = warp_sum(s1);
           if (!(s0 > 1.0f) || !(s1 > 0.f)) break;
-          const float step = threshold_step(s0, s1, expo_class, expo);
+          const float root = expo_class == kExpo1 ? s0
+                             : expo_class == kExpo2 ? sqrtf(s0)
+                             : expo_class == kExpo4 ? sqrtf(sqrtf(s0)) : __powf(s0, 1.0f / expo);
+          const float step = (s0 - s0 / root) / s1;      // threshold_step
           tau += step;
           if (step <= 1e-4f) break;
         }
@@ -235,29 +246,31 @@ __device__ __noinline__ RowState shrink_lists(RowState r, Entry* list, float a, 
           const float mid = 0.5f * (lo + hi);
           float s0 = 0.f;
 #pragma unroll
-          for (int s = 0; s < kSlots; ++s) {
+          for (int s = 0; s < kPer; ++s) {
             const float y = fmaf(aa, e[s].y, -mid);
-            if (y > 0.f) s0 += powf(y, expo);
+            if (y > 0.f) s0 += __powf(y, expo);
           }
           s0 = warp_sum(s0);
           if (s0 > 1.0f) lo = mid; else hi = mid;
         }
         tau = lo;
       }
-      // a hair below the Newton iterate: rounding must never push the bound past the true threshold
-      new_thr = fmaxf(th, (tau - 4e-6f * fmaxf(1.0f, fabsf(tau))) * inv_aa);
+      // a hair below the Newton iterate: rounding must never push the bound past the true threshold (general exponents:
+      // the fast powers are good to about 1e-5 of the mass, and d tau <= d mass where the mass is 1 or more)
+      const float hair = 4e-6f * fmaxf(1.0f, fabsf(tau)) + (expo_class == kExpoGeneral ? 5e-5f : 0.f);
+      new_thr = fmaxf(th, (tau - hair) * inv_aa);
       __syncwarp();
       kept = 0;
       if (!sure_dense) {
 #pragma unroll
-        for (int s = 0; s < kSlots; ++s) {
+        for (int s = 0; s < kPer; ++s) {
           const bool keep = e[s].y > new_thr;
           const unsigned m = __ballot_sync(0xffffffffu, keep);
           if (keep) l[kept + __popc(m & ((1u << lane) - 1u))] = e[s];
           kept += __popc(m);
         }
       }
-      if (kept > kHalfKeep || sure_dense) {
+      if (kept > kListKeep || sure_dense) {
         kept = -1;
         new_thr = INFINITY;
       }
@@ -271,20 +284,34 @@ __device__ __noinline__ RowState shrink_lists(RowState r, Entry* list, float a, 
   return r;
 }
 
-template <int HD, bool kDump, bool kAlibi>
+// The eight column groups of a 64-column step (the first is group G0 of the tile): see the consumers
+template <int G0>
+__device__ __forceinline__ void scan_groups(const float (&g)[8], float thr, uint32_t& at, uint32_t my_slot, uint32_t& groups,
+                                            const float (&v)[64]) {
+  const uint32_t last = my_slot + (kSlots - 1) * kSlotStep;
+  sts_record8_if_greater<kSlotHi, kSlotStep, G0 + 0>(g[0], thr, at, last, groups, &v[0]);
+  sts_record8_if_greater<kSlotHi, kSlotStep, G0 + 1>(g[1], thr, at, last, groups, &v[8]);
+  sts_record8_if_greater<kSlotHi, kSlotStep, G0 + 2>(g[2], thr, at, last, groups, &v[16]);
+  sts_record8_if_greater<kSlotHi, kSlotStep, G0 + 3>(g[3], thr, at, last, groups, &v[24]);
+  sts_record8_if_greater<kSlotHi, kSlotStep, G0 + 4>(g[4], thr, at, last, groups, &v[32]);
+  sts_record8_if_greater<kSlotHi, kSlotStep, G0 + 5>(g[5], thr, at, last, groups, &v[40]);
+  sts_record8_if_greater<kSlotHi, kSlotStep, G0 + 6>(g[6], thr, at, last, groups, &v[48]);
+  sts_record8_if_greater<kSlotHi, kSlotStep, G0 + 7>(g[7], thr, at, last, groups, &v[56]);
+}
+
+template <int HD, bool kDump, bool kAlibi, bool kSearch>
 __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constant__ CUtensorMap map_q,
                                                             const __grid_constant__ CUtensorMap map_k,
                                                             const __grid_constant__ CUtensorMap map_ks,
-                                                            const SweepArgs a) {
+                                                            const __grid_constant__ SweepArgs a) {
   using C = Cfg<HD>;
   extern __shared__ uint8_t smem_raw[];
   // everything in shared memory is addressed by 32-bit shared-window addresses derived from one base
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t q_smem = sbase;                                   // [kQTiles][kHalves][BM rows x 128 B]
   const uint32_t k_smem = sbase + kQTiles * C::kQBytes;            // [kStages][kHalves][BN rows x 128 B]
-  // running maximum of each half-row, tagged with the work item it belongs to: {item id, float bits}
-  const uint32_t m_share = k_smem + C::kStages * C::kKBytes;       // u64 [kQTiles][2][BM]
-  const uint32_t bars = m_share + C::kShareBytes;                  // mbarriers, 8 bytes each
+  const uint32_t slots = k_smem + C::kStages * C::kKBytes;         // [kConsumerWarps][kSlotBytes]
+  const uint32_t bars = slots + kConsumerWarps * kSlotBytes;       // mbarriers, 8 bytes each
   const uint32_t q_full = bars;                            // [kQTiles]
   const uint32_t q_empty = q_full + 8 * kQTiles;           // [kQTiles]
   const uint32_t s_full = q_empty + 8 * kQTiles;           // [kQTiles]
@@ -301,7 +328,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
   static_assert((4 * kQTiles + 2 * C::kStages + 2 * kSchedSlots) * 8 + kSchedSlots * 4 + 8 + 16 <= C::kBarBytes,
                 "barrier area");
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);   // (the same in every lane, and known to be)
   const int lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
@@ -309,7 +336,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
       mbar_init(q_full + 8 * t, 1);
       mbar_init(q_empty + 8 * t, 1);
       mbar_init(s_full + 8 * t, 1);
-      mbar_init(s_empty + 8 * t, 8);                 // one arrival per consumer warp of the Q tile
+      mbar_init(s_empty + 8 * t, 4);                 // one arrival per consumer warp of the Q tile
     }
     for (int t = 0; t < C::kStages; ++t) {
       mbar_init(k_full + 8 * t, 1);
@@ -325,7 +352,6 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
-  if (threadIdx.x < kQTiles * 2 * BM) sts_u64(m_share + 8 * threadIdx.x, ~0ull);   // tag -1: belongs to no work item
   if (warp == 1) {
     tmem_alloc(tmem_slot, kTmemCols);
     tmem_relinquish();
@@ -368,7 +394,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
         }
         // tiles before tf (and sampled tiles before ts0) lie outside the ALiBi window: t counts from there
         const int tf = __shfl_sync(0xffffffffu, first_tile<kAlibi>(a, k), 0);
-        const int ts_all = sample_tiles(a, item);
+        const int ts_all = sample_tiles<kSearch>(a, item);
         const int ts0 = kAlibi ? min(tf / kSampleStride, ts_all) : 0;
         const int ts = ts_all - ts0;
         tiles -= tf;
@@ -445,7 +471,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
           tiles = tx[x] > tiles ? tx[x] : tiles;
         }
         const int tf = __shfl_sync(0xffffffffu, first_tile<kAlibi>(a, k), 0);
-        const int ts_all = sample_tiles(a, item);
+        const int ts_all = sample_tiles<kSearch>(a, item);
         const int ts = ts_all - (kAlibi ? min(tf / kSampleStride, ts_all) : 0);
         tiles -= tf;
         for (int x = 0; x < kQTiles; ++x) tx[x] = tx[x] > 0 ? tx[x] - tf : 0;   // every valid Q tile reaches past tf
@@ -492,23 +518,21 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
       }
     }
   } else {
-    // -------------------------------------------------- consumers: one thread per half of a query row
+    // -------------------------------------------------- consumers: one thread per query row
     const int cw = warp - 2;
-    const int x = cw >> 3;                         // Q tile of this warp
-    const int half = (cw >> 2) & 1;                // which 128 columns of every K tile
+    const int x = cw >> 2;                         // Q tile of this warp
     const int quad = warp & 3;                     // TMEM lane quadrant this warp may read
     const int row_local = quad * 32 + lane;
-    const uint32_t taddr_row = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(x * BN + half * kHalfCols);
-    const uint32_t my_share = m_share + 8 * ((x * 2 + half) * BM + row_local);
-    const uint32_t other_share = m_share + 8 * ((x * 2 + (half ^ 1)) * BM + row_local);
+    const uint32_t taddr_row = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(x * BN);
     const uint32_t my_full = s_full + 8 * x, my_empty = s_empty + 8 * x;
+    const uint32_t my_slot = slots + (uint32_t)(cw * kSlotBytes + 16 * lane);
     uint32_t fphase = 0, wphase = 0;
     int slot = 0;
     bool alive = true;
     while (alive) {
       alive = __all_sync(0xffffffffu, mbar_wait(w_full + 8 * slot, wphase, abort_flag));
       if (!alive) break;
-      const int k = (int)lds_u32(w_item + 4 * slot);
+      const int k = __shfl_sync(0xffffffffu, (int)lds_u32(w_item + 4 * slot), 0);
       __syncwarp();
       if (lane == 0) mbar_arrive(w_empty + 8 * slot);
       if (++slot == kSchedSlots) { slot = 0; wphase ^= 1u; }
@@ -521,23 +545,21 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
       const int h = bh % a.H;
       const int tile_row0 = item * kItemRows + x * BM;
       const int i = tile_row0 + row_local;
-      const bool valid = i < a.N;
-      const size_t grow = (size_t)bh * a.N + (valid ? i : 0);
-      Entry* list = a.entries + grow * kListCap + half * kHalfCap;
+      const int grow = bh * a.N + i;               // (rows past the end never have candidates)
+      Entry* list = a.entries + (size_t)grow * kListCap;
       const int lim = a.causal ? i : a.N - 1;      // largest visible key index
+      // Forward: a value m in the row puts the threshold at m - margin at least (App. A bracket), m_run: the largest so far
       RowState r;
-      r.cnt = 0;
-      r.m_run = -INFINITY;
       r.thr = INFINITY;
-      float ra = 1.f, inv_a = 1.f;
-      if (valid) {
-        ra = a.alpha_m1 * (a.scale[(size_t)(bh / a.H) * a.scale_sb + (size_t)h * a.N + i] * a.sm_scale);
+      r.cnt = 0;
+      float margin = 1.f, m_run = -INFINITY;
+      if (i < a.N) {
+        const float ra = a.alpha_m1 * (a.scale[(size_t)(bh / a.H) * a.scale_sb + (size_t)h * a.N + i] * a.sm_scale);
         if (ra > 0.f && ra < INFINITY) {
-          inv_a = 1.0f / ra;
-          if (a.mode == 0) {
-            r.thr = -INFINITY;
-          } else {
-            const float t_acc = a.tau_in[grow] * inv_a;
+          margin = 1.0f / ra;
+          r.thr = -INFINITY;
+          if constexpr (!kSearch) {
+            const float t_acc = a.tau_in[grow] * margin;
             r.thr = t_acc - 1e-6f * fabsf(t_acc);   // a hair below: the row kernel applies the exact test
           }
         } else {
@@ -547,15 +569,13 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
       // ALiBi (causal): the logit is sm_scale * (acc + slope * (j - i)); everything below works on that sum
       const float slope = kAlibi ? a.dump[h] / a.sm_scale : 0.f;
       const float fi = (float)i;
-      const bool searching = a.mode == 0 && r.cnt == 0 && valid;
-      const bool dump_here = kDump && a.dump != nullptr && bh == a.dump_bh && valid;
-      // first / last visible key over the rows of this Q tile: halves past the last one are skipped,
-      // halves that reach past the first one need the mask
+      // first / last visible key over the rows of this Q tile: chunks past the last one are skipped,
+      // tiles that reach past the first one need the mask
       const int first_lim = a.causal ? tile_row0 : a.N - 1;
       const int last_lim = a.causal ? (tile_row0 + BM - 1 < a.N - 1 ? tile_row0 + BM - 1 : a.N - 1) : a.N - 1;
-      // ---- sampled tiles first (forward mode, long rows): maxima only, nothing is pushed -- every sampled
+      // ---- sampled tiles first (forward mode, long rows): maxima only, nothing is kept -- every sampled
       //      key comes by again in the real stream.  Column c of sampled tile t is key kSampleStride * (t*BN + c).
-      const int ts = sample_tiles(a, item);
+      const int ts = sample_tiles<kSearch>(a, item);
       const int ts0 = kAlibi ? min(tf / kSampleStride, ts) : 0;
       if (kAlibi && a.status && cw == 0 && lane == 0) {
         // K-tile steps of this item left out by the window / still scored
@@ -563,171 +583,196 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
         atomicAdd(a.status + ENTMAX_ATTN_STATUS_SKIPPED_STEPS, tf);
         atomicAdd(a.status + ENTMAX_ATTN_STATUS_SCORED_STEPS, t_item - tf);
       }
-      if (ts > ts0) {
-        // largest sampled group index that is a key this row may look at
+      if (kSearch && ts > ts0) {
+        // largest sampled group index that is a key this row may look at, and the largest all rows may look at
         int glim = lim / kSampleStride;
         if (glim > a.N / kSampleStride - 1) glim = a.N / kSampleStride - 1;
+        const int first_glim = min(first_lim / kSampleStride, a.N / kSampleStride - 1);
         for (int t = ts0; t < ts && alive; ++t) {
           alive = __all_sync(0xffffffffu, mbar_wait(my_full, fphase, abort_flag));
           if (!alive) break;
           fphase ^= 1u;
           tc_fence_after();
-          const int g_base = t * BN + half * kHalfCols;
-          float m_s = -INFINITY;
-          float va[32];
+          const int g_base = t * BN;
+#pragma unroll 1
+          for (int c = 0; c < BN / 64; ++c) {
+            float va[64];
+            tmem_ld64(taddr_row + c * 64, va);
+            tmem_ld_wait64(va);
+            if (kAlibi) {
 #pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            tmem_ld32(taddr_row + c * 32, va);
-            tmem_ld_wait();
-#pragma unroll
-            for (int u = 0; u < 32; ++u) {
-              if (kAlibi) va[u] = fmaf(slope * (float)kSampleStride, (float)u, va[u]);
-              va[u] = (g_base + c * 32 + u <= glim) ? va[u] : -INFINITY;
+              for (int u = 0; u < 64; ++u) va[u] = fmaf(slope * (float)kSampleStride, (float)u, va[u]);
             }
-            float m_c = fmaxf(fmaxf(max8(&va[0]), max8(&va[8])), fmaxf(max8(&va[16]), max8(&va[24])));
-            if (kAlibi) m_c += slope * ((float)(kSampleStride * (g_base + c * 32)) - fi);
-            m_s = fmaxf(m_s, m_c);
+            if (g_base + c * 64 + 63 > first_glim) {
+#pragma unroll
+              for (int u = 0; u < 64; ++u) va[u] = (g_base + c * 64 + u <= glim) ? va[u] : -INFINITY;
+            }
+            float m_c = max8(&va[0]);
+#pragma unroll
+            for (int q = 1; q < 8; ++q) m_c = fmaxf(m_c, max8(&va[8 * q]));
+            if (kAlibi) m_c += slope * ((float)(kSampleStride * (g_base + c * 64)) - fi);
+            m_run = fmaxf(m_run, m_c);
           }
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(my_empty);
-          if (searching) {
-            const unsigned long long o = lds_u64(other_share);
-            const float m_other = (int)(o >> 32) == k ? __uint_as_float((unsigned)o) : -INFINITY;
-            r.m_run = max3(r.m_run, m_s, m_other);
-            r.thr = fmaxf(r.thr, r.m_run - inv_a);
-            sts_u64(my_share, ((unsigned long long)(unsigned)k << 32) | __float_as_uint(r.m_run));
-          }
         }
+        r.thr = fmaxf(r.thr, m_run - margin);
       }
+      // A stream that starts without any bound scans its first tile twice: maxima first, so that the second scan
+      // already has a bound
+      bool blind = kSearch && ts <= ts0;
+      bool crowded = false;                        // the last tile had rows with many candidates
       for (int t = tf; t < tiles && alive; ++t) {
         // the warp leaves together: tcgen05.ld needs all 32 lanes
         alive = __all_sync(0xffffffffu, mbar_wait(my_full, fphase, abort_flag));
         if (!alive) break;
         fphase ^= 1u;
         tc_fence_after();
-        const int col_base = t * BN + half * kHalfCols;
-        bool released = false;
-        if (col_base <= last_lim) {
-          const bool masked = col_base + kHalfCols - 1 > first_lim;
-          // ---- pass 1: 128 columns -> 16 group maxima (8 columns each); four loads of 32 columns (wider
-          //      loads mean fewer TMEM round trips on the path that holds the accumulator)
-          float g[16];
-          float va[32];
+        const int col_base = t * BN;
+        const int nch = min(BN / 32, (last_lim - col_base) / 32 + 1);   // 32-column chunks some row of the tile sees
+        // Away from the mask, as long as candidates are few: one straight pass over the 256 columns without a branch, 64 at a
+        // time with the next 64 on their way.  Maxima of eight columns; eight columns that hold a candidate go to the
+        // thread's next slot as they are, straight from the registers, and are taken apart when the accumulator has been
+        // handed back.  What this kernel's pace hangs on is the time from "accumulator full" to its hand-back, the slowest
+        // warp counting: branches on "some row has a candidate", a second look at TMEM or list stores in between all cost
+        // more there than these predicated stores do.
+        uint32_t at = my_slot, groups = 0u;
+        bool crowd = crowded || col_base + BN - 1 > first_lim || blind || kDump;
+        if (!crowd) {
+          float v0[64], v1[64];
+          tmem_ld64(taddr_row, v0);
 #pragma unroll
-          for (int c = 0; c < 4; ++c) {
+          for (int s = 0; s < 4; ++s) {
+            float (&v)[64] = (s & 1) ? v1 : v0;
+            tmem_ld_wait64(v);
+            if (s < 3) tmem_ld64(taddr_row + 64 * (s + 1), (s & 1) ? v0 : v1);
+            float g[8];
+            if (kAlibi) {
+#pragma unroll
+              for (int u = 0; u < 64; ++u) v[u] = fmaf(slope, (float)u, v[u]);
+              const float t0 = slope * ((float)(col_base + 64 * s) - fi);
+#pragma unroll
+              for (int q = 0; q < 8; ++q) g[q] = max8(&v[8 * q]) + t0;
+            } else {
+#pragma unroll
+              for (int q = 0; q < 8; ++q) g[q] = max8(&v[8 * q]);
+            }
+            if constexpr (kSearch) {
+              m_run = max3(max3(m_run, g[0], g[1]), max3(g[2], g[3], g[4]), max3(g[5], g[6], g[7]));
+              r.thr = fmaxf(r.thr, m_run - margin);
+            }
+            if (s == 0) scan_groups<0>(g, r.thr, at, my_slot, groups, v);
+            else if (s == 1) scan_groups<8>(g, r.thr, at, my_slot, groups, v);
+            else if (s == 2) scan_groups<16>(g, r.thr, at, my_slot, groups, v);
+            else scan_groups<24>(g, r.thr, at, my_slot, groups, v);
+          }
+          // a row had more than its slots take: once more, the other way
+          crowd = __any_sync(0xffffffffu, at > my_slot + kSlots * kSlotStep);
+          if (crowd) at = my_slot;
+        }
+        // Everywhere else 32 columns at a time, with every row appending its candidates to its list directly
+        bool full;
+        int c = crowd ? 0 : nch;
+        if (crowd) crowded = false;
+        do {
+          full = false;
+#pragma unroll 1
+          while (c < nch && !full) {
+            float va[32];
             tmem_ld32(taddr_row + c * 32, va);
             tmem_ld_wait();
+            const int col0 = col_base + c * 32;
             if (kDump) {
-              if (dump_here) {
+              if (a.dump != nullptr && bh == a.dump_bh && i < a.N) {
 #pragma unroll
                 for (int u = 0; u < 32; ++u)
-                  if (col_base + c * 32 + u <= lim) a.dump[(size_t)i * a.N + col_base + c * 32 + u] = va[u];
+                  if (col0 + u <= lim) a.dump[(size_t)i * a.N + col0 + u] = va[u];
               }
             }
             if (kAlibi) {
-              // column part of the bias by an FMA with an immediate; the chunk's constant part joins the maxima
+              // column part of the bias by an FMA with an immediate, then the chunk's constant part
+              const float t0 = slope * ((float)col0 - fi);
 #pragma unroll
-              for (int u = 0; u < 32; ++u) va[u] = fmaf(slope, (float)u, va[u]);
+              for (int u = 0; u < 32; ++u) va[u] = fmaf(slope, (float)u, va[u]) + t0;
             }
-            if (masked) {
+            if (col0 + 31 > first_lim) {
 #pragma unroll
-              for (int u = 0; u < 32; ++u) va[u] = (col_base + c * 32 + u <= lim) ? va[u] : -INFINITY;
+              for (int u = 0; u < 32; ++u) va[u] = (col0 + u <= lim) ? va[u] : -INFINITY;
             }
-#pragma unroll
-            for (int q = 0; q < 4; ++q) g[4 * c + q] = max8(&va[8 * q]);
-            if (kAlibi) {
-              const float t0 = slope * ((float)(col_base + c * 32) - fi);
-#pragma unroll
-              for (int q = 0; q < 4; ++q) g[4 * c + q] += t0;
+            const float m_c = fmaxf(fmaxf(max8(&va[0]), max8(&va[8])), fmaxf(max8(&va[16]), max8(&va[24])));
+            if constexpr (kSearch) {
+              m_run = fmaxf(m_run, m_c);
+              r.thr = fmaxf(r.thr, m_run - margin);
             }
-          }
-          float m_tile = max3(g[0], g[1], g[2]);
+            const bool hit = m_c > r.thr;
+            if (!blind && __any_sync(0xffffffffu, hit)) {
+              // (lists without room for a whole chunk are shrunk first: the chunk is read once more)
+              full = __any_sync(0xffffffffu, r.cnt > kListCap - 32);
+              if (hit && !full) {
+                Entry* dst = list + r.cnt;
+                int n = 0;
 #pragma unroll
-          for (int u = 3; u < 15; u += 2) m_tile = max3(m_tile, g[u], g[u + 1]);
-          m_tile = fmaxf(m_tile, g[15]);
-          if (searching) {
-            // the other half's running maximum (if it already belongs to this item) tightens the bound too
-            const unsigned long long o = lds_u64(other_share);
-            const float m_other = (int)(o >> 32) == k ? __uint_as_float((unsigned)o) : -INFINITY;
-            r.m_run = max3(r.m_run, m_tile, m_other);
-            if (r.cnt >= 0) r.thr = fmaxf(r.thr, r.m_run - inv_a);
-            sts_u64(my_share, ((unsigned long long)(unsigned)k << 32) | __float_as_uint(r.m_run));
-          }
-          // ---- pass 2 (only when some lane saw a candidate): re-read the groups that hold one
-          const bool hit = m_tile > r.thr;
-          if (__any_sync(0xffffffffu, hit)) {
-            unsigned mine = 0;
-#pragma unroll
-            for (int u = 0; u < 16; ++u) mine |= (g[u] > r.thr ? 1u : 0u) << u;
-            unsigned todo = __reduce_or_sync(0xffffffffu, mine);
-            while (todo) {
-              // up to four groups per round trip to TMEM (todo is the same in every lane)
-              int gu[4];
-#pragma unroll
-              for (int w = 0; w < 4; ++w) {
-                gu[w] = todo ? __ffs(todo) - 1 : -1;
-                todo &= todo - 1;
-              }
-              float v8[4][8];
-#pragma unroll
-              for (int w = 0; w < 4; ++w)
-                if (gu[w] >= 0) tmem_ld8(taddr_row + gu[w] * 8, v8[w]);
-              tmem_ld_wait();
-              if (todo == 0) {
-                // the last batch is in registers: hand the accumulator back before the list stores
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(my_empty);
-                released = true;
-              }
-              if (kAlibi) {
-#pragma unroll
-                for (int w = 0; w < 4; ++w) {
-                  const float tw = slope * ((float)(col_base + gu[w] * 8) - fi);
-#pragma unroll
-                  for (int e = 0; e < 8; ++e) v8[w][e] = fmaf(slope, (float)e, v8[w][e]) + tw;
-                }
-              }
-              if (masked) {
-#pragma unroll
-                for (int w = 0; w < 4; ++w)
-#pragma unroll
-                  for (int e = 0; e < 8; ++e)
-                    v8[w][e] = (gu[w] >= 0 && col_base + gu[w] * 8 + e <= lim) ? v8[w][e] : -INFINITY;
-              }
-#pragma unroll
-              for (int w = 0; w < 4; ++w) {
-                if (gu[w] >= 0 && ((mine >> gu[w]) & 1u)) {
-                  const float thr = r.thr;
-                  int cnt = r.cnt;
-#pragma unroll
-                  for (int e = 0; e < 8; ++e) {
-                    if (v8[w][e] > thr) {
-                      *reinterpret_cast<uint2*>(&list[cnt]) =
-                          make_uint2(__float_as_uint(v8[w][e]), (unsigned)(col_base + gu[w] * 8 + e));
-                      ++cnt;
-                    }
+                for (int u = 0; u < 32; ++u) {
+                  if (va[u] > r.thr) {
+                    *reinterpret_cast<uint2*>(dst + n) = make_uint2(__float_as_uint(va[u]), (unsigned)(col0 + u));
+                    ++n;
                   }
-                  r.cnt = cnt;
                 }
+                r.cnt += n;
+                crowded = crowded || n > 2;
               }
-              // at most 32 entries were appended since the last check: the half-list cannot overflow
-              const unsigned need = __ballot_sync(0xffffffffu, r.cnt > kHalfTrigger);
-              if (need) r = shrink_lists(r, list, ra, inv_a, need, a.mode, a.expo_class, a.expo);
+            }
+            if (!full) {
+              ++c;
+              if (kSearch && blind && c == nch) {
+                blind = false;
+                c = 0;
+              }
             }
           }
-        }
-        // the accumulator has been read: hand it back to the MMA issuer (unless pass 2 already did)
-        if (!released) {
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(my_empty);
-        }
+          if (!full) {
+            // the accumulator has been read: hand it back to the MMA issuer
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(my_empty);
+          }
+          // what the slots hold, against the row's bound as it stands now (kListTrigger leaves room for all of it)
+          int n_on = (int)(at - my_slot) / kSlotStep;
+          for (uint32_t from = my_slot; __any_sync(0xffffffffu, n_on > 0); from += kSlotStep, --n_on) {
+            if (n_on > 0) {
+              float v[8];
+              lds_f4(from, v[0], v[1], v[2], v[3]);
+              lds_f4(from + kSlotHi, v[4], v[5], v[6], v[7]);
+              const int key0 = col_base + 8 * (int)((groups >> (5 * (n_on - 1))) & 31u);
+              if (kAlibi) {
+                const float t0 = slope * ((float)(key0 & ~63) - fi);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) v[e] += t0;
+              }
+              Entry* dst = list + r.cnt;
+              int n = 0;
+#pragma unroll
+              for (int e = 0; e < 8; ++e) {
+                if (v[e] > r.thr) {
+                  *reinterpret_cast<uint2*>(dst + n) = make_uint2(__float_as_uint(v[e]), (unsigned)(key0 + e));
+                  ++n;
+                }
+              }
+              r.cnt += n;
+            }
+          }
+          // Lists are shrunk between tiles, so that whether a row goes to the dense path depends on whole tiles of keys; in
+          // the middle of one only where a list has no room for the chunk that is waiting
+          const unsigned need = __ballot_sync(0xffffffffu, r.cnt > (full ? kListCap - 32 : kListTrigger));
+          if (need)
+            r = shrink_lists(r, list, 1.0f / margin, margin, need, kSearch ? 0 : 1, a.expo_class, a.expo);
+        } while (full);
+        crowded = __any_sync(0xffffffffu, crowded);
       }
-      if (valid && alive) {
-        a.half_cnt[grow * 2 + half] = r.cnt;
-        a.half_thr[grow * 2 + half] = r.thr * ra;
+      if (i < a.N && alive) {
+        a.list_cnt[2 * (size_t)grow] = r.cnt;
+        if (kSearch) a.list_thr[grow] = r.thr / margin;   // Eq. 1's units
       }
     }
   }
@@ -905,7 +950,7 @@ cudaError_t make_sample_map(CUtensorMap* map, const void* base, const Problem& p
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-template <int HD, bool kDump, bool kAlibi>
+template <int HD, bool kDump, bool kAlibi, bool kSearch>
 cudaError_t launch_impl(const Problem& p, const void* q, const void* k, SweepArgs& args, cudaStream_t stream) {
   CUtensorMap map_q, map_k, map_ks;
   cudaError_t err = make_map(&map_q, q, p, BM);
@@ -918,7 +963,7 @@ cudaError_t launch_impl(const Problem& p, const void* q, const void* k, SweepArg
   } else {
     map_ks = map_k;   // never used: sample_tiles() is 0 for short sequences
   }
-  err = cudaFuncSetAttribute(sweep_kernel<HD, kDump, kAlibi>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  err = cudaFuncSetAttribute(sweep_kernel<HD, kDump, kAlibi, kSearch>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              Cfg<HD>::kSmemBytes);
   if (err != cudaSuccess) return err;
   int dev = 0, sms = 0;
@@ -927,14 +972,14 @@ cudaError_t launch_impl(const Problem& p, const void* q, const void* k, SweepArg
   err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (err != cudaSuccess) return err;
   const int grid = args.n_items < sms ? args.n_items : sms;
-  sweep_kernel<HD, kDump, kAlibi><<<grid, kThreads, Cfg<HD>::kSmemBytes, stream>>>(map_q, map_k, map_ks, args);
+  sweep_kernel<HD, kDump, kAlibi, kSearch><<<grid, kThreads, Cfg<HD>::kSmemBytes, stream>>>(map_q, map_k, map_ks, args);
   return cudaGetLastError();
 }
 
 }  // namespace
 
 cudaError_t launch_sweep(const Problem& p, const void* q, const void* k, const float* scale, const float* tau_in,
-                         int mode, int32_t* half_cnt, float* half_thr, Entry* entries, int32_t* work_counter,
+                         int mode, int32_t* list_cnt, float* list_thr, Entry* entries, int32_t* work_counter,
                          float* dump, int dump_bh, float* alibi_blob, float* alibi_kmax, int32_t* status,
                          cudaStream_t stream) {
   SweepArgs args;
@@ -948,8 +993,8 @@ cudaError_t launch_sweep(const Problem& p, const void* q, const void* k, const f
   args.scale = scale;
   args.scale_sb = p.scale_sb;
   args.tau_in = tau_in;
-  args.half_cnt = half_cnt;
-  args.half_thr = half_thr;
+  args.list_cnt = list_cnt;
+  args.list_thr = list_thr;
   args.entries = entries;
   args.dump = p.alibi ? alibi_blob : dump;
   args.dump_bh = dump_bh;
@@ -974,12 +1019,13 @@ cudaError_t launch_sweep(const Problem& p, const void* q, const void* k, const f
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return err;
   }
-  if (dump) return p.D == 64 ? launch_impl<64, true, false>(p, q, k, args, stream)
-                             : launch_impl<128, true, false>(p, q, k, args, stream);
-  if (p.alibi) return p.D == 64 ? launch_impl<64, false, true>(p, q, k, args, stream)
-                                : launch_impl<128, false, true>(p, q, k, args, stream);
-  return p.D == 64 ? launch_impl<64, false, false>(p, q, k, args, stream)
-                   : launch_impl<128, false, false>(p, q, k, args, stream);
+#define ENTMAX_SWEEP(DUMP, ALIBI, SEARCH)                                               \
+  (p.D == 64 ? launch_impl<64, DUMP, ALIBI, SEARCH>(p, q, k, args, stream)              \
+             : launch_impl<128, DUMP, ALIBI, SEARCH>(p, q, k, args, stream))
+  if (dump) return ENTMAX_SWEEP(true, false, true);
+  if (p.alibi) return mode == 0 ? ENTMAX_SWEEP(false, true, true) : ENTMAX_SWEEP(false, true, false);
+  return mode == 0 ? ENTMAX_SWEEP(false, false, true) : ENTMAX_SWEEP(false, false, false);
+#undef ENTMAX_SWEEP
 }
 
 }  // namespace entmax
