@@ -51,9 +51,7 @@ static_assert(kTmemCols == 512, "TMEM budget");
 
 // Slots per consumer thread for what its scan of a tile found: eight consecutive accumulators of its row that hold at least
 // one candidate.  Slot s of a warp: two float4 arrays.
-constexpr int kSlots = 4;
 constexpr int kSlotHi = 32 * 16, kSlotStep = 2 * kSlotHi;
-constexpr int kSlotBytes = kSlots * kSlotStep;
 
 template <int HD>
 struct Cfg {
@@ -61,6 +59,8 @@ struct Cfg {
   static constexpr int kQBytes = BM * HD * 2;
   static constexpr int kKBytes = BN * HD * 2;
   static constexpr int kStages = HD == 128 ? 2 : 4;
+  static constexpr int kSlots = HD == 128 ? 4 : 6;        // (what fits, and six 5-bit group numbers in a word)
+  static constexpr int kSlotBytes = kSlots * kSlotStep;
   static constexpr int kBarBytes = 512;
   static constexpr int kSmemBytes =
       kQTiles * kQBytes + kStages * kKBytes + kConsumerWarps * kSlotBytes + 1024 /*align*/ + kBarBytes;
@@ -285,7 +285,7 @@ __device__ __forceinline__ RowState shrink_lists(RowState r, Entry* list, float 
 }
 
 // The eight column groups of a 64-column step (the first is group G0 of the tile): see the consumers
-template <int G0>
+template <int G0, int kSlots>
 __device__ __forceinline__ void scan_groups(const float (&g)[8], float thr, uint32_t& at, uint32_t my_slot, uint32_t& groups,
                                             const float (&v)[64]) {
   const uint32_t last = my_slot + (kSlots - 1) * kSlotStep;
@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
   const uint32_t q_smem = sbase;                                   // [kQTiles][kHalves][BM rows x 128 B]
   const uint32_t k_smem = sbase + kQTiles * C::kQBytes;            // [kStages][kHalves][BN rows x 128 B]
   const uint32_t slots = k_smem + C::kStages * C::kKBytes;         // [kConsumerWarps][kSlotBytes]
-  const uint32_t bars = slots + kConsumerWarps * kSlotBytes;       // mbarriers, 8 bytes each
+  const uint32_t bars = slots + kConsumerWarps * C::kSlotBytes;       // mbarriers, 8 bytes each
   const uint32_t q_full = bars;                            // [kQTiles]
   const uint32_t q_empty = q_full + 8 * kQTiles;           // [kQTiles]
   const uint32_t s_full = q_empty + 8 * kQTiles;           // [kQTiles]
@@ -525,7 +525,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
     const int row_local = quad * 32 + lane;
     const uint32_t taddr_row = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(x * BN);
     const uint32_t my_full = s_full + 8 * x, my_empty = s_empty + 8 * x;
-    const uint32_t my_slot = slots + (uint32_t)(cw * kSlotBytes + 16 * lane);
+    const uint32_t my_slot = slots + (uint32_t)(cw * C::kSlotBytes + 16 * lane);
     uint32_t fphase = 0, wphase = 0;
     int slot = 0;
     bool alive = true;
@@ -638,8 +638,9 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
         // warp counting: branches on "some row has a candidate", a second look at TMEM or list stores in between all cost
         // more there than these predicated stores do.
         uint32_t at = my_slot, groups = 0u;
-        bool crowd = crowded || col_base + BN - 1 > first_lim || blind || kDump;
-        if (!crowd) {
+        bool skip = __all_sync(0xffffffffu, r.thr == INFINITY) && !kDump;   // no row of the warp wants anything any more
+        bool crowd = !skip && (crowded || col_base + BN - 1 > first_lim || blind || kDump);
+        if (!crowd && !skip) {
           float v0[64], v1[64];
           tmem_ld64(taddr_row, v0);
 #pragma unroll
@@ -648,10 +649,11 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
             tmem_ld_wait64(v);
             if (s < 3) tmem_ld64(taddr_row + 64 * (s + 1), (s & 1) ? v0 : v1);
             float g[8];
+            float t0 = 0.f;
             if (kAlibi) {
 #pragma unroll
               for (int u = 0; u < 64; ++u) v[u] = fmaf(slope, (float)u, v[u]);
-              const float t0 = slope * ((float)(col_base + 64 * s) - fi);
+              t0 = slope * ((float)(col_base + 64 * s) - fi);
 #pragma unroll
               for (int q = 0; q < 8; ++q) g[q] = max8(&v[8 * q]) + t0;
             } else {
@@ -659,16 +661,19 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
               for (int q = 0; q < 8; ++q) g[q] = max8(&v[8 * q]);
             }
             if constexpr (kSearch) {
-              m_run = max3(max3(m_run, g[0], g[1]), max3(g[2], g[3], g[4]), max3(g[5], g[6], g[7]));
+              // (a vote per step pays here, 2184 -> 2103 us on 16 x 32768 x 128; in the given-threshold form it cost 40 us)
+              const float m_s = max3(max3(g[0], g[1], g[2]), max3(g[3], g[4], g[5]), fmaxf(g[6], g[7]));
+              m_run = fmaxf(m_run, m_s);
               r.thr = fmaxf(r.thr, m_run - margin);
+              if (!__any_sync(0xffffffffu, m_s > r.thr)) continue;
             }
-            if (s == 0) scan_groups<0>(g, r.thr, at, my_slot, groups, v);
-            else if (s == 1) scan_groups<8>(g, r.thr, at, my_slot, groups, v);
-            else if (s == 2) scan_groups<16>(g, r.thr, at, my_slot, groups, v);
-            else scan_groups<24>(g, r.thr, at, my_slot, groups, v);
+            if (s == 0) scan_groups<0, C::kSlots>(g, r.thr, at, my_slot, groups, v);
+            else if (s == 1) scan_groups<8, C::kSlots>(g, r.thr, at, my_slot, groups, v);
+            else if (s == 2) scan_groups<16, C::kSlots>(g, r.thr, at, my_slot, groups, v);
+            else scan_groups<24, C::kSlots>(g, r.thr, at, my_slot, groups, v);
           }
           // a row had more than its slots take: once more, the other way
-          crowd = __any_sync(0xffffffffu, at > my_slot + kSlots * kSlotStep);
+          crowd = __any_sync(0xffffffffu, at > my_slot + C::kSlots * kSlotStep);
           if (crowd) at = my_slot;
         }
         // Everywhere else 32 columns at a time, with every row appending its candidates to its list directly
@@ -706,6 +711,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
               r.thr = fmaxf(r.thr, m_run - margin);
             }
             const bool hit = m_c > r.thr;
+            int n_new = 0;
             if (!blind && __any_sync(0xffffffffu, hit)) {
               // (lists without room for a whole chunk are shrunk first: the chunk is read once more)
               full = __any_sync(0xffffffffu, r.cnt > kListCap - 32);
@@ -721,10 +727,39 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
                 }
                 r.cnt += n;
                 crowded = crowded || n > 2;
+                n_new = n;
               }
             }
             if (!full) {
               ++c;
+              if (!blind && c == 1 && nch > 1 && __all_sync(0xffffffffu, n_new >= 24 || r.thr == INFINITY)) {
+                // Nearly every key is a candidate (flat logits): before the other chunks are stored, look whether the tile
+                // sends the rows to the dense path anyway.  Given threshold: more candidates than a list may hold.  Search:
+                // tau <= m_run - n^(-1/e) for n listed keys (see shrink_lists), more keys above that than a list may keep.
+                // (Storing them all was most of what such a call spent here: 377 us on 16 x 8192 x 128, backward.)
+                const int n_max = r.cnt + (nch - 1) * 32;
+                const float width = a.expo_class == kExpo2 ? rsqrtf((float)n_max)
+                                    : a.expo_class == kExpo1 ? 1.0f / (float)n_max : __powf((float)n_max, -1.0f / a.expo);
+                const float cut = kSearch ? fmaxf(r.thr, m_run - 0.999f * width * margin) : r.thr;
+                int n = kSearch ? 0 : r.cnt;
+#pragma unroll 1
+                for (int c2 = kSearch ? 0 : 1; c2 < nch; ++c2) {
+                  tmem_ld32(taddr_row + c2 * 32, va);
+                  tmem_ld_wait();
+                  const int col2 = col_base + c2 * 32;
+                  const float t2 = kAlibi ? slope * ((float)col2 - fi) : 0.f;
+#pragma unroll
+                  for (int u = 0; u < 32; ++u) {
+                    const float y = kAlibi ? fmaf(slope, (float)u, va[u]) + t2 : va[u];
+                    n += (y > cut && col2 + u <= lim) ? 1 : 0;
+                  }
+                }
+                if (n > (kSearch ? kListKeep : kListTrigger)) {
+                  r.thr = INFINITY;
+                  r.cnt = -1;
+                }
+                if (__all_sync(0xffffffffu, r.thr == INFINITY)) c = nch;
+              }
               if (kSearch && blind && c == nch) {
                 blind = false;
                 c = 0;
@@ -737,7 +772,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
             __syncwarp();
             if (lane == 0) mbar_arrive(my_empty);
           }
-          // what the slots hold, against the row's bound as it stands now (kListTrigger leaves room for all of it)
+          // what the slots hold goes to the list, filtered with the row's bound as it stands now (kListTrigger leaves room)
           int n_on = (int)(at - my_slot) / kSlotStep;
           for (uint32_t from = my_slot; __any_sync(0xffffffffu, n_on > 0); from += kSlotStep, --n_on) {
             if (n_on > 0) {
