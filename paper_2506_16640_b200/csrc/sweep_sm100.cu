@@ -284,6 +284,55 @@ __device__ __forceinline__ RowState shrink_lists(RowState r, Entry* list, float 
   return r;
 }
 
+// A lower bound of a row's threshold from K values of K different keys of it (-inf: none), in accumulator units: the threshold
+// of those keys alone, by Newton steps from the left (App. A bracket; e < 1: the bracket's lower end itself).  A fixed
+// number of steps: any iterate is a bound.  m_run: raised to the largest of the values.
+template <int EC, int K>
+__device__ __forceinline__ float newton_from_values(const float (&y)[K], float expo) {
+  float s = -1.0f;
+#pragma unroll 1
+  for (int it = 0; it < 3; ++it) {
+    float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+    for (int q = 0; q < K; ++q) {
+      const float d = fmaxf(y[q] - s, 0.f);        // (-inf clamps to 0)
+      float d1 = d;
+      if constexpr (EC == kExpo1) d1 = positive_indicator(d);
+      else if constexpr (EC == kExpo4) d1 = d * d * d;
+      else if constexpr (EC == kExpoGeneral) d1 = d > 0.f ? __powf(d, expo - 1.0f) : 0.f;
+      s0 = fmaf(d1, d, s0);
+      s1 += d1;
+    }
+    const float root = EC == kExpo1 ? s0 : EC == kExpo2 ? sqrtf(s0) : EC == kExpo4 ? sqrtf(sqrtf(s0)) : __powf(s0, 1.0f / expo);
+    const float step = (s0 - s0 / root) / s1;
+    if (step > 0.f) s += step;
+  }
+  return s;
+}
+template <int K>
+__device__ __forceinline__ float bound_from_values(float (&g)[K], float margin, int expo_class, float expo, float& m_run) {
+  float m = g[0];
+#pragma unroll
+  for (int q = 1; q < K; ++q) m = fmaxf(m, g[q]);
+  m_run = fmaxf(m_run, m);
+  // rows of short supports (no more than two of the values within the bracket) gain nothing
+  int n = 0;
+#pragma unroll
+  for (int q = 0; q < K; ++q) n += g[q] > m - margin ? 1 : 0;
+  float s = -1.0f;                                 // threshold below the largest value, in Eq. 1's units
+  if (expo >= 1.0f && __any_sync(0xffffffffu, n > 2)) {
+    const float ra = 1.0f / margin;
+#pragma unroll
+    for (int q = 0; q < K; ++q) g[q] = (g[q] - m) * ra;
+    s = expo_class == kExpo2 ? newton_from_values<kExpo2>(g, expo)
+        : expo_class == kExpo1 ? newton_from_values<kExpo1>(g, expo)
+        : expo_class == kExpo4 ? newton_from_values<kExpo4>(g, expo) : newton_from_values<kExpoGeneral>(g, expo);
+  }
+  // rounding: of the powers (a share of the mass), of s, and of m + s * margin
+  const float hair = (expo_class == kExpoGeneral ? 1e-4f : 1e-5f) * margin + 1e-6f * fabsf(m);
+  return m > -INFINITY ? m + s * margin - hair : -INFINITY;
+}
+
 // The eight column groups of a 64-column step (the first is group G0 of the tile): see the consumers
 template <int G0, int kSlots>
 __device__ __forceinline__ void scan_groups(const float (&g)[8], float thr, uint32_t& at, uint32_t my_slot, uint32_t& groups,
@@ -573,7 +622,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
       // tiles that reach past the first one need the mask
       const int first_lim = a.causal ? tile_row0 : a.N - 1;
       const int last_lim = a.causal ? (tile_row0 + BM - 1 < a.N - 1 ? tile_row0 + BM - 1 : a.N - 1) : a.N - 1;
-      // ---- sampled tiles first (forward mode, long rows): maxima only, nothing is kept -- every sampled
+      // ---- sampled tiles first (forward mode, long rows): maxima only, no key is kept -- every sampled
       //      key comes by again in the real stream.  Column c of sampled tile t is key kSampleStride * (t*BN + c).
       const int ts = sample_tiles<kSearch>(a, item);
       const int ts0 = kAlibi ? min(tf / kSampleStride, ts) : 0;
@@ -588,6 +637,11 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
         int glim = lim / kSampleStride;
         if (glim > a.N / kSampleStride - 1) glim = a.N / kSampleStride - 1;
         const int first_glim = min(first_lim / kSampleStride, a.N / kSampleStride - 1);
+        // maxima of eight classes of sampled keys (eight different keys, near the sample's largest): their threshold is a far
+        // better bound than the largest value alone gives where supports are long
+        float top[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) top[q] = -INFINITY;
         for (int t = ts0; t < ts && alive; ++t) {
           alive = __all_sync(0xffffffffu, mbar_wait(my_full, fphase, abort_flag));
           if (!alive) break;
@@ -599,25 +653,24 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
             float va[64];
             tmem_ld64(taddr_row + c * 64, va);
             tmem_ld_wait64(va);
+            const int g0 = g_base + c * 64;
             if (kAlibi) {
+              const float t0 = slope * ((float)(kSampleStride * g0) - fi);
 #pragma unroll
-              for (int u = 0; u < 64; ++u) va[u] = fmaf(slope * (float)kSampleStride, (float)u, va[u]);
+              for (int u = 0; u < 64; ++u) va[u] = fmaf(slope * (float)kSampleStride, (float)u, va[u]) + t0;
             }
-            if (g_base + c * 64 + 63 > first_glim) {
+            if (g0 + 63 > first_glim) {
 #pragma unroll
-              for (int u = 0; u < 64; ++u) va[u] = (g_base + c * 64 + u <= glim) ? va[u] : -INFINITY;
+              for (int u = 0; u < 64; ++u) va[u] = (g0 + u <= glim) ? va[u] : -INFINITY;
             }
-            float m_c = max8(&va[0]);
 #pragma unroll
-            for (int q = 1; q < 8; ++q) m_c = fmaxf(m_c, max8(&va[8 * q]));
-            if (kAlibi) m_c += slope * ((float)(kSampleStride * (g_base + c * 64)) - fi);
-            m_run = fmaxf(m_run, m_c);
+            for (int q = 0; q < 8; ++q) top[q] = fmaxf(top[q], max8(&va[8 * q]));
           }
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(my_empty);
         }
-        r.thr = fmaxf(r.thr, m_run - margin);
+        r.thr = fmaxf(r.thr, bound_from_values(top, margin, a.expo_class, a.expo, m_run));
       }
       // A stream that starts without any bound scans its first tile twice: maxima first, so that the second scan
       // already has a bound
@@ -638,8 +691,34 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
         // warp counting: branches on "some row has a candidate", a second look at TMEM or list stores in between all cost
         // more there than these predicated stores do.
         uint32_t at = my_slot, groups = 0u;
+        if (blind) {
+          // the first tile of a stream without any bound: maxima of eight classes of its keys, and the threshold of those eight
+          float top[8];
+#pragma unroll
+          for (int q = 0; q < 8; ++q) top[q] = -INFINITY;
+#pragma unroll 1
+          for (int c = 0; c < (nch + 1) / 2; ++c) {
+            float va[64];
+            tmem_ld64(taddr_row + 64 * c, va);
+            tmem_ld_wait64(va);
+            const int col0 = col_base + 64 * c;
+            if (kAlibi) {
+              const float t0 = slope * ((float)col0 - fi);
+#pragma unroll
+              for (int u = 0; u < 64; ++u) va[u] = fmaf(slope, (float)u, va[u]) + t0;
+            }
+            if (col0 + 63 > first_lim) {
+#pragma unroll
+              for (int u = 0; u < 64; ++u) va[u] = (col0 + u <= lim) ? va[u] : -INFINITY;
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q) top[q] = fmaxf(top[q], max8(&va[8 * q]));
+          }
+          r.thr = fmaxf(r.thr, bound_from_values(top, margin, a.expo_class, a.expo, m_run));
+          blind = false;
+        }
         bool skip = __all_sync(0xffffffffu, r.thr == INFINITY) && !kDump;   // no row of the warp wants anything any more
-        bool crowd = !skip && (crowded || col_base + BN - 1 > first_lim || blind || kDump);
+        bool crowd = !skip && (crowded || col_base + BN - 1 > first_lim || kDump);
         if (!crowd && !skip) {
           float v0[64], v1[64];
           tmem_ld64(taddr_row, v0);
@@ -712,7 +791,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
             }
             const bool hit = m_c > r.thr;
             int n_new = 0;
-            if (!blind && __any_sync(0xffffffffu, hit)) {
+            if (__any_sync(0xffffffffu, hit)) {
               // (lists without room for a whole chunk are shrunk first: the chunk is read once more)
               full = __any_sync(0xffffffffu, r.cnt > kListCap - 32);
               if (hit && !full) {
@@ -732,7 +811,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
             }
             if (!full) {
               ++c;
-              if (!blind && c == 1 && nch > 1 && __all_sync(0xffffffffu, n_new >= 24 || r.thr == INFINITY)) {
+              if (c == 1 && nch > 1 && __all_sync(0xffffffffu, n_new >= 24 || r.thr == INFINITY)) {
                 // Nearly every key is a candidate (flat logits): before the other chunks are stored, look whether the tile
                 // sends the rows to the dense path anyway.  Given threshold: more candidates than a list may hold.  Search:
                 // tau <= m_run - n^(-1/e) for n listed keys (see shrink_lists), more keys above that than a list may keep.
@@ -759,10 +838,6 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
                   r.cnt = -1;
                 }
                 if (__all_sync(0xffffffffu, r.thr == INFINITY)) c = nch;
-              }
-              if (kSearch && blind && c == nch) {
-                blind = false;
-                c = 0;
               }
             }
           }
