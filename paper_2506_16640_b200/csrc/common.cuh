@@ -6,6 +6,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <utility>
+
 #include "entmax_attn.h"
 
 namespace entmax {
@@ -181,6 +183,32 @@ __device__ __forceinline__ void atomic_add_slice(float* p, const float (&x)[PER]
   else red_add_v4(p, x[0], x[1], x[2], x[3]);
 }
 
+// ---- launches that overlap the end of the kernel before them
+// Every kernel of this library is launched with programmatic stream serialization: its CTAs may become resident while the
+// kernel before it in the stream still runs, and wait in pdl_begin() until that one has completed and its writes are
+// visible.  Since every kernel waits, the order of a stream is as without it; what is saved is the launch latency and the
+// drain between short kernels (1 to 2 us each of the fifteen of a training step).  pdl_begin() comes before any access to
+// memory that another kernel writes or reads.
+__device__ __forceinline__ void pdl_begin() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem_bytes, cudaStream_t stream,
+                          Args&&... args) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem_bytes;
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+
 // ---- launchers (each enqueues on `stream` and returns the cudaError_t of the launch) -------------
 // scale table c_i [H,N] (scale == nullptr: none) and n_clear words of zeros at `clear`, one launch
 cudaError_t launch_prologue(const Problem& p, const float* beta, const float* gamma, const float* delta, float* scale,
@@ -226,18 +254,17 @@ cudaError_t launch_tile_fwd(const Problem& p, const void* q, const void* k, cons
                             int32_t* work_counter, const int32_t* row_cnt, int32_t* dense_cnt, void* o, float* tau,
                             int32_t* status, cudaStream_t stream);
 
-// Dense-tile backward on the tensor cores (bf16): the rows in row_list[0 .. *row_count) are marked in
-// tile_mask, their 128-row Q tiles listed, and dQ (and dc_rows) of those rows written; their dK and dV
-// contributions are added to the fp32 accumulators.  tile_mask, tile_flag, *tile_count, *work_counter and
-// work_counter[12] must be zero on entry; rho: [B*H*N] floats of scratch.
+// Dense-tile backward on the tensor cores (bf16): dQ (and dc_rows) of the rows marked in tile_mask are written (their Q
+// tiles flagged in tile_flag and listed; the list is reordered); their dK and dV contributions are added to the fp32
+// accumulators.  *work_counter and work_counter[12] must be zero on entry; rho: [B*H*N] floats of scratch.
 cudaError_t launch_tile_bwd(const Problem& p, const void* q, const void* k, const void* v, const void* d_o,
-                            const float* scale, const float* tau, const int32_t* row_list, const int32_t* row_count,
-                            uint32_t* tile_mask, int32_t* tile_flag, int32_t* tile_list, int32_t* tile_count,
+                            const float* scale, const float* tau, const uint32_t* tile_mask, const int32_t* tile_flag,
+                            int32_t* tile_list, const int32_t* tile_count,
                             int32_t* work_counter, float* rho, void* dq,
                             float* acc_dk, float* acc_dv, float* dc_rows, int32_t* status, cudaStream_t stream);
 
-// per-row solve + gather kernels working on the lists (bf16 path); the forward one also lists the
-// 128-row Q tiles that hold rows for the dense-tile path (tile_flag must be zero on entry)
+// per-row solve + gather kernels working on the lists (bf16 path); they also list the 128-row Q tiles that hold rows for
+// the dense-tile path (tile_flag, *tile_count must be zero on entry; backward: the rows are marked in tile_mask, zero too)
 cudaError_t launch_row_fwd(const Problem& p, const void* v, const float* scale, int32_t* row_cnt,
                            const int32_t* list_cnt, const float* list_thr, Entry* entries, void* o, float* tau, int32_t* fb_count,
                            int32_t* fb_list, int32_t* tile_flag, int32_t* tile_list, int32_t* tile_count, int32_t* status,
@@ -245,12 +272,14 @@ cudaError_t launch_row_fwd(const Problem& p, const void* v, const float* scale, 
 cudaError_t launch_row_bwd(const Problem& p, const void* q, const void* k, const void* v, const void* d_o,
                            const float* scale, const float* tau, const int32_t* list_cnt, Entry* entries, void* dq,
                            float* acc_dk, float* acc_dv, float* dc_rows, int32_t* fb_count, int32_t* fb_list,
-                           int32_t* status, int saved, int pitch, cudaStream_t stream);
+                           uint32_t* tile_mask, int32_t* tile_flag, int32_t* tile_list, int32_t* tile_count, int32_t* status,
+                           int saved, int pitch, cudaStream_t stream);
 // compact copy of the forward call's supports (see entmax_attn_save_supports)
 cudaError_t launch_save_supports(const Problem& p, int slots, const int32_t* row_cnt, const Entry* entries,
                                  int32_t* out_cnt, Entry* out_entries, cudaStream_t stream);
 
-// fp32 accumulators [B,H,N,D] contiguous -> strided output tensor of the problem dtype
-cudaError_t launch_store_grad(const Problem& p, const float* acc, void* out, cudaStream_t stream);
+// fp32 accumulators [B,H,N,D] contiguous -> strided output tensors of the problem dtype
+cudaError_t launch_store_grad(const Problem& p, const float* acc_dk, const float* acc_dv, void* dk, void* dv,
+                              cudaStream_t stream);
 
 }  // namespace entmax

@@ -62,6 +62,7 @@ __global__ void __launch_bounds__(kSolveThreads) decode_solve_kernel(DecodeArgs 
                                                                     float* __restrict__ tau_out,
                                                                     int32_t* __restrict__ support_out,
                                                                     int32_t* __restrict__ status) {
+  pdl_begin();
   constexpr int kWarps = kSolveThreads / 32;
   constexpr int kPerThread = kListSlots / kSolveThreads;
   constexpr int kCap = kListSlots;
@@ -371,7 +372,7 @@ extern "C" int entmax_attn_decode_fwd(const entmax_attn_decode_params* params, c
   __nv_bfloat16* ob = static_cast<__nv_bfloat16*>(o);
   // long rows: more threads per row (more loads in flight); many short rows: smaller CTAs
 #define ENTMAX_SOLVE(D, T) \
-  decode_solve_kernel<D, T><<<rows, T, 0, stream>>>(a, vb, scores, chunk_max, ob, tau, support_size, device_status)
+  launch_kernel(decode_solve_kernel<D, T>, rows, T, 0, stream, a, vb, scores, chunk_max, ob, tau, support_size, device_status)
   if (a.NC >= 16384) {
     if (a.D == 64) ENTMAX_SOLVE(64, 512); else ENTMAX_SOLVE(128, 512);
   } else {

@@ -46,6 +46,7 @@ __global__ void __launch_bounds__(kThreadsD, 2) decode_scores_tc_kernel(const __
                                                                        float* __restrict__ scores,
                                                                        float* __restrict__ chunk_max,
                                                                        int32_t* __restrict__ status) {
+  pdl_begin();
   using C = DCfg<HD>;
   extern __shared__ uint8_t smem_raw[];
   __shared__ float smax[4][ENTMAX_ATTN_DECODE_MAX_Q];
@@ -256,7 +257,7 @@ cudaError_t launch_impl(const DecodeArgs& a, const void* q, const void* k, float
   err = cudaFuncSetAttribute(decode_scores_tc_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, DCfg<HD>::kSmemBytes);
   if (err != cudaSuccess) return err;
   const dim3 grid(a.n_chunks, a.H, a.B);
-  decode_scores_tc_kernel<HD><<<grid, kThreadsD, DCfg<HD>::kSmemBytes, stream>>>(map_q, map_k, a, scores, chunk_max,
+  launch_kernel(decode_scores_tc_kernel<HD>, grid, kThreadsD, DCfg<HD>::kSmemBytes, stream, map_q, map_k, a, scores, chunk_max,
                                                                                 status);
   return cudaGetLastError();
 }

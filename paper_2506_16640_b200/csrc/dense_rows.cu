@@ -122,6 +122,7 @@ __global__ void __launch_bounds__(kThreads) dense_fwd_kernel(Problem p, const T*
                                                              const T* __restrict__ v, const float* __restrict__ scale,
                                                              T* __restrict__ o, float* __restrict__ tau_out,
                                                              float* scratch, size_t scratch_floats) {
+  pdl_begin();
   constexpr int PER = D / 32;
   __shared__ float red[2 * kWarps];
   __shared__ float opart[kWarps][D];
@@ -192,6 +193,7 @@ __global__ void __launch_bounds__(kScaleGradThreads) scale_grad_kernel(Problem p
                                                                        float* __restrict__ dbeta,
                                                                        float* __restrict__ dgamma,
                                                                        float* __restrict__ ddelta) {
+  pdl_begin();
   __shared__ double red[kScaleGradThreads / 32];
   __shared__ int last;
   const int h = blockIdx.y;
@@ -240,6 +242,7 @@ __global__ void __launch_bounds__(256) prologue_kernel(Problem p, const float* _
                                                        const float* __restrict__ gamma, const float* __restrict__ delta,
                                                        float* __restrict__ scale, int32_t* __restrict__ clear, int n_clear,
                                                        int32_t* __restrict__ status) {
+  pdl_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (blockIdx.y == 0)
     for (int t = i; t < n_clear; t += gridDim.x * blockDim.x) clear[t] = 0;
@@ -263,7 +266,11 @@ __global__ void __launch_bounds__(256) prologue_kernel(Problem p, const float* _
 }
 
 template <typename T>
-__global__ void store_grad_kernel(Problem p, const float* __restrict__ acc, T* __restrict__ out) {
+__global__ void store_grad_kernel(Problem p, const float* __restrict__ acc_dk, const float* __restrict__ acc_dv,
+                                  T* __restrict__ dk, T* __restrict__ dv) {
+  pdl_begin();
+  const float* __restrict__ acc = blockIdx.y ? acc_dv : acc_dk;
+  T* __restrict__ out = blockIdx.y ? dv : dk;
   const size_t total4 = (size_t)p.B * p.H * p.N * p.D / 4;
   for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < total4; t += (size_t)gridDim.x * blockDim.x) {
     const size_t e = t * 4;
@@ -285,14 +292,14 @@ cudaError_t launch_prologue(const Problem& p, const float* beta, const float* ga
                             int32_t* clear, size_t n_clear, int32_t* status, cudaStream_t stream) {
   const int most = scale ? p.N : (int)(n_clear < 256 * 148 ? n_clear : 256 * 148);
   const dim3 grid((most + 255) / 256, scale ? (p.H + kScaleHeads - 1) / kScaleHeads : 1);
-  prologue_kernel<<<grid, 256, 0, stream>>>(p, beta, gamma, delta, scale, clear, (int)n_clear, status);
+  launch_kernel(prologue_kernel, grid, 256, 0, stream, p, beta, gamma, delta, scale, clear, (int)n_clear, status);
   return cudaGetLastError();
 }
 
 cudaError_t launch_dense_fwd(const Problem& p, const void* q, const void* k, const void* v, const float* scale, void* o,
                              float* tau, float* scratch, size_t scratch_floats, int ctas, cudaStream_t stream) {
 #define ENTMAX_LAUNCH(T, D)                                                                                      \
-  dense_fwd_kernel<T, D><<<ctas, kThreads, 0, stream>>>(p, (const T*)q, (const T*)k, (const T*)v, scale, (T*)o, \
+  launch_kernel(dense_fwd_kernel<T, D>, ctas, kThreads, 0, stream, p, (const T*)q, (const T*)k, (const T*)v, scale, (T*)o, \
                                                         tau, scratch, scratch_floats)
   if (p.dtype == ENTMAX_ATTN_DTYPE_FP32) {
     if (p.D == 64) ENTMAX_LAUNCH(float, 64); else ENTMAX_LAUNCH(float, 128);
@@ -310,16 +317,17 @@ cudaError_t launch_scale_grad(const Problem& p, const float* beta, const float* 
   int ctas = (148 * 4 + p.H - 1) / p.H;
   const int most = (p.N + kScaleGradThreads - 1) / kScaleGradThreads;
   if (ctas > most) ctas = most;
-  scale_grad_kernel<<<dim3(ctas, p.H), kScaleGradThreads, 0, stream>>>(p, beta, gamma, dc_rows, partial, counter, dbeta,
+  launch_kernel(scale_grad_kernel, dim3(ctas, p.H), kScaleGradThreads, 0, stream, p, beta, gamma, dc_rows, partial, counter, dbeta,
                                                                        dgamma, ddelta);
   return cudaGetLastError();
 }
 
-cudaError_t launch_store_grad(const Problem& p, const float* acc, void* out, cudaStream_t stream) {
+cudaError_t launch_store_grad(const Problem& p, const float* acc_dk, const float* acc_dv, void* dk, void* dv,
+                              cudaStream_t stream) {
   const size_t total4 = (size_t)p.B * p.H * p.N * p.D / 4;
-  const int blocks = (int)((total4 + 255) / 256 < 148 * 16 ? (total4 + 255) / 256 : 148 * 16);
-  if (p.dtype == ENTMAX_ATTN_DTYPE_FP32) store_grad_kernel<float><<<blocks, 256, 0, stream>>>(p, acc, (float*)out);
-  else store_grad_kernel<__nv_bfloat16><<<blocks, 256, 0, stream>>>(p, acc, (__nv_bfloat16*)out);
+  const int blocks = (int)((total4 + 255) / 256 < 148 * 8 ? (total4 + 255) / 256 : 148 * 8);
+  if (p.dtype == ENTMAX_ATTN_DTYPE_FP32) launch_kernel(store_grad_kernel<float>, dim3(blocks, 2), 256, 0, stream, p, acc_dk, acc_dv, (float*)dk, (float*)dv);
+  else launch_kernel(store_grad_kernel<__nv_bfloat16>, dim3(blocks, 2), 256, 0, stream, p, acc_dk, acc_dv, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv);
   return cudaGetLastError();
 }
 

@@ -134,7 +134,7 @@ WsLayout make_layout(const Problem& p, bool is_bwd) {
   l.list_thr = take(rows * sizeof(float));
   l.entries = take(rows * kListCap * sizeof(Entry));
   l.fb_count = take(256);
-  l.sweep_counter = l.fb_count + 64;   // same 256-byte block: [0] dense-row count, [16] sweep work counter,
+  l.sweep_counter = l.fb_count + 64;   // same 256-byte block: [16] sweep work counter, [56] long rows,
   l.tile_count = l.fb_count + 128;     // [32] number of listed dense tiles, [48] the dense-tile kernels' work counter
   l.grad_counter = l.fb_count + 32;    // [8] CTAs of the scale gradient that have finished
   // tile flags, list and masks right behind the counters: what a call has to clear is one range
@@ -399,7 +399,7 @@ int bwd_impl(const entmax_attn_params* params, const void* q, const void* k, con
       const uint8_t* sv = static_cast<const uint8_t*>(saved_supports);
       err = launch_row_bwd(p, q, k, v, d_o, scale, tau, reinterpret_cast<const int32_t*>(sv + sl.counts),
                            const_cast<Entry*>(reinterpret_cast<const Entry*>(sv + sl.entries)), dq, acc_dk, acc_dv,
-                           dc_rows, fb_count, fb_list, device_status, 1, ENTMAX_ATTN_SAVED_SLOTS, stream);
+                           dc_rows, fb_count, fb_list, tile_mask, tile_flag, tile_list, tile_count, device_status, 1, ENTMAX_ATTN_SAVED_SLOTS, stream);
       if (err != cudaSuccess) return fail_cuda(err);
     } else if (fwd_workspace) {
       // the forward call's workspace still holds every row's support: no score sweep needed
@@ -407,7 +407,7 @@ int bwd_impl(const entmax_attn_params* params, const void* q, const void* k, con
       const uint8_t* fws = static_cast<const uint8_t*>(fwd_workspace);
       err = launch_row_bwd(p, q, k, v, d_o, scale, tau, reinterpret_cast<const int32_t*>(fws + fl.row_cnt),
                            const_cast<Entry*>(reinterpret_cast<const Entry*>(fws + fl.entries)), dq, acc_dk, acc_dv,
-                           dc_rows, fb_count, fb_list, device_status, 1, kListCap, stream);
+                           dc_rows, fb_count, fb_list, tile_mask, tile_flag, tile_list, tile_count, device_status, 1, kListCap, stream);
       if (err != cudaSuccess) return fail_cuda(err);
     } else {
       if (g_prof_start[1]) cudaEventRecord(g_prof_start[1], stream);
@@ -419,19 +419,17 @@ int bwd_impl(const entmax_attn_params* params, const void* q, const void* k, con
       err = cudaStreamWaitEvent(stream, side->join, 0);     // the accumulators are clear from here on
       if (err != cudaSuccess) return fail_cuda(err);
       err = launch_row_bwd(p, q, k, v, d_o, scale, tau, list_cnt, entries, dq, acc_dk, acc_dv, dc_rows, fb_count,
-                           fb_list, device_status, 0, kListCap, stream);
+                           fb_list, tile_mask, tile_flag, tile_list, tile_count, device_status, 0, kListCap, stream);
       if (err != cudaSuccess) return fail_cuda(err);
     }
     // rows whose support does not fit the lists: dense tiles on the tensor cores
-    err = launch_tile_bwd(p, q, k, v, d_o, scale, tau, fb_list, fb_count, tile_mask, tile_flag, tile_list, tile_count, tile_count + 16,
+    err = launch_tile_bwd(p, q, k, v, d_o, scale, tau, tile_mask, tile_flag, tile_list, tile_count, tile_count + 16,
                           reinterpret_cast<float*>(ws + lay.list_thr) /* idle after the sweep: rho of the dense rows */, dq,
                           acc_dk, acc_dv, dc_rows, device_status, stream);
     if (err != cudaSuccess) return fail_cuda(err);
   }
   if (!in_place) {
-    err = launch_store_grad(p, acc_dk, dk, stream);
-    if (err != cudaSuccess) return fail_cuda(err);
-    err = launch_store_grad(p, acc_dv, dv, stream);
+    err = launch_store_grad(p, acc_dk, acc_dv, dk, dv, stream);
     if (err != cudaSuccess) return fail_cuda(err);
   }
   if (n_param_grads) {

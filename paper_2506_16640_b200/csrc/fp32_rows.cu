@@ -176,6 +176,7 @@ __global__ void __launch_bounds__(kThreads, 3) fp32_fwd_kernel(Problem p, const 
                                                                float* __restrict__ tau_out, int32_t* __restrict__ row_cnt,
                                                                int32_t* __restrict__ dense_cnt, Entry* __restrict__ entries,
                                                                float* scratch, int pitch, int items) {
+  pdl_begin();
   constexpr int PER = D / 32;
   extern __shared__ float4 sm4[];
   float* k_s = reinterpret_cast<float*>(sm4);
@@ -291,6 +292,7 @@ __global__ void __launch_bounds__(kThreads, 3) fp32_bwd_kernel(Problem p, const 
                                                                float* __restrict__ acc_dk, float* __restrict__ acc_dv,
                                                                float* __restrict__ dc_rows, float* scratch, int pitch,
                                                                int items) {
+  pdl_begin();
   constexpr int PL = D / 8;             // elements of a row per lane, eight lanes per key, in chunks of four
   extern __shared__ float4 sm4[];
   float* k_s = reinterpret_cast<float*>(sm4);
@@ -428,8 +430,7 @@ cudaError_t launch_fwd(const Problem& p, const float* q, const float* k, const f
   const long items = (long)p.B * p.H * ((p.N + R - 1) / R);
   cudaError_t err = cudaFuncSetAttribute(fp32_fwd_kernel<D, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (err != cudaSuccess) return err;
-  fp32_fwd_kernel<D, R><<<(int)(items < ctas ? items : ctas), kThreads, bytes, stream>>>(
-      p, q, k, v, scale, o, tau, row_cnt, dense_cnt, entries, scratch, fp32_scratch_pitch(p), (int)items);
+  launch_kernel(fp32_fwd_kernel<D, R>, (int)(items < ctas ? items : ctas), kThreads, bytes, stream, p, q, k, v, scale, o, tau, row_cnt, dense_cnt, entries, scratch, fp32_scratch_pitch(p), (int)items);
   return cudaGetLastError();
 }
 template <int D, int R>
@@ -440,8 +441,7 @@ cudaError_t launch_bwd(const Problem& p, const float* q, const float* k, const f
   const long items = (long)p.B * p.H * ((p.N + R - 1) / R);
   cudaError_t err = cudaFuncSetAttribute(fp32_bwd_kernel<D, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (err != cudaSuccess) return err;
-  fp32_bwd_kernel<D, R><<<(int)(items < ctas ? items : ctas), kThreads, bytes, stream>>>(
-      p, q, k, v, d_o, scale, tau, dq, acc_dk, acc_dv, dc_rows, scratch, fp32_scratch_pitch(p), (int)items);
+  launch_kernel(fp32_bwd_kernel<D, R>, (int)(items < ctas ? items : ctas), kThreads, bytes, stream, p, q, k, v, d_o, scale, tau, dq, acc_dk, acc_dv, dc_rows, scratch, fp32_scratch_pitch(p), (int)items);
   return cudaGetLastError();
 }
 

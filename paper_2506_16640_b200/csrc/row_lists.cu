@@ -3,7 +3,7 @@
 //
 // Forward: exact threshold on the candidates (Eq. 1 with the sum-to-one condition), probabilities, and
 // O_i = sum_j p_ij v_j as a gather over the support only -- every zero of P is skipped, not just
-// all-zero tiles.  A warp takes 16 consecutive rows and serves them by list length (8, 16 or 32 lanes per
+// all-zero tiles.  A warp takes up to 16 consecutive rows and serves them by list length (8, 16 or 32 lanes per
 // row).  alpha = 1.5 and alpha = 2 use the closed form on the sorted candidates (solve_rows_closed); other
 // exponents iterate (Newton from the left of the root, see dense_rows.cu) in two stages.
 // Backward: the entmax Jacobian dS = u (dP - <u,dP>/sum u), u = p^(2-alpha), on the support, dQ by
@@ -85,22 +85,6 @@ __device__ __forceinline__ void atomic_add_vec(float* p, const float (&x)[N]) {
 #pragma unroll
   for (int c = 0; c < N / 4; ++c)
     red_add_v4(p + 4 * c, x[4 * c], x[4 * c + 1], x[4 * c + 2], x[4 * c + 3]);
-}
-
-// The rows of a warp that go to the dense path (mask over the warp's lanes, lane l holding row `grow`): one
-// slot reservation and one status update for all of them.  A counter bumped once per row is a chain of
-// dependent L2 atomics on one address; with every row dense that chain, not the rows' work, set the kernel's time.
-__device__ __forceinline__ void push_dense_rows(unsigned mask, int grow, int32_t* fb_count, int32_t* fb_list,
-                                                int32_t* status, int lane) {
-  if (mask == 0u) return;
-  const int leader = __ffs(mask) - 1;
-  int base = 0;
-  if (lane == leader) {
-    base = atomicAdd(fb_count, __popc(mask));
-    if (status) atomicAdd(status + ENTMAX_ATTN_STATUS_DENSE_ROWS, __popc(mask));
-  }
-  base = __shfl_sync(0xffffffffu, base, leader);
-  if ((mask >> lane) & 1u) fb_list[base + __popc(mask & ((1u << lane) - 1u))] = grow;
 }
 
 // Bitonic sort of 32*S (key j, value y) pairs held as S registers per lane (element index = 32*s + lane),
@@ -555,20 +539,26 @@ __device__ __forceinline__ void push_long_rows(unsigned mask, int grow, int tota
   if ((mask >> lane) & 1u) fb_list[total - 1 - (base + __popc(mask & ((1u << lane) - 1u)))] = grow;
 }
 
-// Forward: the rows of a warp for the dense-tile path (see push_dense_rows).  Their 128-row Q tiles are listed once
-// (tile_flag arbitrates); of the lanes that name the same tile only the lowest asks.
-__device__ __forceinline__ void push_dense_tiles(const Problem& p, unsigned mask, int grow, int32_t* row_cnt,
-                                                 int32_t* fb_count, int32_t* fb_list, int32_t* tile_flag,
-                                                 int32_t* tile_list, int32_t* tile_count, int32_t* status, int lane) {
+// The rows of a warp that go to the dense-tile path (mask over the warp's lanes, lane l holding row `grow`): one status
+// update for all of them -- a counter bumped once per row is a chain of dependent L2 atomics on one address --, their
+// 128-row Q tiles listed once (tile_flag arbitrates; of the lanes that name the same tile only the lowest asks) and, where
+// tile_mask is given, the rows marked in it.
+__device__ __forceinline__ void push_dense_tiles(const Problem& p, unsigned mask, int grow, uint32_t* tile_mask,
+                                                 int32_t* tile_flag, int32_t* tile_list, int32_t* tile_count,
+                                                 int32_t* status, int lane) {
   if (mask == 0u) return;
-  push_dense_rows(mask, grow, fb_count, fb_list, status, lane);
+  if (status && lane == __ffs(mask) - 1) atomicAdd(status + ENTMAX_ATTN_STATUS_DENSE_ROWS, __popc(mask));
   if ((mask >> lane) & 1u) {
-    row_cnt[grow] = -2;
     const int tiles_per_head = (p.N + 127) / 128;
     const int bh = grow / p.N, i = grow - bh * p.N;
-    const int id = bh * tiles_per_head + i / 128;
+    const int id = bh * tiles_per_head + i / 128, r = i % 128;
     const unsigned same = __match_any_sync(mask, id);
     if (lane == __ffs(same) - 1 && atomicExch(tile_flag + id, 1) == 0) tile_list[atomicAdd(tile_count, 1)] = id;
+    if (tile_mask) {
+      const unsigned word = __match_any_sync(mask, 4 * id + (r >> 5));
+      const unsigned bits = __reduce_or_sync(word, 1u << (r & 31));
+      if (lane == __ffs(word) - 1) atomicOr(tile_mask + 4 * (size_t)id + (r >> 5), bits);
+    }
   }
 }
 
@@ -622,6 +612,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32) row_fwd_long_kernel(Problem
                                                                          float* __restrict__ tau_out,
                                                                          const int32_t* __restrict__ fb_count,
                                                                          const int32_t* __restrict__ fb_list) {
+  pdl_begin();
   const int lane = threadIdx.x & 31;
   const int total = p.B * p.H * p.N;
   const int n_long = fb_count[kLongCounter];
@@ -643,16 +634,17 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32) row_fwd_kernel(Problem p, c
                                                                     float* __restrict__ tau_out, int32_t* fb_count,
                                                                     int32_t* fb_list, int32_t* tile_flag,
                                                                     int32_t* tile_list, int32_t* tile_count,
-                                                                    int32_t* status) {
+                                                                    int32_t* status, int rpw) {
+  pdl_begin();
   const int lane = threadIdx.x & 31;
   const int total = p.B * p.H * p.N;
-  const int blocks = (total + 15) / 16;
+  const int blocks = (total + rpw - 1) / rpw;
   for (int blk = blockIdx.x * kWarpsPerCta + (threadIdx.x >> 5); blk < blocks; blk += gridDim.x * kWarpsPerCta) {
-    // A warp takes 16 consecutive rows; lane l (and l + 16) looks at row 16*blk + l.  Rows are then served by
+    // A warp takes rpw (16 or 8) consecutive rows; lane l (and l + 16) looks at row rpw*blk + l.  Rows are then served by
     // list length: four at a time with eight lanes each (1..8 entries), two at a time with sixteen lanes
     // each (9..16 entries), the rest one by one with the whole warp.
     constexpr bool kClosed = EC == kExpo2 || EC == kExpo1;
-    const int my_row = 16 * blk + (lane & 15);
+    const int my_row = (lane & 15) < rpw ? rpw * blk + (lane & 15) : total;
     int mc = 0;
     int cls = 3;                                     // 0: <= 8 entries, 1: <= 16, 2: whole warp / dense, 3: no row
     if (my_row < total) {
@@ -666,7 +658,8 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32) row_fwd_kernel(Problem p, c
       // rows without a usable list go to the dense-tile path, all of the warp's at once
       const unsigned mdense =
           __ballot_sync(0xffffffffu, lane < 16 && my_row < total && mc < 1);
-      push_dense_tiles(p, mdense, my_row, row_cnt, fb_count, fb_list, tile_flag, tile_list, tile_count, status, lane);
+      push_dense_tiles(p, mdense, my_row, nullptr, tile_flag, tile_list, tile_count, status, lane);
+      if ((mdense >> lane) & 1u) row_cnt[my_row] = -2;
       mfull &= ~mdense;
       // ... and the ones with long lists to a launch of their own
       const unsigned mlong = __ballot_sync(0xffffffffu, lane < 16 && ((mfull >> lane) & 1u) && mc > (kClosed ? kLongRow : 32));
@@ -678,7 +671,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32) row_fwd_kernel(Problem p, c
         const unsigned src = __fns(m8, 0, (lane >> 3) + 1);        // the row of this group of eight lanes
         const bool active = src < 32u;
         const int n_list = __shfl_sync(0xffffffffu, mc, active ? src : 0);
-        solve_rows_closed<D, 8, EC>(p, v, scale, entries, o, tau_out, row_cnt, active ? 16 * blk + (int)src : 0, active, n_list, false, lane);
+        solve_rows_closed<D, 8, EC>(p, v, scale, entries, o, tau_out, row_cnt, active ? rpw * blk + (int)src : 0, active, n_list, false, lane);
 #pragma unroll
         for (int t = 0; t < 4; ++t) m8 &= m8 - 1;
       }
@@ -686,7 +679,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32) row_fwd_kernel(Problem p, c
         const unsigned src = __fns(m16, 0, (lane >> 4) + 1);
         const bool active = src < 32u;
         const int n_list = __shfl_sync(0xffffffffu, mc, active ? src : 0);
-        solve_rows_closed<D, 16, EC>(p, v, scale, entries, o, tau_out, row_cnt, active ? 16 * blk + (int)src : 0, active,
+        solve_rows_closed<D, 16, EC>(p, v, scale, entries, o, tau_out, row_cnt, active ? rpw * blk + (int)src : 0, active,
                                      n_list, false, lane);
         m16 &= m16 - 1;
         m16 &= m16 - 1;
@@ -702,7 +695,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32) row_fwd_kernel(Problem p, c
           const int src = 4 * g + (lane >> 3);
           const bool active = (m8 >> src) & 1u;
           const int n_list = __shfl_sync(0xffffffffu, mc, src);
-          solve_rows_sub<D, 8>(p, v, scale, entries, o, tau_out, row_cnt, list_thr, active ? 16 * blk + src : 0, active, n_list, lane);
+          solve_rows_sub<D, 8>(p, v, scale, entries, o, tau_out, row_cnt, list_thr, active ? rpw * blk + src : 0, active, n_list, lane);
         } else {
           mfull |= (m8 | m16) & gm;
         }
@@ -711,7 +704,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32) row_fwd_kernel(Problem p, c
     while (mfull) {
       const int src = __ffs(mfull) - 1;
       mfull &= mfull - 1;
-      const int grow = 16 * blk + src;
+      const int grow = rpw * blk + src;
       const int n_list = __shfl_sync(0xffffffffu, mc, src);
       row_fwd_whole_warp<D, EC>(p, v, scale, row_cnt, list_thr, entries, o, tau_out, grow, n_list, lane);
     }
@@ -972,16 +965,18 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 4) row_bwd_kernel(
     const __nv_bfloat16* __restrict__ v, const __nv_bfloat16* __restrict__ d_o, const float* __restrict__ scale,
     const float* __restrict__ tau_in, const int32_t* __restrict__ list_cnt, const Entry* __restrict__ entries,
     __nv_bfloat16* __restrict__ dq, float* __restrict__ acc_dk, float* __restrict__ acc_dv,
-    float* __restrict__ dc_rows, int32_t* fb_count, int32_t* fb_list, int32_t* status, int saved, int pitch) {
+    float* __restrict__ dc_rows, int32_t* fb_count, int32_t* fb_list, uint32_t* tile_mask, int32_t* tile_flag,
+    int32_t* tile_list, int32_t* tile_count, int32_t* status, int saved, int pitch, int rpw) {
+  pdl_begin();
   // saved != 0: `list_cnt` is the forward pass's final support size per row (one int per row, -2 = dense
   // row) and `entries` its compacted support lists; `pitch` = list slots per row in `entries`
   const int lane = threadIdx.x & 31;
   const int total = p.B * p.H * p.N;
-  const int blocks = (total + 15) / 16;
+  const int blocks = (total + rpw - 1) / rpw;
   for (int blk = blockIdx.x * kWarpsPerCta + (threadIdx.x >> 5); blk < blocks; blk += gridDim.x * kWarpsPerCta) {
-    // A warp takes 16 consecutive rows; lane l (and l + 16) looks at row 16*blk + l.  Rows are served by list
+    // A warp takes rpw (16 or 8) consecutive rows; lane l (and l + 16) looks at row rpw*blk + l.  Rows are served by list
     // length: four at a time (<= 8 entries), two at a time (<= 16), one at a time (<= 32, or the long form).
-    const int my_row = 16 * blk + (lane & 15);
+    const int my_row = (lane & 15) < rpw ? rpw * blk + (lane & 15) : total;
     int mc = 0;
     int cls = 4;                                     // 0: <= 8 entries, 1: <= 16, 2: <= 32, 3: more / dense, 4: no row
     if (my_row < total) {
@@ -995,7 +990,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 4) row_bwd_kernel(
     {
       // rows without a usable list go to the dense path, all of the warp's at once
       const unsigned mdense = __ballot_sync(0xffffffffu, lane < 16 && my_row < total && mc < 0);
-      push_dense_rows(mdense, my_row, fb_count, fb_list, status, lane);
+      push_dense_tiles(p, mdense, my_row, tile_mask, tile_flag, tile_list, tile_count, status, lane);
       mlong &= ~mdense;
       // ... and the ones with long lists to a launch of their own (see push_long_rows)
       push_long_rows(mlong | m32, my_row, total, fb_count, fb_list, lane);
@@ -1005,7 +1000,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 4) row_bwd_kernel(
       const bool active = src < 32u;
       const int n_list = __shfl_sync(0xffffffffu, mc, active ? src : 0);
       bwd_rows_sub<D, 8>(p, q, k, v, d_o, scale, tau_in, entries, dq, acc_dk, acc_dv, dc_rows,
-                         active ? 16 * blk + (int)src : 0, active, n_list, saved != 0, pitch, lane);
+                         active ? rpw * blk + (int)src : 0, active, n_list, saved != 0, pitch, lane);
 #pragma unroll
       for (int t = 0; t < 4; ++t) m8 &= m8 - 1;
     }
@@ -1014,7 +1009,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 4) row_bwd_kernel(
       const bool active = src < 32u;
       const int n_list = __shfl_sync(0xffffffffu, mc, active ? src : 0);
       bwd_rows_sub<D, 16>(p, q, k, v, d_o, scale, tau_in, entries, dq, acc_dk, acc_dv, dc_rows,
-                          active ? 16 * blk + (int)src : 0, active, n_list, saved != 0, pitch, lane);
+                          active ? rpw * blk + (int)src : 0, active, n_list, saved != 0, pitch, lane);
       m16 &= m16 - 1;
       m16 &= m16 - 1;
     }
@@ -1030,6 +1025,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 4) row_bwd_long_kernel(
     __nv_bfloat16* __restrict__ dq, float* __restrict__ acc_dk, float* __restrict__ acc_dv,
     float* __restrict__ dc_rows, const int32_t* __restrict__ fb_count, const int32_t* __restrict__ fb_list, int saved,
     int pitch) {
+  pdl_begin();
   const int lane = threadIdx.x & 31;
   const int total = p.B * p.H * p.N;
   const int n_long = fb_count[kLongCounter];
@@ -1050,6 +1046,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 4) row_bwd_long_kernel(
 __global__ void save_supports_kernel(int rows, int slots, const int32_t* __restrict__ row_cnt,
                                      const Entry* __restrict__ entries, int32_t* __restrict__ out_cnt,
                                      Entry* __restrict__ out_entries) {
+  pdl_begin();
   const long total = (long)rows * slots;
   for (long t = (long)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (long)gridDim.x * blockDim.x) {
     const int row = (int)(t / slots), slot = (int)(t - (long)row * slots);
@@ -1060,9 +1057,14 @@ __global__ void save_supports_kernel(int rows, int slots, const int32_t* __restr
   }
 }
 
-inline int row_grid(const Problem& p) {
-  const long total = ((long)p.B * p.H * p.N + 3) / 4;   // one warp per group of four rows
-  const long ctas = (total + kWarpsPerCta - 1) / kWarpsPerCta;
+// Rows per warp.  A warp works its rows off in four to eight rounds of dependent loads, so while the grid fits the machine at
+// once its time is that of one warp: 8 rows per warp there (8 x 12 x 1024 x 64: forward 54 -> 50 us, backward 80 -> 74 us;
+// 16 x 8192 x 128 39 -> 32 and 55 -> 46).  16 rows pack best into rounds and win where the grid is several waves long; 4 lose
+// more in packing than they save (2 x 12 x 3001 x 64: 37 -> 47 and 93 -> 112 us).
+inline int rows_per_warp(const Problem& p) { return (long)p.B * p.H * p.N >= 148L * 64 * 16 ? 16 : 8; }
+inline int row_grid(const Problem& p, int rpw) {
+  const long warps = ((long)p.B * p.H * p.N + rpw - 1) / rpw;
+  const long ctas = (warps + kWarpsPerCta - 1) / kWarpsPerCta;
   const long cap = 148L * 8 * 8;
   return (int)(ctas < cap ? ctas : cap);
 }
@@ -1073,12 +1075,13 @@ cudaError_t launch_row_fwd(const Problem& p, const void* v, const float* scale, 
                            const int32_t* list_cnt, const float* list_thr, Entry* entries, void* o, float* tau,
                            int32_t* fb_count, int32_t* fb_list, int32_t* tile_flag, int32_t* tile_list,
                            int32_t* tile_count, int32_t* status, cudaStream_t stream) {
-  const int grid = row_grid(p);
+  const int rpw = rows_per_warp(p);
+  const int grid = row_grid(p, rpw);
 #define ENTMAX_ROW_FWD(D, EC)                                                                                         \
-  row_fwd_kernel<D, EC><<<grid, kWarpsPerCta * 32, 0, stream>>>(p, (const __nv_bfloat16*)v, scale, row_cnt, list_cnt, \
+  launch_kernel(row_fwd_kernel<D, EC>, grid, kWarpsPerCta * 32, 0, stream, p, (const __nv_bfloat16*)v, scale, row_cnt, list_cnt, \
                                                                 list_thr, entries, (__nv_bfloat16*)o, tau, fb_count,  \
                                                                 fb_list,                                              \
-                                                                tile_flag, tile_list, tile_count, status)
+                                                                tile_flag, tile_list, tile_count, status, rpw)
   if (p.D == 64) {
     if (p.expo_class == kExpo2) ENTMAX_ROW_FWD(64, kExpo2);
     else if (p.expo_class == kExpo1) ENTMAX_ROW_FWD(64, kExpo1);
@@ -1094,7 +1097,7 @@ cudaError_t launch_row_fwd(const Problem& p, const void* v, const float* scale, 
   // the rows it listed as long, one warp each (normally none or a few: the launch then ends at once)
   const int lgrid = grid < 148 * 4 ? grid : 148 * 4;
 #define ENTMAX_ROW_FWD_LONG(D, EC)                                                                                     \
-  row_fwd_long_kernel<D, EC><<<lgrid, kWarpsPerCta * 32, 0, stream>>>(p, (const __nv_bfloat16*)v, scale, row_cnt,       \
+  launch_kernel(row_fwd_long_kernel<D, EC>, lgrid, kWarpsPerCta * 32, 0, stream, p, (const __nv_bfloat16*)v, scale, row_cnt,       \
                                                                       list_cnt, list_thr, entries, (__nv_bfloat16*)o,  \
                                                                       tau, fb_count, fb_list)
   if (p.D == 64) {
@@ -1115,34 +1118,34 @@ cudaError_t launch_save_supports(const Problem& p, int slots, const int32_t* row
   const int rows = p.B * p.H * p.N;
   const long total = (long)rows * slots;
   const int blocks = (int)((total + 255) / 256 < 148L * 16 ? (total + 255) / 256 : 148L * 16);
-  save_supports_kernel<<<blocks, 256, 0, stream>>>(rows, slots, row_cnt, entries, out_cnt, out_entries);
+  launch_kernel(save_supports_kernel, blocks, 256, 0, stream, rows, slots, row_cnt, entries, out_cnt, out_entries);
   return cudaGetLastError();
 }
 
 cudaError_t launch_row_bwd(const Problem& p, const void* q, const void* k, const void* v, const void* d_o,
                            const float* scale, const float* tau, const int32_t* list_cnt, Entry* entries, void* dq,
                            float* acc_dk, float* acc_dv, float* dc_rows, int32_t* fb_count, int32_t* fb_list,
-                           int32_t* status, int saved, int pitch, cudaStream_t stream) {
-  const int grid = row_grid(p);
+                           uint32_t* tile_mask, int32_t* tile_flag, int32_t* tile_list, int32_t* tile_count, int32_t* status,
+                           int saved, int pitch, cudaStream_t stream) {
+  const int rpw = rows_per_warp(p);
+  const int grid = row_grid(p, rpw);
   if (p.D == 64)
-    row_bwd_kernel<64><<<grid, kWarpsPerCta * 32, 0, stream>>>(
-        p, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, (const __nv_bfloat16*)d_o, scale,
-        tau, list_cnt, entries, (__nv_bfloat16*)dq, acc_dk, acc_dv, dc_rows, fb_count, fb_list, status, saved, pitch);
+    launch_kernel(row_bwd_kernel<64>, grid, kWarpsPerCta * 32, 0, stream, p, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, (const __nv_bfloat16*)d_o, scale,
+        tau, list_cnt, entries, (__nv_bfloat16*)dq, acc_dk, acc_dv, dc_rows, fb_count,
+        fb_list, tile_mask, tile_flag, tile_list, tile_count, status, saved, pitch, rpw);
   else
-    row_bwd_kernel<128><<<grid, kWarpsPerCta * 32, 0, stream>>>(
-        p, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, (const __nv_bfloat16*)d_o, scale,
-        tau, list_cnt, entries, (__nv_bfloat16*)dq, acc_dk, acc_dv, dc_rows, fb_count, fb_list, status, saved, pitch);
+    launch_kernel(row_bwd_kernel<128>, grid, kWarpsPerCta * 32, 0, stream, p, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, (const __nv_bfloat16*)d_o, scale,
+        tau, list_cnt, entries, (__nv_bfloat16*)dq, acc_dk, acc_dv, dc_rows, fb_count,
+        fb_list, tile_mask, tile_flag, tile_list, tile_count, status, saved, pitch, rpw);
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) return err;
   // the rows it listed as long, one warp each (normally none or a few: the launch then ends at once)
   const int lgrid = grid < 148 * 4 ? grid : 148 * 4;
   if (p.D == 64)
-    row_bwd_long_kernel<64><<<lgrid, kWarpsPerCta * 32, 0, stream>>>(
-        p, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, (const __nv_bfloat16*)d_o, scale,
+    launch_kernel(row_bwd_long_kernel<64>, lgrid, kWarpsPerCta * 32, 0, stream, p, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, (const __nv_bfloat16*)d_o, scale,
         tau, list_cnt, entries, (__nv_bfloat16*)dq, acc_dk, acc_dv, dc_rows, fb_count, fb_list, saved, pitch);
   else
-    row_bwd_long_kernel<128><<<lgrid, kWarpsPerCta * 32, 0, stream>>>(
-        p, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, (const __nv_bfloat16*)d_o, scale,
+    launch_kernel(row_bwd_long_kernel<128>, lgrid, kWarpsPerCta * 32, 0, stream, p, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, (const __nv_bfloat16*)d_o, scale,
         tau, list_cnt, entries, (__nv_bfloat16*)dq, acc_dk, acc_dv, dc_rows, fb_count, fb_list, saved, pitch);
   return cudaGetLastError();
 }

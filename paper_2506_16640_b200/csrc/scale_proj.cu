@@ -129,6 +129,7 @@ __global__ void __launch_bounds__(kProjThreads) scale_proj_fwd_kernel(ProjArgs a
                                                                       const float* __restrict__ w_gamma,
                                                                       const float* __restrict__ delta,
                                                                       float* __restrict__ c_rows) {
+  pdl_begin();
   const int lane = threadIdx.x & 31;
   const long tokens = (long)a.B * a.N;
   const int rounds = (a.H + kHeads - 1) / kHeads;
@@ -161,6 +162,7 @@ __global__ void __launch_bounds__(kProjThreads) scale_proj_bwd_kernel(ProjArgs a
                                                                       float* __restrict__ dw_beta,
                                                                       float* __restrict__ dw_gamma,
                                                                       float* __restrict__ ddelta, T* __restrict__ dx) {
+  pdl_begin();
   extern __shared__ float4 sm4[];
   float* g_s = reinterpret_cast<float*>(sm4);      // [2][H][kChunk]: dL/d(pre beta), dL/d(pre gamma)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -297,7 +299,7 @@ int entmax_attn_scale_proj_fwd(const entmax_attn_proj_params* params, const void
   if (ctas > 148L * 16) ctas = 148L * 16;
   const bool vec = rows_aligned(a, {x, w_beta, w_gamma});
 #define ENTMAX_PROJ_FWD(T, VEC)                                                                                  \
-  scale_proj_fwd_kernel<T, VEC><<<(int)ctas, kProjThreads, 0, stream>>>(a, static_cast<const T*>(x), w_beta, w_gamma, delta, \
+  launch_kernel(scale_proj_fwd_kernel<T, VEC>, (int)ctas, kProjThreads, 0, stream, a, static_cast<const T*>(x), w_beta, w_gamma, delta, \
                                                                         c_rows)
   if (params->x_dtype == ENTMAX_ATTN_DTYPE_FP32) {
     if (vec) ENTMAX_PROJ_FWD(float, 4); else ENTMAX_PROJ_FWD(float, 1);
@@ -326,7 +328,7 @@ int entmax_attn_scale_proj_bwd(const entmax_attn_proj_params* params, const void
   const size_t smem = sizeof(float) * 2 * kChunk * a.H;
   const bool vec = rows_aligned(a, {x, w_beta, w_gamma, dw_beta, dw_gamma, dx});
 #define ENTMAX_PROJ_BWD(T, VEC, COLS)                                                                                 \
-  scale_proj_bwd_kernel<T, VEC, COLS><<<ctas, kProjThreads, smem, stream>>>(a, static_cast<const T*>(x), w_beta, w_gamma, \
+  launch_kernel(scale_proj_bwd_kernel<T, VEC, COLS>, ctas, kProjThreads, smem, stream, a, static_cast<const T*>(x), w_beta, w_gamma, \
                                                                             d_scale_rows, dw_beta, dw_gamma, ddelta,      \
                                                                             static_cast<T*>(dx))
   if (params->x_dtype == ENTMAX_ATTN_DTYPE_FP32) {

@@ -353,6 +353,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
                                                             const __grid_constant__ CUtensorMap map_k,
                                                             const __grid_constant__ CUtensorMap map_ks,
                                                             const __grid_constant__ SweepArgs a) {
+  pdl_begin();
   using C = Cfg<HD>;
   extern __shared__ uint8_t smem_raw[];
   // everything in shared memory is addressed by 32-bit shared-window addresses derived from one base
@@ -911,6 +912,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
 template <int HD>
 __global__ void __launch_bounds__(BN) key_norm_kernel(const __nv_bfloat16* __restrict__ k, int H, int N, long long sb,
                                                       long long sh, long long sn, int k_tiles, float* __restrict__ kmax) {
+  pdl_begin();
   __shared__ float red[BN / 32];
   const int bh = blockIdx.x / k_tiles, t = blockIdx.x - bh * k_tiles;
   const int b = bh / H, h = bh - b * H;
@@ -954,6 +956,7 @@ __global__ void __launch_bounds__(kItemRows) alibi_window_kernel(const __nv_bflo
                                                                  const float* __restrict__ slopes,
                                                                  const float* __restrict__ kmax, int k_tiles,
                                                                  float* __restrict__ blob) {
+  pdl_begin();
   __shared__ int red[kItemRows / 32];
   int bh, item;
   decode_item(a, blockIdx.x, bh, item);
@@ -1082,7 +1085,7 @@ cudaError_t launch_impl(const Problem& p, const void* q, const void* k, SweepArg
   err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (err != cudaSuccess) return err;
   const int grid = args.n_items < sms ? args.n_items : sms;
-  sweep_kernel<HD, kDump, kAlibi, kSearch><<<grid, kThreads, Cfg<HD>::kSmemBytes, stream>>>(map_q, map_k, map_ks, args);
+  launch_kernel(sweep_kernel<HD, kDump, kAlibi, kSearch>, grid, kThreads, Cfg<HD>::kSmemBytes, stream, map_q, map_k, map_ks, args);
   return cudaGetLastError();
 }
 
@@ -1118,12 +1121,12 @@ cudaError_t launch_sweep(const Problem& p, const void* q, const void* k, const f
     const __nv_bfloat16* qb = static_cast<const __nv_bfloat16*>(q);
     const __nv_bfloat16* kb = static_cast<const __nv_bfloat16*>(k);
     if (p.D == 64) {
-      key_norm_kernel<64><<<p.B * p.H * k_tiles, BN, 0, stream>>>(kb, p.H, p.N, p.sb, p.sh, p.sn, k_tiles, alibi_kmax);
-      alibi_window_kernel<64><<<args.n_items, kItemRows, 0, stream>>>(qb, kb, args, p.sb, p.sh, p.sn, p.alibi, alibi_kmax,
+      launch_kernel(key_norm_kernel<64>, p.B * p.H * k_tiles, BN, 0, stream, kb, p.H, p.N, p.sb, p.sh, p.sn, k_tiles, alibi_kmax);
+      launch_kernel(alibi_window_kernel<64>, args.n_items, kItemRows, 0, stream, qb, kb, args, p.sb, p.sh, p.sn, p.alibi, alibi_kmax,
                                                                       k_tiles, alibi_blob);
     } else {
-      key_norm_kernel<128><<<p.B * p.H * k_tiles, BN, 0, stream>>>(kb, p.H, p.N, p.sb, p.sh, p.sn, k_tiles, alibi_kmax);
-      alibi_window_kernel<128><<<args.n_items, kItemRows, 0, stream>>>(qb, kb, args, p.sb, p.sh, p.sn, p.alibi, alibi_kmax,
+      launch_kernel(key_norm_kernel<128>, p.B * p.H * k_tiles, BN, 0, stream, kb, p.H, p.N, p.sb, p.sh, p.sn, k_tiles, alibi_kmax);
+      launch_kernel(alibi_window_kernel<128>, args.n_items, kItemRows, 0, stream, qb, kb, args, p.sb, p.sh, p.sn, p.alibi, alibi_kmax,
                                                                        k_tiles, alibi_blob);
     }
     cudaError_t err = cudaGetLastError();

@@ -112,28 +112,13 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   return *reinterpret_cast<const uint32_t*>(&hh);
 }
 
-// Marks the rows of row_list[0 .. *row_count) in the per-tile masks and lists every tile once.
-__global__ void mark_tiles_kernel(int N, int tiles_per_head, const int32_t* __restrict__ row_list,
-                                  const int32_t* __restrict__ row_count, uint32_t* __restrict__ tile_mask,
-                                  int32_t* __restrict__ tile_flag, int32_t* __restrict__ tile_list,
-                                  int32_t* __restrict__ tile_count) {
-  const int total = *row_count;
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
-    const int grow = row_list[t];
-    const int bh = grow / N, i = grow - bh * N;
-    const int id = bh * tiles_per_head + i / TM;
-    const int r = i % TM;
-    atomicOr(tile_mask + 4 * (size_t)id + (r >> 5), 1u << (r & 31));
-    if (atomicExch(tile_flag + id, 1) == 0) tile_list[atomicAdd(tile_count, 1)] = id;
-  }
-}
-
 template <int HD, int EC>
 __global__ void __launch_bounds__(kThreadsB, 1) tile_bwd_kernel(const __grid_constant__ CUtensorMap map_q,
                                                                const __grid_constant__ CUtensorMap map_k,
                                                                const __grid_constant__ CUtensorMap map_v,
                                                                const __grid_constant__ CUtensorMap map_do,
                                                                const TileBwdArgs a) {
+  pdl_begin();
   using C = BCfg<HD>;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -173,6 +158,7 @@ __global__ void __launch_bounds__(kThreadsB, 1) tile_bwd_kernel(const __grid_con
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   const int n_tiles = *a.tile_count;
+  if (n_tiles == 0) return;                            // (before barriers, TMEM and the rest are set up)
 
   if (threadIdx.x == 0) {
     mbar_init(qdo_full, 1);
@@ -664,6 +650,7 @@ __global__ void __launch_bounds__(kThreadsB, 1) tile_bwd_kv_kernel(const __grid_
                                                                   const __grid_constant__ CUtensorMap map_dk,
                                                                   const __grid_constant__ CUtensorMap map_dv,
                                                                   const TileBwdArgs a) {
+  pdl_begin();
   using C = BCfg<HD>;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -692,7 +679,8 @@ __global__ void __launch_bounds__(kThreadsB, 1) tile_bwd_kv_kernel(const __grid_
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   const int n_bh = a.B * a.H;
-  const int n_items = (*a.tile_count > 0) ? n_bh * a.tiles_per_head : 0;   // nothing marked: nothing to do
+  const int n_items = n_bh * a.tiles_per_head;
+  if (*a.tile_count == 0) return;                      // nothing marked: nothing to do
 
   if (threadIdx.x == 0) {
     mbar_init(qdo_full, 1);
@@ -1075,14 +1063,14 @@ cudaError_t launch_tile_bwd_impl(const Problem& p, const void* q, const void* k,
   if (err != cudaSuccess) return err;
   const long all_tiles = (long)p.B * p.H * args.tiles_per_head;
   const int grid = (int)(all_tiles < sms ? all_tiles : sms);
-  tile_bwd_kernel<HD, EC><<<grid, kThreadsB, BCfg<HD>::kSmemBytes, stream>>>(map_q, map_k, map_v, map_do, args);
+  launch_kernel(tile_bwd_kernel<HD, EC>, grid, kThreadsB, BCfg<HD>::kSmemBytes, stream, map_q, map_k, map_v, map_do, args);
   err = cudaGetLastError();
   if (err != cudaSuccess) return err;
   // dK and dV of the same Q tiles, key-major (needs the rho the kernel above leaves behind)
   err = cudaFuncSetAttribute(tile_bwd_kv_kernel<HD, EC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              BCfg<HD>::kSmemBytes);
   if (err != cudaSuccess) return err;
-  tile_bwd_kv_kernel<HD, EC><<<grid, kThreadsB, BCfg<HD>::kSmemBytes, stream>>>(map_q, map_k, map_v, map_do, map_dk,
+  launch_kernel(tile_bwd_kv_kernel<HD, EC>, grid, kThreadsB, BCfg<HD>::kSmemBytes, stream, map_q, map_k, map_v, map_do, map_dk,
                                                                                 map_dv, args);
   return cudaGetLastError();
 }
@@ -1090,16 +1078,12 @@ cudaError_t launch_tile_bwd_impl(const Problem& p, const void* q, const void* k,
 }  // namespace
 
 cudaError_t launch_tile_bwd(const Problem& p, const void* q, const void* k, const void* v, const void* d_o,
-                            const float* scale, const float* tau, const int32_t* row_list, const int32_t* row_count,
-                            uint32_t* tile_mask, int32_t* tile_flag, int32_t* tile_list, int32_t* tile_count,
+                            const float* scale, const float* tau, const uint32_t* tile_mask, const int32_t* tile_flag,
+                            int32_t* tile_list, const int32_t* tile_count,
                             int32_t* work_counter, float* rho, void* dq, float* acc_dk, float* acc_dv, float* dc_rows,
                             int32_t* status, cudaStream_t stream) {
   const int tiles_per_head = (p.N + TM - 1) / TM;
-  mark_tiles_kernel<<<148, 256, 0, stream>>>(p.N, tiles_per_head, row_list, row_count, tile_mask, tile_flag, tile_list,
-                                             tile_count);
-  cudaError_t err = cudaGetLastError();
-  if (err != cudaSuccess) return err;
-  err = order_tiles(p, tile_flag, tile_list, tile_count, stream);
+  cudaError_t err = order_tiles(p, tile_flag, tile_list, tile_count, stream);
   if (err != cudaSuccess) return err;
   TileBwdArgs args;
   args.B = p.B; args.H = p.H; args.N = p.N;

@@ -119,6 +119,7 @@ __global__ void __launch_bounds__(kThreadsT, 1) tile_fwd_kernel(const __grid_con
                                                                const __grid_constant__ CUtensorMap map_v,
                                                                const __grid_constant__ CUtensorMap map_ks,
                                                                const TileArgsK a) {
+  pdl_begin();
   using C = TCfg<HD>;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -155,6 +156,7 @@ __global__ void __launch_bounds__(kThreadsT, 1) tile_fwd_kernel(const __grid_con
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   const int n_tiles = *a.tile_count;
+  if (n_tiles == 0) return;                            // (the usual case: 5 us with barriers, TMEM and the rest, 2 without)
 
   if (threadIdx.x == 0) {
     mbar_init(q_full, 1);
@@ -917,6 +919,7 @@ __global__ void __launch_bounds__(kThreadsT, 1) tile_fwd_kernel(const __grid_con
 __global__ void __launch_bounds__(1024) order_tiles_kernel(const int32_t* __restrict__ tile_flag, int tiles_per_head,
                                                            int n_bh, int32_t* __restrict__ tile_list,
                                                            const int32_t* __restrict__ tile_count) {
+  pdl_begin();
   __shared__ int warp_sum[32];
   __shared__ int base;
   if (*tile_count == 0) return;
@@ -973,7 +976,7 @@ cudaError_t launch_tile_impl(const Problem& p, const void* q, const void* k, con
   if (err != cudaSuccess) return err;
   const long all_tiles = (long)p.B * p.H * args.tiles_per_head;
   const int grid = (int)(all_tiles < sms ? all_tiles : sms);
-  tile_fwd_kernel<HD, EC><<<grid, kThreadsT, TCfg<HD>::kSmemBytes, stream>>>(map_q, map_k, map_v, map_ks, args);
+  launch_kernel(tile_fwd_kernel<HD, EC>, grid, kThreadsT, TCfg<HD>::kSmemBytes, stream, map_q, map_k, map_v, map_ks, args);
   return cudaGetLastError();
 }
 
@@ -1054,7 +1057,7 @@ cudaError_t make_sampled_tile_map(CUtensorMap* map, const void* base, int D, int
 cudaError_t order_tiles(const Problem& p, const int32_t* tile_flag, int32_t* tile_list, const int32_t* tile_count,
                         cudaStream_t stream) {
   if (!p.causal) return cudaSuccess;   // every Q tile sees the same keys: any order will do
-  order_tiles_kernel<<<1, 1024, 0, stream>>>(tile_flag, (p.N + TM - 1) / TM, p.B * p.H, tile_list, tile_count);
+  launch_kernel(order_tiles_kernel, 1, 1024, 0, stream, tile_flag, (p.N + TM - 1) / TM, p.B * p.H, tile_list, tile_count);
   return cudaGetLastError();
 }
 
