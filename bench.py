@@ -414,9 +414,9 @@ def run_ours(args):
         "e2e": {"value": flops_all / (e2e_ms_all * 1e-3) / 1e12, "unit": UNIT, "ms_per_step": e2e_ms_all,
                 "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h},
         # forward: scale table, score sweep, row solve, its long-list rows, tile order, dense tiles; backward: scale
-        # table, score sweep, row gradients, their long-list rows, tile marking, tile order, dense tiles (query-major
-        # and key-major kernels), two gradient stores
-        "gpu_launches": 16 * K,
+        # table, score sweep, row gradients, their long-list rows, tile order, dense tiles (query-major and key-major
+        # kernels), gradient store
+        "gpu_launches": 14 * K,
         "clocks": clocks,
     }
     if density is not None:

@@ -3,9 +3,7 @@
 //
 // Forward: exact threshold on the candidates (Eq. 1 with the sum-to-one condition), probabilities, and
 // O_i = sum_j p_ij v_j as a gather over the support only -- every zero of P is skipped, not just
-// all-zero tiles.  A warp takes up to 16 consecutive rows and serves them by list length (8, 16 or 32 lanes per
-// row).  alpha = 1.5 and alpha = 2 use the closed form on the sorted candidates (solve_rows_closed); other
-// exponents iterate (Newton from the left of the root, see dense_rows.cu) in two stages.
+// all-zero tiles.  A thread solves a row (lists of up to 32 entries, in registers), then lanes share the gathers of a row.
 // Backward: the entmax Jacobian dS = u (dP - <u,dP>/sum u), u = p^(2-alpha), on the support, dQ by
 // gathering K rows, dK / dV by vector atomics into fp32 accumulators.
 #include "common.cuh"
@@ -87,132 +85,111 @@ __device__ __forceinline__ void atomic_add_vec(float* p, const float (&x)[N]) {
     red_add_v4(p + 4 * c, x[4 * c], x[4 * c + 1], x[4 * c + 2], x[4 * c + 3]);
 }
 
-// Bitonic sort of 32*S (key j, value y) pairs held as S registers per lane (element index = 32*s + lane),
-// ascending by key.  Keys are distinct key indices (padding uses INT_MAX and sorts to the end).
-template <int S>
-__device__ __forceinline__ void sort_by_key(int (&jj)[S], float (&y)[S], int lane) {
-#pragma unroll
-  for (int k = 2; k <= 32 * S; k <<= 1) {
-#pragma unroll
-    for (int st = k >> 1; st > 0; st >>= 1) {
-      if (st >= 32) {
-        // partner sits in another register of the same lane
-#pragma unroll
-        for (int s = 0; s < S; ++s) {
-          const int ps = s ^ (st >> 5);
-          if (ps > s) {
-            const bool up = (((32 * s) & k) == 0);
-            const bool swap = up ? (jj[s] > jj[ps]) : (jj[s] < jj[ps]);
-            const int tj = swap ? jj[ps] : jj[s];
-            const float ty = swap ? y[ps] : y[s];
-            jj[ps] = swap ? jj[s] : jj[ps];
-            y[ps] = swap ? y[s] : y[ps];
-            jj[s] = tj;
-            y[s] = ty;
-          }
-        }
-      } else {
-#pragma unroll
-        for (int s = 0; s < S; ++s) {
-          const int idx = 32 * s + lane;
-          const int oj = __shfl_xor_sync(0xffffffffu, jj[s], st);
-          const float oy = __shfl_xor_sync(0xffffffffu, y[s], st);
-          const bool up = ((idx & k) == 0);
-          const bool lower = ((lane & st) == 0);
-          // the lower index keeps the smaller key when sorting upwards, the larger one otherwise
-          const bool take_other = (lower == up) ? (oj < jj[s]) : (oj > jj[s]);
-          jj[s] = take_other ? oj : jj[s];
-          y[s] = take_other ? oy : y[s];
-        }
-      }
-    }
-  }
-}
+// Row solve.  The lists the sweep leaves are deterministic (a row's candidates depend on that row alone, in key order), so a
+// threshold iterated on the whole list is reproducible to the bit.
+constexpr float kBoundMargin = 4e-6f;   // rounding of the bound the sweep ended with
 
-// The forward row solve runs in two stages so that its result does not depend on what else the sweep
-// happened to leave in the lists (their order and their surplus entries vary from run to run):
-//   stage A  Newton on all candidates, in list order -> tau_A, accurate to fp32 rounding;
-//   stage B  the entries above tau_A minus a small margin are compacted and sorted by key index, and
-//            Newton runs again on this set alone, from the bracket's lower end (App. A: tau >= y_max - 1);
-//            its summation order is fixed by the sorted set, so O and tau come out bit-identical
-//            unless an entry lies within rounding noise of the margin cut.
-constexpr float kKeepMargin = 4e-6f;
-
-// Threshold of Eq. 1 on the entries held by the warp, started at the bracket's lower end y_max - 1 (App. A):
-// Newton from the left for e >= 1, bracketed for e < 1 (tau_iter_update)
-template <int S>
-__device__ __forceinline__ float newton_warp(const Problem& p, const float (&y)[S], float ymax,
-                                             float known_below = -INFINITY) {
-  // known_below: a value the threshold is known not to lie below (mass >= 1 there); -inf: the bracket's own lower end
-  TauIter st = tau_iter_start(ymax);
-  st.tau = st.lo = fmaxf(st.lo, known_below);
-  for (int it = 0; it < kMaxNewton; ++it) {
-    float s0 = 0.f, s1 = 0.f;
-#pragma unroll
-    for (int s = 0; s < S; ++s) {
-      const float d = y[s] - st.tau;
-      if (d > 0.f) {
-        float ye, ye1;
-        pow_pair(d, p.expo_class, p.expo, ye, ye1);
-        s0 += ye;
-        s1 += ye1;
-      }
-    }
-    s0 = warp_sum(s0);
-    s1 = warp_sum(s1);
-    if (!tau_iter_update(st, s0, s1, p.expo_class, p.expo, 1e-7f)) break;
-  }
-  return st.tau;
-}
-
-// Stage A on S*32 candidate slots.  Leaves the kept entries (y in Eq. 1's units) compacted from slot 0
-// of the row's list and returns how many there are.
-template <int S>
-__device__ __forceinline__ int prefilter_row(const Problem& p, Entry* list, int n_list, float a, int lane,
-                                             float bound) {
-  float y[S];
-  int jj[S];
+// Threshold of Eq. 1 on the n <= K list entries of one row, by one thread with the entries in registers (n = 0: a lane without
+// a row, which only takes part in the votes); the list is left compacted to the support, y in Eq. 1's units.  Newton from the
+// left starting at the bound the sweep ended with (e < 1: bracketed, tau_iter_update).  Sums over a row need no shuffles this
+// way: eight to thirty-two lanes per row spent two chains of them on every iteration, or sorted the list first (alpha = 1.25,
+// 16 x 20011 x 128: 580 + 92 us with the long rows -> 227 + 66; alpha = 1.5, 16 x 32768 x 128: 222 + 105 -> 255 + 32).
+template <int K, int EC>
+__device__ __forceinline__ int solve_row(const Problem& p, Entry* list, int n, float a, float bound, float& tau) {
+  float y[K];
   float ymax = -INFINITY;
 #pragma unroll
-  for (int s = 0; s < S; ++s) {
-    const int e = lane + 32 * s;
-    y[s] = -INFINITY;
-    jj[s] = 0x7fffffff;
-    if (e < n_list) {
-      const Entry en = list[e];
-      y[s] = a * en.y;
-      jj[s] = en.j;
-    }
-    ymax = fmaxf(ymax, y[s]);
+  for (int e = 0; e < K; e += 2) {
+    float4 q = make_float4(-INFINITY, 0.f, -INFINITY, 0.f);
+    if (e < n) q = *reinterpret_cast<const float4*>(list + e);     // {y, j, y, j}
+    y[e] = e < n ? a * q.x : -INFINITY;
+    y[e + 1] = e + 1 < n ? a * q.z : -INFINITY;
+    ymax = fmaxf(ymax, fmaxf(y[e], y[e + 1]));
   }
-  ymax = warp_max(ymax);
-  __syncwarp();   // every slot is in registers before the list is overwritten
-  // stage A may start from the bound the sweep ended with (a lower bound of the row's threshold, and every key above
-  // it is in the list): only its cut is used, so where it starts does not reach the result
-  const float tau_a = newton_warp<S>(p, y, ymax, bound);
-  const float cut = tau_a - kKeepMargin * fmaxf(1.0f, fabsf(tau_a));
-  int kept = 0;
+  TauIter st = tau_iter_start(ymax);
+  st.tau = st.lo = fmaxf(st.lo, bound);
+  bool done = n == 0;
+  for (int it = 0; it < kMaxNewton; ++it) {
+    float s0[2] = {0.f, 0.f}, s1[2] = {0.f, 0.f};
 #pragma unroll
-  for (int s = 0; s < S; ++s) {
-    const bool keep = y[s] > cut;
-    const unsigned m = __ballot_sync(0xffffffffu, keep);
-    if (keep) {
-      const int pos = kept + __popc(m & ((1u << lane) - 1u));
-      list[pos].y = y[s];
-      list[pos].j = jj[s];
+    for (int e = 0; e < K; ++e) {
+      const float d = fmaxf(y[e] - st.tau, 0.f);
+      float ye, ye1;
+      pow_pair_c<EC>(d, d > 0.f, p.expo, ye, ye1);
+      s0[e & 1] += ye;
+      s1[e & 1] += ye1;
     }
-    kept += __popc(m);
+    if (!done) done = !tau_iter_update(st, s0[0] + s0[1], s1[0] + s1[1], p.expo_class, p.expo, 1e-7f);
+    if (__all_sync(0xffffffffu, done)) break;
   }
-  __syncwarp();
-  return kept;
+  tau = st.tau;
+  int cnt = 0;
+#pragma unroll
+  for (int e = 0; e < K; ++e) {
+    if (e < n && y[e] > tau) {
+      Entry en;
+      en.y = y[e];
+      en.j = list[e].j;
+      list[cnt++] = en;
+    }
+  }
+  return cnt;
 }
 
-// Stage B on the `kept` compacted entries (kept <= 32*S): sort by key index, threshold, probabilities,
-// O_i as a gather over the support, support written back sorted by key index.
-template <int D, int S>
-__device__ __forceinline__ void finish_row(const Problem& p, const __nv_bfloat16* __restrict__ vbase, Entry* list,
-                                           int kept_in, __nv_bfloat16* o_row, float* tau_slot, int32_t* cnt_slot,
-                                           int lane) {
+// O_i of 32 / W rows at once, W lanes per row, from the supports solve_row left (cnt <= W entries; cnt = 0: no row).
+template <int D, int W, int EC>
+__device__ __forceinline__ void gather_rows(const Problem& p, const __nv_bfloat16* __restrict__ v,
+                                            const Entry* __restrict__ entries, __nv_bfloat16* __restrict__ o, int grow, int cnt,
+                                            float tau, int lane) {
+  constexpr int PL = D / W;                        // elements of a V / O row per lane
+  constexpr int kBatch = 4;                        // V rows in flight
+  const int sl = lane & (W - 1);
+  const int base = lane & (32 - W);
+  const int bh = grow / p.N, i = grow - bh * p.N, b = bh / p.H, h = bh - b * p.H;
+  float pe = 0.f;
+  int j = 0;
+  if (sl < cnt) {
+    const Entry en = entries[(size_t)grow * kListCap + sl];
+    float pe1;
+    pow_pair_c<EC>(en.y - tau, true, p.expo, pe, pe1);
+    j = en.j;
+  }
+  float acc[PL];
+#pragma unroll
+  for (int t = 0; t < PL; ++t) acc[t] = 0.f;
+  const size_t hbase = (size_t)b * p.sb + (size_t)h * p.sh + sl * PL;
+#pragma unroll 1
+  for (int t0 = 0; t0 < W; t0 += kBatch) {
+    if (!__any_sync(0xffffffffu, t0 < cnt)) break;
+    float vs[kBatch][PL], pj[kBatch];
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u) {
+      pj[u] = __shfl_sync(0xffffffffu, pe, base + t0 + u);
+      const int kj = __shfl_sync(0xffffffffu, j, base + t0 + u);
+#pragma unroll
+      for (int e = 0; e < PL; ++e) vs[u][e] = 0.f;
+      if (t0 + u < cnt) {
+        if constexpr (PL >= 8) load_bf16_vec<PL>(v + hbase + (size_t)kj * p.sn, vs[u]);
+        else load_bf16<PL>(v + hbase + (size_t)kj * p.sn, vs[u]);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u)
+#pragma unroll
+      for (int e = 0; e < PL; ++e) acc[e] = fmaf(pj[u], vs[u][e], acc[e]);
+  }
+  if (cnt > 0) {
+    __nv_bfloat16* o_row = o + hbase + (size_t)i * p.sn;
+    if constexpr (PL >= 8) store_bf16_vec<PL>(o_row, acc);
+    else store_bf16<PL>(o_row, acc);
+  }
+}
+
+// One row with the whole warp, up to 32 S list entries: threshold, support, output.
+template <int D, int S, int EC>
+__device__ __forceinline__ void long_row(const Problem& p, const __nv_bfloat16* __restrict__ v, Entry* list, int n, float a,
+                                         float bound, __nv_bfloat16* __restrict__ o, float* __restrict__ tau_slot,
+                                         int32_t* __restrict__ cnt_slot, size_t hbase, int i, int lane) {
   constexpr int PER = D / 32;
   float y[S];
   int jj[S];
@@ -221,303 +198,74 @@ __device__ __forceinline__ void finish_row(const Problem& p, const __nv_bfloat16
   for (int s = 0; s < S; ++s) {
     const int e = lane + 32 * s;
     y[s] = -INFINITY;
-    jj[s] = 0x7fffffff;
-    if (e < kept_in) {
+    jj[s] = 0;
+    if (e < n) {
       const Entry en = list[e];
-      y[s] = en.y;
+      y[s] = a * en.y;
       jj[s] = en.j;
     }
     ymax = fmaxf(ymax, y[s]);
   }
   ymax = warp_max(ymax);
-  __syncwarp();
-  sort_by_key<S>(jj, y, lane);
-  const float tau = newton_warp<S>(p, y, ymax);
+  __syncwarp();   // every entry is in registers before the list is overwritten
+  TauIter st = tau_iter_start(ymax);
+  st.tau = st.lo = fmaxf(st.lo, bound);
+  for (int it = 0; it < kMaxNewton; ++it) {
+    float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+      const float d = fmaxf(y[s] - st.tau, 0.f);
+      float ye, ye1;
+      pow_pair_c<EC>(d, d > 0.f, p.expo, ye, ye1);
+      s0 += ye;
+      s1 += ye1;
+    }
+    s0 = warp_sum(s0);
+    s1 = warp_sum(s1);
+    if (!tau_iter_update(st, s0, s1, p.expo_class, p.expo, 1e-7f)) break;
+  }
+  const float tau = st.tau;
   float acc[PER];
 #pragma unroll
   for (int t = 0; t < PER; ++t) acc[t] = 0.f;
+  const __nv_bfloat16* vbase = v + hbase + lane * PER;
   int kept = 0;
 #pragma unroll
   for (int s = 0; s < S; ++s) {
-    const float d = y[s] - tau;
-    float pe = 0.f, pe1;
-    if (d > 0.f) pow_pair(d, p.expo_class, p.expo, pe, pe1);
-    const unsigned m = __ballot_sync(0xffffffffu, d > 0.f);
+    const float d = fmaxf(y[s] - tau, 0.f);
+    float pe, pe1;
+    pow_pair_c<EC>(d, d > 0.f, p.expo, pe, pe1);
+    unsigned m = __ballot_sync(0xffffffffu, d > 0.f);
     if (d > 0.f) {
       const int pos = kept + __popc(m & ((1u << lane) - 1u));
       list[pos].y = y[s];
       list[pos].j = jj[s];
     }
     kept += __popc(m);
-    unsigned rest = m;
-    while (rest) {
-      const int src = __ffs(rest) - 1;
-      rest &= rest - 1;
-      const float pj = __shfl_sync(0xffffffffu, pe, src);
-      const int kj = __shfl_sync(0xffffffffu, jj[s], src);
-      float vs[PER];
-      load_bf16<PER>(vbase + (size_t)kj * p.sn, vs);
+    while (m) {
+      // eight V rows in flight
+      float vs[8][PER], pj[8];
 #pragma unroll
-      for (int t = 0; t < PER; ++t) acc[t] = fmaf(pj, vs[t], acc[t]);
+      for (int u = 0; u < 8; ++u) {
+        const int src = m ? __ffs(m) - 1 : 0;
+        const int kj = __shfl_sync(0xffffffffu, jj[s], src);
+        pj[u] = __shfl_sync(0xffffffffu, pe, src);
+        if (!m) pj[u] = 0.f;
+#pragma unroll
+        for (int t = 0; t < PER; ++t) vs[u][t] = 0.f;
+        if (m) load_bf16<PER>(vbase + (size_t)kj * p.sn, vs[u]);
+        m &= m - 1;
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+#pragma unroll
+        for (int t = 0; t < PER; ++t) acc[t] = fmaf(pj[u], vs[u][t], acc[t]);
     }
   }
-  store_bf16<PER>(o_row, acc);
+  store_bf16<PER>(o + hbase + (size_t)i * p.sn + lane * PER, acc);
   if (lane == 0) {
     *tau_slot = tau;
     *cnt_slot = kept;
-  }
-}
-
-// Out-of-line forms for the rare rows with more than 32 candidates (kept out of the hot loop's code)
-__device__ __noinline__ int prefilter_long(const Problem& p, Entry* list, int n_list, float a, int lane,
-                                           float bound) {
-  const int n = n_list;
-  if (n <= 64) return prefilter_row<2>(p, list, n_list, a, lane, bound);
-  if (n <= 128) return prefilter_row<4>(p, list, n_list, a, lane, bound);
-  return prefilter_row<kSlots>(p, list, n_list, a, lane, bound);
-}
-template <int D>
-__device__ __noinline__ void finish_long(const Problem& p, const __nv_bfloat16* __restrict__ vbase, Entry* list, int kept,
-                                         __nv_bfloat16* o_row, float* tau_slot, int32_t* cnt_slot, int lane) {
-  if (kept <= 64) finish_row<D, 2>(p, vbase, list, kept, o_row, tau_slot, cnt_slot, lane);
-  else if (kept <= 128) finish_row<D, 4>(p, vbase, list, kept, o_row, tau_slot, cnt_slot, lane);
-  else finish_row<D, kSlots>(p, vbase, list, kept, o_row, tau_slot, cnt_slot, lane);
-}
-
-// One row with the whole warp.
-template <int D>
-__device__ __forceinline__ void solve_row_full(const Problem& p, const __nv_bfloat16* __restrict__ vbase, Entry* list,
-                                               int n_list, float a, float bound, __nv_bfloat16* o_row,
-                                               float* tau_slot, int32_t* cnt_slot, int lane) {
-  const int n = n_list;
-  int kept;
-  if (n <= 32) kept = prefilter_row<1>(p, list, n_list, a, lane, bound);
-  else if (n <= 64) kept = prefilter_row<2>(p, list, n_list, a, lane, bound);
-  else if (n <= 128) kept = prefilter_row<4>(p, list, n_list, a, lane, bound);
-  else kept = prefilter_row<kSlots>(p, list, n_list, a, lane, bound);
-  if (kept <= 32) finish_row<D, 1>(p, vbase, list, kept, o_row, tau_slot, cnt_slot, lane);
-  else if (kept <= 64) finish_row<D, 2>(p, vbase, list, kept, o_row, tau_slot, cnt_slot, lane);
-  else if (kept <= 128) finish_row<D, 4>(p, vbase, list, kept, o_row, tau_slot, cnt_slot, lane);
-  else finish_row<D, kSlots>(p, vbase, list, kept, o_row, tau_slot, cnt_slot, lane);
-}
-
-// The same iteration for 32 / W rows at once (W lanes per row); `done` rows keep their tau.
-template <int W>
-__device__ __forceinline__ float newton_sub(const Problem& p, float y, float ymax, bool done,
-                                            float known_below = -INFINITY) {
-  TauIter st = tau_iter_start(ymax);
-  st.tau = st.lo = fmaxf(st.lo, known_below);
-  for (int it = 0; it < kMaxNewton; ++it) {
-    const float d = y - st.tau;
-    float ye = 0.f, ye1 = 0.f;
-    if (d > 0.f) pow_pair(d, p.expo_class, p.expo, ye, ye1);
-    const float s0 = sub_sum<W>(ye), s1 = sub_sum<W>(ye1);
-    if (!done) done = !tau_iter_update(st, s0, s1, p.expo_class, p.expo, 1e-7f);
-    if (__all_sync(0xffffffffu, done)) break;
-  }
-  return st.tau;
-}
-
-// 32 / W rows at once, W lanes per row (W = 8 or 16), for rows with 1..W list entries; same two stages.
-template <int D, int W>
-__device__ __forceinline__ void solve_rows_sub(const Problem& p, const __nv_bfloat16* __restrict__ v,
-                                                const float* __restrict__ scale, Entry* __restrict__ entries,
-                                                __nv_bfloat16* __restrict__ o, float* __restrict__ tau_out,
-                                                int32_t* __restrict__ row_cnt, const float* __restrict__ list_thr,
-                                                int grow, bool active, int n_list, int lane) {
-  constexpr int PL = D / W;                        // elements of a V / O row per lane
-  const int sl = lane & (W - 1);
-  const int base = lane & (32 - W);
-  const int n = active ? n_list : 0;
-  const int bh = grow / p.N, i = grow - bh * p.N, b = bh / p.H, h = bh - b * p.H;
-  const float a = active ? (p.alpha - 1.0f) * (scale[(size_t)b * p.scale_sb + (size_t)h * p.N + i] * p.sm_scale) : 1.0f;
-  Entry* list = entries + (size_t)grow * kListCap;
-  float y = -INFINITY;
-  int j = 0x7fffffff;
-  if (sl < n) {
-    const Entry en = list[sl];
-    y = a * en.y;
-    j = en.j;
-  }
-  __syncwarp();   // every entry is in registers before the compaction below overwrites the lists
-  // stage A
-  // stage A starts from the bound the sweep ended with (see prefilter_row)
-  float bound = -INFINITY;
-  if (active) {
-    bound = list_thr[grow];
-    bound -= kKeepMargin * fmaxf(1.0f, fabsf(bound));
-  }
-  const float tau_a = newton_sub<W>(p, y, sub_max<W>(y), !active, bound);
-  const bool keep = active && y > tau_a - kKeepMargin * fmaxf(1.0f, fabsf(tau_a));
-  // keep only those: they move to the end-stable front when sorted with the others' keys pushed to infinity
-  j = keep ? j : 0x7fffffff;
-  y = keep ? y : -INFINITY;
-  // bitonic sort of the W (j, y) pairs of each row, ascending by key index
-#pragma unroll
-  for (int k = 2; k <= W; k <<= 1) {
-#pragma unroll
-    for (int st = k >> 1; st > 0; st >>= 1) {
-      const int oj = __shfl_xor_sync(0xffffffffu, j, st);
-      const float oy = __shfl_xor_sync(0xffffffffu, y, st);
-      const bool up = ((sl & k) == 0);
-      const bool lower = ((sl & st) == 0);
-      const bool take_other = (lower == up) ? (oj < j) : (oj > j);
-      j = take_other ? oj : j;
-      y = take_other ? oy : y;
-    }
-  }
-  // stage B
-  const float tau = newton_sub<W>(p, y, sub_max<W>(y), !active);
-  const float d = y - tau;
-  const bool in = active && d > 0.f;
-  float pe = 0.f, pe1;
-  if (in) pow_pair(d, p.expo_class, p.expo, pe, pe1);
-  const unsigned m = __ballot_sync(0xffffffffu, in);
-  const unsigned msub = (m >> base) & ((1u << W) - 1u);
-  if (in) {
-    // compact the list to the exact support, y in Eq. 1's units
-    const int pos = __popc(msub & ((1u << sl) - 1u));
-    list[pos].y = y;
-    list[pos].j = j;
-  }
-  float acc[PL];
-#pragma unroll
-  for (int t = 0; t < PL; ++t) acc[t] = 0.f;
-  const __nv_bfloat16* vbase = v + (size_t)b * p.sb + (size_t)h * p.sh + sl * PL;
-#pragma unroll
-  for (int t = 0; t < W; ++t) {
-    const bool has = (msub >> t) & 1u;
-    if (!__any_sync(0xffffffffu, has)) continue;
-    const float pj = __shfl_sync(0xffffffffu, pe, base + t);
-    const int kj = __shfl_sync(0xffffffffu, j, base + t);
-    if (has) {
-      float vs[PL];
-      if constexpr (PL >= 8) load_bf16_vec<PL>(vbase + (size_t)kj * p.sn, vs);
-      else load_bf16<PL>(vbase + (size_t)kj * p.sn, vs);
-#pragma unroll
-      for (int u = 0; u < PL; ++u) acc[u] = fmaf(pj, vs[u], acc[u]);
-    }
-  }
-  if (active) {
-    __nv_bfloat16* o_row = o + (size_t)b * p.sb + (size_t)h * p.sh + (size_t)i * p.sn + sl * PL;
-    if constexpr (PL >= 8) store_bf16_vec<PL>(o_row, acc);
-    else store_bf16<PL>(o_row, acc);
-    if (sl == 0) {
-      tau_out[grow] = tau;
-      row_cnt[grow] = __popc(msub);
-    }
-  }
-}
-
-// Closed-form row solve for e = 2 (alpha = 1.5) and e = 1 (alpha = 2), 32 / W rows at once with W lanes per row
-// (W = 8, 16 or 32) and at most W list entries per row.  With the entries sorted by decreasing y and
-// u_j = y_max - y_j, the threshold that makes the top k sum to one is, in units below the maximum,
-//   e = 2:  t_k = (U1 + sqrt(U1^2 - k (U2 - 1))) / k      (the root of sum_{j<=k} (t - u_j)^2 = 1 with t >= u_k)
-//   e = 1:  t_k = (1 + U1) / k                             (sum_{j<=k} (t - u_j) = 1)
-// with U1, U2 the prefix sums of u and u^2; the support size k* is the number of k with u_k < t_k (they form a
-// prefix) and tau = y_max - t_{k*} -- Eq. 1's threshold without iterating.  Only the top k* entries enter the
-// result, so candidates outside the support, which differ from run to run, do not change a bit of it.
-// `prescaled`: the list already holds y in Eq. 1's units from slot 0.
-template <int D, int W, int EC>
-__device__ __forceinline__ void solve_rows_closed(const Problem& p, const __nv_bfloat16* __restrict__ v,
-                                                  const float* __restrict__ scale, Entry* __restrict__ entries,
-                                                  __nv_bfloat16* __restrict__ o, float* __restrict__ tau_out,
-                                                  int32_t* __restrict__ row_cnt, int grow, bool active, int n_list,
-                                                  bool prescaled, int lane) {
-  static_assert(EC == kExpo2 || EC == kExpo1, "closed forms exist for e = 2 and e = 1");
-  constexpr int PL = D / W;                        // elements of a V / O row per lane
-  constexpr unsigned kWMask = W == 32 ? 0xffffffffu : ((1u << (W & 31)) - 1u);
-  const int sl = lane & (W - 1);
-  const int base = lane & (32 - W);
-  const int n = active ? n_list : 0;
-  const int bh = grow / p.N, i = grow - bh * p.N, b = bh / p.H, h = bh - b * p.H;
-  const float a = (active && !prescaled)
-                      ? (p.alpha - 1.0f) * (scale[(size_t)b * p.scale_sb + (size_t)h * p.N + i] * p.sm_scale) : 1.0f;
-  Entry* list = entries + (size_t)grow * kListCap;
-  float y = -INFINITY;
-  int j = 0x7fffffff;
-  if (sl < n) {
-    const Entry en = list[sl];
-    y = a * en.y;
-    j = en.j;
-  }
-  __syncwarp();   // every entry is in registers before the compaction below overwrites the lists
-  const float ymax = sub_max<W>(y);
-  // bitonic sort of the W (y, j) pairs of each row: decreasing y, equal values by increasing key index
-#pragma unroll
-  for (int k = 2; k <= W; k <<= 1) {
-#pragma unroll
-    for (int st = k >> 1; st > 0; st >>= 1) {
-      const int oj = __shfl_xor_sync(0xffffffffu, j, st);
-      const float oy = __shfl_xor_sync(0xffffffffu, y, st);
-      const bool up = ((sl & k) == 0);
-      const bool lower = ((sl & st) == 0);
-      const bool other_first = oy > y || (oy == y && oj < j);
-      const bool mine_first = y > oy || (y == oy && j < oj);
-      const bool take_other = (lower == up) ? other_first : mine_first;
-      j = take_other ? oj : j;
-      y = take_other ? oy : y;
-    }
-  }
-  const bool have = sl < n;
-  const float u = have ? ymax - y : 0.f;
-  float u1 = u, u2 = u * u;
-#pragma unroll
-  for (int off = 1; off < W; off <<= 1) {
-    const float t1 = __shfl_up_sync(0xffffffffu, u1, off, W);
-    const float t2 = __shfl_up_sync(0xffffffffu, u2, off, W);
-    if (sl >= off) {
-      u1 += t1;
-      u2 += t2;
-    }
-  }
-  const float kf = (float)(sl + 1);
-  float tk;
-  if constexpr (EC == kExpo2) {
-    const float disc = fmaf(u1, u1, -kf * (u2 - 1.0f));
-    tk = disc >= 0.f ? (u1 + sqrtf(disc)) / kf : -INFINITY;
-  } else {
-    tk = (1.0f + u1) / kf;
-  }
-  const unsigned okm = (__ballot_sync(0xffffffffu, have && u < tk) >> base) & kWMask;
-  const int kstar = okm == kWMask ? W : __ffs(~okm) - 1;          // leading ones; >= 1 for a row with entries
-  const float tprime = __shfl_sync(0xffffffffu, tk, base + (kstar > 0 ? kstar - 1 : 0));
-  const float tau = ymax - tprime;
-  const bool in = active && sl < kstar;
-  const float d = tprime - u;
-  const float pe = in ? (EC == kExpo2 ? d * d : d) : 0.f;
-  if (in) {
-    // the list becomes the exact support (by decreasing y), y in Eq. 1's units
-    list[sl].y = y;
-    list[sl].j = j;
-  }
-  float acc[PL];
-#pragma unroll
-  for (int t = 0; t < PL; ++t) acc[t] = 0.f;
-  const __nv_bfloat16* vbase = v + (size_t)b * p.sb + (size_t)h * p.sh + sl * PL;
-  // (not unrolled: a handful of iterations run, and the three widths of this function share the instruction cache)
-#pragma unroll 1
-  for (int t = 0; t < W; ++t) {
-    const bool has = active && t < kstar;
-    if (!__any_sync(0xffffffffu, has)) break;                      // supports are prefixes: nothing further either
-    const float pj = __shfl_sync(0xffffffffu, pe, base + t);
-    const int kj = __shfl_sync(0xffffffffu, j, base + t);
-    if (has) {
-      float vs[PL];
-      if constexpr (PL >= 8) load_bf16_vec<PL>(vbase + (size_t)kj * p.sn, vs);
-      else load_bf16<PL>(vbase + (size_t)kj * p.sn, vs);
-#pragma unroll
-      for (int u_ = 0; u_ < PL; ++u_) acc[u_] = fmaf(pj, vs[u_], acc[u_]);
-    }
-  }
-  if (active) {
-    __nv_bfloat16* o_row = o + (size_t)b * p.sb + (size_t)h * p.sh + (size_t)i * p.sn + sl * PL;
-    if constexpr (PL >= 8) store_bf16_vec<PL>(o_row, acc);
-    else store_bf16<PL>(o_row, acc);
-    if (sl == 0) {
-      tau_out[grow] = tau;
-      row_cnt[grow] = kstar;
-    }
   }
 }
 
@@ -528,7 +276,7 @@ __device__ __forceinline__ void solve_rows_closed(const Problem& p, const __nv_b
 // row) and a second launch gives each of them a warp of its own.  kLongCounter: their count, in the counter block
 // that starts at fb_count.
 constexpr int kLongCounter = 56;
-constexpr int kLongRow = 16;   // list entries from which a row counts as long
+constexpr int kLongRow = 32;   // list entries from which a row counts as long
 __device__ __forceinline__ void push_long_rows(unsigned mask, int grow, int total, int32_t* fb_count, int32_t* fb_list,
                                                int lane) {
   if (mask == 0u) return;
@@ -562,44 +310,6 @@ __device__ __forceinline__ void push_dense_tiles(const Problem& p, unsigned mask
   }
 }
 
-// One row with the whole warp: lists of more than 16 entries (closed forms) or any list the sub-warp Newton
-// solver did not take.
-template <int D, int EC>
-__device__ __forceinline__ void row_fwd_whole_warp(const Problem& p, const __nv_bfloat16* __restrict__ v,
-                                                   const float* __restrict__ scale, int32_t* __restrict__ row_cnt,
-                                                   const float* __restrict__ list_thr, Entry* __restrict__ entries,
-                                                   __nv_bfloat16* __restrict__ o, float* __restrict__ tau_out, int grow,
-                                                   int n_list, int lane) {
-  constexpr int PER = D / 32;
-  constexpr bool kClosed = EC == kExpo2 || EC == kExpo1;
-  const int bh = grow / p.N, i = grow - bh * p.N, b = bh / p.H, h = bh - b * p.H;
-  const float a = (p.alpha - 1.0f) * (scale[(size_t)b * p.scale_sb + (size_t)h * p.N + i] * p.sm_scale);
-  Entry* list = entries + (size_t)grow * kListCap;
-  float bound = list_thr[grow];
-  bound -= kKeepMargin * fmaxf(1.0f, fabsf(bound));
-  if constexpr (kClosed) {
-    // up to 32 entries: closed form with the whole warp; more: Newton prefilter first, and the closed form
-    // if what it keeps fits the warp
-    const int n = n_list;
-    if (n <= 32) {
-      solve_rows_closed<D, 32, EC>(p, v, scale, entries, o, tau_out, row_cnt, grow, true, n_list, false, lane);
-      return;
-    }
-    const int kept = prefilter_long(p, list, n_list, a, lane, bound);
-    if (kept <= 32) {
-      solve_rows_closed<D, 32, EC>(p, v, scale, entries, o, tau_out, row_cnt, grow, true, kept, true, lane);
-      return;
-    }
-    const __nv_bfloat16* vbase = v + (size_t)b * p.sb + (size_t)h * p.sh + lane * PER;
-    __nv_bfloat16* o_row = o + (size_t)b * p.sb + (size_t)h * p.sh + (size_t)i * p.sn + lane * PER;
-    finish_long<D>(p, vbase, list, kept, o_row, tau_out + grow, row_cnt + grow, lane);
-  } else {
-    const __nv_bfloat16* vbase = v + (size_t)b * p.sb + (size_t)h * p.sh + lane * PER;
-    __nv_bfloat16* o_row = o + (size_t)b * p.sb + (size_t)h * p.sh + (size_t)i * p.sn + lane * PER;
-    solve_row_full<D>(p, vbase, list, n_list, a, bound, o_row, tau_out + grow, row_cnt + grow, lane);
-  }
-}
-
 // The rows row_fwd_kernel listed as long (push_long_rows): one warp per row.
 template <int D, int EC>
 __global__ void __launch_bounds__(kWarpsPerCta * 32) row_fwd_long_kernel(Problem p, const __nv_bfloat16* __restrict__ v,
@@ -618,11 +328,19 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32) row_fwd_long_kernel(Problem
   const int n_long = fb_count[kLongCounter];
   for (int t = blockIdx.x * kWarpsPerCta + (threadIdx.x >> 5); t < n_long; t += gridDim.x * kWarpsPerCta) {
     const int grow = fb_list[total - 1 - t];
-    row_fwd_whole_warp<D, EC>(p, v, scale, row_cnt, list_thr, entries, o, tau_out, grow, list_cnt[2 * (size_t)grow], lane);
+    const int n = list_cnt[2 * (size_t)grow];
+    const int bh = grow / p.N, i = grow - bh * p.N, b = bh / p.H, h = bh - b * p.H;
+    const float a = (p.alpha - 1.0f) * (scale[(size_t)b * p.scale_sb + (size_t)h * p.N + i] * p.sm_scale);
+    float bound = list_thr[grow];
+    bound -= kBoundMargin * fmaxf(1.0f, fabsf(bound));
+    Entry* list = entries + (size_t)grow * kListCap;
+    const size_t hbase = (size_t)b * p.sb + (size_t)h * p.sh;
+    if (n <= 64) long_row<D, 2, EC>(p, v, list, n, a, bound, o, tau_out + grow, row_cnt + grow, hbase, i, lane);
+    else if (n <= 128) long_row<D, 4, EC>(p, v, list, n, a, bound, o, tau_out + grow, row_cnt + grow, hbase, i, lane);
+    else long_row<D, kSlots, EC>(p, v, list, n, a, bound, o, tau_out + grow, row_cnt + grow, hbase, i, lane);
   }
 }
 
-// EC: kExpo2 / kExpo1 select the closed-form solvers, kExpoGeneral the Newton ones (any exponent)
 template <int D, int EC>
 __global__ void __launch_bounds__(kWarpsPerCta * 32) row_fwd_kernel(Problem p, const __nv_bfloat16* __restrict__ v,
                                                                     const float* __restrict__ scale,
@@ -640,73 +358,67 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32) row_fwd_kernel(Problem p, c
   const int total = p.B * p.H * p.N;
   const int blocks = (total + rpw - 1) / rpw;
   for (int blk = blockIdx.x * kWarpsPerCta + (threadIdx.x >> 5); blk < blocks; blk += gridDim.x * kWarpsPerCta) {
-    // A warp takes rpw (16 or 8) consecutive rows; lane l (and l + 16) looks at row rpw*blk + l.  Rows are then served by
-    // list length: four at a time with eight lanes each (1..8 entries), two at a time with sixteen lanes
-    // each (9..16 entries), the rest one by one with the whole warp.
-    constexpr bool kClosed = EC == kExpo2 || EC == kExpo1;
-    const int my_row = (lane & 15) < rpw ? rpw * blk + (lane & 15) : total;
-    int mc = 0;
-    int cls = 3;                                     // 0: <= 8 entries, 1: <= 16, 2: whole warp / dense, 3: no row
-    if (my_row < total) {
-      mc = list_cnt[2 * (size_t)my_row];
-      cls = (mc < 1 || mc > 16) ? 2 : mc <= 8 ? 0 : 1;
-    }
-    unsigned m8 = __ballot_sync(0xffffffffu, lane < 16 && cls == 0);
-    unsigned m16 = __ballot_sync(0xffffffffu, lane < 16 && cls == 1);
-    unsigned mfull = __ballot_sync(0xffffffffu, lane < 16 && cls == 2);
+    // A warp takes rpw (32, 16 or 8) consecutive rows; lane l looks at row rpw*blk + l and solves it.  The rows' outputs are
+    // then gathered by support size: four rows at a time with eight lanes each (up to 8 entries), two with sixteen (up to
+    // 16), one with the whole warp.
+    const int my_row = lane < rpw ? rpw * blk + lane : total;
+    int n = 0;
+    if (my_row < total) n = list_cnt[2 * (size_t)my_row];
     {
-      // rows without a usable list go to the dense-tile path, all of the warp's at once
-      const unsigned mdense =
-          __ballot_sync(0xffffffffu, lane < 16 && my_row < total && mc < 1);
+      // rows without a usable list go to the dense-tile path, all of the warp's at once, the ones with long lists to a
+      // launch of their own
+      const unsigned mdense = __ballot_sync(0xffffffffu, my_row < total && n < 1);
       push_dense_tiles(p, mdense, my_row, nullptr, tile_flag, tile_list, tile_count, status, lane);
       if ((mdense >> lane) & 1u) row_cnt[my_row] = -2;
-      mfull &= ~mdense;
-      // ... and the ones with long lists to a launch of their own
-      const unsigned mlong = __ballot_sync(0xffffffffu, lane < 16 && ((mfull >> lane) & 1u) && mc > (kClosed ? kLongRow : 32));
+      const unsigned mlong = __ballot_sync(0xffffffffu, n > kLongRow);
       push_long_rows(mlong, my_row, total, fb_count, fb_list, lane);
-      mfull &= ~mlong;
+      if (n < 0 || n > kLongRow) n = 0;
     }
-    if constexpr (kClosed) {
-      while (m8) {
-        const unsigned src = __fns(m8, 0, (lane >> 3) + 1);        // the row of this group of eight lanes
-        const bool active = src < 32u;
-        const int n_list = __shfl_sync(0xffffffffu, mc, active ? src : 0);
-        solve_rows_closed<D, 8, EC>(p, v, scale, entries, o, tau_out, row_cnt, active ? rpw * blk + (int)src : 0, active, n_list, false, lane);
-#pragma unroll
-        for (int t = 0; t < 4; ++t) m8 &= m8 - 1;
-      }
-      while (m16) {
-        const unsigned src = __fns(m16, 0, (lane >> 4) + 1);
-        const bool active = src < 32u;
-        const int n_list = __shfl_sync(0xffffffffu, mc, active ? src : 0);
-        solve_rows_closed<D, 16, EC>(p, v, scale, entries, o, tau_out, row_cnt, active ? rpw * blk + (int)src : 0, active,
-                                     n_list, false, lane);
-        m16 &= m16 - 1;
-        m16 &= m16 - 1;
-      }
-    } else {
-      // Newton solvers: rows that iterate together wait for the slowest, so only groups of four consecutive
-      // rows that all have at most eight entries share a warp; every other row takes the whole warp.
-      const unsigned none = __ballot_sync(0xffffffffu, lane < 16 && cls == 3);
-#pragma unroll
-      for (int g = 0; g < 4; ++g) {
-        const unsigned gm = 0xFu << (4 * g);
-        if ((m8 & gm) != 0u && ((m8 | none) & gm) == gm) {
-          const int src = 4 * g + (lane >> 3);
-          const bool active = (m8 >> src) & 1u;
-          const int n_list = __shfl_sync(0xffffffffu, mc, src);
-          solve_rows_sub<D, 8>(p, v, scale, entries, o, tau_out, row_cnt, list_thr, active ? rpw * blk + src : 0, active, n_list, lane);
-        } else {
-          mfull |= (m8 | m16) & gm;
-        }
-      }
+    float a = 1.0f, bound = -INFINITY, tau = 0.f;
+    if (n > 0) {
+      const int bh = my_row / p.N, i = my_row - bh * p.N, b = bh / p.H, h = bh - b * p.H;
+      a = (p.alpha - 1.0f) * (scale[(size_t)b * p.scale_sb + (size_t)h * p.N + i] * p.sm_scale);
+      bound = list_thr[my_row];
+      bound -= kBoundMargin * fmaxf(1.0f, fabsf(bound));
     }
-    while (mfull) {
-      const int src = __ffs(mfull) - 1;
-      mfull &= mfull - 1;
-      const int grow = rpw * blk + src;
-      const int n_list = __shfl_sync(0xffffffffu, mc, src);
-      row_fwd_whole_warp<D, EC>(p, v, scale, row_cnt, list_thr, entries, o, tau_out, grow, n_list, lane);
+    Entry* list = entries + (size_t)(my_row < total ? my_row : 0) * kListCap;
+    const int n_max = __reduce_max_sync(0xffffffffu, n);
+    int cnt = 0;
+    if (n_max > 16) cnt = solve_row<32, EC>(p, list, n, a, bound, tau);
+    else if (n_max > 8) cnt = solve_row<16, EC>(p, list, n, a, bound, tau);
+    else if (n_max > 0) cnt = solve_row<8, EC>(p, list, n, a, bound, tau);
+    if (n > 0) {
+      tau_out[my_row] = tau;
+      row_cnt[my_row] = cnt;
+    }
+    __syncwarp();   // the supports are ordered before the other lanes' loads
+    unsigned m8 = __ballot_sync(0xffffffffu, cnt > 0 && cnt <= 8);
+    unsigned m16 = __ballot_sync(0xffffffffu, cnt > 8 && cnt <= 16);
+    unsigned m32 = __ballot_sync(0xffffffffu, cnt > 16);
+    while (m8) {
+      const unsigned src = __fns(m8, 0, (lane >> 3) + 1);        // the row of this group of eight lanes
+      const bool active = src < 32u;
+      const int c = __shfl_sync(0xffffffffu, cnt, active ? src : 0);
+      const float t = __shfl_sync(0xffffffffu, tau, active ? src : 0);
+      gather_rows<D, 8, EC>(p, v, entries, o, active ? rpw * blk + (int)src : 0, active ? c : 0, t, lane);
+#pragma unroll
+      for (int z = 0; z < 4; ++z) m8 &= m8 - 1;
+    }
+    while (m16) {
+      const unsigned src = __fns(m16, 0, (lane >> 4) + 1);
+      const bool active = src < 32u;
+      const int c = __shfl_sync(0xffffffffu, cnt, active ? src : 0);
+      const float t = __shfl_sync(0xffffffffu, tau, active ? src : 0);
+      gather_rows<D, 16, EC>(p, v, entries, o, active ? rpw * blk + (int)src : 0, active ? c : 0, t, lane);
+      m16 &= m16 - 1;
+      m16 &= m16 - 1;
+    }
+    while (m32) {
+      const int src = __ffs(m32) - 1;
+      m32 &= m32 - 1;
+      const int c = __shfl_sync(0xffffffffu, cnt, src);
+      const float t = __shfl_sync(0xffffffffu, tau, src);
+      gather_rows<D, 32, EC>(p, v, entries, o, rpw * blk + src, c, t, lane);
     }
   }
 }
@@ -1061,7 +773,10 @@ __global__ void save_supports_kernel(int rows, int slots, const int32_t* __restr
 // once its time is that of one warp: 8 rows per warp there (8 x 12 x 1024 x 64: forward 54 -> 50 us, backward 80 -> 74 us;
 // 16 x 8192 x 128 39 -> 32 and 55 -> 46).  16 rows pack best into rounds and win where the grid is several waves long; 4 lose
 // more in packing than they save (2 x 12 x 3001 x 64: 37 -> 47 and 93 -> 112 us).
-inline int rows_per_warp(const Problem& p) { return (long)p.B * p.H * p.N >= 148L * 64 * 16 ? 16 : 8; }
+inline int rows_per_warp(const Problem& p, int most) {
+  const long rows = (long)p.B * p.H * p.N;
+  return rows >= 148L * 64 * most ? most : rows >= 148L * 64 * 16 ? 16 : 8;
+}
 inline int row_grid(const Problem& p, int rpw) {
   const long warps = ((long)p.B * p.H * p.N + rpw - 1) / rpw;
   const long ctas = (warps + kWarpsPerCta - 1) / kWarpsPerCta;
@@ -1075,7 +790,7 @@ cudaError_t launch_row_fwd(const Problem& p, const void* v, const float* scale, 
                            const int32_t* list_cnt, const float* list_thr, Entry* entries, void* o, float* tau,
                            int32_t* fb_count, int32_t* fb_list, int32_t* tile_flag, int32_t* tile_list,
                            int32_t* tile_count, int32_t* status, cudaStream_t stream) {
-  const int rpw = rows_per_warp(p);
+  const int rpw = rows_per_warp(p, 32);
   const int grid = row_grid(p, rpw);
 #define ENTMAX_ROW_FWD(D, EC)                                                                                         \
   launch_kernel(row_fwd_kernel<D, EC>, grid, kWarpsPerCta * 32, 0, stream, p, (const __nv_bfloat16*)v, scale, row_cnt, list_cnt, \
@@ -1085,10 +800,12 @@ cudaError_t launch_row_fwd(const Problem& p, const void* v, const float* scale, 
   if (p.D == 64) {
     if (p.expo_class == kExpo2) ENTMAX_ROW_FWD(64, kExpo2);
     else if (p.expo_class == kExpo1) ENTMAX_ROW_FWD(64, kExpo1);
+    else if (p.expo_class == kExpo4) ENTMAX_ROW_FWD(64, kExpo4);
     else ENTMAX_ROW_FWD(64, kExpoGeneral);
   } else {
     if (p.expo_class == kExpo2) ENTMAX_ROW_FWD(128, kExpo2);
     else if (p.expo_class == kExpo1) ENTMAX_ROW_FWD(128, kExpo1);
+    else if (p.expo_class == kExpo4) ENTMAX_ROW_FWD(128, kExpo4);
     else ENTMAX_ROW_FWD(128, kExpoGeneral);
   }
 #undef ENTMAX_ROW_FWD
@@ -1103,10 +820,12 @@ cudaError_t launch_row_fwd(const Problem& p, const void* v, const float* scale, 
   if (p.D == 64) {
     if (p.expo_class == kExpo2) ENTMAX_ROW_FWD_LONG(64, kExpo2);
     else if (p.expo_class == kExpo1) ENTMAX_ROW_FWD_LONG(64, kExpo1);
+    else if (p.expo_class == kExpo4) ENTMAX_ROW_FWD_LONG(64, kExpo4);
     else ENTMAX_ROW_FWD_LONG(64, kExpoGeneral);
   } else {
     if (p.expo_class == kExpo2) ENTMAX_ROW_FWD_LONG(128, kExpo2);
     else if (p.expo_class == kExpo1) ENTMAX_ROW_FWD_LONG(128, kExpo1);
+    else if (p.expo_class == kExpo4) ENTMAX_ROW_FWD_LONG(128, kExpo4);
     else ENTMAX_ROW_FWD_LONG(128, kExpoGeneral);
   }
 #undef ENTMAX_ROW_FWD_LONG
@@ -1127,7 +846,7 @@ cudaError_t launch_row_bwd(const Problem& p, const void* q, const void* k, const
                            float* acc_dk, float* acc_dv, float* dc_rows, int32_t* fb_count, int32_t* fb_list,
                            uint32_t* tile_mask, int32_t* tile_flag, int32_t* tile_list, int32_t* tile_count, int32_t* status,
                            int saved, int pitch, cudaStream_t stream) {
-  const int rpw = rows_per_warp(p);
+  const int rpw = rows_per_warp(p, 16);
   const int grid = row_grid(p, rpw);
   if (p.D == 64)
     launch_kernel(row_bwd_kernel<64>, grid, kWarpsPerCta * 32, 0, stream, p, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, (const __nv_bfloat16*)d_o, scale,
