@@ -463,16 +463,29 @@ __device__ __noinline__ void bwd_row_full(const Problem& p, const __nv_bfloat16*
   for (int s = 0; s < kSlots; ++s) {
     unsigned rest = __ballot_sync(0xffffffffu, yv[s] > 0.f);
     while (rest) {
-      const int src = __ffs(rest) - 1;
-      rest &= rest - 1;
-      const int kj = __shfl_sync(0xffffffffu, jj[s], src);
-      float vs[PER];
-      load_bf16<PER>(v + hbase + (size_t)kj * p.sn, vs);
-      float dp = 0.f;
+      // four V rows in flight
+      float vs[4][PER], dp[4];
+      int src[4];
 #pragma unroll
-      for (int t = 0; t < PER; ++t) dp = fmaf(gs[t], vs[t], dp);
-      dp = warp_sum(dp);
-      if (lane == src) dpv[s] = dp;
+      for (int z = 0; z < 4; ++z) {
+        src[z] = rest ? __ffs(rest) - 1 : -1;
+        const int kj = __shfl_sync(0xffffffffu, jj[s], src[z] < 0 ? 0 : src[z]);
+#pragma unroll
+        for (int t = 0; t < PER; ++t) vs[z][t] = 0.f;
+        if (rest) load_bf16<PER>(v + hbase + (size_t)kj * p.sn, vs[z]);
+        rest &= rest - 1;
+      }
+#pragma unroll
+      for (int z = 0; z < 4; ++z) {
+        dp[z] = 0.f;
+#pragma unroll
+        for (int t = 0; t < PER; ++t) dp[z] = fmaf(gs[t], vs[z][t], dp[z]);
+      }
+#pragma unroll
+      for (int z = 0; z < 4; ++z) {
+        dp[z] = warp_sum(dp[z]);
+        if (lane == src[z]) dpv[s] = dp[z];
+      }
     }
   }
   float pe[kSlots], u[kSlots];
@@ -505,21 +518,36 @@ __device__ __noinline__ void bwd_row_full(const Problem& p, const __nv_bfloat16*
     const float gds_own = g * u[s] * (dpv[s] - rho);
     unsigned rest = __ballot_sync(0xffffffffu, yv[s] > 0.f);
     while (rest) {
-      const int src = __ffs(rest) - 1;
-      rest &= rest - 1;
-      const int kj = __shfl_sync(0xffffffffu, jj[s], src);
-      const float gds = __shfl_sync(0xffffffffu, gds_own, src);
-      const float pj = __shfl_sync(0xffffffffu, pe[s], src);
-      float ks[PER], dkv[PER], dvv[PER];
-      load_bf16<PER>(k + hbase + (size_t)kj * p.sn, ks);
+      float ks[4][PER];
+      unsigned r4 = rest;
 #pragma unroll
-      for (int t = 0; t < PER; ++t) {
-        acc[t] = fmaf(gds, ks[t], acc[t]);
-        dkv[t] = gds * qs[t];
-        dvv[t] = pj * gs[t];
+      for (int z = 0; z < 4; ++z) {
+        const int kj = __shfl_sync(0xffffffffu, jj[s], r4 ? __ffs(r4) - 1 : 0);
+#pragma unroll
+        for (int t = 0; t < PER; ++t) ks[z][t] = 0.f;
+        if (r4) load_bf16<PER>(k + hbase + (size_t)kj * p.sn, ks[z]);
+        r4 &= r4 - 1;
       }
-      atomic_add_slice<PER>(acc_dk + (arow + kj) * D + lane * PER, dkv);
-      atomic_add_slice<PER>(acc_dv + (arow + kj) * D + lane * PER, dvv);
+#pragma unroll
+      for (int z = 0; z < 4; ++z) {
+        if (rest) {
+          const int src = __ffs(rest) - 1;
+          rest &= rest - 1;
+          const int kj = __shfl_sync(0xffffffffu, jj[s], src);
+          const float gds = __shfl_sync(0xffffffffu, gds_own, src);
+          const float pj = __shfl_sync(0xffffffffu, pe[s], src);
+          float x[PER];
+#pragma unroll
+          for (int t = 0; t < PER; ++t) {
+            acc[t] = fmaf(gds, ks[z][t], acc[t]);
+            x[t] = gds * qs[t];
+          }
+          atomic_add_slice<PER>(acc_dk + (arow + kj) * D + lane * PER, x);
+#pragma unroll
+          for (int t = 0; t < PER; ++t) x[t] = pj * gs[t];
+          atomic_add_slice<PER>(acc_dv + (arow + kj) * D + lane * PER, x);
+        }
+      }
     }
   }
   store_bf16<PER>(dq + hbase + (size_t)i * p.sn, acc);
@@ -616,22 +644,49 @@ __device__ __forceinline__ void bwd_rows_sub(const Problem& p, const __nv_bfloat
   }
   const bool in = yv > 0.f;
   const unsigned msub = (__ballot_sync(0xffffffffu, in) >> base) & kWMask;
-  // dP_ij = <dO_i, v_j> on the support
+  // dP_ij = <dO_i, v_j> on the support.  A warp per row keeps four V (and below, K) rows in flight (long-row kernel 113 -> 77 us on
+  // 2 x 12 x 3001 x 64); rows that share a warp hold longer slices, and batches of them spill (630 -> 797 us on 16 x 32768 x 128)
   float dpv = 0.f;
-#pragma unroll 4
-  for (int t = 0; t < W; ++t) {
-    if (!__any_sync(0xffffffffu, (msub >> t) != 0u)) break;        // no row has entries from slot t on
-    const bool has = (msub >> t) & 1u;
-    const int kj = __shfl_sync(0xffffffffu, j, base + t);
-    float dp = 0.f;
-    if (has) {
-      float vs[PL];
-      load_share<PL, W>(v + hbase + (size_t)kj * p.sn, sl, vs);
+  if constexpr (W == 32) {
+#pragma unroll 1
+    for (int t0 = 0; t0 < W; t0 += 4) {
+      if ((msub >> t0) == 0u) break;
+      float vs[4][PL], dp[4];
 #pragma unroll
-      for (int u = 0; u < PL; ++u) dp = fmaf(gs[u], vs[u], dp);
+      for (int z = 0; z < 4; ++z) {
+        const int kj = __shfl_sync(0xffffffffu, j, t0 + z);
+#pragma unroll
+        for (int w = 0; w < PL; ++w) vs[z][w] = 0.f;
+        if ((msub >> (t0 + z)) & 1u) load_share<PL, W>(v + hbase + (size_t)kj * p.sn, sl, vs[z]);
+      }
+#pragma unroll
+      for (int z = 0; z < 4; ++z) {
+        dp[z] = 0.f;
+#pragma unroll
+        for (int w = 0; w < PL; ++w) dp[z] = fmaf(gs[w], vs[z][w], dp[z]);
+      }
+#pragma unroll
+      for (int z = 0; z < 4; ++z) {
+        dp[z] = sub_sum<W>(dp[z]);
+        if (sl == t0 + z) dpv = dp[z];
+      }
     }
-    dp = sub_sum<W>(dp);
-    if (sl == t) dpv = dp;
+  } else {
+#pragma unroll 4
+    for (int t = 0; t < W; ++t) {
+      if (!__any_sync(0xffffffffu, (msub >> t) != 0u)) break;        // no row has entries from slot t on
+      const bool has = (msub >> t) & 1u;
+      const int kj = __shfl_sync(0xffffffffu, j, base + t);
+      float dp = 0.f;
+      if (has) {
+        float vs[PL];
+        load_share<PL, W>(v + hbase + (size_t)kj * p.sn, sl, vs);
+#pragma unroll
+        for (int u = 0; u < PL; ++u) dp = fmaf(gs[u], vs[u], dp);
+      }
+      dp = sub_sum<W>(dp);
+      if (sl == t) dpv = dp;
+    }
   }
   float pe = 0.f, u = 0.f;
   if (in) pow_pair(yv, p.expo_class, p.expo, pe, u);
@@ -647,24 +702,57 @@ __device__ __forceinline__ void bwd_rows_sub(const Problem& p, const __nv_bfloat
 #pragma unroll
   for (int t = 0; t < PL; ++t) acc[t] = 0.f;
   const size_t arow = (size_t)bh * p.N;
-#pragma unroll 4
-  for (int t = 0; t < W; ++t) {
-    if (!__any_sync(0xffffffffu, (msub >> t) != 0u)) break;
-    const bool has = (msub >> t) & 1u;
-    const int kj = __shfl_sync(0xffffffffu, j, base + t);
-    const float gds = __shfl_sync(0xffffffffu, gds_own, base + t);
-    const float pj = __shfl_sync(0xffffffffu, pe, base + t);
-    if (has) {
-      float ks[PL], dkv[PL], dvv[PL];
-      load_share<PL, W>(k + hbase + (size_t)kj * p.sn, sl, ks);
+  if constexpr (W == 32) {
+#pragma unroll 1
+    for (int t0 = 0; t0 < W; t0 += 4) {
+      if ((msub >> t0) == 0u) break;
+      float ks[4][PL];
 #pragma unroll
-      for (int w = 0; w < PL; ++w) {
-        acc[w] = fmaf(gds, ks[w], acc[w]);
-        dkv[w] = gds * qs[w];
-        dvv[w] = pj * gs[w];
+      for (int z = 0; z < 4; ++z) {
+        const int kj = __shfl_sync(0xffffffffu, j, t0 + z);
+#pragma unroll
+        for (int w = 0; w < PL; ++w) ks[z][w] = 0.f;
+        if ((msub >> (t0 + z)) & 1u) load_share<PL, W>(k + hbase + (size_t)kj * p.sn, sl, ks[z]);
       }
-      add_share<PL, W>(acc_dk + (arow + kj) * D, sl, dkv);
-      add_share<PL, W>(acc_dv + (arow + kj) * D, sl, dvv);
+#pragma unroll
+      for (int z = 0; z < 4; ++z) {
+        const int kj = __shfl_sync(0xffffffffu, j, t0 + z);
+        const float gds = __shfl_sync(0xffffffffu, gds_own, t0 + z);
+        const float pj = __shfl_sync(0xffffffffu, pe, t0 + z);
+        if ((msub >> (t0 + z)) & 1u) {
+          float x[PL];
+#pragma unroll
+          for (int w = 0; w < PL; ++w) {
+            acc[w] = fmaf(gds, ks[z][w], acc[w]);
+            x[w] = gds * qs[w];
+          }
+          add_share<PL, W>(acc_dk + (arow + kj) * D, sl, x);
+#pragma unroll
+          for (int w = 0; w < PL; ++w) x[w] = pj * gs[w];
+          add_share<PL, W>(acc_dv + (arow + kj) * D, sl, x);
+        }
+      }
+    }
+  } else {
+#pragma unroll 4
+    for (int t = 0; t < W; ++t) {
+      if (!__any_sync(0xffffffffu, (msub >> t) != 0u)) break;
+      const bool has = (msub >> t) & 1u;
+      const int kj = __shfl_sync(0xffffffffu, j, base + t);
+      const float gds = __shfl_sync(0xffffffffu, gds_own, base + t);
+      const float pj = __shfl_sync(0xffffffffu, pe, base + t);
+      if (has) {
+        float ks[PL], dkv[PL], dvv[PL];
+        load_share<PL, W>(k + hbase + (size_t)kj * p.sn, sl, ks);
+#pragma unroll
+        for (int w = 0; w < PL; ++w) {
+          acc[w] = fmaf(gds, ks[w], acc[w]);
+          dkv[w] = gds * qs[w];
+          dvv[w] = pj * gs[w];
+        }
+        add_share<PL, W>(acc_dk + (arow + kj) * D, sl, dkv);
+        add_share<PL, W>(acc_dv + (arow + kj) * D, sl, dvv);
+      }
     }
   }
   if (active) store_share<PL, W>(dq + hbase + (size_t)i * p.sn, sl, acc);
