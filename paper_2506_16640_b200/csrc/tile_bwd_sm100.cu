@@ -660,11 +660,12 @@ __global__ void __launch_bounds__(kThreadsB, 1) tile_bwd_kv_kernel(const __grid_
   const uint32_t v_smem = k_smem + C::kQBytes;
   const uint32_t p_smem = v_smem + C::kQBytes;           // P tile, [128 rows][128 keys] bf16, swizzled
   const uint32_t ds_smem = p_smem + kTileBytes;           // g dS tile (bf16), same layout; with P the staging tile
-  const uint32_t bars = ds_smem + 2 * kTileBytes;         // (the query-major kernel's layout: the third tile is unused)
-  const uint32_t qdo_full = bars, qdo_empty = bars + 8;
+  const uint32_t q1_smem = ds_smem + kTileBytes;          // second stage of the Q tile
+  const uint32_t bars = q1_smem + kTileBytes;
+  const uint32_t do_full = bars, do_empty = bars + 8;
   const uint32_t kv_full = bars + 16, kv_empty = bars + 24;
-  const uint32_t sd_full = bars + 32, sd_empty = bars + 40;
-  const uint32_t pds_full = bars + 48, pds_empty = bars + 56;
+  const uint32_t s_full = bars + 32, s_empty = bars + 40;
+  const uint32_t p_full = bars + 48, p_empty = bars + 56;
   const uint32_t acc_full = bars + 64, acc_empty = bars + 72;
   const uint32_t tmem_slot = bars + 96;
   const uint32_t abort_flag = bars + 100;
@@ -674,6 +675,10 @@ __global__ void __launch_bounds__(kThreadsB, 1) tile_bwd_kv_kernel(const __grid_
   const uint32_t w_empty = bars + 136;        // [2]
   const uint32_t w_item = bars + 152;         // int32 [2]: item, -1 = no more work
   const uint32_t x_bar = bars + 160;
+  const uint32_t dp_full = bars + 168, dp_empty = bars + 176;
+  const uint32_t ds_full = bars + 184, ds_empty = bars + 192;
+  const uint32_t q_full = bars + 200;         // [2]
+  const uint32_t q_empty = bars + 216;        // [2]
   constexpr int kTmemDK = 2 * TN, kTmemDV = 2 * TN + 128;
 
   const int warp = threadIdx.x >> 5;
@@ -683,19 +688,25 @@ __global__ void __launch_bounds__(kThreadsB, 1) tile_bwd_kv_kernel(const __grid_
   if (*a.tile_count == 0) return;                      // nothing marked: nothing to do
 
   if (threadIdx.x == 0) {
-    mbar_init(qdo_full, 1);
-    mbar_init(qdo_empty, 1);
+    mbar_init(do_full, 1);
+    mbar_init(do_empty, 1);
     mbar_init(kv_full, 1);
     mbar_init(kv_empty, 1);
-    mbar_init(sd_full, 1);
-    mbar_init(sd_empty, kConsWarps);
-    mbar_init(pds_full, kConsWarps);
-    mbar_init(pds_empty, 1);
+    mbar_init(s_full, 1);
+    mbar_init(s_empty, kConsWarps);
+    mbar_init(dp_full, 1);
+    mbar_init(dp_empty, kConsWarps);
+    mbar_init(p_full, kConsWarps);
+    mbar_init(p_empty, 1);
+    mbar_init(ds_full, kConsWarps);
+    mbar_init(ds_empty, 1);
     mbar_init(acc_full, 1);
     mbar_init(acc_empty, kConsWarps);
     mbar_init(x_bar, kConsWarps);
     mbar_init(drain_bar, 1);
     for (int t = 0; t < 2; ++t) {
+      mbar_init(q_full + 8 * t, 1);
+      mbar_init(q_empty + 8 * t, 1);
       mbar_init(w_full + 8 * t, 1);
       mbar_init(w_empty + 8 * t, 1 + kConsWarps);
     }
@@ -723,8 +734,9 @@ __global__ void __launch_bounds__(kThreadsB, 1) tile_bwd_kv_kernel(const __grid_
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
-    uint32_t kvphase = 0, qphase = 0, wphase = 0;
-    int slot = 0;
+    uint32_t kvphase = 0, dophase = 0, wphase = 0;
+    uint32_t qbits = 0;      // bit st: times stage st of Q has been armed, mod 2
+    int slot = 0, qst = 0;
     bool alive = true;
     auto wait_all = [&](uint32_t bar, uint32_t parity) -> bool {
       return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag));
@@ -758,23 +770,34 @@ __global__ void __launch_bounds__(kThreadsB, 1) tile_bwd_kv_kernel(const __grid_
       }
       __syncwarp();
       while (qt < a.tiles_per_head && alive) {
-        alive = wait_all(qdo_empty, qphase ^ 1u);
+        // the next pair's Q arrives under this pair's element code (two stages); its dO as soon as dV has taken this one
+        alive = wait_all(q_empty + 8 * qst, ((qbits >> qst) & 1u) ^ 1u);
         if (!alive) break;
-        qphase ^= 1u;
+        qbits ^= 1u << qst;
         if (elect_one()) {
-          mbar_expect_tx(qdo_full, 2 * C::kQBytes);
-          for (int hf = 0; hf < C::kHalves; ++hf) {
-            tma_load_4d(q_smem + hf * (TM * 128), &map_q, qdo_full, hf * 64, qt * TM, h, b);
-            tma_load_4d(do_smem + hf * (TM * 128), &map_do, qdo_full, hf * 64, qt * TM, h, b);
-          }
+          const uint32_t dst = qst ? q1_smem : q_smem;
+          mbar_expect_tx(q_full + 8 * qst, C::kQBytes);
+          for (int hf = 0; hf < C::kHalves; ++hf)
+            tma_load_4d(dst + hf * (TM * 128), &map_q, q_full + 8 * qst, hf * 64, qt * TM, h, b);
+        }
+        __syncwarp();
+        qst ^= 1;
+        alive = wait_all(do_empty, dophase ^ 1u);
+        if (!alive) break;
+        dophase ^= 1u;
+        if (elect_one()) {
+          mbar_expect_tx(do_full, C::kQBytes);
+          for (int hf = 0; hf < C::kHalves; ++hf)
+            tma_load_4d(do_smem + hf * (TM * 128), &map_do, do_full, hf * 64, qt * TM, h, b);
         }
         __syncwarp();
         qt = __shfl_sync(0xffffffffu, next_marked(bh, qt + 1), 0);
       }
     }
     if (!alive && lane == 0) {
-      bool ok = mbar_drain(qdo_full, qphase ^ 1u);
+      bool ok = mbar_drain(do_full, dophase ^ 1u);
       ok &= mbar_drain(kv_full, kvphase ^ 1u);
+      for (int st = 0; st < 2; ++st) ok &= mbar_drain(q_full + 8 * st, ((qbits >> st) & 1u) ^ 1u);
       if (!ok) sts_u32(drain_fail, 1u);
     }
   } else if (warp == 1) {
@@ -784,10 +807,11 @@ __global__ void __launch_bounds__(kThreadsB, 1) tile_bwd_kv_kernel(const __grid_
     const uint64_t hi = (uint64_t)kDescHi << 32;
     const uint64_t q_d = hi | smem_desc_lo(q_smem), do_d = hi | smem_desc_lo(do_smem);
     const uint64_t k_d = hi | smem_desc_lo(k_smem), v_d = hi | smem_desc_lo(v_smem);
-    const uint64_t q_n_d = hi | mn_desc_lo(q_smem), do_n_d = hi | mn_desc_lo(do_smem);
+    const uint64_t q1_d = hi | smem_desc_lo(q1_smem);
+    const uint64_t q_n_d = hi | mn_desc_lo(q_smem), q1_n_d = hi | mn_desc_lo(q1_smem), do_n_d = hi | mn_desc_lo(do_smem);
     const uint64_t ds_m_d = hi | mn_desc_lo(ds_smem), p_m_d = hi | mn_desc_lo(p_smem);
-    uint32_t kvphase = 0, qphase = 0, sdphase = 0, pdsphase = 0, accphase = 0, wphase = 0;
-    int slot = 0;
+    uint32_t kvphase = 0, qbits = 0, dophase = 0, sphase = 0, dpphase = 0, pphase = 0, dsphase = 0, accphase = 0, wphase = 0;
+    int slot = 0, qst = 0;      // qst: the Q stage the next S reads
     bool alive = true;
     auto wait_all = [&](uint32_t bar, uint32_t parity) -> bool {
       return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag));
@@ -805,60 +829,105 @@ __global__ void __launch_bounds__(kThreadsB, 1) tile_bwd_kv_kernel(const __grid_
       if (qt >= a.tiles_per_head) continue;
       alive = wait_all(kv_full, kvphase);
       kvphase ^= 1u;
-      // the previous item's dK and dV must have been read before this item's first contraction overwrites them
-      if (alive) alive = wait_all(acc_empty, accphase ^ 1u);
-      accphase ^= 1u;
       if (!alive) break;
-      bool first = true;
-      while (qt < a.tiles_per_head && alive) {
-        alive = wait_all(qdo_full, qphase);
-        qphase ^= 1u;
-        if (alive) alive = wait_all(sd_empty, sdphase ^ 1u);
-        if (!alive) break;
-        sdphase ^= 1u;
+      // S = Q K^T of the next pair
+      auto issue_s = [&]() -> bool {
+        bool ok = wait_all(q_full + 8 * qst, (qbits >> qst) & 1u);
+        qbits ^= 1u << qst;
+        if (ok) ok = wait_all(s_empty, sphase ^ 1u);
+        sphase ^= 1u;
+        if (!ok) return false;
+        tc_fence_after();
+        const uint64_t qs_d = qst ? q1_d : q_d;
+        if (elect_one()) {
+#pragma unroll
+          for (int kk = 0; kk < HD / 16; ++kk) {
+            const uint32_t off = (kk >> 2) * ((TM * 128) >> 4) + (kk & 3) * 2;
+            umma_bf16_desc(tmem_base + C::kTmemS, qs_d + off, k_d + off, id_kk, kk > 0 ? 1u : 0u);
+          }
+          umma_commit(s_full);
+        }
+        __syncwarp();
+        qst ^= 1;
+        return true;
+      };
+      // dP = dO V^T of the same pair
+      auto issue_dp = [&]() -> bool {
+        bool ok = wait_all(do_full, dophase);
+        dophase ^= 1u;
+        if (ok) ok = wait_all(dp_empty, dpphase ^ 1u);
+        dpphase ^= 1u;
+        if (!ok) return false;
         tc_fence_after();
         if (elect_one()) {
 #pragma unroll
           for (int kk = 0; kk < HD / 16; ++kk) {
             const uint32_t off = (kk >> 2) * ((TM * 128) >> 4) + (kk & 3) * 2;
-            umma_bf16_desc(tmem_base + C::kTmemS, q_d + off, k_d + off, id_kk, kk > 0 ? 1u : 0u);
-          }
-#pragma unroll
-          for (int kk = 0; kk < HD / 16; ++kk) {
-            const uint32_t off = (kk >> 2) * ((TM * 128) >> 4) + (kk & 3) * 2;
             umma_bf16_desc(tmem_base + C::kTmemDP, do_d + off, v_d + off, id_kk, kk > 0 ? 1u : 0u);
           }
-          umma_commit(sd_full);
+          umma_commit(dp_full);
         }
         __syncwarp();
-        // P and g dS of this pair are in shared memory
-        alive = wait_all(pds_full, pdsphase);
-        pdsphase ^= 1u;
+        return true;
+      };
+      alive = issue_s();
+      if (alive) alive = issue_dp();
+      bool first = true;
+      while (alive) {
+        const int nxt = __shfl_sync(0xffffffffu, next_marked(bh, qt + 1), 0);
+        const bool more = nxt < a.tiles_per_head;
+        const uint64_t qn = qst ? q_n_d : q1_n_d;      // this pair's Q: the stage before the next one
+        const int cur = qst ^ 1;
+        if (!more) {
+          if (elect_one()) umma_commit(kv_empty);      // the item's last S and dP: K and V are free behind them
+          __syncwarp();
+        }
+        // P of this pair is in shared memory
+        alive = wait_all(p_full, pphase);
+        pphase ^= 1u;
+        if (alive && first) {
+          // the previous item's dK and dV must have been read before this item's first contraction overwrites them
+          alive = wait_all(acc_empty, accphase ^ 1u);
+          accphase ^= 1u;
+        }
         if (!alive) break;
         tc_fence_after();
         if (elect_one()) {
 #pragma unroll
           for (int kk = 0; kk < TM / 16; ++kk) {
             const uint32_t off = kk * ((16 * 128) >> 4);                             // 16 query rows
-            umma_bf16_desc(tmem_base + kTmemDK, ds_m_d + off, q_n_d + off, id_mn, (!first || kk > 0) ? 1u : 0u);
+            umma_bf16_desc(tmem_base + kTmemDV, p_m_d + off, do_n_d + off, id_mn, (!first || kk > 0) ? 1u : 0u);
           }
+          umma_commit(do_empty);
+          umma_commit(p_empty);
+        }
+        __syncwarp();
+        if (more) {
+          alive = issue_s();
+          if (!alive) break;
+        }
+        // g dS of this pair is in shared memory
+        alive = wait_all(ds_full, dsphase);
+        dsphase ^= 1u;
+        if (!alive) break;
+        tc_fence_after();
+        if (elect_one()) {
 #pragma unroll
           for (int kk = 0; kk < TM / 16; ++kk) {
             const uint32_t off = kk * ((16 * 128) >> 4);
-            umma_bf16_desc(tmem_base + kTmemDV, p_m_d + off, do_n_d + off, id_mn, (!first || kk > 0) ? 1u : 0u);
+            umma_bf16_desc(tmem_base + kTmemDK, ds_m_d + off, qn + off, id_mn, (!first || kk > 0) ? 1u : 0u);
           }
-          umma_commit(pds_empty);
-          umma_commit(qdo_empty);
+          umma_commit(q_empty + 8 * cur);
+          umma_commit(ds_empty);
         }
         __syncwarp();
         first = false;
-        qt = __shfl_sync(0xffffffffu, next_marked(bh, qt + 1), 0);
+        if (!more) break;
+        qt = nxt;
+        alive = issue_dp();
       }
       if (!alive) break;
-      if (elect_one()) {
-        umma_commit(acc_full);
-        umma_commit(kv_empty);
-      }
+      if (elect_one()) umma_commit(acc_full);
       __syncwarp();
     }
     if (!alive && lane == 0) {
@@ -871,7 +940,7 @@ __global__ void __launch_bounds__(kThreadsB, 1) tile_bwd_kv_kernel(const __grid_
     const int quarter = (warp - 2) >> 2;
     const int row_local = quad * 32 + lane;
     const uint32_t taddr_row = tmem_base + ((uint32_t)(quad * 32) << 16);
-    uint32_t sdphase = 0, pdsphase = 0, accphase = 0, wphase = 0, xphase = 0;
+    uint32_t sphase = 0, dpphase = 0, pphase = 0, dsphase = 0, accphase = 0, wphase = 0, xphase = 0;
     int slot = 0;
     bool alive = true;
     while (alive) {
@@ -887,86 +956,121 @@ __global__ void __launch_bounds__(kThreadsB, 1) tile_bwd_kv_kernel(const __grid_
       int qt = __shfl_sync(0xffffffffu, next_marked(bh, first_q(kt)), 0);
       if (qt >= a.tiles_per_head) continue;
       const float slope = a.alibi ? a.alibi[h] / a.sm_scale : 0.f;   // bias in accumulator units
+      // this thread's query row of a Q tile (TMEM lane = query row, as in the query-major pass), read one Q tile ahead
+      float c_n = 0.f, tau_n = 0.f, rho_n = 0.f;
+      uint32_t mask_n = 0u;
+      int flag_n = 0;
+      auto fetch = [&](int tq) {
+        const int r = tq * TM + row_local;
+        const int rc = r < a.N ? r : a.N - 1;
+        c_n = a.scale[(size_t)b * a.scale_sb + (size_t)h * a.N + rc];
+        tau_n = a.tau[(size_t)bh * a.N + rc];
+        rho_n = a.rho[(size_t)bh * a.N + rc];
+        mask_n = r < a.N ? a.tile_mask[4 * (size_t)(bh * a.tiles_per_head + tq) + (row_local >> 5)] : 0u;
+        flag_n = tq + 1 < a.tiles_per_head ? a.tile_flag[bh * a.tiles_per_head + tq + 1] : 0;
+      };
+      fetch(qt);
       while (qt < a.tiles_per_head && alive) {
-        // this thread's query row of the Q tile: TMEM lane = query row, as in the query-major pass
         const int i = qt * TM + row_local;
-        const bool valid = i < a.N;
-        const int id = bh * a.tiles_per_head + qt;
-        const bool marked = valid && ((a.tile_mask[4 * (size_t)id + (row_local >> 5)] >> (row_local & 31)) & 1u);
-        const size_t grow = (size_t)bh * a.N + (valid ? i : 0);
+        const bool marked = (mask_n >> (row_local & 31)) & 1u;
         const int lim = a.causal ? i : a.N - 1;
-        const float c_i = valid ? a.scale[(size_t)b * a.scale_sb + (size_t)h * a.N + i] : 0.f;
-        const float ra = a.alpha_m1 * (c_i * a.sm_scale);
-        const float g = c_i * a.sm_scale;
-        const float tau = marked ? a.tau[grow] : 0.f;
-        const float rho = marked ? a.rho[grow] : 0.f;
-        const float ra_m = marked ? ra : 0.f;
-        alive = __all_sync(0xffffffffu, mbar_wait(sd_full, sdphase, abort_flag));
+        const float g = c_n * a.sm_scale;
+        const float ra_m = marked ? a.alpha_m1 * g : 0.f;
+        const float tau = marked ? tau_n : 0.f;
+        const float rho = marked ? rho_n : 0.f;
+        // the next marked Q tile: mostly the next one, whose flag came with this tile's values
+        int nxt = qt + 1;
+        if (flag_n == 0) nxt = __shfl_sync(0xffffffffu, next_marked(bh, nxt), 0);
+        if (nxt < a.tiles_per_head) fetch(nxt);
+        alive = __all_sync(0xffffffffu, mbar_wait(s_full, sphase, abort_flag));
         if (!alive) break;
-        sdphase ^= 1u;
+        sphase ^= 1u;
         tc_fence_after();
-        // P and dS of the previous pair must have been consumed before their buffers are rewritten
-        alive = __all_sync(0xffffffffu, mbar_wait(pds_empty, pdsphase ^ 1u, abort_flag));
-        pdsphase ^= 1u;
+        const int col0 = kt * TN + quarter * 32;
+        const bool edge = col0 + 31 > lim;
+        const uint32_t blk = (uint32_t)(quarter >> 1) * (TM * 128) + (uint32_t)row_local * 128u;
+        const uint32_t unit0 = (uint32_t)((quarter & 1) * 4), swz = (uint32_t)(row_local & 7);
+        // this thread's 32 columns: P from S; u = P^(2-alpha) stays in registers for dS
+        float ye1[32];
+        tmem_ld32(taddr_row + C::kTmemS + quarter * 32, ye1);
+        tmem_ld_wait();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(s_empty);           // S has been read
+        if (slope != 0.f) {
+#pragma unroll
+          for (int u = 0; u < 32; ++u) ye1[u] = fmaf(slope, (float)(col0 + u - i), ye1[u]);
+        }
+        // P of the previous pair must have been consumed before its buffer is rewritten
+        alive = __all_sync(0xffffffffu, mbar_wait(p_empty, pphase ^ 1u, abort_flag));
+        pphase ^= 1u;
         if (!alive) break;
-#pragma unroll 1
+#pragma unroll
+        for (int u4 = 0; u4 < 4; ++u4) {
+          float pv[8];
+          if (EC != kExpoGeneral && !edge) {
+            // away from the mask (an unmarked row has a = 0, tau = 0 here: every entry clamps to zero)
+#pragma unroll
+            for (int z = 0; z < 8; ++z) {
+              const float m = fmaxf(fmaf(ra_m, ye1[u4 * 8 + z], -tau), 0.f);
+              const float y1 = clamped_pow_m1<EC>(m);
+              pv[z] = y1 * m;
+              ye1[u4 * 8 + z] = y1;
+            }
+          } else {
+#pragma unroll
+            for (int z = 0; z < 8; ++z) {
+              const int u = u4 * 8 + z;
+              const float yr = fmaf(ra_m, ye1[u], -tau);
+              const bool ok = marked && yr > 0.f && (!edge || col0 + u <= lim);
+              float ye, y1;
+              pow_pair_c<EC>(ok ? yr : 0.f, ok, a.expo, ye, y1);
+              pv[z] = ye;
+              ye1[u] = y1;
+            }
+          }
+          asm volatile("st.shared::cta.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(p_smem + blk + (((unit0 + u4) ^ swz) << 4)),
+                       "r"(pack_bf16(pv[0], pv[1])), "r"(pack_bf16(pv[2], pv[3])), "r"(pack_bf16(pv[4], pv[5])),
+                       "r"(pack_bf16(pv[6], pv[7]))
+                       : "memory");
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(p_full);
+        // g dS = g u (dP - rho)
+        alive = __all_sync(0xffffffffu, mbar_wait(dp_full, dpphase, abort_flag));
+        dpphase ^= 1u;
+        if (!alive) break;
+        tc_fence_after();
+        alive = __all_sync(0xffffffffu, mbar_wait(ds_empty, dsphase ^ 1u, abort_flag));
+        dsphase ^= 1u;
+        if (!alive) break;
+#pragma unroll
         for (int hc = 0; hc < 2; ++hc) {
-          float sa[16], dp[16];
-          tmem_ld16(taddr_row + C::kTmemS + quarter * 32 + hc * 16, sa);
+          float dp[16];
           tmem_ld16(taddr_row + C::kTmemDP + quarter * 32 + hc * 16, dp);
           tmem_ld_wait();
-          const int col0 = kt * TN + quarter * 32 + hc * 16;
-          if (slope != 0.f) {
-#pragma unroll
-            for (int u = 0; u < 16; ++u) sa[u] = fmaf(slope, (float)(col0 + u - i), sa[u]);
+          if (hc == 1) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(dp_empty);      // dP has been read
           }
-          const bool edge = col0 + 15 > lim;
-          const uint32_t blk = (uint32_t)(quarter >> 1) * (TM * 128) + (uint32_t)row_local * 128u;
 #pragma unroll
           for (int u4 = 0; u4 < 2; ++u4) {
-            float pv[8], dv[8];
-            if (EC != kExpoGeneral && !edge) {
-              // away from the mask (an unmarked row has a = 0, tau = 0 here: every entry clamps to zero)
+            float dv[8];
 #pragma unroll
-              for (int z = 0; z < 8; ++z) {
-                const int u = u4 * 8 + z;
-                const float m = fmaxf(fmaf(ra_m, sa[u], -tau), 0.f);
-                const float ye1 = clamped_pow_m1<EC>(m);
-                pv[z] = ye1 * m;
-                dv[z] = g * (ye1 * (dp[u] - rho));
-              }
-            } else {
-#pragma unroll
-              for (int z = 0; z < 8; ++z) {
-                const int u = u4 * 8 + z;
-                const float yr = fmaf(ra, sa[u], -tau);
-                const bool ok = marked && yr > 0.f && (!edge || col0 + u <= lim);
-                float ye, ye1;
-                pow_pair_c<EC>(ok ? yr : 0.f, ok, a.expo, ye, ye1);
-                pv[z] = ye;
-                dv[z] = g * (ye1 * (dp[u] - rho));
-              }
-            }
-            const uint32_t unit = (uint32_t)((quarter & 1) * 4 + hc * 2 + u4);
-            const uint32_t off = blk + ((unit ^ (uint32_t)(row_local & 7)) << 4);
-            asm volatile("st.shared::cta.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(p_smem + off),
-                         "r"(pack_bf16(pv[0], pv[1])), "r"(pack_bf16(pv[2], pv[3])), "r"(pack_bf16(pv[4], pv[5])),
-                         "r"(pack_bf16(pv[6], pv[7]))
-                         : "memory");
-            asm volatile("st.shared::cta.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(ds_smem + off),
+            for (int z = 0; z < 8; ++z) dv[z] = g * (ye1[hc * 16 + u4 * 8 + z] * (dp[u4 * 8 + z] - rho));
+            asm volatile("st.shared::cta.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(
+                             ds_smem + blk + (((unit0 + hc * 2 + u4) ^ swz) << 4)),
                          "r"(pack_bf16(dv[0], dv[1])), "r"(pack_bf16(dv[2], dv[3])), "r"(pack_bf16(dv[4], dv[5])),
                          "r"(pack_bf16(dv[6], dv[7]))
                          : "memory");
           }
         }
-        tc_fence_before();
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
-        if (lane == 0) {
-          mbar_arrive(sd_empty);
-          mbar_arrive(pds_full);
-        }
-        qt = __shfl_sync(0xffffffffu, next_marked(bh, qt + 1), 0);
+        if (lane == 0) mbar_arrive(ds_full);
+        qt = nxt;
       }
       if (!alive) break;
       // ---- dK and dV of the K tile: TMEM lane = key; through a staging tile (the P and g dS buffers, free once the
