@@ -38,6 +38,7 @@ constexpr int kConsGroups = 4;                       // threads per TMEM lane
 constexpr int kConsWarps = 4 * kConsGroups;           // four lane quadrants each
 constexpr int kThreadsB = (2 + kConsWarps) * 32;      // TMA warp, MMA warp, the consumer warps
 constexpr int kTileBytes = TM * TN * 2;   // P or dS tile, bf16
+constexpr int kKStages = 3, kVStages = 2;  // K and V rings of the query-major kernel
 
 template <int HD>
 struct BCfg {
@@ -47,6 +48,7 @@ struct BCfg {
   static constexpr int kSmemBytes = 4 * kQBytes + 3 * kTileBytes + 1024 + kBarBytes;
   static_assert(kSmemBytes <= 232448, "shared memory of one CTA");
   static constexpr int kTmemS = 0, kTmemDP = TN, kTmemDQ = 2 * TN;
+  static constexpr int kTmemDS = 3 * TN, kTmemDL = 3 * TN + TN / 2;   // g dS and its rounding remainder, bf16, two keys a column
 };
 
 struct TileBwdArgs {
@@ -124,17 +126,15 @@ __global__ void __launch_bounds__(kThreadsB, 1) tile_bwd_kernel(const __grid_con
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t q_smem = sbase;
   const uint32_t do_smem = q_smem + C::kQBytes;
-  const uint32_t k_smem = do_smem + C::kQBytes;
-  const uint32_t v_smem = k_smem + C::kQBytes;
-  const uint32_t p_smem = v_smem + C::kQBytes;           // (the key-major kernel's P tile; here: second K stage)
-  const uint32_t ds_smem = p_smem + kTileBytes;           // g dS tile (bf16), same layout
-  const uint32_t dl_smem = ds_smem + kTileBytes;          // what the bf16 rounding of g dS left over, same layout
-  const uint32_t bars = dl_smem + kTileBytes;
+  const uint32_t k_smem = do_smem + C::kQBytes;            // K ring, three stages
+  const uint32_t v_smem = k_smem + kKStages * C::kQBytes;  // V ring, two stages
+  const uint32_t bars = sbase + 4 * C::kQBytes + 3 * kTileBytes;
+  static_assert((2 + kKStages + kVStages) * C::kQBytes <= 4 * C::kQBytes + 3 * kTileBytes, "tiles in front of the barriers");
   const uint32_t qdo_full = bars, qdo_empty = bars + 8;
-  const uint32_t k_full0 = bars + 16, k_empty0 = bars + 24;
-  const uint32_t sd_full = bars + 32, sd_empty = bars + 40;
-  const uint32_t pds_full = bars + 48, pds_empty = bars + 56;
-  const uint32_t dq_full = bars + 80, dq_empty = bars + 88;
+  const uint32_t k_full = bars + 16;          // [3]
+  const uint32_t k_empty = bars + 40;         // [3]
+  const uint32_t v_full = bars + 64;          // [2]
+  const uint32_t v_empty = bars + 80;         // [2]
   const uint32_t tmem_slot = bars + 96;
   const uint32_t abort_flag = bars + 100;
   const uint32_t drain_bar = bars + 104;      // teardown: every MMA issued so far has finished
@@ -143,17 +143,10 @@ __global__ void __launch_bounds__(kThreadsB, 1) tile_bwd_kernel(const __grid_con
   const uint32_t w_empty = bars + 136;        // [2] ... and read by the MMA issuer and every consumer warp
   const uint32_t w_item = bars + 152;         // int32 [2]: tile id, -1 = no more work
   const uint32_t x_bar = bars + 160;          // the threads of a row have written their partial sums
-  const uint32_t v_full0 = bars + 168, v_empty0 = bars + 176;
-  // Pass A has a second K / V stage: the P tile's buffer (the key-major kernel's; idle here) and the g dS buffer, which
-  // is idle until pass B and free again when the item's last contraction has finished -- which the producer waits for
-  // before it loads anything of the next item.
-  const uint32_t k_full1 = bars + 184, k_empty1 = bars + 192, v_full1 = bars + 200, v_empty1 = bars + 208;
-  auto k_full = [&](int st) { return st ? k_full1 : k_full0; };
-  auto k_empty = [&](int st) { return st ? k_empty1 : k_empty0; };
-  auto v_full = [&](int st) { return st ? v_full1 : v_full0; };
-  auto v_empty = [&](int st) { return st ? v_empty1 : v_empty0; };
-  auto k_stage = [&](int st) { return st ? p_smem : k_smem; };
-  auto v_stage = [&](int st) { return st ? ds_smem : v_smem; };
+  const uint32_t sd_full = bars + 168;        // [2] S and dP of a tile in stage 0 (columns 0..255) or 1 (256..511)
+  const uint32_t sd_empty = bars + 184;       // [2]
+  const uint32_t pds_full = bars + 200, pds_empty = bars + 208;
+  const uint32_t dq_full = bars + 216, dq_empty = bars + 224;
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -163,14 +156,16 @@ __global__ void __launch_bounds__(kThreadsB, 1) tile_bwd_kernel(const __grid_con
   if (threadIdx.x == 0) {
     mbar_init(qdo_full, 1);
     mbar_init(qdo_empty, 1);
-    for (int st = 0; st < 2; ++st) {
-      mbar_init(k_full(st), 1);
-      mbar_init(k_empty(st), 1);
-      mbar_init(v_full(st), 1);
-      mbar_init(v_empty(st), 1);
+    for (int st = 0; st < kKStages; ++st) {
+      mbar_init(k_full + 8 * st, 1);
+      mbar_init(k_empty + 8 * st, 1);
     }
-    mbar_init(sd_full, 1);
-    mbar_init(sd_empty, kConsWarps);
+    for (int st = 0; st < 2; ++st) {
+      mbar_init(v_full + 8 * st, 1);
+      mbar_init(v_empty + 8 * st, 1);
+      mbar_init(sd_full + 8 * st, 1);
+      mbar_init(sd_empty + 8 * st, kConsWarps);
+    }
     mbar_init(pds_full, kConsWarps);
     mbar_init(pds_empty, 1);
     mbar_init(dq_full, 1);
@@ -206,11 +201,11 @@ __global__ void __launch_bounds__(kThreadsB, 1) tile_bwd_kernel(const __grid_con
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
     // (the whole warp runs the control flow, one elected lane issues the copies: see the MMA issuer).  K and V
-    // tiles have barriers of their own: in pass B the V tile is free again once dP has been formed and the K tile
-    // once dQ has taken it, so the next tile's copies run under the dK / dV contractions of this one.
+    // tiles have rings of their own: a V tile is free again once dP has been formed, in pass B a K tile only once
+    // dQ has taken it, a tile later.
     {
       uint32_t kbits = 0, vbits = 0 /* bit st: times the stage's barrier has been armed, mod 2 */, qphase = 0, wphase = 0;
-      int slot = 0;
+      int slot = 0, kst = 0, vst = 0;
       bool alive = true;
       auto wait_all = [&](uint32_t bar, uint32_t parity) -> bool {
         return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag));
@@ -245,38 +240,34 @@ __global__ void __launch_bounds__(kThreadsB, 1) tile_bwd_kernel(const __grid_con
         __syncwarp();
         for (int t = 0; t < 2 * tiles && alive; ++t) {
           const int kt = t < tiles ? t : t - tiles;
-          // K alternates between its two stages in both passes (the second one is a tile this kernel has no other use
-          // for); V does so in pass A only: its second stage is the dS tile of pass B, where a V tile is free again as
-          // soon as dP has been formed
-          const int st = t < tiles ? (t & 1) : 0, kst = t & 1;
-          alive = wait_all(v_empty(st), ((vbits >> st) & 1u) ^ 1u);
+          alive = wait_all(v_empty + 8 * vst, ((vbits >> vst) & 1u) ^ 1u);
           if (!alive) break;
-          vbits ^= 1u << st;
+          vbits ^= 1u << vst;
           if (elect_one()) {
-            mbar_expect_tx(v_full(st), C::kQBytes);
+            mbar_expect_tx(v_full + 8 * vst, C::kQBytes);
             for (int hf = 0; hf < C::kHalves; ++hf)
-              tma_load_4d(v_stage(st) + hf * (TN * 128), &map_v, v_full(st), hf * 64, kt * TN, h, b);
+              tma_load_4d(v_smem + vst * C::kQBytes + hf * (TN * 128), &map_v, v_full + 8 * vst, hf * 64, kt * TN, h, b);
           }
           __syncwarp();
-          alive = wait_all(k_empty(kst), ((kbits >> kst) & 1u) ^ 1u);
+          vst ^= 1;
+          alive = wait_all(k_empty + 8 * kst, ((kbits >> kst) & 1u) ^ 1u);
           if (!alive) break;
           kbits ^= 1u << kst;
           if (elect_one()) {
-            mbar_expect_tx(k_full(kst), C::kQBytes);
+            mbar_expect_tx(k_full + 8 * kst, C::kQBytes);
             for (int hf = 0; hf < C::kHalves; ++hf)
-              tma_load_4d(k_stage(kst) + hf * (TN * 128), &map_k, k_full(kst), hf * 64, kt * TN, h, b);
+              tma_load_4d(k_smem + kst * C::kQBytes + hf * (TN * 128), &map_k, k_full + 8 * kst, hf * 64, kt * TN, h, b);
           }
           __syncwarp();
+          if (++kst == kKStages) kst = 0;
         }
       }
       if (!alive && lane == 0) {
         // a wait ran out somewhere in the CTA: the copies this warp armed barriers for must land before shared
         // memory goes away (after n arms a phase word holds n mod 2 and the last armed phase has the other parity)
         bool ok = mbar_drain(qdo_full, qphase ^ 1u);
-        for (int st = 0; st < 2; ++st) {
-          ok &= mbar_drain(k_full(st), ((kbits >> st) & 1u) ^ 1u);
-          ok &= mbar_drain(v_full(st), ((vbits >> st) & 1u) ^ 1u);
-        }
+        for (int st = 0; st < kKStages; ++st) ok &= mbar_drain(k_full + 8 * st, ((kbits >> st) & 1u) ^ 1u);
+        for (int st = 0; st < kVStages; ++st) ok &= mbar_drain(v_full + 8 * st, ((vbits >> st) & 1u) ^ 1u);
         if (!ok) sts_u32(drain_fail, 1u);
       }
     }
@@ -291,12 +282,11 @@ __global__ void __launch_bounds__(kThreadsB, 1) tile_bwd_kernel(const __grid_con
       const uint64_t hi = (uint64_t)kDescHi << 32;
       const uint64_t q_d = hi | smem_desc_lo(q_smem), do_d = hi | smem_desc_lo(do_smem);
       const uint64_t k_d = hi | smem_desc_lo(k_smem), v_d = hi | smem_desc_lo(v_smem);
-      const uint64_t ds_d = hi | smem_desc_lo(ds_smem), dl_d = hi | smem_desc_lo(dl_smem);
-      const uint64_t k_n_d = hi | mn_desc_lo(k_smem), k1_n_d = hi | mn_desc_lo(p_smem);
-      uint32_t kbits = 0, vbits = 0 /* bit st: phase of the stage's barrier to wait for */, qphase = 0, sdphase = 0,
+      const uint64_t k_n_d = hi | mn_desc_lo(k_smem);
+      constexpr uint32_t kStageD = C::kQBytes >> 4;         // from one ring stage to the next, in descriptor units
+      uint32_t kbits = 0, vbits = 0 /* bit st: phase of the stage's barrier to wait for */, sdbits = 0, qphase = 0,
                pdsphase = 0, dqphase = 0, wphase = 0;
-      const uint64_t k1_d = hi | smem_desc_lo(p_smem), v1_d = hi | smem_desc_lo(ds_smem);   // stage 1 of pass A
-      int slot = 0;
+      int slot = 0, kst = 0, vst = 0, kq = 0;     // kq: the K stage the next dQ reads
       bool alive = true;
       auto wait_all = [&](uint32_t bar, uint32_t parity) -> bool {
         return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag));
@@ -315,53 +305,62 @@ __global__ void __launch_bounds__(kThreadsB, 1) tile_bwd_kernel(const __grid_con
         qphase ^= 1u;
         if (!alive) break;
         // S = Q K^T and dP = dO V^T of tile t (pass A: t < tiles, pass B: the same tiles again)
+        // Pass A alternates between two accumulator stages; the second one covers the dQ, dS and remainder columns, all
+        // idle until pass B, which has the first stage only.
         auto issue_sd = [&](int t) -> bool {
           const bool pass_b = t >= tiles;
-          const int st = pass_b ? 0 : (t & 1), kst = t & 1;
-          bool ok = wait_all(k_full(kst), (kbits >> kst) & 1u);
+          const int sst = pass_b ? 0 : (t & 1);
+          bool ok = wait_all(k_full + 8 * kst, (kbits >> kst) & 1u);
           kbits ^= 1u << kst;
-          if (ok) ok = wait_all(v_full(st), (vbits >> st) & 1u);
-          vbits ^= 1u << st;
-          const uint64_t ks_d = kst ? k1_d : k_d, vs_d = st ? v1_d : v_d;
-          if (ok) ok = wait_all(sd_empty, sdphase ^ 1u);
+          if (ok) ok = wait_all(v_full + 8 * vst, (vbits >> vst) & 1u);
+          vbits ^= 1u << vst;
+          if (ok) ok = wait_all(sd_empty + 8 * sst, ((sdbits >> sst) & 1u) ^ 1u);
+          sdbits ^= 1u << sst;
           if (!ok) return false;
-          sdphase ^= 1u;
+          const uint64_t ks_d = k_d + kst * kStageD, vs_d = v_d + vst * kStageD;
+          const uint32_t acc = tmem_base + sst * (2 * TN);
           tc_fence_after();
           if (elect_one()) {
 #pragma unroll
             for (int kk = 0; kk < HD / 16; ++kk) {
               const uint32_t off = (kk >> 2) * ((TM * 128) >> 4) + (kk & 3) * 2;
-              umma_bf16_desc(tmem_base + C::kTmemS, q_d + off, ks_d + off, id_kk, kk > 0 ? 1u : 0u);
+              umma_bf16_desc(acc + C::kTmemS, q_d + off, ks_d + off, id_kk, kk > 0 ? 1u : 0u);
             }
 #pragma unroll
             for (int kk = 0; kk < HD / 16; ++kk) {
               const uint32_t off = (kk >> 2) * ((TM * 128) >> 4) + (kk & 3) * 2;
-              umma_bf16_desc(tmem_base + C::kTmemDP, do_d + off, vs_d + off, id_kk, kk > 0 ? 1u : 0u);
+              umma_bf16_desc(acc + C::kTmemDP, do_d + off, vs_d + off, id_kk, kk > 0 ? 1u : 0u);
             }
-            umma_commit(sd_full);
-            umma_commit(v_empty(st));          // dP has been formed: the V tile is free
-            if (!pass_b) umma_commit(k_empty(kst));
+            umma_commit(sd_full + 8 * sst);
+            umma_commit(v_empty + 8 * vst);      // dP has been formed: the V tile is free
+            if (!pass_b) umma_commit(k_empty + 8 * kst);
           }
           __syncwarp();
+          if (t == tiles) kq = kst;
+          if (++kst == kKStages) kst = 0;
+          vst ^= 1;
           return true;
         };
-        for (int t = 0; t < tiles && alive; ++t) alive = issue_sd(t);
-        if (alive) {
-          // the previous item's dQ must have been read before this item's first dQ MMA overwrites it
-          alive = wait_all(dq_empty, dqphase ^ 1u);
-          dqphase ^= 1u;
+        for (int t = 0; t < tiles && alive; ++t) {
+          if (t == 1) {
+            // the previous item's dQ must have been read before the second stage overwrites it
+            alive = wait_all(dq_empty, dqphase ^ 1u);
+            if (!alive) break;
+          }
+          alive = issue_sd(t);
         }
+        if (alive && tiles == 1) alive = wait_all(dq_empty, dqphase ^ 1u);
+        dqphase ^= 1u;
         if (alive) alive = issue_sd(tiles);
         for (int t = tiles; t < 2 * tiles && alive; ++t) {
-          // the next tile's S and dP are issued before this tile's dS is waited for (its K tile sits in the other
-          // stage), so that they run while the consumers form dS
+          // the next tile's S and dP are issued before this tile's dS is waited for, so that they run while the
+          // consumers form dS
           if (t + 1 < 2 * tiles) {
             alive = issue_sd(t + 1);
             if (!alive) break;
           }
-          const int kst = t & 1;
-          const uint64_t kn_d = kst ? k1_n_d : k_n_d;
-          // g dS of this tile and its rounding remainder are in shared memory
+          const uint64_t kn_d = k_n_d + kq * kStageD;
+          // g dS of this tile and its rounding remainder are in TMEM
           alive = wait_all(pds_full, pdsphase);
           pdsphase ^= 1u;
           if (!alive) break;
@@ -369,24 +368,24 @@ __global__ void __launch_bounds__(kThreadsB, 1) tile_bwd_kernel(const __grid_con
           if (elect_one()) {
 #pragma unroll
             for (int kk = 0; kk < TN / 16; ++kk) {
-              const uint32_t a_off = (kk >> 2) * ((TM * 128) >> 4) + (kk & 3) * 2;   // 64 keys per 128-byte row
               const uint32_t b_off = kk * ((16 * 128) >> 4);                           // 16 keys = 16 rows of 128 B
-              umma_bf16_desc(tmem_base + C::kTmemDQ, ds_d + a_off, kn_d + b_off, id_kn, (t > tiles || kk > 0) ? 1u : 0u);
+              umma_bf16_ts(tmem_base + C::kTmemDQ, tmem_base + C::kTmemDS + kk * 8, kn_d + b_off, id_kn,
+                           (t > tiles || kk > 0) ? 1u : 0u);
             }
             // the rounding remainder of g dS as a second operand: the rows of dS sum to zero, so when a row's keys
             // are nearly equal vectors (retrieval: several copies of one key) dQ is what is left after a
             // cancellation, and the bf16 rounding of dS alone (2^-9 of every term) would be a large part of it
 #pragma unroll
             for (int kk = 0; kk < TN / 16; ++kk) {
-              const uint32_t a_off = (kk >> 2) * ((TM * 128) >> 4) + (kk & 3) * 2;
               const uint32_t b_off = kk * ((16 * 128) >> 4);
-              umma_bf16_desc(tmem_base + C::kTmemDQ, dl_d + a_off, kn_d + b_off, id_kn, 1u);
+              umma_bf16_ts(tmem_base + C::kTmemDQ, tmem_base + C::kTmemDL + kk * 8, kn_d + b_off, id_kn, 1u);
             }
-            umma_commit(k_empty(kst));         // dQ has taken the K tile
+            umma_commit(k_empty + 8 * kq);     // dQ has taken the K tile
             umma_commit(pds_empty);
             if (t == 2 * tiles - 1) umma_commit(dq_full);
           }
           __syncwarp();
+          if (++kq == kKStages) kq = 0;
         }
         if (elect_one()) umma_commit(qdo_empty);
         __syncwarp();
@@ -405,35 +404,30 @@ __global__ void __launch_bounds__(kThreadsB, 1) tile_bwd_kernel(const __grid_con
     const int quarter = (warp - 2) >> 2;
     const int row_local = quad * 32 + lane;
     const uint32_t taddr_row = tmem_base + ((uint32_t)(quad * 32) << 16);
-    uint32_t sdphase = 0, pdsphase = 0, dqphase = 0, wphase = 0, xphase = 0;
+    uint32_t sdbits = 0, pdsphase = 0, dqphase = 0, wphase = 0, xphase = 0;
     int slot = 0;
     bool alive = true;
-    // The four threads of a row swap partial sums through shared memory.  The slots live in the remainder tile's
-    // buffer, which is idle whenever a swap happens (between the passes: not yet written; after the item's last
-    // contraction: no longer read); a second round of the barrier keeps a fast warp from rewriting the buffer while
-    // a slow one still reads it.  All four threads add the same four numbers in the same order.
-    auto swap4 = [&](float x0, float x1, float& r0, float& r1) -> bool {
-      const uint32_t mine = dl_smem + (uint32_t)(quarter * TM + row_local) * 8u;
-      sts_u32(mine, __float_as_uint(x0));
-      sts_u32(mine + 4, __float_as_uint(x1));
+    // The four threads of a row swap partial sums through TMEM, each in the first two of 32 columns of its own at
+    // `col`; all four add the same four numbers in the same order.  Between the passes those are the columns of the
+    // second stage's S that only the thread itself has read; after the item's last contraction they are the dS columns.
+    // What overwrites them next (the first dQ; the next item's second stage) waits for every warp.
+    auto swap4 = [&](int col, float x0, float x1, float& r0, float& r1) -> bool {
+      tmem_st2(taddr_row + col + quarter * 32, __float_as_uint(x0), __float_as_uint(x1));
+      tmem_st_wait();
+      tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(x_bar);
-      bool ok = __all_sync(0xffffffffu, mbar_wait(x_bar, xphase, abort_flag));
+      const bool ok = __all_sync(0xffffffffu, mbar_wait(x_bar, xphase, abort_flag));
       xphase ^= 1u;
       if (!ok) return false;
-      float a0[kConsGroups], a1[kConsGroups];
+      tc_fence_after();
+      uint32_t a0[kConsGroups], a1[kConsGroups];
 #pragma unroll
-      for (int gq = 0; gq < kConsGroups; ++gq) {
-        a0[gq] = __uint_as_float(lds_u32(dl_smem + (uint32_t)(gq * TM + row_local) * 8u));
-        a1[gq] = __uint_as_float(lds_u32(dl_smem + (uint32_t)(gq * TM + row_local) * 8u + 4u));
-      }
-      r0 = (a0[0] + a0[1]) + (a0[2] + a0[3]);
-      r1 = (a1[0] + a1[1]) + (a1[2] + a1[3]);
-      __syncwarp();
-      if (lane == 0) mbar_arrive(x_bar);
-      ok = __all_sync(0xffffffffu, mbar_wait(x_bar, xphase, abort_flag));
-      xphase ^= 1u;
-      return ok;
+      for (int gq = 0; gq < kConsGroups; ++gq) tmem_ld2(taddr_row + col + gq * 32, a0[gq], a1[gq]);
+      tmem_ld_wait();
+      r0 = (__uint_as_float(a0[0]) + __uint_as_float(a0[1])) + (__uint_as_float(a0[2]) + __uint_as_float(a0[3]));
+      r1 = (__uint_as_float(a1[0]) + __uint_as_float(a1[1])) + (__uint_as_float(a1[2]) + __uint_as_float(a1[3]));
+      return true;
     };
     while (alive) {
       alive = __all_sync(0xffffffffu, mbar_wait(w_full + 8 * slot, wphase, abort_flag));
@@ -465,29 +459,41 @@ __global__ void __launch_bounds__(kThreadsB, 1) tile_bwd_kernel(const __grid_con
         if (t == tiles) {
           // rho of the row from the four threads' shares of sum u and sum u dP
           float su_all, sud_all;
-          alive = swap4(su, sud, su_all, sud_all);
+          alive = swap4(2 * TN, su, sud, su_all, sud_all);
           if (!alive) break;
           rho = su_all > 0.f ? sud_all / su_all : 0.f;
           if (marked && quarter == 0) a.rho[grow] = rho;   // for the key-major kernel
         }
-        alive = __all_sync(0xffffffffu, mbar_wait(sd_full, sdphase, abort_flag));
+        const int sst = pass_b ? 0 : (t & 1);
+        alive = __all_sync(0xffffffffu, mbar_wait(sd_full + 8 * sst, (sdbits >> sst) & 1u, abort_flag));
         if (!alive) break;
-        sdphase ^= 1u;
+        sdbits ^= 1u << sst;
         tc_fence_after();
-        // this thread's 32 columns, 16 at a time
-#pragma unroll 1
-        for (int hc = 0; hc < 2; ++hc) {
-          float sa[16], dp[16];
-          tmem_ld16(taddr_row + C::kTmemS + quarter * 32 + hc * 16, sa);
-          tmem_ld16(taddr_row + C::kTmemDP + quarter * 32 + hc * 16, dp);
+        const uint32_t acc = taddr_row + sst * (2 * TN) + quarter * 32;
+        // this thread's 32 columns, 16 at a time; with the second 16 in registers the accumulators are handed back
+        float sa[16], dp[16];
+        auto load = [&](int hc) {
+          __syncwarp();
+          tmem_ld16(acc + C::kTmemS + hc * 16, sa);
+          tmem_ld16(acc + C::kTmemDP + hc * 16, dp);
           tmem_ld_wait();
-          const int col0 = kt * TN + quarter * 32 + hc * 16;
+          if (hc == 1) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(sd_empty + 8 * sst);
+          }
           if (slope != 0.f) {
+            const int col0 = kt * TN + quarter * 32 + hc * 16;
 #pragma unroll
             for (int u = 0; u < 16; ++u) sa[u] = fmaf(slope, (float)(col0 + u - i), sa[u]);
           }
-          const bool edge = col0 + 15 > lim;
-          if (!pass_b) {
+        };
+        if (!pass_b) {
+#pragma unroll 1
+          for (int hc = 0; hc < 2; ++hc) {
+            load(hc);
+            const int col0 = kt * TN + quarter * 32 + hc * 16;
+            const bool edge = col0 + 15 > lim;
             // four independent partial sums each, so that the additions do not form one serial chain
             float p0[4] = {0.f, 0.f, 0.f, 0.f}, p1[4] = {0.f, 0.f, 0.f, 0.f};
             if (EC != kExpoGeneral && !edge) {
@@ -512,72 +518,61 @@ __global__ void __launch_bounds__(kThreadsB, 1) tile_bwd_kernel(const __grid_con
             }
             su += (p0[0] + p0[1]) + (p0[2] + p0[3]);
             sud += (p1[0] + p1[1]) + (p1[2] + p1[3]);
+          }
+          continue;
+        }
+        // g dS and what its bf16 rounding leaves over, both bf16, two entries to a register
+        auto form_ds = [&](int hc, uint32_t (&dsv)[8], uint32_t (&dlv)[8]) {
+          const int col0 = kt * TN + quarter * 32 + hc * 16;
+          const bool edge = col0 + 15 > lim;
+          float dv[16];
+          if (EC != kExpoGeneral && !edge) {
+            // away from the mask (an unmarked row has a = 0, tau = 0 here: every entry clamps to zero)
+#pragma unroll
+            for (int u = 0; u < 16; ++u) {
+              const float m = fmaxf(fmaf(ra_m, sa[u], -tau), 0.f);
+              const float ds = clamped_pow_m1<EC>(m) * (dp[u] - rho);
+              dv[u] = g * ds;
+              dcs[u & 1] = fmaf(ds, sa[u], dcs[u & 1]);
+            }
           } else {
-            // P and g dS -> bf16 -> shared memory, K-major with 128-byte swizzle: row r, 16-byte unit u of
-            // the 64-key block sits at r*128 + ((u ^ (r & 7)) * 16)
-            const uint32_t blk = (uint32_t)(quarter >> 1) * (TM * 128) + (uint32_t)row_local * 128u;
 #pragma unroll
-            for (int u4 = 0; u4 < 2; ++u4) {
-              float dv[8], dl[8];
-              if (EC != kExpoGeneral && !edge) {
-                // away from the mask (an unmarked row has a = 0, tau = 0 here: every entry clamps to zero)
-#pragma unroll
-                for (int z = 0; z < 8; ++z) {
-                  const int u = u4 * 8 + z;
-                  const float m = fmaxf(fmaf(ra_m, sa[u], -tau), 0.f);
-                  const float ds = clamped_pow_m1<EC>(m) * (dp[u] - rho);
-                  dv[z] = g * ds;
-                  dcs[z & 1] = fmaf(ds, sa[u], dcs[z & 1]);
-                }
-              } else {
-#pragma unroll
-                for (int z = 0; z < 8; ++z) {
-                  const int u = u4 * 8 + z;
-                  const float yr = fmaf(ra, sa[u], -tau);
-                  const bool ok = marked && yr > 0.f && (!edge || col0 + u <= lim);
-                  float ye, ye1;
-                  pow_pair_c<EC>(ok ? yr : 0.f, ok, a.expo, ye, ye1);
-                  const float ds = ye1 * (dp[u] - rho);
-                  dv[z] = g * ds;
-                  dcs[z & 1] = fmaf(ds, sa[u], dcs[z & 1]);
-                }
-              }
-              // what the bf16 rounding of g dS leaves over, two entries at a time
-#pragma unroll
-              for (int z = 0; z < 8; z += 2) {
-                const float2 r2 = __bfloat1622float2(__floats2bfloat162_rn(dv[z], dv[z + 1]));
-                dl[z] = dv[z] - r2.x;
-                dl[z + 1] = dv[z + 1] - r2.y;
-              }
-              if (hc == 0 && u4 == 0) {
-                // g dS of the previous tile and its remainder must have been consumed before their buffers are
-                // rewritten (waited for here, not before the loads: that tile's dQ contraction runs under this
-                // tile's first element code)
-                alive = __all_sync(0xffffffffu, mbar_wait(pds_empty, pdsphase ^ 1u, abort_flag));
-                pdsphase ^= 1u;
-              }
-              if (!alive) continue;
-              const uint32_t unit = (uint32_t)((quarter & 1) * 4 + hc * 2 + u4);
-              const uint32_t off = blk + ((unit ^ (uint32_t)(row_local & 7)) << 4);
-              asm volatile("st.shared::cta.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(ds_smem + off),
-                           "r"(pack_bf16(dv[0], dv[1])), "r"(pack_bf16(dv[2], dv[3])), "r"(pack_bf16(dv[4], dv[5])),
-                           "r"(pack_bf16(dv[6], dv[7]))
-                           : "memory");
-              asm volatile("st.shared::cta.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dl_smem + off),
-                           "r"(pack_bf16(dl[0], dl[1])), "r"(pack_bf16(dl[2], dl[3])), "r"(pack_bf16(dl[4], dl[5])),
-                           "r"(pack_bf16(dl[6], dl[7]))
-                           : "memory");
+            for (int u = 0; u < 16; ++u) {
+              const float yr = fmaf(ra, sa[u], -tau);
+              const bool ok = marked && yr > 0.f && (!edge || col0 + u <= lim);
+              float ye, ye1;
+              pow_pair_c<EC>(ok ? yr : 0.f, ok, a.expo, ye, ye1);
+              const float ds = ye1 * (dp[u] - rho);
+              dv[u] = g * ds;
+              dcs[u & 1] = fmaf(ds, sa[u], dcs[u & 1]);
             }
           }
-        }
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            const __nv_bfloat162 r = __floats2bfloat162_rn(dv[2 * u], dv[2 * u + 1]);
+            const float2 r2 = __bfloat1622float2(r);
+            dsv[u] = *reinterpret_cast<const uint32_t*>(&r);
+            dlv[u] = pack_bf16(dv[2 * u] - r2.x, dv[2 * u + 1] - r2.y);
+          }
+        };
+        uint32_t ds0[8], dl0[8];
+        load(0);
+        form_ds(0, ds0, dl0);
+        load(1);
+        // g dS of the previous tile and its remainder must have been consumed before their columns are rewritten
+        // (waited for here: that tile's dQ contraction runs under this tile's first element code)
+        alive = __all_sync(0xffffffffu, mbar_wait(pds_empty, pdsphase ^ 1u, abort_flag));
+        pdsphase ^= 1u;
         if (!alive) break;
-        // S and dP have been read
-        tc_fence_before();
+        tc_fence_after();
+        tmem_st8(taddr_row + C::kTmemDS + quarter * 16, ds0);
+        tmem_st8(taddr_row + C::kTmemDL + quarter * 16, dl0);
+        form_ds(1, ds0, dl0);
         __syncwarp();
-        if (lane == 0) mbar_arrive(sd_empty);
-        if (!pass_b) continue;
-        // make the P / dS stores visible to the tensor core (async proxy), then hand the tiles over
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        tmem_st8(taddr_row + C::kTmemDS + quarter * 16 + 8, ds0);
+        tmem_st8(taddr_row + C::kTmemDL + quarter * 16 + 8, dl0);
+        tmem_st_wait();
+        tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(pds_full);
       }
@@ -601,17 +596,17 @@ __global__ void __launch_bounds__(kThreadsB, 1) tile_bwd_kernel(const __grid_con
                            pack_bf16(va[u8 * 8 + 4], va[u8 * 8 + 5]), pack_bf16(va[u8 * 8 + 6], va[u8 * 8 + 7]));
         }
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(dq_empty);
       // dL/dc_i = sum_j dS_ij z_ij with z_ij = sm_scale * (accumulator + bias in accumulator units); every
-      // contraction of the item has finished (dq_full), so the swap buffer is free
+      // contraction of the item has finished (dq_full), so the dS columns are free for the swap
       if (a.dc_rows) {
         float dc_all, unused;
-        alive = swap4(dcs[0] + dcs[1], 0.f, dc_all, unused);
+        alive = swap4(C::kTmemDS, dcs[0] + dcs[1], 0.f, dc_all, unused);
         if (!alive) break;
         if (marked && quarter == 0) a.dc_rows[grow] = dc_all * a.sm_scale;
       }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(dq_empty);
       if (a.status && threadIdx.x == 64) atomicAdd(a.status + ENTMAX_ATTN_STATUS_TILES, 1);
     }
   }
