@@ -276,7 +276,7 @@ int entmax_attn_workspace_layout(const entmax_attn_params* params, entmax_attn_w
  *   tau          out, device float32 [batch, heads, q_len]
  *   support_size out, device int32 [batch, heads, q_len] or NULL: number of keys with p > 0
  *   workspace    device scratch, 256-byte aligned, >= entmax_attn_decode_workspace_bytes(params)
- *                (one fp32 score per query row and cached key, chunk maxima)
+ *                (one fp32 score per query row and cached key, and the maximum of every 32 keys)
  * K is read once (the HBM traffic that bounds this shape), V only on the support.  Results are
  * bitwise reproducible.  device_status word ENTMAX_ATTN_STATUS_DENSE_ROWS counts query rows whose
  * candidate set did not fit on chip (they are solved on the score row in the workspace instead).

@@ -4,9 +4,10 @@
 // (n_i = pos + 1).  The path is bound by reading K once from HBM:
 //   decode_scores_tc_kernel   (decode_scores_sm100.cu) streams K through TMA and tcgen05, writes
 //                             y = a_t (q.k + bias), a_t = (alpha-1) c_t sm_scale, to a score row in the
-//                             workspace and the maximum of every chunk of keys;
+//                             workspace and the maximum of every 32 keys;
 //   decode_solve_kernel       one CTA per query row: y_max, the candidates above the lower end of the bracket
-//                             of App. A (tau >= y_max - 1), Newton from the left on them (e-norm step), then
+//                             of App. A (tau >= y_max - 1; only 128-key tiles whose maximum lies above it are read),
+//                             Newton from the left on them (e-norm step), then
 //                             p = [y - tau]_+^e and O = sum_j p_j v_j as a gather of the support's V rows.
 // V is read only on the support.  Rows with more candidates than the CTA's list holds run the same
 // Newton iteration and output loop over the whole score row instead.
@@ -57,7 +58,7 @@ __device__ __forceinline__ float2 block_sum2(float x, float y, float2 (*red)[kSo
 template <int D, int kSolveThreads>
 __global__ void __launch_bounds__(kSolveThreads) decode_solve_kernel(DecodeArgs a, const __nv_bfloat16* __restrict__ v,
                                                                     const float* __restrict__ scores,
-                                                                    const float* __restrict__ chunk_max,
+                                                                    const float* __restrict__ tile_max,
                                                                     __nv_bfloat16* __restrict__ o,
                                                                     float* __restrict__ tau_out,
                                                                     int32_t* __restrict__ support_out,
@@ -85,10 +86,14 @@ __global__ void __launch_bounds__(kSolveThreads) decode_solve_kernel(DecodeArgs 
   const int nv = len - a.QL + t + 1;                // visible keys
   const float* y_row = scores + (size_t)row * a.score_stride;
   if (tid == 0) s_overflow = 0;
-  // ---- y_max from the chunk maxima
+  // ---- y_max from the tile maxima
   float m = -INFINITY;
-  const int chunks = (nv + a.chunk_keys - 1) / a.chunk_keys;
-  for (int c = tid; c < chunks; c += kSolveThreads) m = fmaxf(m, chunk_max[(size_t)row * a.n_chunks + c]);
+  const int tiles = (nv + 127) / 128;
+  const float4* row_max = reinterpret_cast<const float4*>(tile_max) + (size_t)row * a.n_tiles;
+  for (int c = tid; c < tiles; c += kSolveThreads) {
+    const float4 x = row_max[c];
+    m = fmaxf(m, fmaxf(fmaxf(x.x, x.y), fmaxf(x.z, x.w)));
+  }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
   if (lane == 0) wmax[warp] = m;
@@ -100,29 +105,44 @@ __global__ void __launch_bounds__(kSolveThreads) decode_solve_kernel(DecodeArgs 
   const float floor_y = ymax - 1.0f;
   int cnt = 0;
   {
-    // eight 16-byte loads in flight per thread; a thread meets its keys in increasing order
+    // Tile t is warp t mod kWarps's, a lane 4 of its 128 keys; 32 of the warp's tiles are tested at a time and those that
+    // hold a candidate read, four at a time (a thread meets its keys in increasing order).  The kernel took 12 us on 16 rows
+    // of 32768 keys with the whole rows read, 9 now; 18 and 14 on 512 rows of 16384.
     const float4* y_row4 = reinterpret_cast<const float4*>(y_row);
-    const int groups = (nv + 3) / 4;
-    const float4 none = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-    for (int g0 = tid; g0 < groups; g0 += 8 * kSolveThreads) {
-      float4 yv[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int g = g0 + u * kSolveThreads;
-        yv[u] = g < groups ? y_row4[g] : none;
+    for (int k0 = 0; warp + k0 * kWarps < tiles; k0 += 32) {
+      const int mine = warp + (k0 + lane) * kWarps;
+      bool any = false;
+      if (mine < tiles) {
+        const float4 x = row_max[mine];
+        any = fmaxf(fmaxf(x.x, x.y), fmaxf(x.z, x.w)) > floor_y;
       }
+      unsigned todo = __ballot_sync(0xffffffffu, any);
+      while (todo) {
+        int at[4];
+        float4 yv[4];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const float ye[4] = {yv[u].x, yv[u].y, yv[u].z, yv[u].w};
+        for (int u = 0; u < 4; ++u) {
+          at[u] = -1;
+          yv[u] = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+          if (todo) {
+            at[u] = (warp + (k0 + __ffs(todo) - 1) * kWarps) * 32 + lane;
+            todo &= todo - 1;
+            if (4 * at[u] < nv) yv[u] = y_row4[at[u]];
+          }
+        }
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int j = 4 * (g0 + u * kSolveThreads) + e;
-          if (j < nv && ye[e] > floor_y) {
-            if (cnt < kPerThread) {
-              cand_y[tid * kPerThread + cnt] = ye[e];
-              cand_j[tid * kPerThread + cnt] = j;
+        for (int u = 0; u < 4; ++u) {
+          const float ye[4] = {yv[u].x, yv[u].y, yv[u].z, yv[u].w};
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int j = 4 * at[u] + e;
+            if (j < nv && ye[e] > floor_y) {
+              if (cnt < kPerThread) {
+                cand_y[tid * kPerThread + cnt] = ye[e];
+                cand_j[tid * kPerThread + cnt] = j;
+              }
+              ++cnt;
             }
-            ++cnt;
           }
         }
       }
@@ -270,22 +290,41 @@ __global__ void __launch_bounds__(kSolveThreads) decode_solve_kernel(DecodeArgs 
 }
 
 struct DecodeLayout {
-  size_t chunk_max, scores, total;
+  size_t tile_max, scores, total;
   size_t score_stride;
-  int chunk_keys, n_chunks;
+  int chunk_tiles, n_chunks, n_tiles;
 };
 
-// A CTA of the score kernel takes up to 1024 keys, fewer when the problem would otherwise leave SMs idle.
+// A CTA of the score kernel takes 1024 keys where that makes four waves' worth of CTAs at least.  Below that a wave more
+// or less, and each CTA's start (barriers, TMEM, the first K tile from HBM: about a tile's time), are what the kernel
+// waits for: the number of CTAs per (sequence, head) is the one that needs the fewest tile times, wave by wave of the
+// 2 x 148 resident CTAs, and the kernel deals a sequence's tiles to them evenly, however full the cache is.
+// 16 heads x 32768 keys, 128 columns: 1024 CTAs of four tiles 31 us, 18 CTAs per head of up to 15 tiles 26 us.
 DecodeLayout decode_layout(int B, int H, int QL, int NC) {
   DecodeLayout l;
   const size_t rows = (size_t)B * H * QL;
-  l.chunk_keys = 1024;
-  while (l.chunk_keys > 128 && (long long)B * H * ((NC + l.chunk_keys - 1) / l.chunk_keys) < 4 * 148) l.chunk_keys /= 2;
-  l.n_chunks = (NC + l.chunk_keys - 1) / l.chunk_keys;
+  const long long bh = (long long)B * H;
+  l.n_tiles = (NC + 127) / 128;
+  l.chunk_tiles = 8;
+  l.n_chunks = (l.n_tiles + 7) / 8;
+  if (bh * l.n_chunks < 4 * 148) {
+    l.chunk_tiles = 0;
+    long long best = 0;
+    for (int w = 1; w <= 4; ++w) {
+      long long n = w * 296 / bh;
+      if (n > l.n_tiles) n = l.n_tiles;
+      if (n < 1) continue;
+      const long long cost = w * ((l.n_tiles + n - 1) / n + 1);
+      if (best == 0 || cost < best) {
+        best = cost;
+        l.n_chunks = (int)n;
+      }
+    }
+  }
   l.score_stride = ((size_t)NC + 31) / 32 * 32;
   size_t off = 0;
   auto take = [&off](size_t bytes) { size_t at = off; off = (off + bytes + 255) / 256 * 256; return at; };
-  l.chunk_max = take(rows * l.n_chunks * sizeof(float));
+  l.tile_max = take(rows * l.n_tiles * 4 * sizeof(float));
   l.scores = take(rows * l.score_stride * sizeof(float));
   l.total = off;
   return l;
@@ -349,8 +388,9 @@ extern "C" int entmax_attn_decode_fwd(const entmax_attn_decode_params* params, c
   a.kv_len = kv_len;
   a.alibi = alibi_slopes;
   a.beta = beta; a.gamma = gamma; a.delta = delta;
-  a.chunk_keys = lay.chunk_keys;
+  a.chunk_tiles = lay.chunk_tiles;
   a.n_chunks = lay.n_chunks;
+  a.n_tiles = lay.n_tiles;
   a.score_stride = lay.score_stride;
   int dev = 0, major = 0;
   cudaError_t err = cudaGetDevice(&dev);
@@ -359,20 +399,20 @@ extern "C" int entmax_attn_decode_fwd(const entmax_attn_decode_params* params, c
   if (major != 10) return ENTMAX_ATTN_EUNSUPPORTED;          // the score kernel needs tcgen05 / TMA
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
   uint8_t* ws = static_cast<uint8_t*>(workspace);
-  float* chunk_max = reinterpret_cast<float*>(ws + lay.chunk_max);
+  float* tile_max = reinterpret_cast<float*>(ws + lay.tile_max);
   float* scores = reinterpret_cast<float*>(ws + lay.scores);
   if (device_status) {
     err = cudaMemsetAsync(device_status, 0, sizeof(int32_t) * ENTMAX_ATTN_STATUS_WORDS, stream);
     if (err != cudaSuccess) return fail_cuda(err);
   }
   const int rows = a.B * a.H * a.QL;
-  err = launch_decode_scores_tc(a, q, k, scores, chunk_max, device_status, stream);
+  err = launch_decode_scores_tc(a, q, k, scores, tile_max, device_status, stream);
   if (err != cudaSuccess) return fail_cuda(err);
   const __nv_bfloat16* vb = static_cast<const __nv_bfloat16*>(v);
   __nv_bfloat16* ob = static_cast<__nv_bfloat16*>(o);
   // long rows: more threads per row (more loads in flight); many short rows: smaller CTAs
 #define ENTMAX_SOLVE(D, T) \
-  launch_kernel(decode_solve_kernel<D, T>, rows, T, 0, stream, a, vb, scores, chunk_max, ob, tau, support_size, device_status)
+  launch_kernel(decode_solve_kernel<D, T>, rows, T, 0, stream, a, vb, scores, tile_max, ob, tau, support_size, device_status)
   if (a.NC >= 16384) {
     if (a.D == 64) ENTMAX_SOLVE(64, 512); else ENTMAX_SOLVE(128, 512);
   } else {

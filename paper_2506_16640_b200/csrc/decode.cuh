@@ -13,8 +13,9 @@ struct DecodeArgs {
   const int32_t* kv_len;           // [B] or nullptr
   const float* alibi;              // [H] or nullptr
   const float *beta, *gamma, *delta;   // [H] each, or all nullptr (c = 1)
-  int chunk_keys;                  // keys per chunk maximum (a multiple of 128)
+  int chunk_tiles;                 // 128-key tiles per CTA of the score kernel; 0: a sequence's tiles dealt evenly to n_chunks CTAs
   int n_chunks;
+  int n_tiles;                     // 128-key tiles of the cache = entries of a row's list of tile maxima
   size_t score_stride;             // floats per score row
 };
 
@@ -28,8 +29,8 @@ __device__ __forceinline__ int seq_len(const DecodeArgs& a, int b, int32_t* stat
 }
 
 // Score stream on the tensor cores: K tiles of 128 keys as the M side of tcgen05 MMAs against the (zero-padded)
-// query rows, one thread per key afterwards.  Writes the score rows and the chunk maxima.
-cudaError_t launch_decode_scores_tc(const DecodeArgs& a, const void* q, const void* k, float* scores, float* chunk_max,
+// query rows, one thread per key afterwards.  Writes the score rows and the maxima of every 32 keys (four to a tile).
+cudaError_t launch_decode_scores_tc(const DecodeArgs& a, const void* q, const void* k, float* scores, float* tile_max,
                                     int32_t* status, cudaStream_t stream);
 
 }  // namespace entmax

@@ -8,7 +8,8 @@
 // CTAs per SM), so the kernel runs at the speed K can be read from HBM.
 //
 // CTA: warp 0 TMA producer, warp 1 MMA issuer, warps 2..5 one thread per key of the tile.  A CTA takes
-// chunk_keys consecutive keys of one (sequence, head).  Every wait is bounded (sm100_ptx.cuh).
+// consecutive tiles of one (sequence, head): eight of them, or, where that would leave less than a few CTAs per SM, its
+// share of the sequence's tiles (decode_layout).  Every wait is bounded (sm100_ptx.cuh).
 #include <cuda.h>
 
 #include "decode.cuh"
@@ -44,19 +45,18 @@ __global__ void __launch_bounds__(kThreadsD, 2) decode_scores_tc_kernel(const __
                                                                        const __grid_constant__ CUtensorMap map_k,
                                                                        const DecodeArgs a,
                                                                        float* __restrict__ scores,
-                                                                       float* __restrict__ chunk_max,
+                                                                       float* __restrict__ tile_max,
                                                                        int32_t* __restrict__ status) {
   pdl_begin();
   using C = DCfg<HD>;
   extern __shared__ uint8_t smem_raw[];
-  __shared__ float smax[4][ENTMAX_ATTN_DECODE_MAX_Q];
   const int chunk = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
   const int len = seq_len(a, b, status);
-  const int key0 = chunk * a.chunk_keys;
-  if (key0 >= len) return;                                  // whole CTA: nothing allocated yet
-  int tiles = a.chunk_keys / kTile;
-  const int left = (len - key0 + kTile - 1) / kTile;
-  if (left < tiles) tiles = left;
+  const int len_tiles = (len + kTile - 1) / kTile;
+  int tiles = a.chunk_tiles ? a.chunk_tiles : (len_tiles + a.n_chunks - 1) / a.n_chunks;
+  const int tile0 = chunk * tiles, key0 = tile0 * kTile;
+  if (tile0 >= len_tiles) return;                           // whole CTA: nothing allocated yet
+  if (len_tiles - tile0 < tiles) tiles = len_tiles - tile0;
 
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t k_smem = sbase;                            // [kStagesD] K tiles
@@ -178,12 +178,9 @@ __global__ void __launch_bounds__(kThreadsD, 2) decode_scores_tc_kernel(const __
       }
       a_lane = a.alpha_m1 * (c * a.sm_scale);
     }
-    float at[ENTMAX_ATTN_DECODE_MAX_Q], vmax[ENTMAX_ATTN_DECODE_MAX_Q];
+    float at[ENTMAX_ATTN_DECODE_MAX_Q];
 #pragma unroll
-    for (int t = 0; t < ENTMAX_ATTN_DECODE_MAX_Q; ++t) {
-      at[t] = __shfl_sync(0xffffffffu, a_lane, t);
-      vmax[t] = -INFINITY;
-    }
+    for (int t = 0; t < ENTMAX_ATTN_DECODE_MAX_Q; ++t) at[t] = __shfl_sync(0xffffffffu, a_lane, t);
     uint32_t sphase[2] = {0, 0};
     int buf = 0;
     bool alive = true;
@@ -200,30 +197,22 @@ __global__ void __launch_bounds__(kThreadsD, 2) decode_scores_tc_kernel(const __
       if (lane == 0) mbar_arrive(s_empty + 8 * buf);
       buf ^= 1;
       const int j = key0 + t * kTile + row_local;
-      if (j < len) {
 #pragma unroll
-        for (int tq = 0; tq < ENTMAX_ATTN_DECODE_MAX_Q; ++tq) {
-          if (tq < a.QL) {
-            const int pos = pos0 + tq;
-            const float y = j <= pos ? at[tq] * fmaf(slope, (float)(j - pos), acc[tq]) : -INFINITY;
-            scores[((size_t)bh * a.QL + tq) * a.score_stride + j] = y;
-            vmax[tq] = fmaxf(vmax[tq], y);
+      for (int tq = 0; tq < ENTMAX_ATTN_DECODE_MAX_Q; ++tq) {
+        if (tq < a.QL) {
+          const int pos = pos0 + tq;
+          const size_t row = (size_t)bh * a.QL + tq;
+          float y = -INFINITY;
+          if (j < len) {
+            if (j <= pos) y = at[tq] * fmaf(slope, (float)(j - pos), acc[tq]);
+            scores[row * a.score_stride + j] = y;
           }
+          // the warp's 32 keys: their maximum, by which the solve finds the tiles worth reading (one warp reduction: five
+          // shuffles per query instead cost 5 us of 79 on 8 x 16 x 16384 keys, four queries)
+          asm volatile("redux.sync.max.f32 %0, %0, 0xffffffff;" : "+f"(y));
+          if (lane == 0) tile_max[(row * a.n_tiles + tile0 + t) * 4 + quad] = y;
         }
       }
-    }
-    // chunk maximum per query: the warp, then the four warps
-#pragma unroll
-    for (int tq = 0; tq < ENTMAX_ATTN_DECODE_MAX_Q; ++tq) {
-      float m = vmax[tq];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-      if (lane == 0) smax[quad][tq] = m;
-    }
-    asm volatile("bar.sync 1, 128;" ::: "memory");
-    if (alive && row_local < a.QL) {
-      const float m = fmaxf(fmaxf(smax[0][row_local], smax[1][row_local]), fmaxf(smax[2][row_local], smax[3][row_local]));
-      chunk_max[((size_t)bh * a.QL + row_local) * a.n_chunks + chunk] = m;
     }
   }
 
@@ -247,7 +236,7 @@ __global__ void __launch_bounds__(kThreadsD, 2) decode_scores_tc_kernel(const __
 }
 
 template <int HD>
-cudaError_t launch_impl(const DecodeArgs& a, const void* q, const void* k, float* scores, float* chunk_max,
+cudaError_t launch_impl(const DecodeArgs& a, const void* q, const void* k, float* scores, float* tile_max,
                         int32_t* status, cudaStream_t stream) {
   CUtensorMap map_q, map_k;
   cudaError_t err = make_tile_map(&map_q, q, a.D, a.QL, a.H, a.B, a.D, (int64_t)a.QL * a.D, (int64_t)a.H * a.QL * a.D, kQPad);
@@ -257,17 +246,17 @@ cudaError_t launch_impl(const DecodeArgs& a, const void* q, const void* k, float
   err = cudaFuncSetAttribute(decode_scores_tc_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, DCfg<HD>::kSmemBytes);
   if (err != cudaSuccess) return err;
   const dim3 grid(a.n_chunks, a.H, a.B);
-  launch_kernel(decode_scores_tc_kernel<HD>, grid, kThreadsD, DCfg<HD>::kSmemBytes, stream, map_q, map_k, a, scores, chunk_max,
+  launch_kernel(decode_scores_tc_kernel<HD>, grid, kThreadsD, DCfg<HD>::kSmemBytes, stream, map_q, map_k, a, scores, tile_max,
                                                                                 status);
   return cudaGetLastError();
 }
 
 }  // namespace
 
-cudaError_t launch_decode_scores_tc(const DecodeArgs& a, const void* q, const void* k, float* scores, float* chunk_max,
+cudaError_t launch_decode_scores_tc(const DecodeArgs& a, const void* q, const void* k, float* scores, float* tile_max,
                                     int32_t* status, cudaStream_t stream) {
-  return a.D == 64 ? launch_impl<64>(a, q, k, scores, chunk_max, status, stream)
-                   : launch_impl<128>(a, q, k, scores, chunk_max, status, stream);
+  return a.D == 64 ? launch_impl<64>(a, q, k, scores, tile_max, status, stream)
+                   : launch_impl<128>(a, q, k, scores, tile_max, status, stream);
 }
 
 }  // namespace entmax

@@ -151,3 +151,18 @@ def test_decode_long_cache_sampled_heads():
     got = _run(inp, lens, 2, 1.5)
     assert int(got["status"][binding.STATUS_FLAGS]) == 0
     _check(inp, lens, 2, 1.5, got, heads=[0, 7, 15])
+
+
+@pytest.mark.parametrize("B,H,N,d,q_len", [(2, 8, 4737, 64, 2), (2, 148, 257, 64, 1), (4, 148, 129, 128, 3),
+                                           (1, 1, 66177, 64, 2)])
+def test_decode_split_of_the_keys_at_its_edges(B, H, N, d, q_len):
+    # tiles dealt to more CTAs than divide them (38 to 37), more (sequence, head) pairs than one wave holds, eight-tile
+    # CTAs with a one-key second tile, and a row with more than 32 tiles for every warp of the solve; sequences of every
+    # length down to the new rows alone
+    inp = _problem(B, H, N, d, plant=3, seed=N)
+    heads = sorted({0, H // 2, H - 1})
+    for ragged in (False, True):
+        lens = _lengths(B, N, q_len, N, ragged)
+        got = _run(inp, lens, q_len, 1.5)
+        assert int(got["status"][binding.STATUS_FLAGS]) == 0
+        _check(inp, lens, q_len, 1.5, got, heads=heads)
