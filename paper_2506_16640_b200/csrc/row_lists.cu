@@ -341,8 +341,10 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32) row_fwd_long_kernel(Problem
   }
 }
 
+// (register cap: as for row_bwd_kernel.  Without one the solve takes 127 registers and two CTAs fill an SM: 47 us against 37
+// now on 8 x 12 x 1024 x 64, 152 against 120 on 4 x 16 x 8192 x 64; at head_dim 128 227 against 212 on 16 x 20011)
 template <int D, int EC>
-__global__ void __launch_bounds__(kWarpsPerCta * 32) row_fwd_kernel(Problem p, const __nv_bfloat16* __restrict__ v,
+__global__ void __launch_bounds__(kWarpsPerCta * 32, D == 64 ? 4 : 3) row_fwd_kernel(Problem p, const __nv_bfloat16* __restrict__ v,
                                                                     const float* __restrict__ scale,
                                                                     int32_t* __restrict__ row_cnt,
                                                                     const int32_t* __restrict__ list_cnt,
@@ -553,23 +555,6 @@ __device__ __noinline__ void bwd_row_full(const Problem& p, const __nv_bfloat16*
   store_bf16<PER>(dq + hbase + (size_t)i * p.sn, acc);
 }
 
-// PL consecutive elements of a row: loads, stores and accumulator adds for any slice width used here
-template <int PL>
-__device__ __forceinline__ void load_slice_bf16(const __nv_bfloat16* p, float (&x)[PL]) {
-  if constexpr (PL >= 8) load_bf16_vec<PL>(p, x);
-  else load_bf16<PL>(p, x);
-}
-template <int PL>
-__device__ __forceinline__ void store_slice_bf16(__nv_bfloat16* p, const float (&x)[PL]) {
-  if constexpr (PL >= 8) store_bf16_vec<PL>(p, x);
-  else store_bf16<PL>(p, x);
-}
-template <int PL>
-__device__ __forceinline__ void add_slice(float* p, const float (&x)[PL]) {
-  if constexpr (PL >= 8) atomic_add_vec<PL>(p, x);
-  else atomic_add_slice<PL>(p, x);
-}
-
 // A lane's share of a row of D elements, W lanes per row: PL = D / W elements.  They are taken as chunks of four
 // that interleave across the lanes (chunk c of lane sl = elements [4 W c + 4 sl, +4)), so that what the W lanes
 // move in one instruction is contiguous: 16-byte reductions of neighbouring lanes fall into the same 32-byte
@@ -610,7 +595,130 @@ __device__ __forceinline__ void add_share(float* row, int sl, const float (&x)[P
   }
 }
 
-// Backward of 32 / W rows at once, W lanes per row (W = 8, 16 or 32), for rows with at most W list entries.
+// Backward of a row with 17 to 32 list entries: one lane per entry, the row's elements split over the whole warp.
+template <int D>
+__device__ __forceinline__ void bwd_row_warp(const Problem& p, const __nv_bfloat16* __restrict__ q,
+                                             const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v,
+                                             const __nv_bfloat16* __restrict__ d_o, const float* __restrict__ scale,
+                                             const float* __restrict__ tau_in, const Entry* __restrict__ entries,
+                                             __nv_bfloat16* __restrict__ dq, float* __restrict__ acc_dk,
+                                             float* __restrict__ acc_dv, float* __restrict__ dc_rows, int grow, int n,
+                                             bool saved, int pitch, int lane) {
+  constexpr int PL = D / 32;                       // elements of a row per lane
+  const int bh = grow / p.N, i = grow - bh * p.N, b = bh / p.H, h = bh - b * p.H;
+  const float g = scale[(size_t)b * p.scale_sb + (size_t)h * p.N + i] * p.sm_scale;
+  const float a = (p.alpha - 1.0f) * g;
+  const float tau = tau_in[grow];
+  const size_t hbase = (size_t)b * p.sb + (size_t)h * p.sh;
+  float qs[PL], gs[PL];
+  load_share<PL, 32>(q + hbase + (size_t)i * p.sn, lane, qs);
+  load_share<PL, 32>(d_o + hbase + (size_t)i * p.sn, lane, gs);
+  const Entry* list = entries + (size_t)grow * pitch;
+  float yv = -1.0f, zz = 0.f;
+  int j = 0;
+  if (lane < n) {
+    const Entry en = list[lane];
+    // a list saved by the forward pass holds y = (alpha-1) s in Eq. 1's units, a fresh one raw <q_i, k_j>
+    yv = saved ? en.y - tau : fmaf(a, en.y, -tau);
+    j = en.j;
+    zz = saved ? en.y / a : en.y;                  // raw <q_i, k_j>
+  }
+  const bool in = yv > 0.f;
+  const unsigned m = __ballot_sync(0xffffffffu, in);
+  // dP_ij = <dO_i, v_j> on the support, four V (and below, K) rows in flight: the loads are a chain of L2 round trips
+  // otherwise (long-row kernel 113 -> 77 us on 2 x 12 x 3001 x 64)
+  float dpv = 0.f;
+#pragma unroll 1
+  for (int t0 = 0; t0 < 32; t0 += 4) {
+    if ((m >> t0) == 0u) break;
+    float vs[4][PL], dp[4];
+#pragma unroll
+    for (int z = 0; z < 4; ++z) {
+      const int kj = __shfl_sync(0xffffffffu, j, t0 + z);
+#pragma unroll
+      for (int w = 0; w < PL; ++w) vs[z][w] = 0.f;
+      if ((m >> (t0 + z)) & 1u) load_share<PL, 32>(v + hbase + (size_t)kj * p.sn, lane, vs[z]);
+    }
+#pragma unroll
+    for (int z = 0; z < 4; ++z) {
+      dp[z] = 0.f;
+#pragma unroll
+      for (int w = 0; w < PL; ++w) dp[z] = fmaf(gs[w], vs[z][w], dp[z]);
+    }
+#pragma unroll
+    for (int z = 0; z < 4; ++z) {
+      dp[z] = warp_sum(dp[z]);
+      if (lane == t0 + z) dpv = dp[z];
+    }
+  }
+  float pe = 0.f, u = 0.f;
+  if (in) pow_pair(yv, p.expo_class, p.expo, pe, u);
+  const float su = warp_sum(u), sud = warp_sum(u * dpv);
+  const float rho = su > 0.f ? sud / su : 0.f;
+  const float gds_own = g * u * (dpv - rho);
+  if (dc_rows) {
+    // dL/dc_i = sum_j dS_ij z_ij with z_ij = <q_i,k_j> sm_scale (chain rule through s = c z)
+    const float dc = warp_sum(u * (dpv - rho) * zz);
+    if (lane == 0) dc_rows[grow] = dc * p.sm_scale;
+  }
+  float acc[PL];
+#pragma unroll
+  for (int t = 0; t < PL; ++t) acc[t] = 0.f;
+  const size_t arow = (size_t)bh * p.N;
+#pragma unroll 1
+  for (int t0 = 0; t0 < 32; t0 += 4) {
+    if ((m >> t0) == 0u) break;
+    float ks[4][PL];
+#pragma unroll
+    for (int z = 0; z < 4; ++z) {
+      const int kj = __shfl_sync(0xffffffffu, j, t0 + z);
+#pragma unroll
+      for (int w = 0; w < PL; ++w) ks[z][w] = 0.f;
+      if ((m >> (t0 + z)) & 1u) load_share<PL, 32>(k + hbase + (size_t)kj * p.sn, lane, ks[z]);
+    }
+#pragma unroll
+    for (int z = 0; z < 4; ++z) {
+      const int kj = __shfl_sync(0xffffffffu, j, t0 + z);
+      const float gds = __shfl_sync(0xffffffffu, gds_own, t0 + z);
+      const float pj = __shfl_sync(0xffffffffu, pe, t0 + z);
+      if ((m >> (t0 + z)) & 1u) {
+        float x[PL];
+#pragma unroll
+        for (int w = 0; w < PL; ++w) {
+          acc[w] = fmaf(gds, ks[z][w], acc[w]);
+          x[w] = gds * qs[w];
+        }
+        add_share<PL, 32>(acc_dk + (arow + kj) * D, lane, x);
+#pragma unroll
+        for (int w = 0; w < PL; ++w) x[w] = pj * gs[w];
+        add_share<PL, 32>(acc_dv + (arow + kj) * D, lane, x);
+      }
+    }
+  }
+  store_share<PL, 32>(dq + hbase + (size_t)i * p.sn, lane, acc);
+}
+
+// A lane's share of a row as it lies in memory, 2 PL bytes (same interleaving as load_share): half the registers of its
+// floats, so that several rows can be in flight.
+template <int PL>
+struct PackedShare {
+  uint2 c[PL / 4];
+};
+template <int PL, int W>
+__device__ __forceinline__ void load_packed(const __nv_bfloat16* row, int sl, PackedShare<PL>& x) {
+#pragma unroll
+  for (int c = 0; c < PL / 4; ++c) x.c[c] = *reinterpret_cast<const uint2*>(row + 4 * W * c + 4 * sl);
+}
+template <int PL>
+__device__ __forceinline__ float packed_at(const PackedShare<PL>& x, int e) {
+  const uint32_t w = (e & 2) ? x.c[e >> 2].y : x.c[e >> 2].x;
+  return __uint_as_float((e & 1) ? (w & 0xffff0000u) : (w << 16));
+}
+
+// Backward of 32 / W rows at once, W lanes per row (W = 8 or 16), for rows with at most W list entries.  Bound by the
+// latency of the gathers: four V rows, then four (head_dim 64) or two K rows are in flight at a time, and q_i, dO_i and
+// the gathered rows stay packed until they are used (as floats batches of four spill).  One row at a time before ->
+// now: 8 x 12 x 1024 x 64 74 -> 57 us, 4 x 16 x 8192 x 64 281 -> 217, 16 x 32768 x 128 632 -> 570.
 template <int D, int W>
 __device__ __forceinline__ void bwd_rows_sub(const Problem& p, const __nv_bfloat16* __restrict__ q,
                                              const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v,
@@ -620,7 +728,8 @@ __device__ __forceinline__ void bwd_rows_sub(const Problem& p, const __nv_bfloat
                                              float* __restrict__ acc_dv, float* __restrict__ dc_rows, int grow,
                                              bool active, int n_list, bool saved, int pitch, int lane) {
   constexpr int PL = D / W;                        // elements of a row per lane
-  constexpr unsigned kWMask = W == 32 ? 0xffffffffu : ((1u << (W & 31)) - 1u);
+  constexpr int kBatch = PL <= 8 ? 4 : 2;          // rows in flight
+  constexpr unsigned kWMask = (1u << W) - 1u;
   const int sl = lane & (W - 1);
   const int base = lane & (32 - W);
   const int n = active ? n_list : 0;
@@ -629,9 +738,9 @@ __device__ __forceinline__ void bwd_rows_sub(const Problem& p, const __nv_bfloat
   const float a = (p.alpha - 1.0f) * g;
   const float tau = active ? tau_in[grow] : 0.f;
   const size_t hbase = (size_t)b * p.sb + (size_t)h * p.sh;
-  float qs[PL], gs[PL];
-  load_share<PL, W>(q + hbase + (size_t)i * p.sn, sl, qs);
-  load_share<PL, W>(d_o + hbase + (size_t)i * p.sn, sl, gs);
+  PackedShare<PL> qs, gs;
+  load_packed<PL, W>(q + hbase + (size_t)i * p.sn, sl, qs);
+  load_packed<PL, W>(d_o + hbase + (size_t)i * p.sn, sl, gs);
   const Entry* list = entries + (size_t)grow * pitch;
   float yv = -1.0f, zz = 0.f;
   int j = 0;
@@ -644,52 +753,38 @@ __device__ __forceinline__ void bwd_rows_sub(const Problem& p, const __nv_bfloat
   }
   const bool in = yv > 0.f;
   const unsigned msub = (__ballot_sync(0xffffffffu, in) >> base) & kWMask;
-  // dP_ij = <dO_i, v_j> on the support.  A warp per row keeps four V (and below, K) rows in flight (long-row kernel 113 -> 77 us on
-  // 2 x 12 x 3001 x 64); rows that share a warp hold longer slices, and batches of them spill (630 -> 797 us on 16 x 32768 x 128)
+  // slots of the fullest row of the warp
+  const int last = 32 - __clz(__reduce_or_sync(0xffffffffu, msub));
+  // dP_ij = <dO_i, v_j> on the support.  (A slot without an entry names key 0: its row is loaded and the product dropped.)
   float dpv = 0.f;
-  if constexpr (W == 32) {
 #pragma unroll 1
-    for (int t0 = 0; t0 < W; t0 += 4) {
-      if ((msub >> t0) == 0u) break;
-      float vs[4][PL], dp[4];
+  for (int t0 = 0; t0 < last; t0 += kBatch) {
+    PackedShare<PL> vs[kBatch];
 #pragma unroll
-      for (int z = 0; z < 4; ++z) {
-        const int kj = __shfl_sync(0xffffffffu, j, t0 + z);
+    for (int z = 0; z < kBatch; ++z)
+      load_packed<PL, W>(v + hbase + (size_t)__shfl_sync(0xffffffffu, j, base + t0 + z) * p.sn, sl, vs[z]);
+    float dp[kBatch];
 #pragma unroll
-        for (int w = 0; w < PL; ++w) vs[z][w] = 0.f;
-        if ((msub >> (t0 + z)) & 1u) load_share<PL, W>(v + hbase + (size_t)kj * p.sn, sl, vs[z]);
-      }
+    for (int z = 0; z < kBatch; ++z) {
+      dp[z] = 0.f;
 #pragma unroll
-      for (int z = 0; z < 4; ++z) {
-        dp[z] = 0.f;
-#pragma unroll
-        for (int w = 0; w < PL; ++w) dp[z] = fmaf(gs[w], vs[z][w], dp[z]);
-      }
-#pragma unroll
-      for (int z = 0; z < 4; ++z) {
-        dp[z] = sub_sum<W>(dp[z]);
-        if (sl == t0 + z) dpv = dp[z];
-      }
+      for (int e = 0; e < PL; ++e) dp[z] = fmaf(packed_at(gs, e), packed_at(vs[z], e), dp[z]);
     }
-  } else {
-#pragma unroll 4
-    for (int t = 0; t < W; ++t) {
-      if (!__any_sync(0xffffffffu, (msub >> t) != 0u)) break;        // no row has entries from slot t on
-      const bool has = (msub >> t) & 1u;
-      const int kj = __shfl_sync(0xffffffffu, j, base + t);
-      float dp = 0.f;
-      if (has) {
-        float vs[PL];
-        load_share<PL, W>(v + hbase + (size_t)kj * p.sn, sl, vs);
-#pragma unroll
-        for (int u = 0; u < PL; ++u) dp = fmaf(gs[u], vs[u], dp);
-      }
-      dp = sub_sum<W>(dp);
-      if (sl == t) dpv = dp;
+    // the batch's sums over the row's lanes in one butterfly: lane sl ends up with the one of slot t0 + sl mod kBatch
+    const bool odd = sl & 1;
+    float r = (odd ? dp[1] : dp[0]) + __shfl_xor_sync(0xffffffffu, odd ? dp[0] : dp[1], 1);
+    if constexpr (kBatch == 4) {
+      const float s23 = (odd ? dp[3] : dp[2]) + __shfl_xor_sync(0xffffffffu, odd ? dp[2] : dp[3], 1);
+      const bool upper = sl & 2;
+      r = (upper ? s23 : r) + __shfl_xor_sync(0xffffffffu, upper ? r : s23, 2);
     }
+#pragma unroll
+    for (int o = kBatch; o < W; o <<= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+    if ((sl & ~(kBatch - 1)) == t0) dpv = r;
   }
   float pe = 0.f, u = 0.f;
   if (in) pow_pair(yv, p.expo_class, p.expo, pe, u);
+  else dpv = 0.f;
   const float su = sub_sum<W>(u), sud = sub_sum<W>(u * dpv);
   const float rho = su > 0.f ? sud / su : 0.f;
   const float gds_own = g * u * (dpv - rho);
@@ -702,65 +797,40 @@ __device__ __forceinline__ void bwd_rows_sub(const Problem& p, const __nv_bfloat
 #pragma unroll
   for (int t = 0; t < PL; ++t) acc[t] = 0.f;
   const size_t arow = (size_t)bh * p.N;
-  if constexpr (W == 32) {
 #pragma unroll 1
-    for (int t0 = 0; t0 < W; t0 += 4) {
-      if ((msub >> t0) == 0u) break;
-      float ks[4][PL];
+  for (int t0 = 0; t0 < last; t0 += kBatch) {
+    PackedShare<PL> ks[kBatch];
 #pragma unroll
-      for (int z = 0; z < 4; ++z) {
-        const int kj = __shfl_sync(0xffffffffu, j, t0 + z);
+    for (int z = 0; z < kBatch; ++z)
+      load_packed<PL, W>(k + hbase + (size_t)__shfl_sync(0xffffffffu, j, base + t0 + z) * p.sn, sl, ks[z]);
 #pragma unroll
-        for (int w = 0; w < PL; ++w) ks[z][w] = 0.f;
-        if ((msub >> (t0 + z)) & 1u) load_share<PL, W>(k + hbase + (size_t)kj * p.sn, sl, ks[z]);
-      }
+    for (int z = 0; z < kBatch; ++z) {
+      const int kj = __shfl_sync(0xffffffffu, j, base + t0 + z);
+      const float gds = __shfl_sync(0xffffffffu, gds_own, base + t0 + z);
+      const float pj = __shfl_sync(0xffffffffu, pe, base + t0 + z);
+      if ((msub >> (t0 + z)) & 1u) {
+        float* dk_row = acc_dk + (arow + kj) * D + 4 * sl;
+        float* dv_row = acc_dv + (arow + kj) * D + 4 * sl;
 #pragma unroll
-      for (int z = 0; z < 4; ++z) {
-        const int kj = __shfl_sync(0xffffffffu, j, t0 + z);
-        const float gds = __shfl_sync(0xffffffffu, gds_own, t0 + z);
-        const float pj = __shfl_sync(0xffffffffu, pe, t0 + z);
-        if ((msub >> (t0 + z)) & 1u) {
-          float x[PL];
+        for (int c = 0; c < PL / 4; ++c) {
 #pragma unroll
-          for (int w = 0; w < PL; ++w) {
-            acc[w] = fmaf(gds, ks[z][w], acc[w]);
-            x[w] = gds * qs[w];
-          }
-          add_share<PL, W>(acc_dk + (arow + kj) * D, sl, x);
-#pragma unroll
-          for (int w = 0; w < PL; ++w) x[w] = pj * gs[w];
-          add_share<PL, W>(acc_dv + (arow + kj) * D, sl, x);
+          for (int e = 4 * c; e < 4 * c + 4; ++e) acc[e] = fmaf(gds, packed_at(ks[z], e), acc[e]);
+          red_add_v4(dk_row + 4 * W * c, gds * packed_at(qs, 4 * c), gds * packed_at(qs, 4 * c + 1),
+                     gds * packed_at(qs, 4 * c + 2), gds * packed_at(qs, 4 * c + 3));
+          red_add_v4(dv_row + 4 * W * c, pj * packed_at(gs, 4 * c), pj * packed_at(gs, 4 * c + 1),
+                     pj * packed_at(gs, 4 * c + 2), pj * packed_at(gs, 4 * c + 3));
         }
-      }
-    }
-  } else {
-#pragma unroll 4
-    for (int t = 0; t < W; ++t) {
-      if (!__any_sync(0xffffffffu, (msub >> t) != 0u)) break;
-      const bool has = (msub >> t) & 1u;
-      const int kj = __shfl_sync(0xffffffffu, j, base + t);
-      const float gds = __shfl_sync(0xffffffffu, gds_own, base + t);
-      const float pj = __shfl_sync(0xffffffffu, pe, base + t);
-      if (has) {
-        float ks[PL], dkv[PL], dvv[PL];
-        load_share<PL, W>(k + hbase + (size_t)kj * p.sn, sl, ks);
-#pragma unroll
-        for (int w = 0; w < PL; ++w) {
-          acc[w] = fmaf(gds, ks[w], acc[w]);
-          dkv[w] = gds * qs[w];
-          dvv[w] = pj * gs[w];
-        }
-        add_share<PL, W>(acc_dk + (arow + kj) * D, sl, dkv);
-        add_share<PL, W>(acc_dv + (arow + kj) * D, sl, dvv);
       }
     }
   }
   if (active) store_share<PL, W>(dq + hbase + (size_t)i * p.sn, sl, acc);
 }
 
-// (register cap: four CTAs per SM -- this kernel waits on gathers and reductions, occupancy is what hides them)
+// (register cap: this kernel waits on gathers and reductions, warps are what hides them.  Four CTAs per SM at head_dim 64,
+// where three take 60 us instead of 57 on 8 x 12 x 1024; three at 128, where the cap of four spills: 640 us against 570 on
+// 16 x 32768)
 template <int D>
-__global__ void __launch_bounds__(kWarpsPerCta * 32, 4) row_bwd_kernel(
+__global__ void __launch_bounds__(kWarpsPerCta * 32, D == 64 ? 4 : 3) row_bwd_kernel(
     Problem p, const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k,
     const __nv_bfloat16* __restrict__ v, const __nv_bfloat16* __restrict__ d_o, const float* __restrict__ scale,
     const float* __restrict__ tau_in, const int32_t* __restrict__ list_cnt, const Entry* __restrict__ entries,
@@ -833,8 +903,8 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 4) row_bwd_long_kernel(
     const int grow = fb_list[total - 1 - t];
     const int n_list = list_cnt[saved ? (size_t)grow : 2 * (size_t)grow];
     if (n_list <= 32)
-      bwd_rows_sub<D, 32>(p, q, k, v, d_o, scale, tau_in, entries, dq, acc_dk, acc_dv, dc_rows, grow, true, n_list,
-                          saved != 0, pitch, lane);
+      bwd_row_warp<D>(p, q, k, v, d_o, scale, tau_in, entries, dq, acc_dk, acc_dv, dc_rows, grow, n_list, saved != 0, pitch,
+                      lane);
     else
       bwd_row_full<D>(p, q, k, v, d_o, scale, tau_in, entries, dq, acc_dk, acc_dv, dc_rows, grow, n_list, saved != 0,
                       pitch, lane);
