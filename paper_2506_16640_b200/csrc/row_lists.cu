@@ -136,6 +136,70 @@ __device__ __forceinline__ int solve_row(const Problem& p, Entry* list, int n, f
   return cnt;
 }
 
+// A lane's share of a row of D elements, W lanes per row: PL = D / W elements.  They are taken as chunks of four
+// that interleave across the lanes (chunk c of lane sl = elements [4 W c + 4 sl, +4)), so that what the W lanes
+// move in one instruction is contiguous: 16-byte reductions of neighbouring lanes fall into the same 32-byte
+// sector instead of half-filling one each, loads and stores stay coalesced.  (PL < 4: one contiguous piece.)
+template <int PL, int W>
+__device__ __forceinline__ void load_share(const __nv_bfloat16* row, int sl, float (&x)[PL]) {
+  if constexpr (PL < 4) {
+    load_bf16<PL>(row + sl * PL, x);
+  } else {
+#pragma unroll
+    for (int c = 0; c < PL / 4; ++c) {
+      float t[4];
+      load_bf16<4>(row + 4 * W * c + 4 * sl, t);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) x[4 * c + e] = t[e];
+    }
+  }
+}
+template <int PL, int W>
+__device__ __forceinline__ void store_share(__nv_bfloat16* row, int sl, const float (&x)[PL]) {
+  if constexpr (PL < 4) {
+    store_bf16<PL>(row + sl * PL, x);
+  } else {
+#pragma unroll
+    for (int c = 0; c < PL / 4; ++c) {
+      const float t[4] = {x[4 * c], x[4 * c + 1], x[4 * c + 2], x[4 * c + 3]};
+      store_bf16<4>(row + 4 * W * c + 4 * sl, t);
+    }
+  }
+}
+template <int PL, int W>
+__device__ __forceinline__ void add_share(float* row, int sl, const float (&x)[PL]) {
+  if constexpr (PL < 4) {
+    atomic_add_slice<PL>(row + sl * PL, x);
+  } else {
+#pragma unroll
+    for (int c = 0; c < PL / 4; ++c) red_add_v4(row + 4 * W * c + 4 * sl, x[4 * c], x[4 * c + 1], x[4 * c + 2], x[4 * c + 3]);
+  }
+}
+
+// A lane's share of a row as it lies in memory (the interleaving of load_share), two elements to a register: half the
+// registers of its floats, so that several rows can be in flight.
+template <int PL>
+struct PackedShare {
+  uint32_t w[PL / 2];
+};
+template <int PL, int W>
+__device__ __forceinline__ void load_packed(const __nv_bfloat16* row, int sl, PackedShare<PL>& x) {
+  if constexpr (PL < 4) {
+    x.w[0] = *reinterpret_cast<const uint32_t*>(row + 2 * sl);
+  } else {
+#pragma unroll
+    for (int c = 0; c < PL / 4; ++c) {
+      const uint2 r = *reinterpret_cast<const uint2*>(row + 4 * W * c + 4 * sl);
+      x.w[2 * c] = r.x;
+      x.w[2 * c + 1] = r.y;
+    }
+  }
+}
+template <int PL>
+__device__ __forceinline__ float packed_at(const PackedShare<PL>& x, int e) {
+  return __uint_as_float((e & 1) ? (x.w[e >> 1] & 0xffff0000u) : (x.w[e >> 1] << 16));
+}
+
 // O_i of 32 / W rows at once, W lanes per row, from the supports solve_row left (cnt <= W entries; cnt = 0: no row).
 template <int D, int W, int EC>
 __device__ __forceinline__ void gather_rows(const Problem& p, const __nv_bfloat16* __restrict__ v,
@@ -157,32 +221,26 @@ __device__ __forceinline__ void gather_rows(const Problem& p, const __nv_bfloat1
   float acc[PL];
 #pragma unroll
   for (int t = 0; t < PL; ++t) acc[t] = 0.f;
-  const size_t hbase = (size_t)b * p.sb + (size_t)h * p.sh + sl * PL;
+  const size_t hbase = (size_t)b * p.sb + (size_t)h * p.sh;
 #pragma unroll 1
   for (int t0 = 0; t0 < W; t0 += kBatch) {
     if (!__any_sync(0xffffffffu, t0 < cnt)) break;
-    float vs[kBatch][PL], pj[kBatch];
+    PackedShare<PL> vs[kBatch];
+    float pj[kBatch];
 #pragma unroll
     for (int u = 0; u < kBatch; ++u) {
       pj[u] = __shfl_sync(0xffffffffu, pe, base + t0 + u);
       const int kj = __shfl_sync(0xffffffffu, j, base + t0 + u);
 #pragma unroll
-      for (int e = 0; e < PL; ++e) vs[u][e] = 0.f;
-      if (t0 + u < cnt) {
-        if constexpr (PL >= 8) load_bf16_vec<PL>(v + hbase + (size_t)kj * p.sn, vs[u]);
-        else load_bf16<PL>(v + hbase + (size_t)kj * p.sn, vs[u]);
-      }
+      for (int e = 0; e < PL / 2; ++e) vs[u].w[e] = 0u;
+      if (t0 + u < cnt) load_packed<PL, W>(v + hbase + (size_t)kj * p.sn, sl, vs[u]);
     }
 #pragma unroll
     for (int u = 0; u < kBatch; ++u)
 #pragma unroll
-      for (int e = 0; e < PL; ++e) acc[e] = fmaf(pj[u], vs[u][e], acc[e]);
+      for (int e = 0; e < PL; ++e) acc[e] = fmaf(pj[u], packed_at(vs[u], e), acc[e]);
   }
-  if (cnt > 0) {
-    __nv_bfloat16* o_row = o + hbase + (size_t)i * p.sn;
-    if constexpr (PL >= 8) store_bf16_vec<PL>(o_row, acc);
-    else store_bf16<PL>(o_row, acc);
-  }
+  if (cnt > 0) store_share<PL, W>(o + hbase + (size_t)i * p.sn, sl, acc);
 }
 
 // One row with the whole warp, up to 32 S list entries: threshold, support, output.
@@ -555,46 +613,6 @@ __device__ __noinline__ void bwd_row_full(const Problem& p, const __nv_bfloat16*
   store_bf16<PER>(dq + hbase + (size_t)i * p.sn, acc);
 }
 
-// A lane's share of a row of D elements, W lanes per row: PL = D / W elements.  They are taken as chunks of four
-// that interleave across the lanes (chunk c of lane sl = elements [4 W c + 4 sl, +4)), so that what the W lanes
-// move in one instruction is contiguous: 16-byte reductions of neighbouring lanes fall into the same 32-byte
-// sector instead of half-filling one each, loads and stores stay coalesced.  (PL < 4: one contiguous piece.)
-template <int PL, int W>
-__device__ __forceinline__ void load_share(const __nv_bfloat16* row, int sl, float (&x)[PL]) {
-  if constexpr (PL < 4) {
-    load_bf16<PL>(row + sl * PL, x);
-  } else {
-#pragma unroll
-    for (int c = 0; c < PL / 4; ++c) {
-      float t[4];
-      load_bf16<4>(row + 4 * W * c + 4 * sl, t);
-#pragma unroll
-      for (int e = 0; e < 4; ++e) x[4 * c + e] = t[e];
-    }
-  }
-}
-template <int PL, int W>
-__device__ __forceinline__ void store_share(__nv_bfloat16* row, int sl, const float (&x)[PL]) {
-  if constexpr (PL < 4) {
-    store_bf16<PL>(row + sl * PL, x);
-  } else {
-#pragma unroll
-    for (int c = 0; c < PL / 4; ++c) {
-      const float t[4] = {x[4 * c], x[4 * c + 1], x[4 * c + 2], x[4 * c + 3]};
-      store_bf16<4>(row + 4 * W * c + 4 * sl, t);
-    }
-  }
-}
-template <int PL, int W>
-__device__ __forceinline__ void add_share(float* row, int sl, const float (&x)[PL]) {
-  if constexpr (PL < 4) {
-    atomic_add_slice<PL>(row + sl * PL, x);
-  } else {
-#pragma unroll
-    for (int c = 0; c < PL / 4; ++c) red_add_v4(row + 4 * W * c + 4 * sl, x[4 * c], x[4 * c + 1], x[4 * c + 2], x[4 * c + 3]);
-  }
-}
-
 // Backward of a row with 17 to 32 list entries: one lane per entry, the row's elements split over the whole warp.
 template <int D>
 __device__ __forceinline__ void bwd_row_warp(const Problem& p, const __nv_bfloat16* __restrict__ q,
@@ -696,23 +714,6 @@ __device__ __forceinline__ void bwd_row_warp(const Problem& p, const __nv_bfloat
     }
   }
   store_share<PL, 32>(dq + hbase + (size_t)i * p.sn, lane, acc);
-}
-
-// A lane's share of a row as it lies in memory, 2 PL bytes (same interleaving as load_share): half the registers of its
-// floats, so that several rows can be in flight.
-template <int PL>
-struct PackedShare {
-  uint2 c[PL / 4];
-};
-template <int PL, int W>
-__device__ __forceinline__ void load_packed(const __nv_bfloat16* row, int sl, PackedShare<PL>& x) {
-#pragma unroll
-  for (int c = 0; c < PL / 4; ++c) x.c[c] = *reinterpret_cast<const uint2*>(row + 4 * W * c + 4 * sl);
-}
-template <int PL>
-__device__ __forceinline__ float packed_at(const PackedShare<PL>& x, int e) {
-  const uint32_t w = (e & 2) ? x.c[e >> 2].y : x.c[e >> 2].x;
-  return __uint_as_float((e & 1) ? (w & 0xffff0000u) : (w << 16));
 }
 
 // Backward of 32 / W rows at once, W lanes per row (W = 8 or 16), for rows with at most W list entries.  Bound by the
