@@ -44,97 +44,6 @@ __device__ __forceinline__ float sub_sum(float x) {
   for (int o = 1; o < W; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
   return x;
 }
-template <int W>
-__device__ __forceinline__ float sub_max(float x) {
-#pragma unroll
-  for (int o = 1; o < W; o <<= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, o));
-  return x;
-}
-// N consecutive bf16 (N = 8 or 16, 16-byte aligned) <-> floats
-template <int N>
-__device__ __forceinline__ void load_bf16_vec(const __nv_bfloat16* p, float (&x)[N]) {
-#pragma unroll
-  for (int c = 0; c < N / 8; ++c) {
-    const uint4 raw = *reinterpret_cast<const uint4*>(p + 8 * c);
-    const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[t]));
-      x[8 * c + 2 * t] = f.x;
-      x[8 * c + 2 * t + 1] = f.y;
-    }
-  }
-}
-template <int N>
-__device__ __forceinline__ void store_bf16_vec(__nv_bfloat16* p, const float (&x)[N]) {
-#pragma unroll
-  for (int c = 0; c < N / 8; ++c) {
-    uint32_t w[4];
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const __nv_bfloat162 h = __floats2bfloat162_rn(x[8 * c + 2 * t], x[8 * c + 2 * t + 1]);
-      w[t] = *reinterpret_cast<const uint32_t*>(&h);
-    }
-    *reinterpret_cast<uint4*>(p + 8 * c) = make_uint4(w[0], w[1], w[2], w[3]);
-  }
-}
-template <int N>
-__device__ __forceinline__ void atomic_add_vec(float* p, const float (&x)[N]) {
-#pragma unroll
-  for (int c = 0; c < N / 4; ++c)
-    red_add_v4(p + 4 * c, x[4 * c], x[4 * c + 1], x[4 * c + 2], x[4 * c + 3]);
-}
-
-// Row solve.  The lists the sweep leaves are deterministic (a row's candidates depend on that row alone, in key order), so a
-// threshold iterated on the whole list is reproducible to the bit.
-constexpr float kBoundMargin = 4e-6f;   // rounding of the bound the sweep ended with
-
-// Threshold of Eq. 1 on the n <= K list entries of one row, by one thread with the entries in registers (n = 0: a lane without
-// a row, which only takes part in the votes); the list is left compacted to the support, y in Eq. 1's units.  Newton from the
-// left starting at the bound the sweep ended with (e < 1: bracketed, tau_iter_update).  Sums over a row need no shuffles this
-// way: eight to thirty-two lanes per row spent two chains of them on every iteration, or sorted the list first (alpha = 1.25,
-// 16 x 20011 x 128: 580 + 92 us with the long rows -> 227 + 66; alpha = 1.5, 16 x 32768 x 128: 222 + 105 -> 255 + 32).
-template <int K, int EC>
-__device__ __forceinline__ int solve_row(const Problem& p, Entry* list, int n, float a, float bound, float& tau) {
-  float y[K];
-  float ymax = -INFINITY;
-#pragma unroll
-  for (int e = 0; e < K; e += 2) {
-    float4 q = make_float4(-INFINITY, 0.f, -INFINITY, 0.f);
-    if (e < n) q = *reinterpret_cast<const float4*>(list + e);     // {y, j, y, j}
-    y[e] = e < n ? a * q.x : -INFINITY;
-    y[e + 1] = e + 1 < n ? a * q.z : -INFINITY;
-    ymax = fmaxf(ymax, fmaxf(y[e], y[e + 1]));
-  }
-  TauIter st = tau_iter_start(ymax);
-  st.tau = st.lo = fmaxf(st.lo, bound);
-  bool done = n == 0;
-  for (int it = 0; it < kMaxNewton; ++it) {
-    float s0[2] = {0.f, 0.f}, s1[2] = {0.f, 0.f};
-#pragma unroll
-    for (int e = 0; e < K; ++e) {
-      const float d = fmaxf(y[e] - st.tau, 0.f);
-      float ye, ye1;
-      pow_pair_c<EC>(d, d > 0.f, p.expo, ye, ye1);
-      s0[e & 1] += ye;
-      s1[e & 1] += ye1;
-    }
-    if (!done) done = !tau_iter_update(st, s0[0] + s0[1], s1[0] + s1[1], p.expo_class, p.expo, 1e-7f);
-    if (__all_sync(0xffffffffu, done)) break;
-  }
-  tau = st.tau;
-  int cnt = 0;
-#pragma unroll
-  for (int e = 0; e < K; ++e) {
-    if (e < n && y[e] > tau) {
-      Entry en;
-      en.y = y[e];
-      en.j = list[e].j;
-      list[cnt++] = en;
-    }
-  }
-  return cnt;
-}
 
 // A lane's share of a row of D elements, W lanes per row: PL = D / W elements.  They are taken as chunks of four
 // that interleave across the lanes (chunk c of lane sl = elements [4 W c + 4 sl, +4)), so that what the W lanes
@@ -198,6 +107,57 @@ __device__ __forceinline__ void load_packed(const __nv_bfloat16* row, int sl, Pa
 template <int PL>
 __device__ __forceinline__ float packed_at(const PackedShare<PL>& x, int e) {
   return __uint_as_float((e & 1) ? (x.w[e >> 1] & 0xffff0000u) : (x.w[e >> 1] << 16));
+}
+
+// Row solve.  The lists the sweep leaves are deterministic (a row's candidates depend on that row alone, in key order), so a
+// threshold iterated on the whole list is reproducible to the bit.
+constexpr float kBoundMargin = 4e-6f;   // rounding of the bound the sweep ended with
+
+// Threshold of Eq. 1 on the n <= K list entries of one row, by one thread with the entries in registers (n = 0: a lane without
+// a row, which only takes part in the votes); the list is left compacted to the support, y in Eq. 1's units.  Newton from the
+// left starting at the bound the sweep ended with (e < 1: bracketed, tau_iter_update).  Sums over a row need no shuffles this
+// way: eight to thirty-two lanes per row spent two chains of them on every iteration, or sorted the list first (alpha = 1.25,
+// 16 x 20011 x 128: 580 + 92 us with the long rows -> 227 + 66; alpha = 1.5, 16 x 32768 x 128: 222 + 105 -> 255 + 32).
+template <int K, int EC>
+__device__ __forceinline__ int solve_row(const Problem& p, Entry* list, int n, float a, float bound, float& tau) {
+  float y[K];
+  float ymax = -INFINITY;
+#pragma unroll
+  for (int e = 0; e < K; e += 2) {
+    float4 q = make_float4(-INFINITY, 0.f, -INFINITY, 0.f);
+    if (e < n) q = *reinterpret_cast<const float4*>(list + e);     // {y, j, y, j}
+    y[e] = e < n ? a * q.x : -INFINITY;
+    y[e + 1] = e + 1 < n ? a * q.z : -INFINITY;
+    ymax = fmaxf(ymax, fmaxf(y[e], y[e + 1]));
+  }
+  TauIter st = tau_iter_start(ymax);
+  st.tau = st.lo = fmaxf(st.lo, bound);
+  bool done = n == 0;
+  for (int it = 0; it < kMaxNewton; ++it) {
+    float s0[2] = {0.f, 0.f}, s1[2] = {0.f, 0.f};
+#pragma unroll
+    for (int e = 0; e < K; ++e) {
+      const float d = fmaxf(y[e] - st.tau, 0.f);
+      float ye, ye1;
+      pow_pair_c<EC>(d, d > 0.f, p.expo, ye, ye1);
+      s0[e & 1] += ye;
+      s1[e & 1] += ye1;
+    }
+    if (!done) done = !tau_iter_update(st, s0[0] + s0[1], s1[0] + s1[1], p.expo_class, p.expo, 1e-7f);
+    if (__all_sync(0xffffffffu, done)) break;
+  }
+  tau = st.tau;
+  int cnt = 0;
+#pragma unroll
+  for (int e = 0; e < K; ++e) {
+    if (e < n && y[e] > tau) {
+      Entry en;
+      en.y = y[e];
+      en.j = list[e].j;
+      list[cnt++] = en;
+    }
+  }
+  return cnt;
 }
 
 // O_i of 32 / W rows at once, W lanes per row, from the supports solve_row left (cnt <= W entries; cnt = 0: no row).
@@ -286,7 +246,6 @@ __device__ __forceinline__ void long_row(const Problem& p, const __nv_bfloat16* 
   float acc[PER];
 #pragma unroll
   for (int t = 0; t < PER; ++t) acc[t] = 0.f;
-  const __nv_bfloat16* vbase = v + hbase + lane * PER;
   int kept = 0;
 #pragma unroll
   for (int s = 0; s < S; ++s) {
@@ -302,7 +261,8 @@ __device__ __forceinline__ void long_row(const Problem& p, const __nv_bfloat16* 
     kept += __popc(m);
     while (m) {
       // eight V rows in flight
-      float vs[8][PER], pj[8];
+      PackedShare<PER> vs[8];
+      float pj[8];
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         const int src = m ? __ffs(m) - 1 : 0;
@@ -310,17 +270,17 @@ __device__ __forceinline__ void long_row(const Problem& p, const __nv_bfloat16* 
         pj[u] = __shfl_sync(0xffffffffu, pe, src);
         if (!m) pj[u] = 0.f;
 #pragma unroll
-        for (int t = 0; t < PER; ++t) vs[u][t] = 0.f;
-        if (m) load_bf16<PER>(vbase + (size_t)kj * p.sn, vs[u]);
+        for (int t = 0; t < PER / 2; ++t) vs[u].w[t] = 0u;
+        if (m) load_packed<PER, 32>(v + hbase + (size_t)kj * p.sn, lane, vs[u]);
         m &= m - 1;
       }
 #pragma unroll
       for (int u = 0; u < 8; ++u)
 #pragma unroll
-        for (int t = 0; t < PER; ++t) acc[t] = fmaf(pj[u], vs[u][t], acc[t]);
+        for (int t = 0; t < PER; ++t) acc[t] = fmaf(pj[u], packed_at(vs[u], t), acc[t]);
     }
   }
-  store_bf16<PER>(o + hbase + (size_t)i * p.sn + lane * PER, acc);
+  store_share<PER, 32>(o + hbase + (size_t)i * p.sn, lane, acc);
   if (lane == 0) {
     *tau_slot = tau;
     *cnt_slot = kept;
@@ -370,7 +330,7 @@ __device__ __forceinline__ void push_dense_tiles(const Problem& p, unsigned mask
 
 // The rows row_fwd_kernel listed as long (push_long_rows): one warp per row.
 template <int D, int EC>
-__global__ void __launch_bounds__(kWarpsPerCta * 32) row_fwd_long_kernel(Problem p, const __nv_bfloat16* __restrict__ v,
+__global__ void __launch_bounds__(kWarpsPerCta * 32, 4) row_fwd_long_kernel(Problem p, const __nv_bfloat16* __restrict__ v,
                                                                          const float* __restrict__ scale,
                                                                          int32_t* __restrict__ row_cnt,
                                                                          const int32_t* __restrict__ list_cnt,
@@ -483,75 +443,91 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, D == 64 ? 4 : 3) row_fwd_ke
   }
 }
 
-// Backward of one row with the whole warp: the entmax Jacobian on the support.
-template <int D>
-__device__ __noinline__ void bwd_row_full(const Problem& p, const __nv_bfloat16* __restrict__ q,
+// Backward of one row with the whole warp, for rows with at most 32 S list entries: entry e on lane e mod 32, the row's
+// elements split over the 32 lanes.  Bound by the latency of the gathers: four V rows, then four K rows are in flight
+// (packed), and four sums share one butterfly.  Float rows and a reduction each -> now: 2 x 12 x 3001 x 64 73 -> 60 us,
+// 8 x 65536 x 64 (retrieval) 182 -> 137, 16 x 32768 x 128 36 -> 27.  Eight rows in flight need more registers, and with
+// three CTAs on an SM instead of four lose more than they gain: 82 and 215 us.
+template <int D, int S>
+__device__ __forceinline__ void bwd_row_wide(const Problem& p, const __nv_bfloat16* __restrict__ q,
                                              const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v,
                                              const __nv_bfloat16* __restrict__ d_o, const float* __restrict__ scale,
                                              const float* __restrict__ tau_in, const Entry* __restrict__ entries,
                                              __nv_bfloat16* __restrict__ dq, float* __restrict__ acc_dk,
-                                             float* __restrict__ acc_dv, float* __restrict__ dc_rows, int grow, int n_list, bool saved, int pitch, int lane) {
-  constexpr int PER = D / 32;
+                                             float* __restrict__ acc_dv, float* __restrict__ dc_rows, int grow, int n,
+                                             bool saved, int pitch, int lane) {
+  constexpr int PL = D / 32;                       // elements of a row per lane
+  constexpr int kBatch = 4;
   const int bh = grow / p.N, i = grow - bh * p.N, b = bh / p.H, h = bh - b * p.H;
   const float g = scale[(size_t)b * p.scale_sb + (size_t)h * p.N + i] * p.sm_scale;
   const float a = (p.alpha - 1.0f) * g;
   const float tau = tau_in[grow];
-  const size_t hbase = (size_t)b * p.sb + (size_t)h * p.sh + lane * PER;
-  float qs[PER], gs[PER];
-  load_bf16<PER>(q + hbase + (size_t)i * p.sn, qs);
-  load_bf16<PER>(d_o + hbase + (size_t)i * p.sn, gs);
+  const size_t hbase = (size_t)b * p.sb + (size_t)h * p.sh;
+  PackedShare<PL> qs, gs;
+  load_packed<PL, 32>(q + hbase + (size_t)i * p.sn, lane, qs);
+  load_packed<PL, 32>(d_o + hbase + (size_t)i * p.sn, lane, gs);
   const Entry* list = entries + (size_t)grow * pitch;
-  float yv[kSlots], dpv[kSlots], zz[kSlots];
-  int jj[kSlots];
+  float yv[S], zz[S], dpv[S];
+  int jj[S];
+  unsigned in[S];
 #pragma unroll
-  for (int s = 0; s < kSlots; ++s) {
-    const int e = lane + 32 * s;  
+  for (int s = 0; s < S; ++s) {
     yv[s] = -1.0f;
-    jj[s] = 0;
-    dpv[s] = 0.f;
     zz[s] = 0.f;
-    if (e < n_list) {
-      const Entry en = list[e];
+    dpv[s] = 0.f;
+    jj[s] = 0;
+    if (lane + 32 * s < n) {
+      const Entry en = list[lane + 32 * s];
       // a list saved by the forward pass holds y = (alpha-1) s in Eq. 1's units, a fresh one raw <q_i, k_j>
       yv[s] = saved ? en.y - tau : fmaf(a, en.y, -tau);
       jj[s] = en.j;
       zz[s] = saved ? en.y / a : en.y;               // raw <q_i, k_j>
     }
+    in[s] = __ballot_sync(0xffffffffu, yv[s] > 0.f);
   }
+  auto load_batch = [&](const __nv_bfloat16* rows, int j, unsigned rest, int t0, PackedShare<PL> (&x)[kBatch]) {
+#pragma unroll
+    for (int z = 0; z < kBatch; ++z) {
+      const int kj = __shfl_sync(0xffffffffu, j, t0 + z);
+#pragma unroll
+      for (int w = 0; w < PL / 2; ++w) x[z].w[w] = 0u;
+      if ((rest >> z) & 1u) load_packed<PL, 32>(rows + hbase + (size_t)kj * p.sn, lane, x[z]);
+    }
+  };
   // dP_ij = <dO_i, v_j> on the support
 #pragma unroll
-  for (int s = 0; s < kSlots; ++s) {
-    unsigned rest = __ballot_sync(0xffffffffu, yv[s] > 0.f);
-    while (rest) {
-      // four V rows in flight
-      float vs[4][PER], dp[4];
-      int src[4];
+  for (int s = 0; s < S; ++s) {
+#pragma unroll 1
+    for (int t0 = 0; t0 < 32; t0 += kBatch) {
+      const unsigned rest = in[s] >> t0;
+      if (rest == 0u) break;
+      PackedShare<PL> vs[kBatch];
+      load_batch(v, jj[s], rest, t0, vs);
+      float dp[kBatch];
 #pragma unroll
-      for (int z = 0; z < 4; ++z) {
-        src[z] = rest ? __ffs(rest) - 1 : -1;
-        const int kj = __shfl_sync(0xffffffffu, jj[s], src[z] < 0 ? 0 : src[z]);
-#pragma unroll
-        for (int t = 0; t < PER; ++t) vs[z][t] = 0.f;
-        if (rest) load_bf16<PER>(v + hbase + (size_t)kj * p.sn, vs[z]);
-        rest &= rest - 1;
-      }
-#pragma unroll
-      for (int z = 0; z < 4; ++z) {
+      for (int z = 0; z < kBatch; ++z) {
         dp[z] = 0.f;
 #pragma unroll
-        for (int t = 0; t < PER; ++t) dp[z] = fmaf(gs[t], vs[z][t], dp[z]);
+        for (int e = 0; e < PL; ++e) dp[z] = fmaf(packed_at(gs, e), packed_at(vs[z], e), dp[z]);
       }
+      // the batch's sums over the warp in one butterfly: lane l ends up with the one of slot t0 + l mod kBatch
 #pragma unroll
-      for (int z = 0; z < 4; ++z) {
-        dp[z] = warp_sum(dp[z]);
-        if (lane == src[z]) dpv[s] = dp[z];
+      for (int o = 1; o < kBatch; o <<= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int z = 0; z < kBatch; z += 2 * o)
+          dp[z] = (up ? dp[z + o] : dp[z]) + __shfl_xor_sync(0xffffffffu, up ? dp[z] : dp[z + o], o);
       }
+      float r = dp[0];
+#pragma unroll
+      for (int o = kBatch; o < 32; o <<= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+      if ((lane & ~(kBatch - 1)) == t0) dpv[s] = r;
     }
   }
-  float pe[kSlots], u[kSlots];
+  float pe[S], u[S];
   float su = 0.f, sud = 0.f;
 #pragma unroll
-  for (int s = 0; s < kSlots; ++s) {
+  for (int s = 0; s < S; ++s) {
     pe[s] = 0.f;
     u[s] = 0.f;
     if (yv[s] > 0.f) pow_pair(yv[s], p.expo_class, p.expo, pe[s], u[s]);
@@ -565,151 +541,40 @@ __device__ __noinline__ void bwd_row_full(const Problem& p, const __nv_bfloat16*
     // dL/dc_i = sum_j dS_ij z_ij with z_ij = <q_i,k_j> sm_scale (chain rule through s = c z)
     float dc = 0.f;
 #pragma unroll
-    for (int s = 0; s < kSlots; ++s) dc = fmaf(u[s] * (dpv[s] - rho), zz[s], dc);
+    for (int s = 0; s < S; ++s) dc = fmaf(u[s] * (dpv[s] - rho), zz[s], dc);
     dc = warp_sum(dc);
-    if (lane == 0) dc_rows[grow] = dc * p.sm_scale;
-  }
-  float acc[PER];
-#pragma unroll
-  for (int t = 0; t < PER; ++t) acc[t] = 0.f;
-  const size_t arow = (size_t)bh * p.N;
-#pragma unroll
-  for (int s = 0; s < kSlots; ++s) {
-    const float gds_own = g * u[s] * (dpv[s] - rho);
-    unsigned rest = __ballot_sync(0xffffffffu, yv[s] > 0.f);
-    while (rest) {
-      float ks[4][PER];
-      unsigned r4 = rest;
-#pragma unroll
-      for (int z = 0; z < 4; ++z) {
-        const int kj = __shfl_sync(0xffffffffu, jj[s], r4 ? __ffs(r4) - 1 : 0);
-#pragma unroll
-        for (int t = 0; t < PER; ++t) ks[z][t] = 0.f;
-        if (r4) load_bf16<PER>(k + hbase + (size_t)kj * p.sn, ks[z]);
-        r4 &= r4 - 1;
-      }
-#pragma unroll
-      for (int z = 0; z < 4; ++z) {
-        if (rest) {
-          const int src = __ffs(rest) - 1;
-          rest &= rest - 1;
-          const int kj = __shfl_sync(0xffffffffu, jj[s], src);
-          const float gds = __shfl_sync(0xffffffffu, gds_own, src);
-          const float pj = __shfl_sync(0xffffffffu, pe[s], src);
-          float x[PER];
-#pragma unroll
-          for (int t = 0; t < PER; ++t) {
-            acc[t] = fmaf(gds, ks[z][t], acc[t]);
-            x[t] = gds * qs[t];
-          }
-          atomic_add_slice<PER>(acc_dk + (arow + kj) * D + lane * PER, x);
-#pragma unroll
-          for (int t = 0; t < PER; ++t) x[t] = pj * gs[t];
-          atomic_add_slice<PER>(acc_dv + (arow + kj) * D + lane * PER, x);
-        }
-      }
-    }
-  }
-  store_bf16<PER>(dq + hbase + (size_t)i * p.sn, acc);
-}
-
-// Backward of a row with 17 to 32 list entries: one lane per entry, the row's elements split over the whole warp.
-template <int D>
-__device__ __forceinline__ void bwd_row_warp(const Problem& p, const __nv_bfloat16* __restrict__ q,
-                                             const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v,
-                                             const __nv_bfloat16* __restrict__ d_o, const float* __restrict__ scale,
-                                             const float* __restrict__ tau_in, const Entry* __restrict__ entries,
-                                             __nv_bfloat16* __restrict__ dq, float* __restrict__ acc_dk,
-                                             float* __restrict__ acc_dv, float* __restrict__ dc_rows, int grow, int n,
-                                             bool saved, int pitch, int lane) {
-  constexpr int PL = D / 32;                       // elements of a row per lane
-  const int bh = grow / p.N, i = grow - bh * p.N, b = bh / p.H, h = bh - b * p.H;
-  const float g = scale[(size_t)b * p.scale_sb + (size_t)h * p.N + i] * p.sm_scale;
-  const float a = (p.alpha - 1.0f) * g;
-  const float tau = tau_in[grow];
-  const size_t hbase = (size_t)b * p.sb + (size_t)h * p.sh;
-  float qs[PL], gs[PL];
-  load_share<PL, 32>(q + hbase + (size_t)i * p.sn, lane, qs);
-  load_share<PL, 32>(d_o + hbase + (size_t)i * p.sn, lane, gs);
-  const Entry* list = entries + (size_t)grow * pitch;
-  float yv = -1.0f, zz = 0.f;
-  int j = 0;
-  if (lane < n) {
-    const Entry en = list[lane];
-    // a list saved by the forward pass holds y = (alpha-1) s in Eq. 1's units, a fresh one raw <q_i, k_j>
-    yv = saved ? en.y - tau : fmaf(a, en.y, -tau);
-    j = en.j;
-    zz = saved ? en.y / a : en.y;                  // raw <q_i, k_j>
-  }
-  const bool in = yv > 0.f;
-  const unsigned m = __ballot_sync(0xffffffffu, in);
-  // dP_ij = <dO_i, v_j> on the support, four V (and below, K) rows in flight: the loads are a chain of L2 round trips
-  // otherwise (long-row kernel 113 -> 77 us on 2 x 12 x 3001 x 64)
-  float dpv = 0.f;
-#pragma unroll 1
-  for (int t0 = 0; t0 < 32; t0 += 4) {
-    if ((m >> t0) == 0u) break;
-    float vs[4][PL], dp[4];
-#pragma unroll
-    for (int z = 0; z < 4; ++z) {
-      const int kj = __shfl_sync(0xffffffffu, j, t0 + z);
-#pragma unroll
-      for (int w = 0; w < PL; ++w) vs[z][w] = 0.f;
-      if ((m >> (t0 + z)) & 1u) load_share<PL, 32>(v + hbase + (size_t)kj * p.sn, lane, vs[z]);
-    }
-#pragma unroll
-    for (int z = 0; z < 4; ++z) {
-      dp[z] = 0.f;
-#pragma unroll
-      for (int w = 0; w < PL; ++w) dp[z] = fmaf(gs[w], vs[z][w], dp[z]);
-    }
-#pragma unroll
-    for (int z = 0; z < 4; ++z) {
-      dp[z] = warp_sum(dp[z]);
-      if (lane == t0 + z) dpv = dp[z];
-    }
-  }
-  float pe = 0.f, u = 0.f;
-  if (in) pow_pair(yv, p.expo_class, p.expo, pe, u);
-  const float su = warp_sum(u), sud = warp_sum(u * dpv);
-  const float rho = su > 0.f ? sud / su : 0.f;
-  const float gds_own = g * u * (dpv - rho);
-  if (dc_rows) {
-    // dL/dc_i = sum_j dS_ij z_ij with z_ij = <q_i,k_j> sm_scale (chain rule through s = c z)
-    const float dc = warp_sum(u * (dpv - rho) * zz);
     if (lane == 0) dc_rows[grow] = dc * p.sm_scale;
   }
   float acc[PL];
 #pragma unroll
   for (int t = 0; t < PL; ++t) acc[t] = 0.f;
   const size_t arow = (size_t)bh * p.N;
+#pragma unroll
+  for (int s = 0; s < S; ++s) {
+    const float gds_own = g * u[s] * (dpv[s] - rho);
 #pragma unroll 1
-  for (int t0 = 0; t0 < 32; t0 += 4) {
-    if ((m >> t0) == 0u) break;
-    float ks[4][PL];
+    for (int t0 = 0; t0 < 32; t0 += kBatch) {
+      const unsigned rest = in[s] >> t0;
+      if (rest == 0u) break;
+      PackedShare<PL> ks[kBatch];
+      load_batch(k, jj[s], rest, t0, ks);
 #pragma unroll
-    for (int z = 0; z < 4; ++z) {
-      const int kj = __shfl_sync(0xffffffffu, j, t0 + z);
+      for (int z = 0; z < kBatch; ++z) {
+        const int kj = __shfl_sync(0xffffffffu, jj[s], t0 + z);
+        const float gds = __shfl_sync(0xffffffffu, gds_own, t0 + z);
+        const float pj = __shfl_sync(0xffffffffu, pe[s], t0 + z);
+        if ((rest >> z) & 1u) {
+          float x[PL];
 #pragma unroll
-      for (int w = 0; w < PL; ++w) ks[z][w] = 0.f;
-      if ((m >> (t0 + z)) & 1u) load_share<PL, 32>(k + hbase + (size_t)kj * p.sn, lane, ks[z]);
-    }
+          for (int e = 0; e < PL; ++e) {
+            acc[e] = fmaf(gds, packed_at(ks[z], e), acc[e]);
+            x[e] = gds * packed_at(qs, e);
+          }
+          add_share<PL, 32>(acc_dk + (arow + kj) * D, lane, x);
 #pragma unroll
-    for (int z = 0; z < 4; ++z) {
-      const int kj = __shfl_sync(0xffffffffu, j, t0 + z);
-      const float gds = __shfl_sync(0xffffffffu, gds_own, t0 + z);
-      const float pj = __shfl_sync(0xffffffffu, pe, t0 + z);
-      if ((m >> (t0 + z)) & 1u) {
-        float x[PL];
-#pragma unroll
-        for (int w = 0; w < PL; ++w) {
-          acc[w] = fmaf(gds, ks[z][w], acc[w]);
-          x[w] = gds * qs[w];
+          for (int e = 0; e < PL; ++e) x[e] = pj * packed_at(gs, e);
+          add_share<PL, 32>(acc_dv + (arow + kj) * D, lane, x);
         }
-        add_share<PL, 32>(acc_dk + (arow + kj) * D, lane, x);
-#pragma unroll
-        for (int w = 0; w < PL; ++w) x[w] = pj * gs[w];
-        add_share<PL, 32>(acc_dv + (arow + kj) * D, lane, x);
       }
     }
   }
@@ -903,12 +768,14 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 4) row_bwd_long_kernel(
   for (int t = blockIdx.x * kWarpsPerCta + (threadIdx.x >> 5); t < n_long; t += gridDim.x * kWarpsPerCta) {
     const int grow = fb_list[total - 1 - t];
     const int n_list = list_cnt[saved ? (size_t)grow : 2 * (size_t)grow];
-    if (n_list <= 32)
-      bwd_row_warp<D>(p, q, k, v, d_o, scale, tau_in, entries, dq, acc_dk, acc_dv, dc_rows, grow, n_list, saved != 0, pitch,
-                      lane);
-    else
-      bwd_row_full<D>(p, q, k, v, d_o, scale, tau_in, entries, dq, acc_dk, acc_dv, dc_rows, grow, n_list, saved != 0,
-                      pitch, lane);
+#define ENTMAX_ROW_BWD_WIDE(S)                                                                                              \
+  bwd_row_wide<D, S>(p, q, k, v, d_o, scale, tau_in, entries, dq, acc_dk, acc_dv, dc_rows, grow, n_list, saved != 0, pitch, \
+                     lane)
+    if (n_list <= 32) ENTMAX_ROW_BWD_WIDE(1);
+    else if (n_list <= 64) ENTMAX_ROW_BWD_WIDE(2);
+    else if (n_list <= 128) ENTMAX_ROW_BWD_WIDE(4);
+    else ENTMAX_ROW_BWD_WIDE(kSlots);
+#undef ENTMAX_ROW_BWD_WIDE
   }
 }
 
