@@ -799,10 +799,11 @@ __global__ void __launch_bounds__(256) save_supports_kernel(int rows, int slots,
   }
 }
 
-// Rows per warp.  A warp works its rows off in four to eight rounds of dependent loads, so while the grid fits the machine at
-// once its time is that of one warp: 8 rows per warp there (8 x 12 x 1024 x 64: forward 54 -> 50 us, backward 80 -> 74 us;
-// 16 x 8192 x 128 39 -> 32 and 55 -> 46).  16 rows pack best into rounds and win where the grid is several waves long; 4 lose
-// more in packing than they save (2 x 12 x 3001 x 64: 37 -> 47 and 93 -> 112 us).
+// Rows per warp (forward up to 32, backward up to 16).  A warp works its rows off in rounds of dependent loads, so while the
+// grid fits the machine at once its time is that of one warp: 8 rows per warp there (with 16: 8 x 12 x 1024 x 64 forward 50 ->
+// 54 us, backward 74 -> 80).  More rows pack better into rounds and win where the grid is several waves long; 4 lose more in
+// packing than they save (2 x 12 x 3001 x 64: 37 -> 47 and 93 -> 112 us).  (Compared before the gathers were packed, which
+// shortened both sides.)
 inline int rows_per_warp(const Problem& p, int most) {
   const long rows = (long)p.B * p.H * p.N;
   return rows >= 148L * 64 * most ? most : rows >= 148L * 64 * 16 ? 16 : 8;

@@ -8,25 +8,25 @@
 //  (2) the threshold of a subset of the row's keys never exceeds the threshold of the whole row (adding
 //      a logit never lowers tau), while keys at or below the threshold do not change it.
 // So while the keys stream by, a thread keeps a lower bound thr on the row's final tau and the list of
-// the keys it has seen with y > thr.  When a list grows past kHalfTrigger entries, Newton steps on the
+// the keys it has seen with y > thr.  When a list grows past kListTrigger, Newton steps on the
 // listed keys, started at thr, raise thr (f is convex and decreasing for e >= 1, so Newton from the left
 // of the root never passes it) and the list is filtered.  A row whose list cannot be brought down to
-// kHalfKeep entries is flagged and later recomputed by the dense-row path.  In backward mode the
+// kListKeep entries is flagged and later recomputed by the dense-row path.  In backward mode the
 // threshold is the tau of the forward pass and the lists are simply the support.
 //
-// CTA layout (576 threads, one CTA per SM, persistent; work items of 2 x 128 query rows are handed out
+// CTA layout (320 threads, one CTA per SM, persistent; work items of 2 x 128 query rows are handed out
 // longest-first through an atomic counter):
 //   warp 0        scheduler + TMA producer: the item's two Q tiles, K tiles of 256 keys through a ring
 //   warp 1        MMA issuer: per K tile one M=128 x N=256 accumulation per Q tile into its own 256
 //                 TMEM columns (2 accumulators = all 512 columns).  N = 256 keeps the operand traffic of
 //                 an MMA (A 4 KB + B 8 KB per 128 tensor-core cycles) below the shared-memory bandwidth.
-//   warps 2..17   consumers, eight warps per Q tile: TMEM lane = query row; the 256 columns of a row are
-//                 split between two threads (columns 0-127 and 128-255 of every K tile), each with its
-//                 own running maximum, threshold, list length (registers) and half-list; the two share
-//                 their running maxima through shared memory so that both thresholds stay tight.
-// A consumer first reduces its 128 columns to 16 group maxima (branch-free), and only when some lane of
-// the warp saw a value above its threshold re-reads the groups that hold candidates (four groups per
-// round trip to TMEM); it hands the accumulator back as soon as the last values it needs are in registers.  While the consumers of one Q tile scan, the tensor core works on the other.
+//   warps 2..9    consumers, four warps per Q tile, one thread per query row (TMEM lane = query row) with the row's
+//                 maximum, threshold and list length in registers (168 of them: ten warps are what allows that).
+// A consumer reads its 256 columns in one straight pass of 64-column TMEM loads: group maxima of eight columns (branch-free),
+// and a group that holds a candidate is parked as it is in one of the thread's slots in shared memory, so that the accumulator
+// is handed back after the pass; the candidates are taken out of the slots and appended to the row's list behind that.  A
+// tile in which some row runs out of slots is taken 32 columns at a time instead.  One thread per row makes a row's list
+// depend on that row alone.  While the consumers of one Q tile scan, the tensor core works on the other.
 // Every mbarrier wait is bounded: on expiry the CTA raises ENTMAX_ATTN_FLAG_WAIT_EXPIRED, all roles
 // leave their loops, the producer waits for the copies it armed barriers for and the MMA issuer for the tensor-core
 // work it issued (each with a bound of its own), TMEM is freed and the CTA returns.
@@ -157,10 +157,10 @@ __device__ __forceinline__ int first_tile(const SweepArgs& a, int k) {
   return 0;
 }
 
-// ------------------------------------------------------------- consumer side: one half-row per thread
+// ------------------------------------------------------------- consumer side: one row per thread
 struct RowState {
   float thr;       // candidates are accumulators above this (accumulator units); +inf: none any more
-  int cnt;         // half-list length; -1 = handed to the dense path
+  int cnt;         // list length; -1 = handed to the dense path
 };
 
 // Warp-cooperative list shrink for the lanes whose list has grown past kListTrigger.  Accumulator

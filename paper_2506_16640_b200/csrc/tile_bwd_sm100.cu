@@ -6,15 +6,22 @@
 //   dL/dc_i = sum_j dS_ij z_ij                      (g_i = c_i * sm_scale, c_i the ASEntmax scale)
 // Two kernels.  tile_bwd_kernel, query-major: a work item is one Q tile of 128 rows that holds at least one such
 // row; two passes over its visible K/V tiles:
-//   pass A   S = Q K^T and dP = dO V^T into TMEM; the row threads accumulate sum u and sum u dP: rho_i (kept for the
-//            second kernel);
-//   pass B   S and dP again; the row threads write g dS (bf16, and what the rounding left over) to shared memory;
-//            dQ += (g dS) K     (A = g dS K-major, B = K tile with the head dim contiguous)   kept in TMEM.
+//   pass A   S = Q K^T and dP = dO V^T into one of two TMEM stages; the row threads accumulate sum u and sum u dP: rho_i
+//            (kept for the second kernel);
+//   pass B   S and dP again; the row threads write g dS (bf16, and what the rounding left over) to TMEM;
+//            dQ += (g dS) K     (A = g dS from TMEM, B = K tile with the head dim contiguous)   kept in TMEM.
+// With g dS out of shared memory there is room for three K and two V stages.  Bound by the operand traffic of the N = 128
+// contractions (an M = N = 128 MMA reads shared memory at its full rate) and the tiles' way from L2 (64 KB per step, about
+// 5 TB/s over the chip): 16 heads x 8192 x 128, every row dense, 953 us with g dS in shared memory and one S / dP stage,
+// 808 now.
 // tile_bwd_kv_kernel, key-major: a work item is one K/V tile; over the marked Q tiles that see it, S and dP once
 // more, P and g dS to shared memory, and
 //            dK_t += (g dS)^T Q (A = the shared tile read M-major, B = Q tile, head dim contiguous)
 //            dV_t += P^T dO     (likewise), accumulated in TMEM over those Q tiles and added to the fp32 dK / dV
 //            accumulators in global memory once per K/V tile, by bulk tensor reductions from a staging tile.
+// P is handed over before dS is formed: dV runs, and dO is free again, under dS; S of the next pair runs under dS as well.
+// Bound by shared memory (four contractions of N = 128 and the P / dS stores: 3100 of 4460 cycles per pair): same case 762 us
+// with the four contractions and the element code of a pair one after the other, 568 now.
 // (One kernel that also formed dK_t and dV_t per (Q tile, K tile) pair was bound by those reductions in L2: 128 KB of
 // them per pair.)  Rows of a Q tile that are not marked contribute zeros (their P and dS rows are written as zero)
 // and their dQ is not stored: the list kernels have already handled them.
