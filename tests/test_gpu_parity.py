@@ -777,3 +777,24 @@ def test_cfg5_shape_reduced_full_backward():
     bwd = parity.run_bwd(inp, 1.5, got["tau"], got["dev"])
     parity.check_fwd_rows(inp, 1.5, got, 1, np.arange(4096))
     parity.check_bwd_head(inp, 1.5, bwd, 1)
+
+
+@pytest.mark.parametrize("alpha", [1.25, 1.5, 2.0, 1.7])
+@pytest.mark.parametrize("N,d,causal", [(33, 64, True), (65, 128, True), (129, 64, True), (255, 128, False), (257, 64, False),
+                                        (4095, 64, True), (4097, 128, True)])
+def test_candidate_lists_and_row_solves_at_their_edges(N, d, causal, alpha):
+    # flattening rows from one temperature to the next: lists (and supports) from a few entries through the sizes at which
+    # the row kernels change form (8, 16, 32, 64, 128) up to the list trigger and into the dense path, within and across
+    # K tiles of 256 keys, with and without the sampled start (from 4096 keys on); the backward pass reads the same lists
+    # (its Jacobian jumps at the threshold for alpha = 2, where too many of such flat rows have a key within rounding of it)
+    with_bwd = N < 300 and alpha < 2.0
+    for sigma in (1.0, 0.45, 0.25):
+        inp = make_inputs(_small("lists", N, d, causal, use_scale=False, sigma=sigma, backward=with_bwd, seed=N + d))
+        got = parity.run_fwd(inp, alpha)
+        rows = np.arange(N) if N < 300 else np.unique(np.r_[np.arange(0, N, 61), 0:140, N - 3 : N])
+        for bh in range(inp.workload.H):
+            parity.check_fwd_rows(inp, alpha, got, bh, rows)
+        if with_bwd:
+            bwd = parity.run_bwd(inp, alpha, got["tau"], got["dev"])
+            for bh in range(inp.workload.H):
+                parity.check_bwd_head(inp, alpha, bwd, bh)
