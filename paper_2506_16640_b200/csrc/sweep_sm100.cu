@@ -812,7 +812,8 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
             }
             if (!full) {
               ++c;
-              if (c == 1 && nch > 1 && __all_sync(0xffffffffu, n_new >= 24 || r.thr == INFINITY)) {
+              // (a dump has to see every chunk)
+              if (!kDump && c == 1 && nch > 1 && __all_sync(0xffffffffu, n_new >= 24 || r.thr == INFINITY)) {
                 // Nearly every key is a candidate (flat logits): before the other chunks are stored, look whether the tile
                 // sends the rows to the dense path anyway.  Given threshold: more candidates than a list may hold.  Search:
                 // tau <= m_run - n^(-1/e) for n listed keys (see shrink_lists), more keys above that than a list may keep.

@@ -46,6 +46,20 @@ def test_score_tiles_match_fp64_dot_products(N, d, causal):
         assert err <= 1e-4 * max(1.0, ref.abs().max().item()), err
 
 
+@pytest.mark.parametrize("sigma", [0.03, 0.3])
+@pytest.mark.parametrize("causal", [True, False])
+@pytest.mark.parametrize("N,d", [(700, 64), (1025, 128)])
+def test_score_tiles_of_rows_without_a_list(N, d, causal, sigma):
+    # flat logits: the rows' lists are given up in their first tile, their scores have to come out all the same
+    inp = make_inputs(_small("scores_flat", N, d, causal, sigma=sigma))
+    dev = parity.to_device(inp)
+    got = binding.entmax_attn_scores_debug(dev["q"], dev["k"], 1, causal).cpu().double()
+    ref = inp.q[0, 1].double() @ inp.k[0, 1].double().T
+    keep = torch.ones(N, N, dtype=torch.bool).tril() if causal else torch.ones(N, N, dtype=torch.bool)
+    assert torch.isnan(got[~keep]).all()
+    assert (got[keep] - ref[keep]).abs().max().item() <= 1e-4 * max(1.0, ref.abs().max().item())
+
+
 # ------------------------------------------------------------------ config 1: fp32, fixed temperature
 def test_cfg1_fp32_all_rows():
     inp = make_inputs(WORKLOADS[1])
