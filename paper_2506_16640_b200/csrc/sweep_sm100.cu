@@ -821,10 +821,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
                 const int n_max = r.cnt + (nch - 1) * 32;
                 const float width = a.expo_class == kExpo2 ? rsqrtf((float)n_max)
                                     : a.expo_class == kExpo1 ? 1.0f / (float)n_max : __powf((float)n_max, -1.0f / a.expo);
-                const float cut = kSearch ? fmaxf(r.thr, m_run - 0.999f * width * margin) : r.thr;
-                int n = kSearch ? 0 : r.cnt;
-#pragma unroll 1
-                for (int c2 = kSearch ? 0 : 1; c2 < nch; ++c2) {
+                auto load_visible = [&](int c2) {      // chunk c2 into va, -inf past the row's last visible key
                   tmem_ld32(taddr_row + c2 * 32, va);
                   tmem_ld_wait();
                   const int col2 = col_base + c2 * 32;
@@ -832,8 +829,26 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
 #pragma unroll
                   for (int u = 0; u < 32; ++u) {
                     const float y = kAlibi ? fmaf(slope, (float)u, va[u]) + t2 : va[u];
-                    n += (y > cut && col2 + u <= lim) ? 1 : 0;
+                    va[u] = col2 + u <= lim ? y : -INFINITY;
                   }
+                };
+                if constexpr (kSearch) {
+                  // (m_run has to be the largest of all the keys that are counted, the chunks to come included: a larger one
+                  // there makes the rest no candidates at all)
+#pragma unroll 1
+                  for (int c2 = 1; c2 < nch; ++c2) {
+                    load_visible(c2);
+                    m_run = fmaxf(m_run, fmaxf(fmaxf(max8(&va[0]), max8(&va[8])), fmaxf(max8(&va[16]), max8(&va[24]))));
+                  }
+                  r.thr = fmaxf(r.thr, m_run - margin);
+                }
+                const float cut = kSearch ? fmaxf(r.thr, m_run - 0.999f * width * margin) : r.thr;
+                int n = kSearch ? 0 : r.cnt;
+#pragma unroll 1
+                for (int c2 = kSearch ? 0 : 1; c2 < nch; ++c2) {
+                  load_visible(c2);
+#pragma unroll
+                  for (int u = 0; u < 32; ++u) n += va[u] > cut ? 1 : 0;
                 }
                 if (n > (kSearch ? kListKeep : kListTrigger)) {
                   r.thr = INFINITY;

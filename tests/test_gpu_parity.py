@@ -812,3 +812,18 @@ def test_candidate_lists_and_row_solves_at_their_edges(N, d, causal, alpha):
             bwd = parity.run_bwd(inp, alpha, got["tau"], got["dev"])
             for bh in range(inp.workload.H):
                 parity.check_bwd_head(inp, alpha, bwd, bh)
+
+
+@pytest.mark.parametrize("alpha", [1.25, 1.5, 1.7, 2.0, 3.0])
+@pytest.mark.parametrize("N,d,low,high", [(500, 64, 256, 256 + 203), (4300, 64, 4096, 4096 + 203), (4200, 128, 0, 251)])
+def test_flat_rows_with_one_large_key_late_in_a_tile_keep_their_lists(N, d, low, high, alpha):
+    # 50 flat keys, faint ones up to key `low`, flat again behind it: the tile that starts there looks as if it sent every row
+    # to the dense path, until its key `high` (in a late chunk, never among the sampled keys) leaves nothing else
+    inp = make_inputs(_small("flat_late_key", N, d, False, use_scale=False, sigma=0.01, seed=61))
+    inp.q += 1.0
+    inp.k[:, :, 50:low] = -3.0
+    inp.k[:, :, high] = 3.0
+    got = parity.run_fwd(inp, alpha)
+    assert int(got["status"][binding.STATUS_DENSE_ROWS]) == 0
+    for idx, _ in binding.read_support(got["params"], got["workspace"], range(0, 2 * N, 7)):
+        assert idx.tolist() == [high]
