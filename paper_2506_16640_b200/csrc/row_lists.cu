@@ -160,11 +160,12 @@ __device__ __forceinline__ int solve_row(const Problem& p, Entry* list, int n, f
   return cnt;
 }
 
-// O_i of 32 / W rows at once, W lanes per row, from the supports solve_row left (cnt <= W entries; cnt = 0: no row).
+// O_i of 32 / W rows at once, W lanes per row, from the supports solve_row left (cnt <= W entries; a row without any, whose
+// y_max - 1 rounds to y_max, gets zeros; not active: no row, cnt = 0).
 template <int D, int W, int EC>
 __device__ __forceinline__ void gather_rows(const Problem& p, const __nv_bfloat16* __restrict__ v,
-                                            const Entry* __restrict__ entries, __nv_bfloat16* __restrict__ o, int grow, int cnt,
-                                            float tau, int lane) {
+                                            const Entry* __restrict__ entries, __nv_bfloat16* __restrict__ o, int grow,
+                                            bool active, int cnt, float tau, int lane) {
   constexpr int PL = D / W;                        // elements of a V / O row per lane
   constexpr int kBatch = 4;                        // V rows in flight
   const int sl = lane & (W - 1);
@@ -200,7 +201,7 @@ __device__ __forceinline__ void gather_rows(const Problem& p, const __nv_bfloat1
 #pragma unroll
       for (int e = 0; e < PL; ++e) acc[e] = fmaf(pj[u], packed_at(vs[u], e), acc[e]);
   }
-  if (cnt > 0) store_share<PL, W>(o + hbase + (size_t)i * p.sn, sl, acc);
+  if (active) store_share<PL, W>(o + hbase + (size_t)i * p.sn, sl, acc);
 }
 
 // One row with the whole warp, up to 32 S list entries: threshold, support, output.
@@ -412,7 +413,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, D == 64 ? 4 : 3) row_fwd_ke
       row_cnt[my_row] = cnt;
     }
     __syncwarp();   // the supports are ordered before the other lanes' loads
-    unsigned m8 = __ballot_sync(0xffffffffu, cnt > 0 && cnt <= 8);
+    unsigned m8 = __ballot_sync(0xffffffffu, n > 0 && cnt <= 8);
     unsigned m16 = __ballot_sync(0xffffffffu, cnt > 8 && cnt <= 16);
     unsigned m32 = __ballot_sync(0xffffffffu, cnt > 16);
     while (m8) {
@@ -420,7 +421,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, D == 64 ? 4 : 3) row_fwd_ke
       const bool active = src < 32u;
       const int c = __shfl_sync(0xffffffffu, cnt, active ? src : 0);
       const float t = __shfl_sync(0xffffffffu, tau, active ? src : 0);
-      gather_rows<D, 8, EC>(p, v, entries, o, active ? rpw * blk + (int)src : 0, active ? c : 0, t, lane);
+      gather_rows<D, 8, EC>(p, v, entries, o, active ? rpw * blk + (int)src : 0, active, active ? c : 0, t, lane);
 #pragma unroll
       for (int z = 0; z < 4; ++z) m8 &= m8 - 1;
     }
@@ -429,7 +430,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, D == 64 ? 4 : 3) row_fwd_ke
       const bool active = src < 32u;
       const int c = __shfl_sync(0xffffffffu, cnt, active ? src : 0);
       const float t = __shfl_sync(0xffffffffu, tau, active ? src : 0);
-      gather_rows<D, 16, EC>(p, v, entries, o, active ? rpw * blk + (int)src : 0, active ? c : 0, t, lane);
+      gather_rows<D, 16, EC>(p, v, entries, o, active ? rpw * blk + (int)src : 0, active, active ? c : 0, t, lane);
       m16 &= m16 - 1;
       m16 &= m16 - 1;
     }
@@ -438,7 +439,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, D == 64 ? 4 : 3) row_fwd_ke
       m32 &= m32 - 1;
       const int c = __shfl_sync(0xffffffffu, cnt, src);
       const float t = __shfl_sync(0xffffffffu, tau, src);
-      gather_rows<D, 32, EC>(p, v, entries, o, rpw * blk + src, c, t, lane);
+      gather_rows<D, 32, EC>(p, v, entries, o, rpw * blk + src, true, c, t, lane);
     }
   }
 }

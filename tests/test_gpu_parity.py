@@ -827,3 +827,18 @@ def test_flat_rows_with_one_large_key_late_in_a_tile_keep_their_lists(N, d, low,
     assert int(got["status"][binding.STATUS_DENSE_ROWS]) == 0
     for idx, _ in binding.read_support(got["params"], got["workspace"], range(0, 2 * N, 7)):
         assert idx.tolist() == [high]
+
+
+def test_row_whose_threshold_rounds_to_its_largest_logit_is_written():
+    # y_max = 2^24 + 4: y_max - 1 rounds to y_max in float32 (to even), while in accumulator units (1.5 * 2^26, margin 6) the
+    # sweep still keeps the key -- a list whose support comes out empty.  O has to be written (as zeros) all the same
+    sm_scale = 0.33333340287208557
+    q = torch.full((1, 1, 5, 64), 1536.0, dtype=torch.bfloat16, device="cuda")
+    k = torch.zeros_like(q)
+    k[:, :, 0] = 1024.0
+    o = torch.full_like(q, float("nan"))
+    params = binding.make_params(q, 1.5, True, sm_scale)
+    ws = binding.alloc_workspace(params, False, q.device)
+    binding.entmax_attn_fwd(q, k, torch.ones_like(q), 1.5, True, sm_scale=sm_scale, o=o, workspace=ws)
+    assert [len(idx) for idx, _ in binding.read_support(params, ws, range(5))] == [0] * 5
+    assert (o == 0).all()
