@@ -252,6 +252,12 @@ def entmax_attn_decode_fwd(q, k, v, alpha, kv_len=None, beta=None, gamma=None, d
     return o, tau, support_size
 
 
+def _param_grads(H: int, device):
+    # three tensors, not views of one: the caller may change, free or save each by itself
+    f32 = torch.float32
+    return torch.empty(H, dtype=f32, device=device), torch.empty(H, dtype=f32, device=device), torch.empty(H, dtype=f32, device=device)
+
+
 def entmax_attn_bwd(q, k, v, tau, d_o, alpha, causal, beta=None, gamma=None, delta=None, *, sm_scale=0.0, n_mode=0,
                     dq=None, dk=None, dv=None, workspace=None, status=None, stream=None):
     """Backward pass.  Returns (dq, dk, dv)."""
@@ -286,7 +292,7 @@ def entmax_attn_bwd_scale(q, k, v, tau, d_o, alpha, causal, beta, gamma, delta, 
         d_scale_rows = torch.empty((B, H, N), dtype=torch.float32, device=q.device)
     grads = None
     if want_param_grads:
-        grads = torch.empty((3, H), dtype=torch.float32, device=q.device).unbind(0)
+        grads = _param_grads(H, q.device)
     if workspace is None:
         workspace = alloc_workspace(params, True, q.device)
     g = grads if grads is not None else (None, None, None)
@@ -384,7 +390,7 @@ def entmax_attn_bwd_ex(q, k, v, tau, d_o, alpha, causal, beta=None, gamma=None, 
     dk = torch.empty_like(q) if dk is None else dk
     dv = torch.empty_like(q) if dv is None else dv
     dc = torch.empty((B, H, N), dtype=torch.float32, device=q.device) if want_scale_rows else None
-    grads = torch.empty((3, H), dtype=torch.float32, device=q.device).unbind(0) if want_param_grads else None
+    grads = _param_grads(H, q.device) if want_param_grads else None
     g = grads if grads is not None else (None, None, None)
     if workspace is None:
         workspace = alloc_workspace(params, True, q.device)

@@ -6,6 +6,7 @@ import torch
 
 import oracle as oracle_mod
 import parity
+from paper_2506_16640_b200 import binding
 from paper_2506_16640_b200.autograd import entmax_attention
 from paper_2506_16640_b200.inputs import Workload, make_inputs
 
@@ -62,3 +63,16 @@ def test_gradient_of_a_per_query_scale_table():
         qh, kh, vh, gh = (t[0, h].float().numpy() for t in (inp.q, inp.k, inp.v, inp.d_o))
         dc_ref, _ = oracle_mod.attn_bwd_scale_head(qh, kh, vh, gh, 1.5, inp.sm_scale, True, scale=inp.head_scale(h))
         parity.grad_close("dc rows", c_rows.grad[0, h].cpu().numpy(), dc_ref)
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_parameter_gradients_are_tensors_of_their_own(dtype):
+    # no views of one another: storages and version counters are theirs, in-place changes under autograd are allowed
+    q, k, v = (torch.randn((1, 2, 65, 64), device="cuda").to(dtype) for _ in range(3))
+    scale = [torch.ones(2, device="cuda", requires_grad=True) for _ in range(3)]
+    o, tau = entmax_attention(q, k, v, *scale, return_tau=True)
+    d_o = torch.randn_like(o)
+    direct = binding.entmax_attn_bwd_scale(q, k, v, tau, d_o, 1.5, True, *scale)[4]
+    for g in torch.autograd.grad(o, scale, d_o) + tuple(direct):
+        assert g._base is None and g.untyped_storage().nbytes() == 2 * 4
+        g += scale[0]
