@@ -196,10 +196,10 @@ __global__ void __launch_bounds__(kScaleGradThreads) scale_grad_kernel(Problem p
   pdl_begin();
   __shared__ double red[kScaleGradThreads / 32];
   __shared__ int last;
-  const int h = blockIdx.y;
+  const int h = blockIdx.x;                        // (heads along x: the other dimensions of a grid end at 65535)
   const double b = beta[h], g = gamma[h];
   double sb = 0.0, sg = 0.0, sd = 0.0;
-  for (int i = blockIdx.x * kScaleGradThreads + threadIdx.x; i < p.N; i += gridDim.x * kScaleGradThreads) {
+  for (int i = blockIdx.y * kScaleGradThreads + threadIdx.x; i < p.N; i += gridDim.y * kScaleGradThreads) {
     double dc = 0.0;
     for (int bb = 0; bb < p.B; ++bb) dc += dc_rows[((size_t)bb * p.H + h) * p.N + i];
     const int n = (p.n_mode || !p.causal) ? p.N : i + 1;
@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(kScaleGradThreads) scale_grad_kernel(Problem p
   sg = block_sum_fp64(sg, red);
   sd = block_sum_fp64(sd, red);
   if (threadIdx.x == 0) {
-    double* mine = partial + 3 * ((size_t)h * gridDim.x + blockIdx.x);
+    double* mine = partial + 3 * ((size_t)h * gridDim.y + blockIdx.y);
     mine[0] = sb;
     mine[1] = sg;
     mine[2] = sd;
@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(kScaleGradThreads) scale_grad_kernel(Problem p
   for (int t = threadIdx.x; t < 3 * p.H; t += kScaleGradThreads) {
     const int hh = t / 3, which = t - 3 * hh;
     double sum = 0.0;
-    for (unsigned c = 0; c < gridDim.x; ++c) sum += __ldcg(partial + 3 * ((size_t)hh * gridDim.x + c) + which);
+    for (unsigned c = 0; c < gridDim.y; ++c) sum += __ldcg(partial + 3 * ((size_t)hh * gridDim.y + c) + which);
     (which == 0 ? dbeta : which == 1 ? dgamma : ddelta)[hh] = (float)sum;
   }
 }
@@ -247,21 +247,22 @@ __global__ void __launch_bounds__(256) prologue_kernel(Problem p, const float* _
   if (blockIdx.y == 0)
     for (int t = i; t < n_clear; t += gridDim.x * blockDim.x) clear[t] = 0;
   if (!scale || i >= p.N) return;
-  const int h0 = blockIdx.y * kScaleHeads;
   const int n = (p.n_mode || !p.causal) ? p.N : i + 1;
   const double lnL = p.has_scale && n > 1 ? log(log((double)n)) : 0.0;
+  for (int h0 = blockIdx.y * kScaleHeads; h0 < p.H; h0 += gridDim.y * kScaleHeads) {
 #pragma unroll
-  for (int t = 0; t < kScaleHeads; ++t) {
-    const int h = h0 + t;
-    if (h >= p.H) break;
-    float c = 1.0f;
-    if (p.has_scale) {
-      double cd = (double)delta[h];
-      if (n > 1) cd += (double)beta[h] * exp((double)gamma[h] * lnL);
-      c = (float)cd;
-      if (!isfinite(c) && status) atomicOr(status + ENTMAX_ATTN_STATUS_FLAGS, ENTMAX_ATTN_FLAG_BAD_SCALE);
+    for (int t = 0; t < kScaleHeads; ++t) {
+      const int h = h0 + t;
+      if (h >= p.H) break;
+      float c = 1.0f;
+      if (p.has_scale) {
+        double cd = (double)delta[h];
+        if (n > 1) cd += (double)beta[h] * exp((double)gamma[h] * lnL);
+        c = (float)cd;
+        if (!isfinite(c) && status) atomicOr(status + ENTMAX_ATTN_STATUS_FLAGS, ENTMAX_ATTN_FLAG_BAD_SCALE);
+      }
+      scale[(size_t)h * p.N + i] = c;
     }
-    scale[(size_t)h * p.N + i] = c;
   }
 }
 
@@ -305,7 +306,8 @@ __global__ void __launch_bounds__(256) store_grad_kernel(Problem p, const float*
 cudaError_t launch_prologue(const Problem& p, const float* beta, const float* gamma, const float* delta, float* scale,
                             int32_t* clear, size_t n_clear, int32_t* status, cudaStream_t stream) {
   const int most = scale ? p.N : (int)(n_clear < 256 * 148 ? n_clear : 256 * 148);
-  const dim3 grid((most + 255) / 256, scale ? (p.H + kScaleHeads - 1) / kScaleHeads : 1);
+  const int groups = scale ? (p.H + kScaleHeads - 1) / kScaleHeads : 1;
+  const dim3 grid((most + 255) / 256, groups < 65535 ? groups : 65535);
   launch_kernel(prologue_kernel, grid, 256, 0, stream, p, beta, gamma, delta, scale, clear, (int)n_clear, status);
   return cudaGetLastError();
 }
@@ -331,7 +333,7 @@ cudaError_t launch_scale_grad(const Problem& p, const float* beta, const float* 
   int ctas = (148 * 4 + p.H - 1) / p.H;
   const int most = (p.N + kScaleGradThreads - 1) / kScaleGradThreads;
   if (ctas > most) ctas = most;
-  launch_kernel(scale_grad_kernel, dim3(ctas, p.H), kScaleGradThreads, 0, stream, p, beta, gamma, dc_rows, partial, counter, dbeta,
+  launch_kernel(scale_grad_kernel, dim3(p.H, ctas), kScaleGradThreads, 0, stream, p, beta, gamma, dc_rows, partial, counter, dbeta,
                                                                        dgamma, ddelta);
   return cudaGetLastError();
 }

@@ -842,3 +842,26 @@ def test_row_whose_threshold_rounds_to_its_largest_logit_is_written():
     binding.entmax_attn_fwd(q, k, torch.ones_like(q), 1.5, True, sm_scale=sm_scale, o=o, workspace=ws)
     assert [len(idx) for idx, _ in binding.read_support(params, ws, range(5))] == [0] * 5
     assert (o == 0).all()
+
+
+@pytest.mark.parametrize("dtype,H", [(torch.bfloat16, 65536 + 37), (torch.float32, 65536 + 37), (torch.bfloat16, 4 * 65535 + 5)])
+def test_more_heads_than_a_grid_dimension_holds(dtype, H):
+    # (sequences folded into the heads): scale table and scale gradients against their formulas, head by head
+    N, gen = 5, torch.Generator(device="cuda").manual_seed(3)
+    q, k, v, d_o = (torch.randn((1, H, N, 64), device="cuda", generator=gen).to(dtype) for _ in range(4))
+    beta, gamma, delta = (torch.rand(H, device="cuda", generator=gen) + 0.5 for _ in range(3))
+    params = binding.make_params(q, 1.5, True)
+    ws = binding.alloc_workspace(params, False, q.device)
+    o, tau = binding.entmax_attn_fwd(q, k, v, 1.5, True, beta, gamma, delta, workspace=ws)
+    at = binding.entmax_attn_workspace_layout(params).scale_offset
+    L = torch.log(torch.arange(1, N + 1, device="cuda", dtype=torch.float64))
+    power = torch.where(L > 0, L.clamp_min(1e-300) ** gamma.double()[:, None], 0.0)             # [H, N]
+    c = ws[at: at + 4 * H * N].view(torch.float32).view(H, N)
+    ref = delta.double()[:, None] + beta.double()[:, None] * power
+    assert (c - ref).abs().max().item() <= 2.0 ** -23 * ref.abs().max().item()                # one rounding
+    *_, dc, grads = binding.entmax_attn_bwd_scale(q, k, v, tau, d_o, 1.5, True, beta, gamma, delta)
+    dc = dc[0].double()
+    lnL = torch.where(L > 0, torch.log(L.clamp_min(1e-300)), 0.0)
+    for got, want in zip(grads, (dc * power, dc * power * beta.double()[:, None] * lnL, dc)):
+        want = want.sum(dim=1)
+        assert (got - want).abs().max().item() <= 1e-6 * want.abs().max().item()              # fp64 sums, one rounding
