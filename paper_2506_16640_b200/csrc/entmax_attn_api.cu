@@ -341,12 +341,18 @@ int bwd_impl(const entmax_attn_params* params, const void* q, const void* k, con
   int32_t* fb_count = reinterpret_cast<int32_t*>(ws + lay.fb_count);
   int32_t* fb_list = reinterpret_cast<int32_t*>(ws + lay.fb_list);
   float* scratch = reinterpret_cast<float*>(ws + lay.scratch);
-  // contiguous float32 outputs are their own accumulators
-  const bool in_place = p.dtype == ENTMAX_ATTN_DTYPE_FP32 && p.sn == p.D && p.sh == (int64_t)p.N * p.D &&
-                        p.sb == (int64_t)p.H * p.N * p.D;
+  const size_t acc_bytes = (size_t)p.B * p.H * p.N * p.D * sizeof(float);
+  // Contiguous float32 outputs are their own accumulators, unless a caller writes a gradient over a tensor this call reads or
+  // over another gradient: accumulators are cleared first and added to until the end.
+  auto apart = [acc_bytes](const void* x, const void* y) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(x), b = reinterpret_cast<uintptr_t>(y);
+    return a + acc_bytes <= b || b + acc_bytes <= a;
+  };
+  bool in_place = p.dtype == ENTMAX_ATTN_DTYPE_FP32 && p.sn == p.D && p.sh == (int64_t)p.N * p.D &&
+                  p.sb == (int64_t)p.H * p.N * p.D && apart(dk, dv);
+  for (const void* t : {q, k, v, d_o, static_cast<const void*>(dq)}) in_place = in_place && apart(dk, t) && apart(dv, t);
   float* acc_dk = in_place ? static_cast<float*>(dk) : reinterpret_cast<float*>(ws + lay.acc_dk);
   float* acc_dv = in_place ? static_cast<float*>(dv) : reinterpret_cast<float*>(ws + lay.acc_dv);
-  const size_t acc_bytes = (size_t)p.B * p.H * p.N * p.D * sizeof(float);
   // per-row scale gradients: into the caller's array, else (when only the parameter gradients are wanted)
   // into the workspace, else not computed
   float* dc_rows = d_scale_rows ? d_scale_rows : (n_param_grads ? reinterpret_cast<float*>(ws + lay.dc_rows) : nullptr);

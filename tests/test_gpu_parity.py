@@ -865,3 +865,15 @@ def test_more_heads_than_a_grid_dimension_holds(dtype, H):
     for got, want in zip(grads, (dc * power, dc * power * beta.double()[:, None] * lnL, dc)):
         want = want.sum(dim=1)
         assert (got - want).abs().max().item() <= 1e-6 * want.abs().max().item()              # fp64 sums, one rounding
+
+
+@pytest.mark.parametrize("N,d", [(130, 64), (777, 128)])
+@pytest.mark.parametrize("dk,dv", [("k", "v"), ("v", "k"), ("q", "d_o"), ("d_o", "q")])
+def test_fp32_gradients_written_over_the_inputs(N, d, dk, dv):
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    t = {n: torch.randn((1, 2, N, d), device="cuda", generator=gen) for n in ("q", "k", "v", "d_o")}
+    _, tau = binding.entmax_attn_fwd(t["q"], t["k"], t["v"], 1.5, True)
+    ref = binding.entmax_attn_bwd(t["q"], t["k"], t["v"], tau, t["d_o"], 1.5, True)
+    got = binding.entmax_attn_bwd(t["q"], t["k"], t["v"], tau, t["d_o"], 1.5, True, dk=t[dk], dv=t[dv])
+    for a, b in zip(got, ref):
+        assert (a - b).abs().max().item() <= 1e-5 * b.abs().max().item()      # sums in another order
