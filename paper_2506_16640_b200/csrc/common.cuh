@@ -49,7 +49,7 @@ struct Problem {
 
 struct WsLayout {
   size_t scale, row_cnt, list_cnt, list_thr, entries, fb_count, sweep_counter, tile_count, grad_counter, tile_flag, tile_list, tile_mask, fb_list, alibi_blob, alibi_kmax, scratch, acc_dk, acc_dv, dc_rows, total;
-  int scratch_ctas;     // CTAs of the float32 kernels (each owns sixteen score rows of the scratch)
+  int scratch_ctas;     // CTAs of the float32 kernels (each owns fp32_scratch_rows() score rows of the scratch)
 };
 
 WsLayout make_layout(const Problem& p, bool is_bwd);
@@ -217,9 +217,10 @@ cudaError_t launch_prologue(const Problem& p, const float* beta, const float* ga
 // dense-row forward on CUDA cores, one score row of scratch per CTA
 cudaError_t launch_dense_fwd(const Problem& p, const void* q, const void* k, const void* v, const float* scale, void* o,
                              float* tau, float* scratch, size_t scratch_floats, int ctas, cudaStream_t stream);
-// float32 problems; scratch: fp32_scratch_ctas() CTAs of sixteen score rows of fp32_scratch_pitch() floats each.
+// float32 problems; scratch: fp32_scratch_ctas() CTAs of fp32_scratch_rows() score rows of fp32_scratch_pitch() floats each.
 // acc_dk, acc_dv: fp32 [B,H,N,D] contiguous, zero on entry
 int fp32_scratch_pitch(const Problem& p);
+int fp32_scratch_rows(const Problem& p);
 int fp32_scratch_ctas(const Problem& p);
 cudaError_t launch_fp32_fwd(const Problem& p, const float* q, const float* k, const float* v, const float* scale, float* o,
                             float* tau, int32_t* row_cnt, int32_t* dense_cnt, Entry* entries, float* scratch, int ctas,

@@ -152,7 +152,7 @@ WsLayout make_layout(const Problem& p, bool is_bwd) {
   l.scratch = off;
   if (p.dtype == ENTMAX_ATTN_DTYPE_FP32) {
     l.scratch_ctas = fp32_scratch_ctas(p);
-    l.scratch = take((size_t)l.scratch_ctas * 16 * fp32_scratch_pitch(p) * sizeof(float));
+    l.scratch = take((size_t)l.scratch_ctas * fp32_scratch_rows(p) * fp32_scratch_pitch(p) * sizeof(float));
   }
   l.acc_dk = l.acc_dv = l.dc_rows = 0;
   if (is_bwd) {

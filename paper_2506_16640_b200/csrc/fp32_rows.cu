@@ -31,6 +31,12 @@ constexpr int kFwdCap = kTileFloats / (2 * kWarps);   // candidates (y, j) a war
 constexpr int kBwdCap = kTileFloats / (3 * kWarps);   // support entries (y, j, dP)
 static_assert(kFwdCap >= 256 && kBwdCap >= 256, "row lists");
 
+template <int D, int R>
+constexpr int smem_bytes() { return (kTileFloats + R * D) * (int)sizeof(float); }
+// CTAs an SM holds (228 KB of shared memory, 1 KB of it reserved per CTA): three, two for sixteen rows of 128
+template <int D, int R>
+constexpr int resident_ctas() { return 3 * (smem_bytes<D, R>() + 1024) <= 233472 ? 3 : 2; }
+
 __device__ __forceinline__ float warp_sum(float x) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
@@ -170,7 +176,7 @@ __device__ __forceinline__ int compact_row(const float* y, int nv, float cut, in
 }
 
 template <int D, int R>
-__global__ void __launch_bounds__(kThreads, 3) fp32_fwd_kernel(Problem p, const float* __restrict__ q,
+__global__ void __launch_bounds__(kThreads, resident_ctas<D, R>()) fp32_fwd_kernel(Problem p, const float* __restrict__ q,
                                                                const float* __restrict__ k, const float* __restrict__ v,
                                                                const float* __restrict__ scale, float* __restrict__ o,
                                                                float* __restrict__ tau_out, int32_t* __restrict__ row_cnt,
@@ -285,7 +291,7 @@ __global__ void __launch_bounds__(kThreads, 3) fp32_fwd_kernel(Problem p, const 
 
 // acc_dk, acc_dv: fp32 [B,H,N,D] contiguous, zero on entry
 template <int D, int R>
-__global__ void __launch_bounds__(kThreads, 3) fp32_bwd_kernel(Problem p, const float* __restrict__ q,
+__global__ void __launch_bounds__(kThreads, resident_ctas<D, R>()) fp32_bwd_kernel(Problem p, const float* __restrict__ q,
                                                                const float* __restrict__ k, const float* __restrict__ v,
                                                                const float* __restrict__ d_o, const float* __restrict__ scale,
                                                                const float* __restrict__ tau_in, float* __restrict__ dq,
@@ -416,9 +422,6 @@ __global__ void __launch_bounds__(kThreads, 3) fp32_bwd_kernel(Problem p, const 
   }
 }
 
-template <int D, int R>
-constexpr int smem_bytes() { return (kTileFloats + R * D) * (int)sizeof(float); }
-
 // Rows per CTA: eight (one per warp) while sixteen would leave SMs without a CTA
 bool eight_rows(const Problem& p) { return (long)p.B * p.H * ((p.N + 15) / 16) < 148; }
 
@@ -447,11 +450,14 @@ cudaError_t launch_bwd(const Problem& p, const float* q, const float* k, const f
 
 }  // namespace
 
-// Three CTAs per SM of sixteen score rows each while that stays within 256 MB, never fewer than one per SM.
 int fp32_scratch_pitch(const Problem& p) { return (p.N + 31) / 32 * 32; }
+int fp32_scratch_rows(const Problem& p) { return eight_rows(p) ? 8 : 16; }
+// 3 x 148 CTAs while their score rows stay within 256 MB, never fewer than one per SM.  (Also where the SMs hold fewer: what
+// waits for a free place evens out the items' lengths.  2 x 4 x 777 x 128 causal: 64 us, with 2 x 148 CTAs 81.)
 int fp32_scratch_ctas(const Problem& p) {
-  const long items = (long)p.B * p.H * ((p.N + 7) / 8);
-  const long per = 16L * fp32_scratch_pitch(p) * 4;
+  const int rows = fp32_scratch_rows(p);
+  const long items = (long)p.B * p.H * ((p.N + rows - 1) / rows);
+  const long per = (long)rows * fp32_scratch_pitch(p) * 4;
   long ctas = (256L << 20) / per;
   ctas = ctas > 148 * 3 ? 148 * 3 : ctas < 148 ? 148 : ctas;
   return (int)(items < ctas ? items : ctas);
