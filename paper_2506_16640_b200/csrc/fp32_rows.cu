@@ -425,6 +425,12 @@ __global__ void __launch_bounds__(kThreads, resident_ctas<D, R>()) fp32_bwd_kern
 // Rows per CTA: eight (one per warp) while sixteen would leave SMs without a CTA
 bool eight_rows(const Problem& p) { return (long)p.B * p.H * ((p.N + 15) / 16) < 148; }
 
+// Long problems, whose score rows leave fewer CTAs than the SMs hold: these start only after the kernel before them.  Beside
+// its last CTAs they would be placed two on one SM and none on another, and stay there for the whole problem (32768 x 64, one
+// head: forward 12.2 ms, placed early 13.5 to 15.2; 3 x 40000 x 128 76 and 90).  Where the grid fills the machine an early
+// start gains (2 x 8 x 2048 x 64: 316 us against 326).
+bool plain_launch(long items, int ctas) { return items > ctas && ctas < 148 * 3; }
+
 template <int D, int R>
 cudaError_t launch_fwd(const Problem& p, const float* q, const float* k, const float* v, const float* scale, float* o,
                        float* tau, int32_t* row_cnt, int32_t* dense_cnt, Entry* entries, float* scratch, int ctas,
@@ -433,7 +439,12 @@ cudaError_t launch_fwd(const Problem& p, const float* q, const float* k, const f
   const long items = (long)p.B * p.H * ((p.N + R - 1) / R);
   cudaError_t err = cudaFuncSetAttribute(fp32_fwd_kernel<D, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (err != cudaSuccess) return err;
-  launch_kernel(fp32_fwd_kernel<D, R>, (int)(items < ctas ? items : ctas), kThreads, bytes, stream, p, q, k, v, scale, o, tau, row_cnt, dense_cnt, entries, scratch, fp32_scratch_pitch(p), (int)items);
+  if (plain_launch(items, ctas))
+    fp32_fwd_kernel<D, R><<<ctas, kThreads, bytes, stream>>>(p, q, k, v, scale, o, tau, row_cnt, dense_cnt, entries, scratch,
+                                                             fp32_scratch_pitch(p), (int)items);
+  else
+    launch_kernel(fp32_fwd_kernel<D, R>, (int)(items < ctas ? items : ctas), kThreads, bytes, stream, p, q, k, v, scale, o, tau, row_cnt, dense_cnt,
+                  entries, scratch, fp32_scratch_pitch(p), (int)items);
   return cudaGetLastError();
 }
 template <int D, int R>
@@ -444,7 +455,12 @@ cudaError_t launch_bwd(const Problem& p, const float* q, const float* k, const f
   const long items = (long)p.B * p.H * ((p.N + R - 1) / R);
   cudaError_t err = cudaFuncSetAttribute(fp32_bwd_kernel<D, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (err != cudaSuccess) return err;
-  launch_kernel(fp32_bwd_kernel<D, R>, (int)(items < ctas ? items : ctas), kThreads, bytes, stream, p, q, k, v, d_o, scale, tau, dq, acc_dk, acc_dv, dc_rows, scratch, fp32_scratch_pitch(p), (int)items);
+  if (plain_launch(items, ctas))
+    fp32_bwd_kernel<D, R><<<ctas, kThreads, bytes, stream>>>(p, q, k, v, d_o, scale, tau, dq, acc_dk, acc_dv, dc_rows, scratch,
+                                                             fp32_scratch_pitch(p), (int)items);
+  else
+    launch_kernel(fp32_bwd_kernel<D, R>, (int)(items < ctas ? items : ctas), kThreads, bytes, stream, p, q, k, v, d_o, scale, tau, dq, acc_dk, acc_dv,
+                  dc_rows, scratch, fp32_scratch_pitch(p), (int)items);
   return cudaGetLastError();
 }
 

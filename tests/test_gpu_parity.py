@@ -877,3 +877,16 @@ def test_fp32_gradients_written_over_the_inputs(N, d, dk, dv):
     got = binding.entmax_attn_bwd(t["q"], t["k"], t["v"], tau, t["d_o"], 1.5, True, dk=t[dk], dv=t[dv])
     for a, b in zip(got, ref):
         assert (a - b).abs().max().item() <= 1e-5 * b.abs().max().item()      # sums in another order
+
+
+def test_fp32_long_problem_with_fewer_ctas_than_the_sms_hold():
+    # past 9362 keys the score rows of 3 x 148 CTAs no longer fit their 256 MB: fewer CTAs, several row tiles each, launched
+    # behind the kernel before them
+    N = 9601
+    inp = make_inputs(_small("fp32_long", N, 64, True, dtype="fp32", H=2, backward=True, seed=77))
+    got = parity.run_fwd(inp, 1.5)
+    bwd = parity.run_bwd(inp, 1.5, got["tau"], got["dev"])
+    rows = np.unique(np.r_[0:40, np.arange(0, N, 331), N - 20 : N])
+    for bh in range(2):
+        parity.check_fwd_rows(inp, 1.5, got, bh, rows)
+        parity.check_bwd_rows(inp, 1.5, bwd, bh, rows)
