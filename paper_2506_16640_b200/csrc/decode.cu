@@ -22,17 +22,19 @@ namespace {
 constexpr int kListSlots = 2048;   // candidate slots of a solve CTA, split evenly among its threads
 constexpr int kMaxNewtonD = 64;
 
-// PER consecutive bf16 values (PER = 2 or 4) as floats
+// PER consecutive bf16 values (PER = 2 or 4), as they lie in memory and as floats
 template <int PER>
-__device__ __forceinline__ void load_bf16_row(const __nv_bfloat16* p, float (&f)[PER]) {
+__device__ __forceinline__ void load_packed_row(const __nv_bfloat16* p, uint32_t (&w)[PER / 2]) {
   if constexpr (PER == 4) {
     const uint2 raw = *reinterpret_cast<const uint2*>(p);
-    f[0] = __uint_as_float(raw.x << 16); f[1] = __uint_as_float(raw.x & 0xffff0000u);
-    f[2] = __uint_as_float(raw.y << 16); f[3] = __uint_as_float(raw.y & 0xffff0000u);
+    w[0] = raw.x;
+    w[1] = raw.y;
   } else {
-    const uint32_t raw = *reinterpret_cast<const uint32_t*>(p);
-    f[0] = __uint_as_float(raw << 16); f[1] = __uint_as_float(raw & 0xffff0000u);
+    w[0] = *reinterpret_cast<const uint32_t*>(p);
   }
+}
+__device__ __forceinline__ float packed_at(const uint32_t* w, int e) {
+  return __uint_as_float((e & 1) ? (w[e >> 1] & 0xffff0000u) : (w[e >> 1] << 16));
 }
 
 // Sum over the CTA in a fixed order; every thread returns the same value.  `slot` alternates between
@@ -55,8 +57,89 @@ __device__ __forceinline__ float2 block_sum2(float x, float y, float2 (*red)[kSo
   return s;
 }
 
+// A row with more candidates than the list holds: the same iteration and output sum over the whole score row.  The CTA's warps
+// leave their shares of O in opart; returns the threshold and (its bits) the support size.  (Out of line, so that it costs the
+// usual path no registers.)  The gather takes the warp's ballot of 64 keys and four V rows at a time: as a loop over single
+// keys every step waited for its score, 457 us of 16 heads x 32768 keys at c = 1 (8 of 16 rows run over), now 108.
 template <int D, int kSolveThreads>
-__global__ void __launch_bounds__(kSolveThreads) decode_solve_kernel(DecodeArgs a, const __nv_bfloat16* __restrict__ v,
+__device__ __noinline__ float2 solve_on_score_row(const float* y_row, int nv, float ymax, int expo_class, float expo,
+                                                  const __nv_bfloat16* v_head, int64_t v_stride,
+                                                  float2 (*red)[kSolveThreads / 32], int* scan, float (*opart)[D]) {
+  constexpr int kWarps = kSolveThreads / 32;
+  constexpr int PER = D / 32;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  TauIter st = tau_iter_start(ymax);
+  for (int it = 0; it < kMaxNewtonD; ++it) {
+    float s0 = 0.f, s1 = 0.f;
+    for (int j0 = tid; j0 < nv; j0 += 4 * kSolveThreads) {
+      float d[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int j = j0 + u * kSolveThreads;
+        d[u] = j < nv ? y_row[j] - st.tau : -INFINITY;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (d[u] > 0.f) {
+          float ye, ye1;
+          pow_pair(d[u], expo_class, expo, ye, ye1);
+          s0 += ye;
+          s1 += ye1;
+        }
+    }
+    const float2 s = block_sum2<kSolveThreads>(s0, s1, red, it & 1);
+    if (!tau_iter_update(st, s.x, s.y, expo_class, expo, 1e-7f)) break;
+  }
+  const float tau = st.tau;
+  const __nv_bfloat16* vbase = v_head + lane * PER;
+  float acc[PER];
+#pragma unroll
+  for (int e = 0; e < PER; ++e) acc[e] = 0.f;
+  int local = 0;
+  // a warp looks at 64 keys together and gathers the V rows of those in the support four at a time
+  for (int j0 = warp * 64; j0 < nv; j0 += kWarps * 64) {
+    float d[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int j = j0 + 32 * u + lane;
+      d[u] = j < nv ? y_row[j] - tau : -INFINITY;
+    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      float ye = 0.f, ye1;
+      if (d[u] > 0.f) pow_pair(d[u], expo_class, expo, ye, ye1);
+      unsigned m = __ballot_sync(0xffffffffu, d[u] > 0.f);
+      local += __popc(m);
+      while (m) {
+        float p[4];
+        uint32_t vw[4][PER / 2];
+#pragma unroll
+        for (int z = 0; z < 4; ++z) {
+          const int src = m ? __ffs(m) - 1 : 0;
+          p[z] = __shfl_sync(0xffffffffu, ye, src);
+#pragma unroll
+          for (int e = 0; e < PER / 2; ++e) vw[z][e] = 0u;
+          if (m) load_packed_row<PER>(vbase + (size_t)(j0 + 32 * u + src) * v_stride, vw[z]);
+          m &= m - 1;
+        }
+#pragma unroll
+        for (int z = 0; z < 4; ++z)
+#pragma unroll
+          for (int e = 0; e < PER; ++e) acc[e] = fmaf(p[z], packed_at(vw[z], e), acc[e]);
+      }
+    }
+  }
+  if (lane == 0) scan[warp] = local;
+#pragma unroll
+  for (int e = 0; e < PER; ++e) opart[warp][lane * PER + e] = acc[e];
+  __syncthreads();
+  int support = 0;
+  for (int w = 0; w < kWarps; ++w) support += scan[w];
+  return make_float2(tau, __int_as_float(support));
+}
+
+template <int D, int kSolveThreads>
+__global__ void __launch_bounds__(kSolveThreads, kSolveThreads == 512 ? 3 : 1) decode_solve_kernel(DecodeArgs a, const __nv_bfloat16* __restrict__ v,
                                                                     const float* __restrict__ scores,
                                                                     const float* __restrict__ tile_max,
                                                                     __nv_bfloat16* __restrict__ o,
@@ -178,6 +261,7 @@ __global__ void __launch_bounds__(kSolveThreads) decode_solve_kernel(DecodeArgs 
   TauIter st;
   st.tau = st.lo = floor_y;      // y_max - 1, the bracket's lower end (App. A)
   st.hi = ymax;
+  const __nv_bfloat16* v_head = v + (size_t)b * a.ksb + (size_t)h * a.ksh;
   float tau = floor_y;
   int support = 0;
   if (!dense) {
@@ -223,59 +307,27 @@ __global__ void __launch_bounds__(kSolveThreads) decode_solve_kernel(DecodeArgs 
     __syncthreads();
     tau = s_tau;
     support = s_support;
-  } else {
-    for (int it = 0; it < kMaxNewtonD; ++it) {
-      float s0 = 0.f, s1 = 0.f;
-      for (int j = tid; j < nv; j += kSolveThreads) {
-        const float d = y_row[j] - st.tau;
-        if (d > 0.f) {
-          float ye, ye1;
-          pow_pair(d, a.expo_class, a.expo, ye, ye1);
-          s0 += ye;
-          s1 += ye1;
-        }
-      }
-      const float2 s = block_sum2<kSolveThreads>(s0, s1, red, it & 1);
-      if (!tau_iter_update(st, s.x, s.y, a.expo_class, a.expo, 1e-7f)) break;
-    }
-    tau = st.tau;
-    __syncthreads();
-  }
-  // ---- O = sum_j p_j v_j
-  const __nv_bfloat16* vbase = v + (size_t)b * a.ksb + (size_t)h * a.ksh + lane * PER;
-  float acc[PER];
+    // ---- O = sum_j p_j v_j
+    float acc[PER];
 #pragma unroll
-  for (int e = 0; e < PER; ++e) acc[e] = 0.f;
-  if (!dense) {
+    for (int e = 0; e < PER; ++e) acc[e] = 0.f;
     for (int c = warp; c < n_cand; c += kWarps) {
       const float p = cand_y[c];
       if (p > 0.f) {
-        float vf[PER];
-        load_bf16_row<PER>(vbase + (size_t)list_j[c] * a.ksn, vf);
+        uint32_t vw[PER / 2];
+        load_packed_row<PER>(v_head + (size_t)list_j[c] * a.ksn + lane * PER, vw);
 #pragma unroll
-        for (int e = 0; e < PER; ++e) acc[e] = fmaf(p, vf[e], acc[e]);
+        for (int e = 0; e < PER; ++e) acc[e] = fmaf(p, packed_at(vw, e), acc[e]);
       }
     }
+#pragma unroll
+    for (int e = 0; e < PER; ++e) opart[warp][lane * PER + e] = acc[e];
   } else {
-    int local = 0;
-    for (int j = warp; j < nv; j += kWarps) {
-      const float d = y_row[j] - tau;
-      if (d > 0.f) {
-        float ye, ye1;
-        pow_pair(d, a.expo_class, a.expo, ye, ye1);
-        float vf[PER];
-        load_bf16_row<PER>(vbase + (size_t)j * a.ksn, vf);
-#pragma unroll
-        for (int e = 0; e < PER; ++e) acc[e] = fmaf(ye, vf[e], acc[e]);
-        ++local;
-      }
-    }
-    if (lane == 0) scan[warp] = local;
-    __syncthreads();
-    for (int w = 0; w < kWarps; ++w) support += scan[w];
+    const float2 solved = solve_on_score_row<D, kSolveThreads>(y_row, nv, ymax, a.expo_class, a.expo, v_head, a.ksn, red, scan,
+                                                              opart);
+    tau = solved.x;
+    support = __float_as_int(solved.y);
   }
-#pragma unroll
-  for (int e = 0; e < PER; ++e) opart[warp][lane * PER + e] = acc[e];
   __syncthreads();
   if (tid < D) {
     float s = 0.f;

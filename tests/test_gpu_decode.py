@@ -166,3 +166,15 @@ def test_decode_split_of_the_keys_at_its_edges(B, H, N, d, q_len):
         got = _run(inp, lens, q_len, 1.5)
         assert int(got["status"][binding.STATUS_FLAGS]) == 0
         _check(inp, lens, q_len, 1.5, got, heads=heads)
+
+
+@pytest.mark.parametrize("alpha", [1.25, 1.5])
+@pytest.mark.parametrize("B,H,N,d,q_len", [(1, 8, 16384, 128, 1), (1, 8, 16421, 64, 2), (2, 8, 8191, 128, 2)])
+def test_decode_rows_with_too_many_candidates_and_a_short_support(B, H, N, d, q_len, alpha):
+    # fixed temperature: a thousand candidates and more within the bracket, some thread's share of the list runs over, and
+    # the row is solved and gathered from the score row, where its support is a few dozen scattered keys
+    inp = _problem(B, H, N, d, use_scale=False, seed=N)
+    lens = _lengths(B, N, q_len, N, B > 1)
+    got = _run(inp, lens, q_len, alpha)
+    assert int(got["status"][binding.STATUS_DENSE_ROWS]) > 0
+    _check(inp, lens, q_len, alpha, got, heads=[0, 3, H - 1])
