@@ -239,7 +239,8 @@ int entmax_attn_bwd_ex(const entmax_attn_params* params, const void* q, const vo
  * support of row i is {j : (alpha-1) s_ij > tau_i}).  Byte offsets from the workspace base:
  *   row_count  int32 [batch*heads*seq]: support size of the row, or -2 when the row was computed by the
  *              dense path and its list is not kept (a row goes there when its candidate list could not
- *              be kept at `keep_limit` entries at some point of the sweep)
+ *              be kept at `keep_limit` entries at some point of the sweep; on long sequences a few rows of
+ *              every 32 may keep more, up to 176)
  *   dense_count int32 [batch*heads*seq][2]: for a row with row_count == -2, the number of keys with p > 0
  *              counted by each of the two threads that formed the row's probabilities; their sum is the
  *              support size (other rows: unspecified)

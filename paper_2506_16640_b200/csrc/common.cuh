@@ -14,11 +14,12 @@ namespace entmax {
 
 // Sparse row lists: kListCap slots per row, the fill level at which the sweep tightens the threshold and filters the list
 // (checked after every K tile), and the length a filtered list may keep -- a row that cannot be brought down to it is
-// handed to the dense path.  The row kernels leave the support compacted from slot 0.
+// handed to the dense path.  Such a row takes its whole 128-row tile there, so the second pair of limits holds where only a
+// few rows of a warp pass the first (see the sweep's consumers).  The row kernels leave the support compacted from slot 0.
 constexpr int kListCap = 256;
-constexpr int kListTrigger = 112;
-constexpr int kListKeep = 96;
-static_assert(kListTrigger + 64 <= kListCap && kListKeep < kListTrigger, "list bounds");
+constexpr int kListTrigger = 112, kListTriggerLong = 176;
+constexpr int kListKeep = 96, kListKeepLong = 144;
+static_assert(kListTriggerLong + 64 <= kListCap && kListKeep < kListTrigger && kListKeepLong < kListTriggerLong, "list bounds");
 
 // One list slot: y = (alpha-1) * s_ij (or the raw accumulator while a sweep is running), j = key index.
 struct __align__(8) Entry {

@@ -167,7 +167,7 @@ struct RowState {
 // units are turned into Eq. 1's units with y = a * acc.  All 32 lanes must call this together.
 // Takes and returns the row state by value: a state whose address escaped would have to be kept in
 // local memory across every asm statement of the scan loop.
-__device__ __forceinline__ RowState shrink_lists(RowState r, Entry* list, float a, float inv_a, unsigned need, int mode,
+__device__ __forceinline__ RowState shrink_lists(RowState r, Entry* list, float a, float inv_a, unsigned need, int keep_limit,
                                               int expo_class, float expo) {
   const int lane = threadIdx.x & 31;
   constexpr int kPer = kListCap / 32;
@@ -180,100 +180,96 @@ __device__ __forceinline__ RowState shrink_lists(RowState r, Entry* list, float 
     const float th = __shfl_sync(0xffffffffu, r.thr, src);
     const float aa = __shfl_sync(0xffffffffu, a, src);
     const float inv_aa = __shfl_sync(0xffffffffu, inv_a, src);
-    float new_thr = INFINITY;
-    int kept = -1;
-    if (mode == 0) {
-      Entry e[kPer];
+    Entry e[kPer];
 #pragma unroll
-      for (int s = 0; s < kPer; ++s) {
-        const int idx = lane + 32 * s;
-        e[s].y = -INFINITY;
-        e[s].j = 0;
-        if (idx < c) e[s] = l[idx];
-      }
-      // A sure case first.  With y_max the largest of the c listed keys, sum_j (y_max - tau)^e >= sum_j [y_j - tau]_+^e
-      // = 1 at the list's own threshold tau*, so tau* <= y_max - c^(-1/e): every listed key above that is in the
-      // list's support.  If those alone are more than a list may keep, the row goes to the dense path without a
-      // solve (rows of flat logits, which would otherwise each pay a full Newton solve just to be handed over).
-      bool sure_dense = false;
-      {
-        float ym = -INFINITY;
+    for (int s = 0; s < kPer; ++s) {
+      const int idx = lane + 32 * s;
+      e[s].y = -INFINITY;
+      e[s].j = 0;
+      if (idx < c) e[s] = l[idx];
+    }
+    // A sure case first.  With y_max the largest of the c listed keys, sum_j (y_max - tau)^e >= sum_j [y_j - tau]_+^e
+    // = 1 at the list's own threshold tau*, so tau* <= y_max - c^(-1/e): every listed key above that is in the
+    // list's support.  If those alone are more than a list may keep, the row goes to the dense path without a
+    // solve (rows of flat logits, which would otherwise each pay a full Newton solve just to be handed over).
+    bool sure_dense = false;
+    {
+      float ym = -INFINITY;
 #pragma unroll
-        for (int s = 0; s < kPer; ++s) ym = fmaxf(ym, e[s].y);
+      for (int s = 0; s < kPer; ++s) ym = fmaxf(ym, e[s].y);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) ym = fmaxf(ym, __shfl_xor_sync(0xffffffffu, ym, o));
-        const float width = expo_class == kExpo2 ? rsqrtf((float)c) : expo_class == kExpo1 ? 1.0f / (float)c
-                                                                                           : __powf((float)c, -1.0f / expo);
-        const float cut = ym - width * inv_aa;
-        int sure = 0;
+      for (int o = 16; o > 0; o >>= 1) ym = fmaxf(ym, __shfl_xor_sync(0xffffffffu, ym, o));
+      const float width = expo_class == kExpo2 ? rsqrtf((float)c) : expo_class == kExpo1 ? 1.0f / (float)c
+                                                                                         : __powf((float)c, -1.0f / expo);
+      const float cut = ym - width * inv_aa;
+      int sure = 0;
 #pragma unroll
-        for (int s = 0; s < kPer; ++s) sure += __popc(__ballot_sync(0xffffffffu, e[s].y > cut));
-        sure_dense = sure > kListKeep;
-      }
-      float tau = th * aa;
-      if (sure_dense) {
-        // nothing to solve
-      } else if (expo >= 1.0f) {
-        for (int it = 0; it < 8; ++it) {
-          float s0 = 0.f, s1 = 0.f;
-#pragma unroll
-          for (int s = 0; s < kPer; ++s) {
-            const float y = fmaf(aa, e[s].y, -tau);
-            if (y > 0.f) {
-              float ye1 = y;
-              if (expo_class == kExpo1) ye1 = 1.0f;
-              else if (expo_class == kExpo4) ye1 = y * y * y;
-              else if (expo_class == kExpoGeneral) ye1 = __powf(y, expo - 1.0f);
-              s0 = fmaf(ye1, y, s0);
-              s1 += ye1;
-            }
-          }
-          s0 = warp_sum(s0);
-          s1 = warp_sum(s1);
-          if (!(s0 > 1.0f) || !(s1 > 0.f)) break;
-          const float root = expo_class == kExpo1 ? s0
-                             : expo_class == kExpo2 ? sqrtf(s0)
-                             : expo_class == kExpo4 ? sqrtf(sqrtf(s0)) : __powf(s0, 1.0f / expo);
-          const float step = (s0 - s0 / root) / s1;      // threshold_step
-          tau += step;
-          if (step <= 1e-4f) break;
-        }
-      } else {
-        // e < 1 (alpha > 2): plain bisection between the current bound (mass of the listed keys >= 1 there) and one
-        // unit above it (tau <= y_max <= bound + 1); the lower end stays a valid bound whatever the rounding does
-        float lo = tau, hi = tau + 1.0f;
-        for (int it = 0; it < 14; ++it) {
-          const float mid = 0.5f * (lo + hi);
-          float s0 = 0.f;
-#pragma unroll
-          for (int s = 0; s < kPer; ++s) {
-            const float y = fmaf(aa, e[s].y, -mid);
-            if (y > 0.f) s0 += __powf(y, expo);
-          }
-          s0 = warp_sum(s0);
-          if (s0 > 1.0f) lo = mid; else hi = mid;
-        }
-        tau = lo;
-      }
-      // a hair below the Newton iterate: rounding must never push the bound past the true threshold (general exponents:
-      // the fast powers are good to about 1e-5 of the mass, and d tau <= d mass where the mass is 1 or more)
-      const float hair = 4e-6f * fmaxf(1.0f, fabsf(tau)) + (expo_class == kExpoGeneral ? 5e-5f : 0.f);
-      new_thr = fmaxf(th, (tau - hair) * inv_aa);
-      __syncwarp();
-      kept = 0;
-      if (!sure_dense) {
+      for (int s = 0; s < kPer; ++s) sure += __popc(__ballot_sync(0xffffffffu, e[s].y > cut));
+      sure_dense = sure > keep_limit;
+    }
+    float tau = th * aa;
+    if (sure_dense) {
+      // nothing to solve
+    } else if (expo >= 1.0f) {
+      for (int it = 0; it < 8; ++it) {
+        float s0 = 0.f, s1 = 0.f;
 #pragma unroll
         for (int s = 0; s < kPer; ++s) {
-          const bool keep = e[s].y > new_thr;
-          const unsigned m = __ballot_sync(0xffffffffu, keep);
-          if (keep) l[kept + __popc(m & ((1u << lane) - 1u))] = e[s];
-          kept += __popc(m);
+          const float y = fmaf(aa, e[s].y, -tau);
+          if (y > 0.f) {
+            float ye1 = y;
+            if (expo_class == kExpo1) ye1 = 1.0f;
+            else if (expo_class == kExpo4) ye1 = y * y * y;
+            else if (expo_class == kExpoGeneral) ye1 = __powf(y, expo - 1.0f);
+            s0 = fmaf(ye1, y, s0);
+            s1 += ye1;
+          }
         }
+        s0 = warp_sum(s0);
+        s1 = warp_sum(s1);
+        if (!(s0 > 1.0f) || !(s1 > 0.f)) break;
+        const float root = expo_class == kExpo1 ? s0
+                           : expo_class == kExpo2 ? sqrtf(s0)
+                           : expo_class == kExpo4 ? sqrtf(sqrtf(s0)) : __powf(s0, 1.0f / expo);
+        const float step = (s0 - s0 / root) / s1;      // threshold_step
+        tau += step;
+        if (step <= 1e-4f) break;
       }
-      if (kept > kListKeep || sure_dense) {
-        kept = -1;
-        new_thr = INFINITY;
+    } else {
+      // e < 1 (alpha > 2): plain bisection between the current bound (mass of the listed keys >= 1 there) and one
+      // unit above it (tau <= y_max <= bound + 1); the lower end stays a valid bound whatever the rounding does
+      float lo = tau, hi = tau + 1.0f;
+      for (int it = 0; it < 14; ++it) {
+        const float mid = 0.5f * (lo + hi);
+        float s0 = 0.f;
+#pragma unroll
+        for (int s = 0; s < kPer; ++s) {
+          const float y = fmaf(aa, e[s].y, -mid);
+          if (y > 0.f) s0 += __powf(y, expo);
+        }
+        s0 = warp_sum(s0);
+        if (s0 > 1.0f) lo = mid; else hi = mid;
       }
+      tau = lo;
+    }
+    // a hair below the Newton iterate: rounding must never push the bound past the true threshold (general exponents:
+    // the fast powers are good to about 1e-5 of the mass, and d tau <= d mass where the mass is 1 or more)
+    const float hair = 4e-6f * fmaxf(1.0f, fabsf(tau)) + (expo_class == kExpoGeneral ? 5e-5f : 0.f);
+    float new_thr = fmaxf(th, (tau - hair) * inv_aa);
+    __syncwarp();
+    int kept = 0;
+    if (!sure_dense) {
+#pragma unroll
+      for (int s = 0; s < kPer; ++s) {
+        const bool keep = e[s].y > new_thr;
+        const unsigned m = __ballot_sync(0xffffffffu, keep);
+        if (keep) l[kept + __popc(m & ((1u << lane) - 1u))] = e[s];
+        kept += __popc(m);
+      }
+    }
+    if (kept > keep_limit || sure_dense) {
+      kept = -1;
+      new_thr = INFINITY;
     }
     if (lane == src) {
       r.cnt = kept;
@@ -677,6 +673,12 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
       // already has a bound
       bool blind = kSearch && ts <= ts0;
       bool crowded = false;                        // the last tile had rows with many candidates
+      // Rows of the warp that may have long lists, and that do (forward).  What a dense tile costs grows with its K tiles, what
+      // a list costs does not.  16 x 32768 x 128 at 70 keys a row (9 % of them past 96): 28.5 + 27.3 ms forward and backward
+      // with none, 26.9 + 13.4 with at most four, 18.1 + 12.0 with eight, 12.9 + 12.0 with sixteen; 16 x 16384 at 99 keys a
+      // row, where most warps give up in the end: backward 9.6 with none, 9.7, 10.0 and 10.9 (with this rule 13.9 + 12.0 and 9.6).
+      const int max_long = min(tiles / 8, 16);
+      unsigned long_rows = 0u;
       for (int t = tf; t < tiles && alive; ++t) {
         // the warp leaves together: tcgen05.ld needs all 32 lanes
         alive = __all_sync(0xffffffffu, mbar_wait(my_full, fphase, abort_flag));
@@ -890,10 +892,32 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
             }
           }
           // Lists are shrunk between tiles, so that whether a row goes to the dense path depends on whole tiles of keys; in
-          // the middle of one only where a list has no room for the chunk that is waiting
-          const unsigned need = __ballot_sync(0xffffffffu, r.cnt > (full ? kListCap - 32 : kListTrigger));
-          if (need)
-            r = shrink_lists(r, list, 1.0f / margin, margin, need, kSearch ? 0 : 1, a.expo_class, a.expo);
+          // the middle of one only where a list has no room for the chunk that is waiting.  A dense row costs its whole Q tile
+          // the work on all of its K tiles, a list its own keys: while at most max_long rows of the warp pass the first limits
+          // they go by the second ones, and when one row has to go, these go with it.
+          if constexpr (kSearch) {
+            const unsigned need = __ballot_sync(0xffffffffu, r.cnt > (full ? kListCap - 32 : ((long_rows >> lane) & 1u)
+                                                                               ? kListTriggerLong : kListTrigger));
+            if (need) {
+              const bool few = __popc(need | long_rows) <= max_long && !__any_sync(0xffffffffu, r.cnt < 0);
+              r = shrink_lists(r, list, 1.0f / margin, margin, need, few ? kListKeepLong : kListKeep, a.expo_class, a.expo);
+              long_rows |= need & __ballot_sync(0xffffffffu, r.cnt > kListKeep);
+            }
+            if (long_rows && __any_sync(0xffffffffu, r.cnt < 0)) {
+              if ((long_rows >> lane) & 1u) {
+                r.cnt = -1;
+                r.thr = INFINITY;
+              }
+              long_rows = 0u;
+            }
+          } else {
+            const unsigned need = __ballot_sync(0xffffffffu, r.cnt > (full ? kListCap - 32 : kListTrigger));
+            if (need && (__popc(need) > max_long || __any_sync(0xffffffffu, r.cnt < 0 || r.cnt > kListTriggerLong)) &&
+                ((need >> lane) & 1u)) {
+              r.cnt = -1;
+              r.thr = INFINITY;
+            }
+          }
         } while (full);
         crowded = __any_sync(0xffffffffu, crowded);
       }

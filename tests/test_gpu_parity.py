@@ -890,3 +890,37 @@ def test_fp32_long_problem_with_fewer_ctas_than_the_sms_hold():
     for bh in range(2):
         parity.check_fwd_rows(inp, 1.5, got, bh, rows)
         parity.check_bwd_rows(inp, 1.5, bwd, bh, rows)
+
+
+def _some_rows_long(N, d, every, m, seed):
+    # every `every`-th row has a flat support of m keys scattered over the sequence, the others only key 0
+    inp = make_inputs(_small("some_long", N, d, False, use_scale=False, sigma=0.01, backward=True, seed=seed))
+    half = d // 2
+    keys = torch.from_numpy(1 + np.random.default_rng(seed).permutation(N - 1))
+    inp.k[:, :, keys[m:], :half] = -3.0
+    inp.k[:, :, 0, :half] = -3.0
+    inp.k[:, :, 0, half:] = 3.0
+    inp.q[..., half:] += 1.0
+    inp.q[:, :, ::every, :half] += 1.0
+    inp.q[:, :, ::every, half:] -= 1.0
+    return inp, keys[:m].sort().values
+
+
+@pytest.mark.parametrize("alpha", [1.25, 1.5, 1.7])
+@pytest.mark.parametrize("N,d,every,m,lists", [(8192, 64, 16, 100, True), (8192, 128, 8, 140, True), (8192, 64, 4, 140, False),
+                                                (4096, 64, 16, 140, True), (1500, 64, 16, 140, False), (8192, 64, 16, 180, False)])
+def test_a_few_long_rows_among_short_ones(N, d, every, m, lists, alpha):
+    # supports past the list limits (96 keys forward, 112 backward): two and four rows of every 32 keep lists of up to 176 where
+    # a Q tile sees 16 and 32 K tiles; more rows, shorter sequences or longer supports go to the dense path
+    inp, keys = _some_rows_long(N, d, every, m, seed=N + m)
+    got = parity.run_fwd(inp, alpha)
+    bwd = parity.run_bwd(inp, alpha, got["tau"], got["dev"])
+    long_rows = np.arange(0, N, every)
+    for out in (got, bwd):
+        assert int(out["status"][binding.STATUS_DENSE_ROWS]) == (0 if lists else 2 * len(long_rows))
+    rows = np.unique(np.r_[0:33, N // 2 : N // 2 + 33, N - 33 : N])
+    for bh in range(2):
+        parity.check_fwd_rows(inp, alpha, got, bh, rows)
+        parity.check_bwd_rows(inp, alpha, bwd, bh, rows)
+    for idx, _ in binding.read_support(got["params"], got["workspace"], long_rows[::7]):
+        assert torch.equal(idx.sort().values, keys) if lists else idx is None
