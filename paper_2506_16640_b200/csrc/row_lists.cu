@@ -16,9 +16,7 @@ constexpr int kWarpsPerCta = 8;
 constexpr int kSlots = kListCap / 32;
 constexpr int kMaxNewton = 400;
 
-// Butterfly sum with ascending strides: for values held by lanes 0..W-1 only (zeros elsewhere) the first
-// log2(W) steps are exactly sub_sum<W>'s tree and the rest add zeros, so the full-warp and the
-// W-lanes-per-row paths give the same bits for the same sorted support.
+// Butterfly sum, strides ascending as in sub_sum below.
 __device__ __forceinline__ float warp_sum(float x) {
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
@@ -29,13 +27,6 @@ __device__ __forceinline__ float warp_max(float x) {
   for (int o = 16; o > 0; o >>= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, o));
   return x;
 }
-
-// the row-slice helpers of common.cuh under the names this file uses
-template <int PER>
-__device__ __forceinline__ void load_bf16(const __nv_bfloat16* p, float (&x)[PER]) { load_slice<PER>(p, x); }
-template <int PER>
-__device__ __forceinline__ void store_bf16(__nv_bfloat16* p, const float (&x)[PER]) { store_slice<PER>(p, x); }
-
 
 // reductions over aligned groups of W lanes (W = 8 or 16); the sum takes ascending strides like warp_sum
 template <int W>
@@ -50,28 +41,14 @@ __device__ __forceinline__ float sub_sum(float x) {
 // move in one instruction is contiguous: 16-byte reductions of neighbouring lanes fall into the same 32-byte
 // sector instead of half-filling one each, loads and stores stay coalesced.  (PL < 4: one contiguous piece.)
 template <int PL, int W>
-__device__ __forceinline__ void load_share(const __nv_bfloat16* row, int sl, float (&x)[PL]) {
-  if constexpr (PL < 4) {
-    load_bf16<PL>(row + sl * PL, x);
-  } else {
-#pragma unroll
-    for (int c = 0; c < PL / 4; ++c) {
-      float t[4];
-      load_bf16<4>(row + 4 * W * c + 4 * sl, t);
-#pragma unroll
-      for (int e = 0; e < 4; ++e) x[4 * c + e] = t[e];
-    }
-  }
-}
-template <int PL, int W>
 __device__ __forceinline__ void store_share(__nv_bfloat16* row, int sl, const float (&x)[PL]) {
   if constexpr (PL < 4) {
-    store_bf16<PL>(row + sl * PL, x);
+    store_slice<PL>(row + sl * PL, x);
   } else {
 #pragma unroll
     for (int c = 0; c < PL / 4; ++c) {
       const float t[4] = {x[4 * c], x[4 * c + 1], x[4 * c + 2], x[4 * c + 3]};
-      store_bf16<4>(row + 4 * W * c + 4 * sl, t);
+      store_slice<4>(row + 4 * W * c + 4 * sl, t);
     }
   }
 }
@@ -85,7 +62,7 @@ __device__ __forceinline__ void add_share(float* row, int sl, const float (&x)[P
   }
 }
 
-// A lane's share of a row as it lies in memory (the interleaving of load_share), two elements to a register: half the
+// A lane's share of a row as it lies in memory (interleaved as above), two elements to a register: half the
 // registers of its floats, so that several rows can be in flight.
 template <int PL>
 struct PackedShare {
@@ -109,15 +86,17 @@ __device__ __forceinline__ float packed_at(const PackedShare<PL>& x, int e) {
   return __uint_as_float((e & 1) ? (x.w[e >> 1] & 0xffff0000u) : (x.w[e >> 1] << 16));
 }
 
-// Row solve.  The lists the sweep leaves are deterministic (a row's candidates depend on that row alone, in key order), so a
-// threshold iterated on the whole list is reproducible to the bit.
+// Row solve.  The lists the sweep leaves are deterministic (a row's candidates, in key order, depend on the 32 rows its warp
+// scanned together and on nothing that varies from call to call), so a threshold iterated on the whole list is reproducible to
+// the bit.
 constexpr float kBoundMargin = 4e-6f;   // rounding of the bound the sweep ended with
 
 // Threshold of Eq. 1 on the n <= K list entries of one row, by one thread with the entries in registers (n = 0: a lane without
 // a row, which only takes part in the votes); the list is left compacted to the support, y in Eq. 1's units.  Newton from the
 // left starting at the bound the sweep ended with (e < 1: bracketed, tau_iter_update).  Sums over a row need no shuffles this
 // way: eight to thirty-two lanes per row spent two chains of them on every iteration, or sorted the list first (alpha = 1.25,
-// 16 x 20011 x 128: 580 + 92 us with the long rows -> 227 + 66; alpha = 1.5, 16 x 32768 x 128: 222 + 105 -> 255 + 32).
+// 16 x 20011 x 128: 580 + 92 us with the long rows -> 227 + 66; alpha = 1.5, 16 x 32768 x 128: 222 + 105 -> 255 + 32 by this
+// step alone, 168 + 22 with the gathers of the kernels below as they are now).
 template <int K, int EC>
 __device__ __forceinline__ int solve_row(const Problem& p, Entry* list, int n, float a, float bound, float& tau) {
   float y[K];

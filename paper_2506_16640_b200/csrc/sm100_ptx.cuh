@@ -46,9 +46,6 @@ __device__ __forceinline__ uint32_t lds_u32(uint32_t addr) {
 __device__ __forceinline__ void sts_u32(uint32_t addr, uint32_t v) {
   asm volatile("st.volatile.shared::cta.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
-__device__ __forceinline__ void sts_f4(uint32_t addr, float x, float y, float z, float w) {
-  asm volatile("st.shared::cta.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
-}
 __device__ __forceinline__ void lds_f4(uint32_t addr, float& x, float& y, float& z, float& w) {
   asm volatile("ld.shared::cta.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x), "=f"(y), "=f"(z), "=f"(w) : "r"(addr) : "memory");
 }
@@ -74,14 +71,6 @@ __device__ __forceinline__ void sts_record8_if_greater(float x, float thr, uint3
       : "f"(x), "f"(thr), "r"(last), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]),
         "n"(HI), "n"(STEP), "n"(GROUP)
       : "memory");
-}
-__device__ __forceinline__ unsigned long long lds_u64(uint32_t addr) {
-  unsigned long long v;
-  asm volatile("ld.volatile.shared::cta.u64 %0, [%1];" : "=l"(v) : "r"(addr) : "memory");
-  return v;
-}
-__device__ __forceinline__ void sts_u64(uint32_t addr, unsigned long long v) {
-  asm volatile("st.volatile.shared::cta.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
 }
 __device__ __forceinline__ uint64_t global_ns() {
   uint64_t t;

@@ -25,8 +25,9 @@
 // A consumer reads its 256 columns in one straight pass of 64-column TMEM loads: group maxima of eight columns (branch-free),
 // and a group that holds a candidate is parked as it is in one of the thread's slots in shared memory, so that the accumulator
 // is handed back after the pass; the candidates are taken out of the slots and appended to the row's list behind that.  A
-// tile in which some row runs out of slots is taken 32 columns at a time instead.  One thread per row makes a row's list
-// depend on that row alone.  While the consumers of one Q tile scan, the tensor core works on the other.
+// tile in which some row runs out of slots is taken 32 columns at a time instead, by a vote of the warp.  So a row's list, in
+// key order, depends on the 32 rows of its warp and on nothing else: not on timing, and not on the other warps.  While the
+// consumers of one Q tile scan, the tensor core works on the other.
 // Every mbarrier wait is bounded: on expiry the CTA raises ENTMAX_ATTN_FLAG_WAIT_EXPIRED, all roles
 // leave their loops, the producer waits for the copies it armed barriers for and the MMA issuer for the tensor-core
 // work it issued (each with a bound of its own), TMEM is freed and the CTA returns.
@@ -125,7 +126,7 @@ __device__ __forceinline__ int qtile_tiles(const SweepArgs& a, int item, int x) 
 // key (a second view of K: the key index split into (index / stride, index % stride), phase 0 taken),
 // maxima only: the running maxima and thresholds the real stream then starts from are already close to
 // their final values, which roughly halves the candidates it pushes (a one-pass stream pushes every new
-// running maximum, about ln n of them per row; after a 1/16 sample about ln 16 are left; measured best among 8, 16, 32, 64).
+// running maximum, about ln n of them per row; after a 1/8 sample about ln 8 are left).
 constexpr int kSampleStride = 8;
 constexpr int kSampleMinKeys = 4096;   // below this the stream is too short for the sample to pay
 template <bool kSearch>
