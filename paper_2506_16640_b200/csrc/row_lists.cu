@@ -86,7 +86,7 @@ __device__ __forceinline__ float packed_at(const PackedShare<PL>& x, int e) {
   return __uint_as_float((e & 1) ? (x.w[e >> 1] & 0xffff0000u) : (x.w[e >> 1] << 16));
 }
 
-// Row solve.  The lists the sweep leaves are deterministic (a row's candidates, in key order, depend on the 32 rows its warp
+// Row solve.  The lists the sweep leaves are deterministic (a row's candidates and their order depend on the 32 rows its warp
 // scanned together and on nothing that varies from call to call), so a threshold iterated on the whole list is reproducible to
 // the bit.
 constexpr float kBoundMargin = 4e-6f;   // rounding of the bound the sweep ended with

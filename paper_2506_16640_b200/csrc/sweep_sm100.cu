@@ -26,7 +26,7 @@
 // and a group that holds a candidate is parked as it is in one of the thread's slots in shared memory, so that the accumulator
 // is handed back after the pass; the candidates are taken out of the slots and appended to the row's list behind that.  A
 // tile in which some row runs out of slots is taken 32 columns at a time instead, by a vote of the warp.  So a row's list, in
-// key order, depends on the 32 rows of its warp and on nothing else: not on timing, and not on the other warps.  While the
+// the order of the tiles, depends on the 32 rows of its warp and on nothing else: not on timing, and not on the other warps.  While the
 // consumers of one Q tile scan, the tensor core works on the other.
 // Every mbarrier wait is bounded: on expiry the CTA raises ENTMAX_ATTN_FLAG_WAIT_EXPIRED, all roles
 // leave their loops, the producer waits for the copies it armed barriers for and the MMA issuer for the tensor-core
@@ -453,7 +453,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
             for (int hf = 0; hf < C::kHalves; ++hf) {
               const uint32_t dst = k_smem + stage * C::kKBytes + hf * (BN * 128);
               if (t < ts) tma_load_5d(dst, &map_ks, k_full + 8 * stage, hf * 64, 0, (ts0 + t) * BN, h, b);
-              else tma_load_4d(dst, &map_k, k_full + 8 * stage, hf * 64, (tf + t - ts) * BN, h, b);
+              else tma_load_4d(dst, &map_k, k_full + 8 * stage, hf * 64, (kAlibi ? tf + tiles - 1 - (t - ts) : t - ts) * BN, h, b);
             }
           }
           __syncwarp();
@@ -680,7 +680,11 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
       // row, where most warps give up in the end: backward 9.6 with none, 9.7, 10.0 and 10.9 (with this rule 13.9 + 12.0 and 9.6).
       const int max_long = min(tiles / 8, 16);
       unsigned long_rows = 0u;
-      for (int t = tf; t < tiles && alive; ++t) {
+      for (int s = 0; s < tiles - tf && alive; ++s) {
+        // ALiBi: the nearest keys first.  Their penalty is the smallest, so that the bound is good from the first tile on; in key
+        // order tile after tile brought new maxima (12 heads x 6000 x 64, alpha 2, half of the heads with slopes: 190 us in key
+        // order, 141 now; 12 x 3000 x 64 at alpha 1.5, where no sample helps: 307 and 118).
+        const int t = kAlibi ? tiles - 1 - s : s;
         // the warp leaves together: tcgen05.ld needs all 32 lanes
         alive = __all_sync(0xffffffffu, mbar_wait(my_full, fphase, abort_flag));
         if (!alive) break;

@@ -530,6 +530,14 @@ def test_alibi_bf16_causal_sparse_rows(N, d, alpha):
     _check_alibi(inp, alpha, True, [0.0, 0.05], None)
 
 
+@pytest.mark.parametrize("alpha", [1.25, 1.7])
+@pytest.mark.parametrize("N,d", [(1, 64), (255, 128), (257, 64), (513, 128), (1027, 64), (4099, 64)])
+def test_alibi_at_the_edges_of_tiles(N, d, alpha):
+    # the sweep takes the K tiles from the diagonal backwards: one tile, a last tile of one row, several tiles, with a sample
+    inp = make_inputs(_small("alibi_edges", N, d, True, backward=True, seed=N + 11))
+    _check_alibi(inp, alpha, True, [0.01, 0.2], None)
+
+
 def test_alibi_window_skips_far_tiles_and_keeps_parity():
     # NAPE-style heads at a length where the hard cutoff bites: slopes 0 (NoPE), 0.5, 0.1 and 0.02.  The sweep starts
     # every work item at the first K tile that can still hold a candidate (norm bound on the logits); forward and
