@@ -72,6 +72,9 @@ __device__ __forceinline__ void sts_record8_if_greater(float x, float thr, uint3
         "n"(HI), "n"(STEP), "n"(GROUP)
       : "memory");
 }
+__device__ __forceinline__ void sts_f4(uint32_t addr, float x, float y, float z, float w) {
+  asm volatile("st.shared::cta.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
+}
 __device__ __forceinline__ uint64_t global_ns() {
   uint64_t t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));

@@ -128,10 +128,17 @@ __device__ __forceinline__ int qtile_tiles(const SweepArgs& a, int item, int x) 
 // their final values, which roughly halves the candidates it pushes (a one-pass stream pushes every new
 // running maximum, about ln n of them per row; after a 1/8 sample about ln 8 are left).
 constexpr int kSampleStride = 8;
+// Shorter sequences instead raise their bound behind crowded tiles, from the largest keys of the tiles so far (see the end of
+// a tile): items of at least kTightenTiles K tiles, while some list is longer than kTightenList.  2 x 12 x 3001 x 64 with a
+// projected scale 260 -> 186 us, 4 x 16 x 2048 x 64 at c = 1 256 -> 173, 16 x 3500 x 128 at c = 1 238 -> 164; rows with few
+// candidates have nothing to gain (8 x 12 x 1024 x 64 69 either way; 82 without these two limits; 2 x 16 x 2000 x 128 with
+// planted keys 90 -> 94).  With a sample ahead it costs more than it gives (8192 keys: 507 -> 543).
+// Below kShortMinKeys an item has too few tiles for that (1024 keys: 257 -> 260 us a training step with it, 960: 167 -> 171).
+constexpr int kTightenTiles = 4, kTightenList = 48, kShortMinKeys = 1536;
 constexpr int kSampleMinKeys = 4096;   // below this the stream is too short for the sample to pay
-template <bool kSearch>
+template <bool kSample>
 __device__ __forceinline__ int sample_tiles(const SweepArgs& a, int item) {
-  if (!kSearch) return 0;
+  if (!kSample) return 0;
   int last_row = item * kItemRows + kItemRows - 1;
   if (last_row > a.N - 1) last_row = a.N - 1;
   const int n_vis = a.causal ? last_row + 1 : a.N;
@@ -345,7 +352,8 @@ __device__ __forceinline__ void scan_groups(const float (&g)[8], float thr, uint
   sts_record8_if_greater<kSlotHi, kSlotStep, G0 + 7>(g[7], thr, at, last, groups, &v[56]);
 }
 
-template <int HD, bool kDump, bool kAlibi, bool kSearch>
+// kShort: sequences of kShortMinKeys to kSampleMinKeys - 1 keys, which have no sampled pass
+template <int HD, bool kDump, bool kAlibi, bool kSearch, bool kShort>
 __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constant__ CUtensorMap map_q,
                                                             const __grid_constant__ CUtensorMap map_k,
                                                             const __grid_constant__ CUtensorMap map_ks,
@@ -441,7 +449,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
         }
         // tiles before tf (and sampled tiles before ts0) lie outside the ALiBi window: t counts from there
         const int tf = __shfl_sync(0xffffffffu, first_tile<kAlibi>(a, k), 0);
-        const int ts_all = sample_tiles<kSearch>(a, item);
+        const int ts_all = sample_tiles<kSearch && !kShort>(a, item);
         const int ts0 = kAlibi ? min(tf / kSampleStride, ts_all) : 0;
         const int ts = ts_all - ts0;
         tiles -= tf;
@@ -518,7 +526,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
           tiles = tx[x] > tiles ? tx[x] : tiles;
         }
         const int tf = __shfl_sync(0xffffffffu, first_tile<kAlibi>(a, k), 0);
-        const int ts_all = sample_tiles<kSearch>(a, item);
+        const int ts_all = sample_tiles<kSearch && !kShort>(a, item);
         const int ts = ts_all - (kAlibi ? min(tf / kSampleStride, ts_all) : 0);
         tiles -= tf;
         for (int x = 0; x < kQTiles; ++x) tx[x] = tx[x] > 0 ? tx[x] - tf : 0;   // every valid Q tile reaches past tf
@@ -622,7 +630,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
       const int last_lim = a.causal ? (tile_row0 + BM - 1 < a.N - 1 ? tile_row0 + BM - 1 : a.N - 1) : a.N - 1;
       // ---- sampled tiles first (forward mode, long rows): maxima only, no key is kept -- every sampled
       //      key comes by again in the real stream.  Column c of sampled tile t is key kSampleStride * (t*BN + c).
-      const int ts = sample_tiles<kSearch>(a, item);
+      const int ts = sample_tiles<kSearch && !kShort>(a, item);
       const int ts0 = kAlibi ? min(tf / kSampleStride, ts) : 0;
       if (kAlibi && a.status && cw == 0 && lane == 0) {
         // K-tile steps of this item left out by the window / still scored
@@ -630,7 +638,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
         atomicAdd(a.status + ENTMAX_ATTN_STATUS_SKIPPED_STEPS, tf);
         atomicAdd(a.status + ENTMAX_ATTN_STATUS_SCORED_STEPS, t_item - tf);
       }
-      if (kSearch && ts > ts0) {
+      if (kSearch && !kShort && ts > ts0) {
         // largest sampled group index that is a key this row may look at, and the largest all rows may look at
         int glim = lim / kSampleStride;
         if (glim > a.N / kSampleStride - 1) glim = a.N / kSampleStride - 1;
@@ -674,6 +682,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
       // already has a bound
       bool blind = kSearch && ts <= ts0;
       bool crowded = false;                        // the last tile had rows with many candidates
+      bool tops_valid = false;
       // Rows of the warp that may have long lists, and that do (forward).  What a dense tile costs grows with its K tiles, what
       // a list costs does not.  16 x 32768 x 128 at 70 keys a row (9 % of them past 96): 28.5 + 27.3 ms forward and backward
       // with none, 26.9 + 13.4 with at most four, 18.1 + 12.0 with eight, 12.9 + 12.0 with sixteen; 16 x 16384 at 99 keys a
@@ -726,6 +735,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
           blind = false;
         }
         bool skip = __all_sync(0xffffffffu, r.thr == INFINITY) && !kDump;   // no row of the warp wants anything any more
+        if constexpr (kShort) tops_valid = tops_valid && crowded;   // (the straight pass uses the slots)
         bool crowd = !skip && (crowded || col_base + BN - 1 > first_lim || kDump);
         if (!crowd && !skip) {
           float v0[64], v1[64];
@@ -792,10 +802,20 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
 #pragma unroll
               for (int u = 0; u < 32; ++u) va[u] = (col0 + u <= lim) ? va[u] : -INFINITY;
             }
-            const float m_c = fmaxf(fmaxf(max8(&va[0]), max8(&va[8])), fmaxf(max8(&va[16]), max8(&va[24])));
+            float h4[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) h4[q] = max8(&va[8 * q]);
+            const float m_c = fmaxf(fmaxf(h4[0], h4[1]), fmaxf(h4[2], h4[3]));
             if constexpr (kSearch) {
               m_run = fmaxf(m_run, m_c);
               r.thr = fmaxf(r.thr, m_run - margin);
+              if (kShort && tiles >= kTightenTiles) {
+                // maxima of eight classes of the keys of this run of crowded tiles, in the (idle) first slot
+                const uint32_t tops = my_slot + ((c & 1) ? kSlotHi : 0);
+                float t4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+                if (tops_valid || c >= 2) lds_f4(tops, t4[0], t4[1], t4[2], t4[3]);
+                sts_f4(tops, fmaxf(t4[0], h4[0]), fmaxf(t4[1], h4[1]), fmaxf(t4[2], h4[2]), fmaxf(t4[3], h4[3]));
+              }
             }
             const bool hit = m_c > r.thr;
             int n_new = 0;
@@ -924,6 +944,18 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
             }
           }
         } while (full);
+        if constexpr (kSearch && kShort) {
+          // The threshold of those eight keys is a bound as well (nothing new before the second tile of the run)
+          if (crowd && tiles >= kTightenTiles) {
+            if (tops_valid && s + 1 < tiles - tf && __any_sync(0xffffffffu, r.cnt > kTightenList)) {
+              float top[8];
+              lds_f4(my_slot, top[0], top[1], top[2], top[3]);
+              lds_f4(my_slot + kSlotHi, top[4], top[5], top[6], top[7]);
+              r.thr = fmaxf(r.thr, bound_from_values(top, margin, a.expo_class, a.expo, m_run));
+            }
+            tops_valid = tops_valid || nch > 1;
+          }
+        }
         crowded = __any_sync(0xffffffffu, crowded);
       }
       if (i < a.N && alive) {
@@ -1108,7 +1140,7 @@ cudaError_t make_sample_map(CUtensorMap* map, const void* base, const Problem& p
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-template <int HD, bool kDump, bool kAlibi, bool kSearch>
+template <int HD, bool kDump, bool kAlibi, bool kSearch, bool kShort>
 cudaError_t launch_impl(const Problem& p, const void* q, const void* k, SweepArgs& args, cudaStream_t stream) {
   CUtensorMap map_q, map_k, map_ks;
   cudaError_t err = make_map(&map_q, q, p, BM);
@@ -1121,7 +1153,7 @@ cudaError_t launch_impl(const Problem& p, const void* q, const void* k, SweepArg
   } else {
     map_ks = map_k;   // never used: sample_tiles() is 0 for short sequences
   }
-  err = cudaFuncSetAttribute(sweep_kernel<HD, kDump, kAlibi, kSearch>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  err = cudaFuncSetAttribute(sweep_kernel<HD, kDump, kAlibi, kSearch, kShort>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              Cfg<HD>::kSmemBytes);
   if (err != cudaSuccess) return err;
   int dev = 0, sms = 0;
@@ -1130,7 +1162,7 @@ cudaError_t launch_impl(const Problem& p, const void* q, const void* k, SweepArg
   err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (err != cudaSuccess) return err;
   const int grid = args.n_items < sms ? args.n_items : sms;
-  launch_kernel(sweep_kernel<HD, kDump, kAlibi, kSearch>, grid, kThreads, Cfg<HD>::kSmemBytes, stream, map_q, map_k, map_ks, args);
+  launch_kernel(sweep_kernel<HD, kDump, kAlibi, kSearch, kShort>, grid, kThreads, Cfg<HD>::kSmemBytes, stream, map_q, map_k, map_ks, args);
   return cudaGetLastError();
 }
 
@@ -1177,12 +1209,13 @@ cudaError_t launch_sweep(const Problem& p, const void* q, const void* k, const f
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return err;
   }
-#define ENTMAX_SWEEP(DUMP, ALIBI, SEARCH)                                               \
-  (p.D == 64 ? launch_impl<64, DUMP, ALIBI, SEARCH>(p, q, k, args, stream)              \
-             : launch_impl<128, DUMP, ALIBI, SEARCH>(p, q, k, args, stream))
-  if (dump) return ENTMAX_SWEEP(true, false, true);
-  if (p.alibi) return mode == 0 ? ENTMAX_SWEEP(false, true, true) : ENTMAX_SWEEP(false, true, false);
-  return mode == 0 ? ENTMAX_SWEEP(false, false, true) : ENTMAX_SWEEP(false, false, false);
+#define ENTMAX_SWEEP(DUMP, ALIBI, SEARCH, SHORT)                                               \
+  (p.D == 64 ? launch_impl<64, DUMP, ALIBI, SEARCH, SHORT>(p, q, k, args, stream)              \
+             : launch_impl<128, DUMP, ALIBI, SEARCH, SHORT>(p, q, k, args, stream))
+  if (dump) return ENTMAX_SWEEP(true, false, true, false);
+  if (mode != 0) return p.alibi ? ENTMAX_SWEEP(false, true, false, false) : ENTMAX_SWEEP(false, false, false, false);
+  if (p.N >= kShortMinKeys && p.N < kSampleMinKeys) return p.alibi ? ENTMAX_SWEEP(false, true, true, true) : ENTMAX_SWEEP(false, false, true, true);
+  return p.alibi ? ENTMAX_SWEEP(false, true, true, false) : ENTMAX_SWEEP(false, false, true, false);
 #undef ENTMAX_SWEEP
 }
 

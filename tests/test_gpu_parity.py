@@ -823,6 +823,19 @@ def test_candidate_lists_and_row_solves_at_their_edges(N, d, causal, alpha):
 
 
 @pytest.mark.parametrize("alpha", [1.25, 1.5, 1.7, 2.0, 3.0])
+@pytest.mark.parametrize("N,d,causal", [(1535, 64, True), (1536, 64, False), (1537, 128, True), (2049, 128, False), (4095, 64, True)])
+def test_crowded_tiles_of_sequences_without_a_sample(N, d, causal, alpha):
+    # flat logits below the length from which rows have a sampled pass: lists past 48 entries within the first tiles, so that the
+    # bound is raised from the largest keys of a run of crowded tiles (from the second of at least four tiles on)
+    for sigma in (1.0, 0.7):
+        inp = make_inputs(_small("crowded", N, d, causal, use_scale=False, sigma=sigma, seed=N + d))
+        got = parity.run_fwd(inp, alpha)
+        rows = np.unique(np.r_[np.arange(0, N, 37), N - 3 : N])
+        for bh in range(inp.workload.H):
+            parity.check_fwd_rows(inp, alpha, got, bh, rows)
+
+
+@pytest.mark.parametrize("alpha", [1.25, 1.5, 1.7, 2.0, 3.0])
 @pytest.mark.parametrize("N,d,low,high", [(500, 64, 256, 256 + 203), (4300, 64, 4096, 4096 + 203), (4200, 128, 0, 251)])
 def test_flat_rows_with_one_large_key_late_in_a_tile_keep_their_lists(N, d, low, high, alpha):
     # 50 flat keys, faint ones up to key `low`, flat again behind it: the tile that starts there looks as if it sent every row
