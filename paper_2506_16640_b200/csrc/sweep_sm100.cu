@@ -128,13 +128,20 @@ __device__ __forceinline__ int qtile_tiles(const SweepArgs& a, int item, int x) 
 // their final values, which roughly halves the candidates it pushes (a one-pass stream pushes every new
 // running maximum, about ln n of them per row; after a 1/8 sample about ln 8 are left).
 constexpr int kSampleStride = 8;
-// Shorter sequences instead raise their bound behind crowded tiles, from the largest keys of the tiles so far (see the end of
-// a tile): items of at least kTightenTiles K tiles, while some list is longer than kTightenList.  2 x 12 x 3001 x 64 with a
-// projected scale 260 -> 186 us, 4 x 16 x 2048 x 64 at c = 1 256 -> 173, 16 x 3500 x 128 at c = 1 238 -> 164; rows with few
-// candidates have nothing to gain (8 x 12 x 1024 x 64 69 either way; 82 without these two limits; 2 x 16 x 2000 x 128 with
-// planted keys 90 -> 94).  With a sample ahead it costs more than it gives (8192 keys: 507 -> 543).
-// Below kShortMinKeys an item has too few tiles for that (1024 keys: 257 -> 260 us a training step with it, 960: 167 -> 171).
-constexpr int kTightenTiles = 4, kTightenList = 48, kShortMinKeys = 1536;
+// Sequences of kShortMinKeys to kSampleMinKeys - 1 keys have no sampled pass.  Their bound comes from the first look at a tile
+// (maxima only, see the consumers), and where the temperature is low most of what is stored is stored because of that.  So
+// they look at a tile first again when the one before left kLookRows rows of the warp crowded, with more than kLookList entries
+// in their lists.  Forward sweep, us, without and with it: 2 x 12 x 3001 x 64 with a projected scale 182 -> 170; at c = 1 16 x
+// 3001 x 64 175 -> 138, 24 x 2000 x 128 124 -> 94, 16 x 4095 x 64 300 -> 226; rows with few candidates hardly ever take it (planted
+// keys, 24 x 2048 x 128 77 and 78, 48 x 3001 x 64 186 and 187).  Kept up in every crowded tile instead, the maxima cost those
+// calls 3 to 14 % (the same two: 84 and 200).  Sixteen rows instead of four: 140, 106 and 238 at c = 1, 180 with the projected
+// scale; two rows: 16 x 3001 x 64 with planted keys 94 -> 103.  Above an exponent of kLookExpo supports are long and eight keys
+// say little about them: with it, alpha = 1.25, 24 x 1536 x 64 55 -> 57, 16 x 3001 x 64 86 -> 91, 16 x 4095 x 64 213 -> 199.
+// Below kShortMinKeys an item has too few tiles for that.  In longer sequences the code alone costs the scan 1 to 4 % at
+// head_dim 64 (16 x 32768 non-causal 2591 -> 2689) against 2 to 6 % gained at c = 1 and 8192 keys, also where only the items
+// without a sample (those that see fewer than kSampleMinKeys keys) take it: they have neither.
+constexpr int kLookRows = 4, kLookList = 32, kShortMinKeys = 1536;
+constexpr float kLookExpo = 2.0f;
 constexpr int kSampleMinKeys = 4096;   // below this the stream is too short for the sample to pay
 template <bool kSample>
 __device__ __forceinline__ int sample_tiles(const SweepArgs& a, int item) {
@@ -679,10 +686,10 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
         r.thr = fmaxf(r.thr, bound_from_values(top, margin, a.expo_class, a.expo, m_run));
       }
       // A stream that starts without any bound scans its first tile twice: maxima first, so that the second scan
-      // already has a bound
-      bool blind = kSearch && ts <= ts0;
+      // already has a bound.  (kShort: later tiles too, see kLookRows.)
+      bool look = kSearch && ts <= ts0;
       bool crowded = false;                        // the last tile had rows with many candidates
-      bool tops_valid = false;
+      bool looked = false;                         // kShort: the first slot holds the class maxima of the tiles looked at so far
       // Rows of the warp that may have long lists, and that do (forward).  What a dense tile costs grows with its K tiles, what
       // a list costs does not.  16 x 32768 x 128 at 70 keys a row (9 % of them past 96): 28.5 + 27.3 ms forward and backward
       // with none, 26.9 + 13.4 with at most four, 18.1 + 12.0 with eight, 12.9 + 12.0 with sixteen; 16 x 16384 at 99 keys a
@@ -708,11 +715,16 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
         // warp counting: branches on "some row has a candidate", a second look at TMEM or list stores in between all cost
         // more there than these predicated stores do.
         uint32_t at = my_slot, groups = 0u;
-        if (blind) {
-          // the first tile of a stream without any bound: maxima of eight classes of its keys, and the threshold of those eight
+        if (look) {
+          // maxima of eight classes of the tile's keys (kShort: of the tiles looked at since the slots were last in use: eight
+          // different keys all the same), and the threshold of those eight
           float top[8];
 #pragma unroll
           for (int q = 0; q < 8; ++q) top[q] = -INFINITY;
+          if (kShort && looked) {
+            lds_f4(my_slot, top[0], top[1], top[2], top[3]);
+            lds_f4(my_slot + kSlotHi, top[4], top[5], top[6], top[7]);
+          }
 #pragma unroll 1
           for (int c = 0; c < (nch + 1) / 2; ++c) {
             float va[64];
@@ -731,13 +743,18 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
 #pragma unroll
             for (int q = 0; q < 8; ++q) top[q] = fmaxf(top[q], max8(&va[8 * q]));
           }
+          if (kShort) {
+            sts_f4(my_slot, top[0], top[1], top[2], top[3]);
+            sts_f4(my_slot + kSlotHi, top[4], top[5], top[6], top[7]);
+            looked = true;
+          }
           r.thr = fmaxf(r.thr, bound_from_values(top, margin, a.expo_class, a.expo, m_run));
-          blind = false;
+          look = false;
         }
         bool skip = __all_sync(0xffffffffu, r.thr == INFINITY) && !kDump;   // no row of the warp wants anything any more
-        if constexpr (kShort) tops_valid = tops_valid && crowded;   // (the straight pass uses the slots)
         bool crowd = !skip && (crowded || col_base + BN - 1 > first_lim || kDump);
         if (!crowd && !skip) {
+          looked = false;                            // (the slots are in use)
           float v0[64], v1[64];
           tmem_ld64(taddr_row, v0);
 #pragma unroll
@@ -802,20 +819,10 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
 #pragma unroll
               for (int u = 0; u < 32; ++u) va[u] = (col0 + u <= lim) ? va[u] : -INFINITY;
             }
-            float h4[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) h4[q] = max8(&va[8 * q]);
-            const float m_c = fmaxf(fmaxf(h4[0], h4[1]), fmaxf(h4[2], h4[3]));
+            const float m_c = fmaxf(fmaxf(max8(&va[0]), max8(&va[8])), fmaxf(max8(&va[16]), max8(&va[24])));
             if constexpr (kSearch) {
               m_run = fmaxf(m_run, m_c);
               r.thr = fmaxf(r.thr, m_run - margin);
-              if (kShort && tiles >= kTightenTiles) {
-                // maxima of eight classes of the keys of this run of crowded tiles, in the (idle) first slot
-                const uint32_t tops = my_slot + ((c & 1) ? kSlotHi : 0);
-                float t4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-                if (tops_valid || c >= 2) lds_f4(tops, t4[0], t4[1], t4[2], t4[3]);
-                sts_f4(tops, fmaxf(t4[0], h4[0]), fmaxf(t4[1], h4[1]), fmaxf(t4[2], h4[2]), fmaxf(t4[3], h4[3]));
-              }
             }
             const bool hit = m_c > r.thr;
             int n_new = 0;
@@ -945,18 +952,13 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
           }
         } while (full);
         if constexpr (kSearch && kShort) {
-          // The threshold of those eight keys is a bound as well (nothing new before the second tile of the run)
-          if (crowd && tiles >= kTightenTiles) {
-            if (tops_valid && s + 1 < tiles - tf && __any_sync(0xffffffffu, r.cnt > kTightenList)) {
-              float top[8];
-              lds_f4(my_slot, top[0], top[1], top[2], top[3]);
-              lds_f4(my_slot + kSlotHi, top[4], top[5], top[6], top[7]);
-              r.thr = fmaxf(r.thr, bound_from_values(top, margin, a.expo_class, a.expo, m_run));
-            }
-            tops_valid = tops_valid || nch > 1;
-          }
+          const unsigned rows = __ballot_sync(0xffffffffu, crowded);
+          crowded = rows != 0u;
+          if (crowded)
+            look = a.expo <= kLookExpo && __popc(rows & __ballot_sync(0xffffffffu, r.cnt > kLookList)) >= kLookRows;
+        } else {
+          crowded = __any_sync(0xffffffffu, crowded);
         }
-        crowded = __any_sync(0xffffffffu, crowded);
       }
       if (i < a.N && alive) {
         a.list_cnt[2 * (size_t)grow] = r.cnt;
@@ -1214,7 +1216,8 @@ cudaError_t launch_sweep(const Problem& p, const void* q, const void* k, const f
              : launch_impl<128, DUMP, ALIBI, SEARCH, SHORT>(p, q, k, args, stream))
   if (dump) return ENTMAX_SWEEP(true, false, true, false);
   if (mode != 0) return p.alibi ? ENTMAX_SWEEP(false, true, false, false) : ENTMAX_SWEEP(false, false, false, false);
-  if (p.N >= kShortMinKeys && p.N < kSampleMinKeys) return p.alibi ? ENTMAX_SWEEP(false, true, true, true) : ENTMAX_SWEEP(false, false, true, true);
+  if (p.N >= kShortMinKeys && p.N < kSampleMinKeys)
+    return p.alibi ? ENTMAX_SWEEP(false, true, true, true) : ENTMAX_SWEEP(false, false, true, true);
   return p.alibi ? ENTMAX_SWEEP(false, true, true, false) : ENTMAX_SWEEP(false, false, true, false);
 #undef ENTMAX_SWEEP
 }

@@ -825,8 +825,9 @@ def test_candidate_lists_and_row_solves_at_their_edges(N, d, causal, alpha):
 @pytest.mark.parametrize("alpha", [1.25, 1.5, 1.7, 2.0, 3.0])
 @pytest.mark.parametrize("N,d,causal", [(1535, 64, True), (1536, 64, False), (1537, 128, True), (2049, 128, False), (4095, 64, True)])
 def test_crowded_tiles_of_sequences_without_a_sample(N, d, causal, alpha):
-    # flat logits below the length from which rows have a sampled pass: lists past 48 entries within the first tiles, so that the
-    # bound is raised from the largest keys of a run of crowded tiles (from the second of at least four tiles on)
+    # flat logits below the length from which rows have a sampled pass: lists past 32 entries within the first tiles, so that
+    # tile after tile is looked at before it is scanned and the bound comes from the largest keys of all of them (alpha = 1.25:
+    # of the first one only)
     for sigma in (1.0, 0.7):
         inp = make_inputs(_small("crowded", N, d, causal, use_scale=False, sigma=sigma, seed=N + d))
         got = parity.run_fwd(inp, alpha)
