@@ -367,6 +367,9 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
                                                             const __grid_constant__ SweepArgs a) {
   pdl_begin();
   using C = Cfg<HD>;
+  // K tiles from the diagonal backwards.  Counting down from an item's last tile needs every Q tile of the item to have the same.
+  constexpr bool kBack = kAlibi && kSearch;
+  static_assert(kItemRows == BN, "the Q tiles of an item end in the same K tile");
   extern __shared__ uint8_t smem_raw[];
   // everything in shared memory is addressed by 32-bit shared-window addresses derived from one base
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -468,7 +471,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
             for (int hf = 0; hf < C::kHalves; ++hf) {
               const uint32_t dst = k_smem + stage * C::kKBytes + hf * (BN * 128);
               if (t < ts) tma_load_5d(dst, &map_ks, k_full + 8 * stage, hf * 64, 0, (ts0 + t) * BN, h, b);
-              else tma_load_4d(dst, &map_k, k_full + 8 * stage, hf * 64, (kAlibi ? tf + tiles - 1 - (t - ts) : t - ts) * BN, h, b);
+              else tma_load_4d(dst, &map_k, k_full + 8 * stage, hf * 64, (kBack ? tf + tiles - 1 - (t - ts) : tf + t - ts) * BN, h, b);
             }
           }
           __syncwarp();
@@ -698,9 +701,9 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
       unsigned long_rows = 0u;
       for (int s = 0; s < tiles - tf && alive; ++s) {
         // ALiBi: the nearest keys first.  Their penalty is the smallest, so that the bound is good from the first tile on; in key
-        // order tile after tile brought new maxima (12 heads x 6000 x 64, alpha 2, half of the heads with slopes: 190 us in key
-        // order, 141 now; 12 x 3000 x 64 at alpha 1.5, where no sample helps: 307 and 118).
-        const int t = kAlibi ? tiles - 1 - s : s;
+        // order tile after tile brought new maxima (12 heads x 6000 x 64, alpha 2, half of the heads with slopes: 191 us in key
+        // order, 138 now).  A given threshold has no bound to gain (and 4 to 7 % to lose on 12 x 32768 x 64, slopes on all heads).
+        const int t = kBack ? tiles - 1 - s : tf + s;
         // the warp leaves together: tcgen05.ld needs all 32 lanes
         alive = __all_sync(0xffffffffu, mbar_wait(my_full, fphase, abort_flag));
         if (!alive) break;

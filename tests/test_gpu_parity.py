@@ -538,6 +538,17 @@ def test_alibi_at_the_edges_of_tiles(N, d, alpha):
     _check_alibi(inp, alpha, True, [0.01, 0.2], None)
 
 
+@pytest.mark.parametrize("alpha", [1.25, 1.5, 1.7, 2.0])
+@pytest.mark.parametrize("N,d", [(1536, 64), (1793, 128), (3001, 64), (4095, 128)])
+def test_alibi_of_sequences_without_a_sample(N, d, alpha):
+    # 1536 to 4095 keys: the first tile is a masked one, later ones are looked at again where lists are long (flat logits, c = 1),
+    # a head without positional term next to one whose window leaves tiles out; the backward sweep has the exact threshold.
+    # (alpha = 2 with flat logits: keys so close to the threshold that its Jacobian jumps within the rounding of a score)
+    for kw in ({"plant": 2}, {"use_scale": False}) if alpha < 2.0 else ({"plant": 2},):
+        inp = make_inputs(_small("alibi_short", N, d, True, backward=True, seed=N + d, **kw))
+        _check_alibi(inp, alpha, True, [0.0, 0.03], None)
+
+
 def test_alibi_window_skips_far_tiles_and_keeps_parity():
     # NAPE-style heads at a length where the hard cutoff bites: slopes 0 (NoPE), 0.5, 0.1 and 0.02.  The sweep starts
     # every work item at the first K tile that can still hold a candidate (norm bound on the logits); forward and
