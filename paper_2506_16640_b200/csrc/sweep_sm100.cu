@@ -172,6 +172,17 @@ __device__ __forceinline__ int first_tile(const SweepArgs& a, int k) {
   return 0;
 }
 
+// Heads with a slope take their K tiles from the diagonal backwards when they search: the nearest keys have the smallest
+// penalty, so that the bound is good from the first tile on; in key order tile after tile brought new maxima (12 heads x 6000
+// x 64, alpha 2, half of the heads with slopes: 191 us in key order, 138 now).  A given threshold has no bound to gain (and 4
+// to 7 % to lose on 12 x 32768 x 64, slopes on all heads).  Nor has a head without slope, which backwards starts with a masked
+// tile: 12 x 2000 x 64 at alpha 1.25 and c = 1, where most rows are dense, 151 -> 173 us with every slope zero.
+template <bool kAlibiSearch>
+__device__ __forceinline__ bool from_diagonal(const SweepArgs& a, int h) {
+  if constexpr (kAlibiSearch) return a.dump[h] > 0.f;
+  return false;
+}
+
 // ------------------------------------------------------------- consumer side: one row per thread
 struct RowState {
   float thr;       // candidates are accumulators above this (accumulator units); +inf: none any more
@@ -367,8 +378,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
                                                             const __grid_constant__ SweepArgs a) {
   pdl_begin();
   using C = Cfg<HD>;
-  // K tiles from the diagonal backwards.  Counting down from an item's last tile needs every Q tile of the item to have the same.
-  constexpr bool kBack = kAlibi && kSearch;
+  // from_diagonal counts down from an item's last K tile
   static_assert(kItemRows == BN, "the Q tiles of an item end in the same K tile");
   extern __shared__ uint8_t smem_raw[];
   // everything in shared memory is addressed by 32-bit shared-window addresses derived from one base
@@ -463,6 +473,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
         const int ts0 = kAlibi ? min(tf / kSampleStride, ts_all) : 0;
         const int ts = ts_all - ts0;
         tiles -= tf;
+        const bool back = from_diagonal<kAlibi && kSearch>(a, h);
         for (int t = 0; t < ts + tiles && alive; ++t) {
           alive = wait_all(k_empty + 8 * stage, kphase ^ 1u);
           if (!alive) break;
@@ -471,7 +482,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
             for (int hf = 0; hf < C::kHalves; ++hf) {
               const uint32_t dst = k_smem + stage * C::kKBytes + hf * (BN * 128);
               if (t < ts) tma_load_5d(dst, &map_ks, k_full + 8 * stage, hf * 64, 0, (ts0 + t) * BN, h, b);
-              else tma_load_4d(dst, &map_k, k_full + 8 * stage, hf * 64, (kBack ? tf + tiles - 1 - (t - ts) : tf + t - ts) * BN, h, b);
+              else tma_load_4d(dst, &map_k, k_full + 8 * stage, hf * 64, (back ? tf + tiles - 1 - (t - ts) : tf + t - ts) * BN, h, b);
             }
           }
           __syncwarp();
@@ -634,6 +645,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
       // ALiBi (causal): the logit is sm_scale * (acc + slope * (j - i)); everything below works on that sum
       const float slope = kAlibi ? a.dump[h] / a.sm_scale : 0.f;
       const float fi = (float)i;
+      const bool back = from_diagonal<kAlibi && kSearch>(a, h);
       // first / last visible key over the rows of this Q tile: chunks past the last one are skipped,
       // tiles that reach past the first one need the mask
       const int first_lim = a.causal ? tile_row0 : a.N - 1;
@@ -700,10 +712,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
       const int max_long = min(tiles / 8, 16);
       unsigned long_rows = 0u;
       for (int s = 0; s < tiles - tf && alive; ++s) {
-        // ALiBi: the nearest keys first.  Their penalty is the smallest, so that the bound is good from the first tile on; in key
-        // order tile after tile brought new maxima (12 heads x 6000 x 64, alpha 2, half of the heads with slopes: 191 us in key
-        // order, 138 now).  A given threshold has no bound to gain (and 4 to 7 % to lose on 12 x 32768 x 64, slopes on all heads).
-        const int t = kBack ? tiles - 1 - s : tf + s;
+        const int t = back ? tiles - 1 - s : tf + s;
         // the warp leaves together: tcgen05.ld needs all 32 lanes
         alive = __all_sync(0xffffffffu, mbar_wait(my_full, fphase, abort_flag));
         if (!alive) break;
