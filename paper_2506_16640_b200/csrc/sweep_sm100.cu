@@ -370,7 +370,7 @@ __device__ __forceinline__ void scan_groups(const float (&g)[8], float thr, uint
   sts_record8_if_greater<kSlotHi, kSlotStep, G0 + 7>(g[7], thr, at, last, groups, &v[56]);
 }
 
-// kShort: sequences of kShortMinKeys to kSampleMinKeys - 1 keys, which have no sampled pass
+// kShort: sequences without a sampled pass, from kShortMinKeys keys on or with slopes (see kLookRows)
 template <int HD, bool kDump, bool kAlibi, bool kSearch, bool kShort>
 __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constant__ CUtensorMap map_q,
                                                             const __grid_constant__ CUtensorMap map_k,
@@ -761,7 +761,10 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
             looked = true;
           }
           r.thr = fmaxf(r.thr, bound_from_values(top, margin, a.expo_class, a.expo, m_run));
-          look = false;
+          // (a stream from the diagonal starts with a masked tile, in which the first rows see few keys: the next one is looked at
+          // as well.  Slopes on all heads, c = 1: 48 x 300 x 64 at alpha 1.25, where the diagonal tile has 44 keys, 100 -> 79 us
+          // (82 in key order); every row dense 48 x 500 x 64 152 -> 120, 12 x 2000 166 -> 128)
+          look = kShort && back && s == 0;
         }
         bool skip = __all_sync(0xffffffffu, r.thr == INFINITY) && !kDump;   // no row of the warp wants anything any more
         bool crowd = !skip && (crowded || col_base + BN - 1 > first_lim || kDump);
@@ -967,7 +970,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
           const unsigned rows = __ballot_sync(0xffffffffu, crowded);
           crowded = rows != 0u;
           if (crowded)
-            look = a.expo <= kLookExpo && __popc(rows & __ballot_sync(0xffffffffu, r.cnt > kLookList)) >= kLookRows;
+            look |= a.expo <= kLookExpo && __popc(rows & __ballot_sync(0xffffffffu, r.cnt > kLookList)) >= kLookRows;
         } else {
           crowded = __any_sync(0xffffffffu, crowded);
         }
@@ -1228,7 +1231,7 @@ cudaError_t launch_sweep(const Problem& p, const void* q, const void* k, const f
              : launch_impl<128, DUMP, ALIBI, SEARCH, SHORT>(p, q, k, args, stream))
   if (dump) return ENTMAX_SWEEP(true, false, true, false);
   if (mode != 0) return p.alibi ? ENTMAX_SWEEP(false, true, false, false) : ENTMAX_SWEEP(false, false, false, false);
-  if (p.N >= kShortMinKeys && p.N < kSampleMinKeys)
+  if ((p.alibi || p.N >= kShortMinKeys) && p.N < kSampleMinKeys)
     return p.alibi ? ENTMAX_SWEEP(false, true, true, true) : ENTMAX_SWEEP(false, false, true, true);
   return p.alibi ? ENTMAX_SWEEP(false, true, true, false) : ENTMAX_SWEEP(false, false, true, false);
 #undef ENTMAX_SWEEP

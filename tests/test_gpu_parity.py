@@ -549,6 +549,14 @@ def test_alibi_of_sequences_without_a_sample(N, d, alpha):
         _check_alibi(inp, alpha, True, [0.0, 0.03], None)
 
 
+@pytest.mark.parametrize("alpha", [1.25, 1.5])
+@pytest.mark.parametrize("N,d,sigma", [(300, 64, 1.0), (500, 128, 0.05), (1027, 64, 0.7)])
+def test_alibi_flat_rows_of_few_tiles(N, d, sigma, alpha):
+    # a stream from the diagonal whose first tile holds few keys, lists that grow long or are given up in the second one
+    inp = make_inputs(_small("alibi_flat", N, d, True, backward=True, use_scale=False, sigma=sigma, seed=N + 5))
+    _check_alibi(inp, alpha, True, [0.0, 0.004], None)
+
+
 def test_alibi_window_skips_far_tiles_and_keeps_parity():
     # NAPE-style heads at a length where the hard cutoff bites: slopes 0 (NoPE), 0.5, 0.1 and 0.02.  The sweep starts
     # every work item at the first K tile that can still hold a candidate (norm bound on the logits); forward and
