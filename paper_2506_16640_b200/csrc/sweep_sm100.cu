@@ -482,7 +482,8 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
             for (int hf = 0; hf < C::kHalves; ++hf) {
               const uint32_t dst = k_smem + stage * C::kKBytes + hf * (BN * 128);
               if (t < ts) tma_load_5d(dst, &map_ks, k_full + 8 * stage, hf * 64, 0, (ts0 + t) * BN, h, b);
-              else tma_load_4d(dst, &map_k, k_full + 8 * stage, hf * 64, (back ? tf + tiles - 1 - (t - ts) : tf + t - ts) * BN, h, b);
+              else
+                tma_load_4d(dst, &map_k, k_full + 8 * stage, hf * 64, (back ? tf + tiles - 1 - (t - ts) : tf + t - ts) * BN, h, b);
             }
           }
           __syncwarp();
@@ -709,10 +710,14 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
       // a list costs does not.  16 x 32768 x 128 at 70 keys a row (9 % of them past 96): 28.5 + 27.3 ms forward and backward
       // with none, 26.9 + 13.4 with at most four, 18.1 + 12.0 with eight, 12.9 + 12.0 with sixteen; 16 x 16384 at 99 keys a
       // row, where most warps give up in the end: backward 9.6 with none, 9.7, 10.0 and 10.9 (with this rule 13.9 + 12.0 and 9.6).
-      const int max_long = min(tiles / 8, 16);
+      // Short sequences (kShort) would have none or one by this, and the first dense row of a call costs it a launch that otherwise
+      // returns at once (2 x 12 x 3001 x 64 with a projected scale: forward 298 us without such a row, 436 with one).  One per K
+      // tile there, up to eight: 16 x 2500 x 128 at alpha 1.4 and c = 1, three rows, 1714 -> 617; 16 x 3500 x 128 non-causal, 136
+      // rows, 2980 -> 1160; calls whose rows are mostly dense all the same lose up to 3 % (slopes, alpha 1.25, 500 keys 230 -> 235).
+      const int max_long = kShort ? min(tiles, 8) : min(tiles / 8, 16);
       unsigned long_rows = 0u;
-      for (int s = 0; s < tiles - tf && alive; ++s) {
-        const int t = back ? tiles - 1 - s : tf + s;
+      for (int step = 0; step < tiles - tf && alive; ++step) {
+        const int t = back ? tiles - 1 - step : tf + step;
         // the warp leaves together: tcgen05.ld needs all 32 lanes
         alive = __all_sync(0xffffffffu, mbar_wait(my_full, fphase, abort_flag));
         if (!alive) break;
@@ -764,7 +769,7 @@ __global__ void __launch_bounds__(kThreads, 1) sweep_kernel(const __grid_constan
           // (a stream from the diagonal starts with a masked tile, in which the first rows see few keys: the next one is looked at
           // as well.  Slopes on all heads, c = 1: 48 x 300 x 64 at alpha 1.25, where the diagonal tile has 44 keys, 100 -> 79 us
           // (82 in key order); every row dense 48 x 500 x 64 152 -> 120, 12 x 2000 166 -> 128)
-          look = kShort && back && s == 0;
+          look = kShort && back && step == 0;
         }
         bool skip = __all_sync(0xffffffffu, r.thr == INFINITY) && !kDump;   // no row of the warp wants anything any more
         bool crowd = !skip && (crowded || col_base + BN - 1 > first_lim || kDump);

@@ -855,6 +855,21 @@ def test_crowded_tiles_of_sequences_without_a_sample(N, d, causal, alpha):
             parity.check_fwd_rows(inp, alpha, got, bh, rows)
 
 
+@pytest.mark.parametrize("N,d,norm", [(1600, 64, 0.36), (2500, 128, 0.38)])
+def test_a_few_long_rows_of_a_short_sequence_keep_their_lists(N, d, norm):
+    # four rows of every 32 flatter than the others: supports of 52 to 137 keys at N, and of no more on the way there
+    inp = make_inputs(_small("few_long", N, d, False, use_scale=False, seed=N + d))
+    rows = np.arange(3, N, 8)
+    flat = inp.q[:, :, rows].double()
+    inp.q *= 4.0
+    inp.q[:, :, rows] = (flat / flat.norm(dim=-1, keepdim=True) * (norm * d ** 0.5)).to(inp.q.dtype)
+    got = parity.run_fwd(inp, 1.5)
+    assert int(got["status"][binding.STATUS_DENSE_ROWS]) == 0
+    assert max(len(idx) for idx, _ in binding.read_support(got["params"], got["workspace"], rows)) > 112
+    for bh in range(inp.workload.H):
+        parity.check_fwd_rows(inp, 1.5, got, bh, rows)
+
+
 @pytest.mark.parametrize("alpha", [1.25, 1.5, 1.7, 2.0, 3.0])
 @pytest.mark.parametrize("N,d,low,high", [(500, 64, 256, 256 + 203), (4300, 64, 4096, 4096 + 203), (4200, 128, 0, 251)])
 def test_flat_rows_with_one_large_key_late_in_a_tile_keep_their_lists(N, d, low, high, alpha):
