@@ -137,7 +137,8 @@ constexpr int kSampleStride = 8;
 // calls 3 to 14 % (the same two: 84 and 200).  Sixteen rows instead of four: 140, 106 and 238 at c = 1, 180 with the projected
 // scale; two rows: 16 x 3001 x 64 with planted keys 94 -> 103.  Above an exponent of kLookExpo supports are long and eight keys
 // say little about them: with it, alpha = 1.25, 24 x 1536 x 64 55 -> 57, 16 x 3001 x 64 86 -> 91, 16 x 4095 x 64 213 -> 199.
-// Below kShortMinKeys an item has too few tiles for that.  In longer sequences the code alone costs the scan 1 to 4 % at
+// Below kShortMinKeys items have few tiles: 24 x 1500 x 64 gained at c = 1 (78 -> 66, sixteen rows) and lost at alpha 1.7 (48 ->
+// 51) and with the paper's scale (50 -> 53).  In longer sequences the code alone costs the scan 1 to 4 % at
 // head_dim 64 (16 x 32768 non-causal 2591 -> 2689) against 2 to 6 % gained at c = 1 and 8192 keys, also where only the items
 // without a sample (those that see fewer than kSampleMinKeys keys) take it: they have neither.
 constexpr int kLookRows = 4, kLookList = 32, kShortMinKeys = 1536;
@@ -1236,6 +1237,9 @@ cudaError_t launch_sweep(const Problem& p, const void* q, const void* k, const f
              : launch_impl<128, DUMP, ALIBI, SEARCH, SHORT>(p, q, k, args, stream))
   if (dump) return ENTMAX_SWEEP(true, false, true, false);
   if (mode != 0) return p.alibi ? ENTMAX_SWEEP(false, true, false, false) : ENTMAX_SWEEP(false, false, false, false);
+  // (slopes below kShortMinKeys: for the second look behind the diagonal tile.  Forward calls of 260 to 1024 keys, slopes on all
+  // heads, geometric mean over key order: 0.81 with it, 0.85 in the other instance.  That one, which has the sample, goes without
+  // it: its code cost 12 x 32768 x 64 1 to 2 %)
   if ((p.alibi || p.N >= kShortMinKeys) && p.N < kSampleMinKeys)
     return p.alibi ? ENTMAX_SWEEP(false, true, true, true) : ENTMAX_SWEEP(false, false, true, true);
   return p.alibi ? ENTMAX_SWEEP(false, true, true, false) : ENTMAX_SWEEP(false, false, true, false);
