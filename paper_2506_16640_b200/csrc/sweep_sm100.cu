@@ -176,8 +176,9 @@ __device__ __forceinline__ int first_tile(const SweepArgs& a, int k) {
 // Heads with a slope take their K tiles from the diagonal backwards when they search: the nearest keys have the smallest
 // penalty, so that the bound is good from the first tile on; in key order tile after tile brought new maxima (12 heads x 6000
 // x 64, alpha 2, half of the heads with slopes: 191 us in key order, 138 now).  A given threshold has no bound to gain (and 4
-// to 7 % to lose on 12 x 32768 x 64, slopes on all heads).  Nor has a head without slope, which backwards starts with a masked
-// tile: 12 x 2000 x 64 at alpha 1.25 and c = 1, where most rows are dense, 151 -> 173 us with every slope zero.
+// to 7 % to lose on 12 x 32768 x 64, slopes on all heads).  A head without slope has no such keys and starts, backwards, with a
+// masked tile: every slope zero, 12 x 2000 x 64 at alpha 1.25 and c = 1, where most rows are dense, 151 -> 173 us; 12 x 32768 x 64
+// with planted keys 1584 -> 1537.
 template <bool kAlibiSearch>
 __device__ __forceinline__ bool from_diagonal(const SweepArgs& a, int h) {
   if constexpr (kAlibiSearch) return a.dump[h] > 0.f;
